@@ -1,0 +1,722 @@
+// The drawing launch of a run at T > 0: one sweep over the vocabulary of every position that needs a token (residual
+// resample of Sec. 3.2, bonus token of Sec. 3.1), then the token itself.
+#ifndef COS_DRAW_CUH
+#define COS_DRAW_CUH
+
+#include "cos_common.cuh"
+
+namespace cosv {
+
+// A token's mass is max(0, sum_i k_i e_i / Z_i), e_i = 2^(x_i c - ref_i), where the channels i are the models (ensemble)
+// or the proposer's and the combined logits (logit level) and the k_i say what is drawn: max(0, r - q), r or q.  The set
+// of tokens with a positive mass is decided with the normalisers the streaming launch left (good to 1e-7; a token whose
+// sign that could change carries no mass to speak of), products rounded one by one so that equal terms cancel exactly.
+// Over that set the mass is linear in the 1/Z_i, so the sweep only adds up e_i over it, next to the refined normalisers.
+//
+// Split: a position is shared by p.draw_parts blocks, its steps (32 lanes x one 16-byte vector of every model) cut into
+// chunks of p.draw_cs; a warp takes consecutive chunks and leaves one record of sums for each, nothing per step.  The host
+// picks block size and parts so that the launch fills the device in one wave (see draw_plan).  The block that completes a
+// position (fence and counter, no waiting) adds its records up, finds the chunk that holds the token, then the step, then the token.
+constexpr int kMaxDrawThreads = 256;
+constexpr int kChunksKept = 4;  // chunks of a thread of the locating block whose masses it keeps in registers
+
+__device__ __forceinline__ double warp_sum(double t) {
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+  return t;
+}
+// Sums of N values over the warp at once: lane L ends up with the sum of value (L * N / 32).
+template <int N>
+__device__ __forceinline__ double warp_sums(double (&v)[N], int lane) {
+  int n = N;
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    const bool upper = (lane & d) != 0;
+    if (n > 1) {
+      n >>= 1;
+#pragma unroll
+      for (int i = 0; i < N / 2; ++i)
+        if (i < n) {
+          const double give = upper ? v[i] : v[i + n], keep = upper ? v[i + n] : v[i];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, give, d);
+        }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], d);
+    }
+  }
+  return v[0];
+}
+
+// What a block knows about its position.
+template <int NCH>
+struct DrawUnit {
+  const char* base;      // logits of model 0 at this position
+  int b, j, uidx;
+  int pis;               // model whose distribution is q
+  int law;               // kDrawResidual, kDrawR or kDrawQ
+  int emit;              // the token drawn here is the row's output (else only the residual mass is wanted)
+  int accepted;
+  float thr;             // plausibility threshold
+  float nref[NCH], bt[NCH], ct[NCH];  // minus the reference exponents, "big" bounds, k / Z in fp32
+};
+
+template <bool ENS>
+__device__ __forceinline__ double coefficient(const KParams& p, int i, int pis, int law) {  // k_i
+  if (ENS) {
+    const double sel = (i == pis) ? 1.0 : 0.0;
+    return i >= p.n ? 0.0 : (law == kDrawResidual ? p.w64[i] - sel : (law == kDrawQ ? sel : p.w64[i]));
+  }
+  return (i == 0) ? (law == kDrawResidual ? -1.0 : (law == kDrawQ ? 1.0 : 0.0)) : (law == kDrawQ ? 0.0 : 1.0);
+}
+
+// Position `u` of the launch; false when nothing is drawn there.  Same values in every thread.
+template <int DT, bool ENS, int NCH>
+__device__ __forceinline__ bool load_unit(const KParams& p, int u, DrawUnit<NCH>& d) {
+  if (!p.draw_all) {
+    d.b = u;
+    d.j = __ldcg(&p.row_draw[u]);
+    if (d.j < 0) return false;
+    d.emit = 1;
+  } else {
+    const int drafts = p.B * p.gamma;  // every draft position, then the bonus positions
+    d.b = u < drafts ? u / p.gamma : u - drafts;
+    d.j = u < drafts ? u % p.gamma : p.gamma;
+    d.emit = (__ldcg(&p.row_draw[d.b]) == d.j) ? 1 : 0;
+    if (d.j == p.gamma && !d.emit) return false;
+  }
+  d.uidx = d.b * p.P + d.j;
+  const UnitStats* st = &p.ustats[d.uidx];
+  const int4 res = __ldcg(&p.unit_res[d.uidx]);
+  if (!res.w) return false;
+  d.accepted = res.x;
+  const int pi = proposer_of(p, d.b, d.j);
+  d.pis = (pi >= 0 && pi < p.n) ? pi : 0;
+  d.law = (d.j == p.gamma) ? (p.bonus_model >= 0 ? kDrawQ : kDrawR) : kDrawResidual;
+  d.base = reinterpret_cast<const char*>(p.logits) +
+           (static_cast<long long>(d.b) * p.s_row + static_cast<long long>(d.j) * p.s_pos) * Elem<DT>::bytes;
+  d.thr = (!ENS && p.mask_model >= 0) ? __ldcg(&st->thr32) : -INFINITY;
+#pragma unroll
+  for (int i = 0; i < NCH; ++i) {
+    const bool live = i < (ENS ? p.n : 2);
+    const double z = live ? __ldcg(&st->s[i]) : 1.0;
+    d.nref[i] = live ? -__ldcg(&st->ref[i]) : 0.f;
+    d.bt[i] = live ? static_cast<float>(z * kBigShare) : INFINITY;
+    d.ct[i] = static_cast<float>(coefficient<ENS>(p, i, d.pis, d.law) / z);
+  }
+  return true;
+}
+
+// fp64 terms of one token from the stored logits: e_i of every channel.  Rare ("big" tokens, more than 2^-8 of a
+// normaliser, and the bonus token's probability); out of line.
+template <int DT, bool ENS, int NCH>
+__device__ __noinline__ void exact_terms(const KParams& p, const DrawUnit<NCH>& u, int e, double* out) {
+  float lv[COS_MAX_MODELS];
+  for (int i = 0; i < p.n; ++i) lv[i] = Elem<DT>::load1(u.base + i * p.s_model * Elem<DT>::bytes, e);
+  if (ENS) {
+#pragma unroll
+    for (int i = 0; i < NCH; ++i)
+      out[i] = (i < p.n) ? exp2(static_cast<double>(lv[i]) * p.cT64 + static_cast<double>(u.nref[i])) : 0.0;
+  } else {
+    double cd = 0.0;
+    for (int i = 0; i < p.n; ++i) cd = fma(p.w64[i], static_cast<double>(lv[i]), cd);
+    const bool in = p.mask_model < 0 || (lv[p.mask_model] >= u.thr);
+    out[0] = exp2(static_cast<double>(lv[u.pis]) * p.cT64 + static_cast<double>(u.nref[0]));
+    out[1] = in ? exp2(cd * p.cT64 + static_cast<double>(u.nref[1])) : 0.0;
+  }
+}
+
+// Mass of one token from its fp64 terms under the refined normalisers `inv` = 1 / Z_i.
+template <bool ENS, int NCH>
+__device__ __forceinline__ double exact_mass(const KParams& p, const double* e, const double* inv, int pis, int law) {
+  double r = 0.0, q = 0.0;
+  if (ENS) {
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      if (i < p.n) {
+        const double pr = e[i] * inv[i];
+        r += p.w64[i] * pr;
+        if (i == pis) q = pr;
+      }
+    }
+  } else {
+    q = e[0] * inv[0];
+    r = e[1] * inv[1];
+  }
+  return law == kDrawR ? r : (law == kDrawQ ? q : fmax(0.0, r - q));
+}
+
+// The arguments of the NCH channels for the E tokens of vector v (any vector of the row; -inf beyond V), one lane.
+template <int DT, bool ENS, int NCH, bool AL>
+__device__ __forceinline__ void vector_args(const KParams& p, const DrawUnit<NCH>& u, int v, float (&x)[NCH][Elem<DT>::E]) {
+  constexpr int E = Elem<DT>::E;
+  const VecRange whole = whole_vectors<DT, AL>(p.V);
+  const long long row_step = p.s_model * Elem<DT>::bytes;
+  if (ENS) {
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      uint4 r = neg_inf_vector<DT>();
+      if (i < p.n) r = load_vector<DT, AL>(u.base + i * row_step, v, p.V, whole);
+#pragma unroll
+      for (int k = 0; k < E; ++k) x[i][k] = entry<DT>(r, k);
+    }
+  } else {
+    auto row = [&](int i) { return load_vector<DT, AL>(u.base + i * row_step, v, p.V, whole); };
+    const uint4 r0 = row(0);
+    const uint4 r1 = p.n >= 2 ? row(1) : r0;
+    f32x2 xq[E / 2], cmb[E / 2];
+    const LogitWeights lw = logit_weights(p, u.pis, u.thr);
+    if (p.mask_model >= 0)
+      logit_args<DT, false, true>(p, lw, r0, r1, row, xq, cmb);
+    else
+      logit_args<DT, false, false>(p, lw, r0, r1, row, xq, cmb);
+#pragma unroll
+    for (int k = 0; k < E; ++k) {  // (beyond V the combination of -inf could be anything)
+      x[0][k] = pair_at(xq[k / 2], k);
+      x[1][k] = (v * E + k < p.V) ? pair_at(cmb[k / 2], k) : -INFINITY;
+    }
+  }
+}
+
+// One vector the fast loop left out, entry by entry: it holds a big entry (in fp64 then), or it is one of the ragged ends
+// of the row.  Its sums go to the thread's slots of `acc`.  Rare; out of line.
+template <int DT, bool ENS, int NCH, bool AL>
+__device__ __noinline__ void slow_vector(const KParams& p, const DrawUnit<NCH>& u, int v, double* acc) {
+  constexpr int E = Elem<DT>::E;
+  const int T = blockDim.x;
+  if (v * E >= p.V) return;
+  float x[NCH][E];
+  vector_args<DT, ENS, NCH, AL>(p, u, v, x);
+  float z[NCH], a[NCH];
+#pragma unroll
+  for (int i = 0; i < NCH; ++i) z[i] = a[i] = 0.f;
+#pragma unroll
+  for (int k = 0; k < E; ++k) {
+    float e[NCH], tot = 0.f;
+    bool big = false;
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      e[i] = ex2_approx(fmaf(x[i][k], p.cT, u.nref[i]));
+      big = big || e[i] > u.bt[i];
+      tot = __fadd_rn(tot, __fmul_rn(u.ct[i], e[i]));
+    }
+    if (big) {
+      double d[NCH], t64 = 0.0;
+      exact_terms<DT, ENS, NCH>(p, u, v * E + k, d);
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) t64 += static_cast<double>(u.ct[i]) * d[i];
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) {
+        acc[i * T] += d[i];
+        if (t64 > 0.0) acc[(NCH + i) * T] += d[i];
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) {
+        z[i] += e[i];
+        if (tot > 0.f) a[i] += e[i];
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NCH; ++i) {
+    acc[i * T] += static_cast<double>(z[i]);
+    acc[(NCH + i) * T] += static_cast<double>(a[i]);
+  }
+}
+
+// The chunks [c_lo, c_hi) of a position by one warp: per channel the normaliser's share and the sum over the tokens with a
+// positive mass, 2 NCH sums for every chunk at rec[chunk * 2 NCH].  The fast loop adds vectors up in fp32; vectors that need the
+// slow path it only remembers until the end of the strip (their sums, in fp64, in the thread's slots of `acc`).
+// What bounds it: loads in flight (two steps of every model at a time) and issue (about 17 instructions per pair of terms).
+// PAIR, MASKED: logit level with exactly two models, and with a mask.
+template <int DT, bool ENS, int NCH, bool AL, bool PAIR, bool MASKED>
+__device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawUnit<NCH>& u, int cs, int c_lo, int c_hi, double* acc,
+                                              double* rec) {
+  constexpr int E = Elem<DT>::E;
+  constexpr int NP = NCH / 2;
+  constexpr int NR = ENS ? NCH : 2;         // vectors of a step kept in registers
+  constexpr int US = (NR == 2) ? 2 : 1;     // steps fetched at a time
+  const int lane = threadIdx.x & 31;
+  const f32x2 c2 = pack2(p.cT, p.cT);
+  const VecRange whole = whole_vectors<DT, AL>(p.V);
+  const char* base = u.base;
+  const long long row_step = p.s_model * Elem<DT>::bytes;
+  f32x2 nref[NP], ct[NP];
+  float bt[NCH];
+#pragma unroll
+  for (int q = 0; q < NP; ++q) {
+    nref[q] = pack2(u.nref[2 * q], u.nref[2 * q + 1]);
+    ct[q] = pack2(u.ct[2 * q], u.ct[2 * q + 1]);
+    bt[2 * q] = u.bt[2 * q];
+    bt[2 * q + 1] = u.bt[2 * q + 1];
+  }
+  const LogitWeights lw = logit_weights(p, u.pis, u.thr);
+  for (int chunk = c_lo; chunk < c_hi; ++chunk) {
+    const int end = (chunk + 1) * cs < p.nsteps ? (chunk + 1) * cs : p.nsteps;
+    double sums[2 * NCH];
+    // in strips of 32 steps: a bit each in the slow-path mask
+    for (int c = chunk * cs; c < end; c += 32) {
+      const int ce = c + 32 < end ? c + 32 : end;
+      unsigned slow = 0u;
+      f32x2 zc[NP], ac[NP];
+#pragma unroll
+      for (int q = 0; q < NP; ++q) zc[q] = ac[q] = pack2(0.f, 0.f);
+      for (int s = c; s < ce; s += US) {
+        uint4 r[US][NR];
+#pragma unroll
+        for (int t = 0; t < US; ++t) {
+          const int v = (s + t) * 32 + lane;
+          const bool in = v >= whole.lo && v < whole.hi;
+#pragma unroll
+          for (int i = 0; i < NR; ++i) {
+            r[t][i] = neg_inf_vector<DT>();
+            if (in && s + t < ce && i < p.n) r[t][i] = load_whole<DT, AL>(base + i * row_step, v);
+          }
+          if (!in && s + t < ce) slow |= 1u << (s + t - c);
+        }
+#pragma unroll
+        for (int t = 0; t < US; ++t) {
+          f32x2 vz[NP], va[NP];
+#pragma unroll
+          for (int q = 0; q < NP; ++q) vz[q] = va[q] = pack2(0.f, 0.f);
+          if (ENS) {
+            // two channels side by side in every packed instruction
+#pragma unroll
+            for (int k = 0; k < E; ++k) {
+              f32x2 e[NP], m[NP];
+#pragma unroll
+              for (int q = 0; q < NP; ++q) {
+                const f32x2 arg = fma2(pack2(entry<DT>(r[t][2 * q], k), entry<DT>(r[t][2 * q + 1], k)), c2, nref[q]);
+                e[q] = pack2(ex2_approx(lo2(arg)), ex2_approx(hi2(arg)));
+                vz[q] = add2(vz[q], e[q]);
+                m[q] = mul2(ct[q], e[q]);
+              }
+              float tot = __fadd_rn(lo2(m[0]), hi2(m[0]));
+#pragma unroll
+              for (int q = 1; q < NP; ++q) tot = __fadd_rn(__fadd_rn(tot, lo2(m[q])), hi2(m[q]));
+#pragma unroll
+              for (int q = 0; q < NP; ++q) add2_if(va[q], e[q], tot);
+            }
+          } else {
+            // two neighbouring tokens side by side
+            f32x2 xq[E / 2], cmb[E / 2];
+            const int v = (s + t) * 32 + lane;
+            const bool in = v >= whole.lo && v < whole.hi && s + t < ce;
+            logit_args<DT, PAIR, MASKED>(p, lw, r[t][0], r[t][1],
+                                         [&](int i) {
+                                           uint4 m = neg_inf_vector<DT>();
+                                           if (in) m = load_whole<DT, AL>(base + i * row_step, v);
+                                           return m;
+                                         },
+                                         xq, cmb);
+            f32x2 zq = pack2(0.f, 0.f), zm = zq;
+            float aq = 0.f, am = 0.f;
+            const f32x2 nq = pack2(lo2(nref[0]), lo2(nref[0])), nm = pack2(hi2(nref[0]), hi2(nref[0]));
+            const f32x2 cq = pack2(-lo2(ct[0]), -lo2(ct[0])), cm = pack2(hi2(ct[0]), hi2(ct[0]));
+#pragma unroll
+            for (int k = 0; k < E / 2; ++k) {
+              const f32x2 tq = fma2(xq[k], c2, nq), tm = fma2(cmb[k], c2, nm);
+              const float q0 = ex2_approx(lo2(tq)), q1 = ex2_approx(hi2(tq)), m0 = ex2_approx(lo2(tm)), m1 = ex2_approx(hi2(tm));
+              const f32x2 eq = pack2(q0, q1), em = pack2(m0, m1);
+              zq = add2(zq, eq);
+              zm = add2(zm, em);
+              const f32x2 pq = mul2(cq, eq), pm = mul2(cm, em);
+              if (lo2(pm) > lo2(pq)) {
+                aq += q0;
+                am += m0;
+              }
+              if (hi2(pm) > hi2(pq)) {
+                aq += q1;
+                am += m1;
+              }
+            }
+            vz[0] = in ? pack2(lo2(zq) + hi2(zq), lo2(zm) + hi2(zm)) : pack2(0.f, 0.f);
+            va[0] = in ? pack2(aq, am) : pack2(0.f, 0.f);
+          }
+          // no term is negative, so a vector that holds a big entry has a big sum
+          bool big = false;
+#pragma unroll
+          for (int q = 0; q < NP; ++q) big = big || lo2(vz[q]) > bt[2 * q] || hi2(vz[q]) > bt[2 * q + 1];
+          if (big) {
+            slow |= 1u << (s + t - c);
+          } else {
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
+              zc[q] = add2(zc[q], vz[q]);
+              ac[q] = add2(ac[q], va[q]);
+            }
+          }
+        }
+      }
+      const int T = blockDim.x;
+      const bool more = c > chunk * cs;
+#pragma unroll
+      for (int q = 0; q < NP; ++q) {
+        sums[2 * q] = static_cast<double>(lo2(zc[q])) + (more ? acc[(2 * q) * T] : 0.0);
+        sums[2 * q + 1] = static_cast<double>(hi2(zc[q])) + (more ? acc[(2 * q + 1) * T] : 0.0);
+        sums[NCH + 2 * q] = static_cast<double>(lo2(ac[q])) + (more ? acc[(NCH + 2 * q) * T] : 0.0);
+        sums[NCH + 2 * q + 1] = static_cast<double>(hi2(ac[q])) + (more ? acc[(NCH + 2 * q + 1) * T] : 0.0);
+      }
+      if (slow || ce < end) {
+#pragma unroll
+        for (int q = 0; q < 2 * NCH; ++q) acc[q * T] = sums[q];
+        while (slow) {
+          const int k = __ffs(slow) - 1;
+          slow &= slow - 1;
+          slow_vector<DT, ENS, NCH, AL>(p, u, (c + k) * 32 + lane, acc);
+        }
+#pragma unroll
+        for (int q = 0; q < 2 * NCH; ++q) sums[q] = acc[q * T];
+      }
+    }
+    __syncwarp();
+    const double mine = warp_sums<2 * NCH>(sums, lane);
+    if (lane % (32 / (2 * NCH)) == 0) rec[static_cast<size_t>(chunk) * (2 * NCH) + lane / (32 / (2 * NCH))] = mine;
+  }
+}
+
+template <int DT, bool ENS, int NCH, bool AL>
+__device__ __forceinline__ void draw_sweep(const KParams& p, const DrawUnit<NCH>& u, int cs, int c_lo, int c_hi, double* acc,
+                                           double* rec) {
+  if (ENS) return draw_sweep_as<DT, ENS, NCH, AL, true, false>(p, u, cs, c_lo, c_hi, acc, rec);
+  if (p.n == 2 && p.mask_model < 0) return draw_sweep_as<DT, ENS, NCH, AL, true, false>(p, u, cs, c_lo, c_hi, acc, rec);
+  if (p.n == 2) return draw_sweep_as<DT, ENS, NCH, AL, true, true>(p, u, cs, c_lo, c_hi, acc, rec);
+  if (p.mask_model < 0) return draw_sweep_as<DT, ENS, NCH, AL, false, false>(p, u, cs, c_lo, c_hi, acc, rec);
+  draw_sweep_as<DT, ENS, NCH, AL, false, true>(p, u, cs, c_lo, c_hi, acc, rec);
+}
+
+// Masses of one lane's tokens of step s under the refined normalisers (coefficients cf = k / Z): small ones in fp32, big
+// ones in fp64; returns the lane's total (fp32 sum of the small ones in token order, then the big ones).
+template <int DT, bool ENS, int NCH, bool AL>
+__device__ __forceinline__ double step_masses(const KParams& p, const DrawUnit<NCH>& u, const float* cf, const double* inv,
+                                              int s, float (&m32)[Elem<DT>::E], unsigned& bigbits,
+                                              double (&mbig)[Elem<DT>::E]) {
+  constexpr int E = Elem<DT>::E;
+  const int v = s * 32 + (threadIdx.x & 31);
+  float x[NCH][E];
+  vector_args<DT, ENS, NCH, AL>(p, u, v, x);
+  bigbits = 0u;
+#pragma unroll
+  for (int k = 0; k < E; ++k) {
+    float tot = 0.f;
+    bool big = false;
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      const float e = ex2_approx(fmaf(x[i][k], p.cT, u.nref[i]));
+      big = big || e > u.bt[i];
+      tot = __fadd_rn(tot, __fmul_rn(cf[i], e));
+    }
+    m32[k] = big ? 0.f : fmaxf(0.f, tot);
+    bigbits |= big ? (1u << k) : 0u;
+    mbig[k] = 0.0;
+  }
+  float ls = 0.f;
+#pragma unroll
+  for (int k = 0; k < E; ++k) ls += m32[k];
+  double own = static_cast<double>(ls);
+  if (bigbits) {
+#pragma unroll
+    for (int k = 0; k < E; ++k)
+      if (bigbits & (1u << k)) {
+        double d[NCH];
+        exact_terms<DT, ENS, NCH>(p, u, v * E + k, d);
+        mbig[k] = exact_mass<ENS, NCH>(p, d, inv, u.pis, u.law);
+        own += mbig[k];
+      }
+  }
+  return own;
+}
+
+// The whole position again by one block, for another law.  Rare; out of line.
+template <int DT, bool ENS, int NCH, bool AL>
+__device__ __noinline__ void draw_sweep_again(const KParams& p, const DrawUnit<NCH>& u, double* acc, double* rec) {
+  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int c_lo = static_cast<int>(static_cast<long long>(p.draw_chunks) * warp / nw);
+  const int c_hi = static_cast<int>(static_cast<long long>(p.draw_chunks) * (warp + 1) / nw);
+  draw_sweep<DT, ENS, NCH, AL>(p, u, p.draw_cs, c_lo, c_hi, acc, rec);
+}
+
+// Shared memory of a block, in front of every thread's 2 NCH slots of the slow path.
+template <int NCH>
+struct DrawShared {
+  DrawUnit<NCH> unit;
+  double part[NCH][kMaxDrawThreads / 32];
+  double wmass[kMaxDrawThreads / 32];
+  double step_mass[32];
+  double base;      // mass before the winning chunk
+  int first, last;  // the winning chunk; the last chunk with mass
+  int go;
+};
+
+// A position whose records are all in: add them up, find the chunk, the step and the token.  Whole block.
+template <int DT, bool ENS, int NCH, bool AL>
+__device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, double* acc, double* rec) {
+  constexpr int E = Elem<DT>::E;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int live = ENS ? p.n : 2;
+  DrawUnit<NCH>& u = sh.unit;
+  const int nch = p.draw_chunks, cs = p.draw_cs;
+  const int per = (nch + blockDim.x - 1) / blockDim.x;  // consecutive chunks of a thread
+  unsigned rnd[4];
+  philox4x32_10(static_cast<unsigned>(p.row_base + u.b), static_cast<unsigned>(u.j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
+  for (int pass = 0; pass < 2; ++pass) {
+    double z[NCH], a[kChunksKept][NCH];
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) z[i] = 0.0;
+    const int c_lo = tid * per, c_hi = c_lo + per < nch ? c_lo + per : nch;
+#pragma unroll
+    for (int q = 0; q < kChunksKept; ++q) {
+      const double* r = rec + static_cast<size_t>(c_lo + q) * (2 * NCH);
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) {
+        a[q][i] = 0.0;
+        if (c_lo + q < c_hi) {
+          z[i] += __ldcg(r + i);
+          a[q][i] = __ldcg(r + NCH + i);
+        }
+      }
+    }
+    for (int c = c_lo + kChunksKept; c < c_hi; ++c)
+      for (int i = 0; i < NCH; ++i) z[i] += __ldcg(rec + static_cast<size_t>(c) * (2 * NCH) + i);
+    {
+      double t[NCH];
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) t[i] = z[i];
+      const double mine = warp_sums<NCH>(t, lane);
+      if (lane % (32 / NCH) == 0) sh.part[lane / (32 / NCH)][warp] = mine;
+    }
+    if (tid == 0) {
+      sh.first = 0x7fffffff;
+      sh.last = -1;
+    }
+    __syncthreads();
+    double inv[NCH], c64[NCH], mass[kChunksKept], mine = 0.0;
+    float cf[NCH];
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      double t = 0.0;
+      for (int w = 0; w < nw; ++w) t += sh.part[i][w];
+      inv[i] = i < live ? 1.0 / t : 0.0;
+      c64[i] = i < live ? coefficient<ENS>(p, i, u.pis, u.law) * inv[i] : 0.0;
+      cf[i] = static_cast<float>(c64[i]);
+    }
+    auto mass_of = [&](const double* w) -> double {  // (products rounded one by one: equal sums under opposite coefficients cancel)
+      double m = __dmul_rn(c64[0], w[0]);
+#pragma unroll
+      for (int i = 1; i < NCH; ++i) m = __dadd_rn(m, __dmul_rn(c64[i], w[i]));
+      return fmax(0.0, m);
+    };
+#pragma unroll
+    for (int q = 0; q < kChunksKept; ++q) {
+      mass[q] = mass_of(a[q]);
+      mine += mass[q];
+    }
+    for (int c = c_lo + kChunksKept; c < c_hi; ++c) mine += mass_of(rec + static_cast<size_t>(c) * (2 * NCH) + NCH);
+    double incl = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const double o = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += o;
+    }
+    if (lane == 31) sh.wmass[warp] = incl;
+    __syncthreads();
+    double before = 0.0, S = 0.0;
+    for (int w = 0; w < nw; ++w) {
+      if (w == warp) before = S;
+      S += sh.wmass[w];
+    }
+    before += incl - mine;
+    const double target = word_to_uniform(rnd[1]) * S;
+    if (pass == 0 && tid == 0 && p.diag && u.j != p.gamma) p.diag[static_cast<long long>(u.uidx) * 4 + 3] = static_cast<float>(S);
+    if (!u.emit) return;
+    // the first chunk whose running total reaches the target; where rounding leaves none, the last chunk with mass
+    int first = -1, last = -1;
+    double first_base = 0.0, last_base = 0.0;
+    auto look = [&](int c, double m) {
+      if (m > 0.0) {
+        last = c;
+        last_base = before;
+        if (first < 0 && before + m >= target) {
+          first = c;
+          first_base = before;
+        }
+      }
+      before += m;
+    };
+#pragma unroll
+    for (int q = 0; q < kChunksKept; ++q) look(c_lo + q, mass[q]);
+    for (int c = c_lo + kChunksKept; c < c_hi; ++c) look(c, mass_of(rec + static_cast<size_t>(c) * (2 * NCH) + NCH));
+    if (first >= 0) atomicMin(&sh.first, first);
+    if (last >= 0) atomicMax(&sh.last, last);
+    __syncthreads();
+    const bool hit = sh.first != 0x7fffffff;
+    const int win = hit ? sh.first : sh.last;
+    if (win < 0 || !(S > 0.0)) {
+      // no residual mass although a token is needed: this block draws from r instead, over the whole position
+      if (u.law != kDrawResidual) return;
+      __syncthreads();
+      if (tid == 0) {
+        if (!u.accepted) atomicOr(&p.row_status[u.b], static_cast<unsigned>(COS_ROW_RESIDUAL_EMPTY));
+        u.law = kDrawR;
+#pragma unroll
+        for (int i = 0; i < NCH; ++i)
+          u.ct[i] = static_cast<float>(coefficient<ENS>(p, i, u.pis, kDrawR) / (i < live ? __ldcg(&p.ustats[u.uidx].s[i]) : 1.0));
+      }
+      __syncthreads();
+      draw_sweep_again<DT, ENS, NCH, AL>(p, u, acc, rec);
+      __syncthreads();
+      continue;
+    }
+    if ((hit ? first : last) == win) sh.base = hit ? first_base : last_base;
+    // the steps of that chunk, dealt out over the warps in up to 32 records of `gsz` steps (one step, nearly always)
+    const int s0 = win * cs, s1 = s0 + cs < p.nsteps ? s0 + cs : p.nsteps, gsz = (cs + 31) / 32;
+    float m32[E];
+    unsigned bigbits = 0u;
+    double mbig[E], own = 0.0;
+    int held = -1;  // the step whose masses the lanes of this warp hold
+#pragma unroll 1
+    for (int t = warp; s0 + t * gsz < s1; t += nw) {
+      double rm = 0.0;
+#pragma unroll 1
+      for (int s = s0 + t * gsz; s < s0 + (t + 1) * gsz && s < s1; ++s) {
+        own = step_masses<DT, ENS, NCH, AL>(p, u, cf, inv, s, m32, bigbits, mbig);
+        rm += warp_sum(own);
+        held = s;
+      }
+      if (lane == 0) sh.step_mass[t] = rm;
+    }
+    __syncthreads();
+    const double v = (s0 + lane * gsz < s1) ? sh.step_mass[lane] : 0.0;
+    double inc = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const double o = __shfl_up_sync(0xffffffffu, inc, d);
+      if (lane >= d) inc += o;
+    }
+    const double base = sh.base;
+    const unsigned ok = __ballot_sync(0xffffffffu, v > 0.0 && base + inc >= target), pos = __ballot_sync(0xffffffffu, v > 0.0);
+    if (pos == 0u) return;
+    const int k = ok ? __ffs(ok) - 1 : 31 - __clz(pos);  // rounding corner: the last record with mass
+    if (k % nw != warp) return;
+    double at = base + __shfl_sync(0xffffffffu, inc - v, k);
+    // one warp goes on: the record's steps in order, an fp64 prefix over the lanes, then the lane's tokens
+    int token = -1, last_tok = -1;
+#pragma unroll 1
+    for (int s = s0 + k * gsz; s < s0 + (k + 1) * gsz && s < s1 && token < 0; ++s) {
+      if (s != held) own = step_masses<DT, ENS, NCH, AL>(p, u, cf, inv, s, m32, bigbits, mbig);
+      held = s;
+      double in = own;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const double o = __shfl_up_sync(0xffffffffu, in, d);
+        if (lane >= d) in += o;
+      }
+      const unsigned lok = __ballot_sync(0xffffffffu, own > 0.0 && at + in >= target), lpos = __ballot_sync(0xffffffffu, own > 0.0);
+      double part = at + (in - own);
+      int found = -1, lastk = -1;
+#pragma unroll
+      for (int q = 0; q < E; ++q) {
+        const double mk = (bigbits & (1u << q)) ? mbig[q] : static_cast<double>(m32[q]);
+        part += mk;
+        if (mk > 0.0) {
+          lastk = (s * 32 + lane) * E + q;
+          if (found < 0 && part >= target) found = lastk;
+        }
+      }
+      if (found < 0) found = lastk;
+      if (lok) token = __shfl_sync(0xffffffffu, found, __ffs(lok) - 1);
+      if (lpos) last_tok = __shfl_sync(0xffffffffu, lastk, 31 - __clz(lpos));
+      at += __shfl_sync(0xffffffffu, in, 31);
+    }
+    if (token < 0) token = last_tok;
+    if (lane == 0 && token >= 0) {
+      p.out_tokens[u.uidx] = token;
+      // Algorithm 2's Score returns the bonus token with its probability under the law it came from
+      if (u.j == p.gamma && p.bonus_prob != nullptr) {
+        double d[NCH];
+        exact_terms<DT, ENS, NCH>(p, u, token, d);
+        p.bonus_prob[u.b] = static_cast<float>(exact_mass<ENS, NCH>(p, d, inv, u.pis, u.law));
+      }
+    }
+    return;
+  }
+}
+
+// PHASE 0: everything in one launch.  1 and 2: the sweep and the rest as two launches (one block per position in the second).
+template <int DT, bool ENS, int NCH, bool AL, int PHASE>
+__global__ void __launch_bounds__(kMaxDrawThreads, NCH == 2 ? 4 : 2) cos_draw_kernel(const __grid_constant__ KParams p) {
+  extern __shared__ __align__(16) unsigned char draw_smem_raw[];
+  DrawShared<NCH>& sh = *reinterpret_cast<DrawShared<NCH>*>(draw_smem_raw);
+  double* acc = reinterpret_cast<double*>(draw_smem_raw + sizeof(DrawShared<NCH>)) + threadIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int parts = PHASE == 2 ? 1 : p.draw_parts;
+  const int slot = blockIdx.x / parts, part = blockIdx.x % parts;
+  // launched while the kernel before it drains; nothing is read or written before that one is complete
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (PHASE == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  {
+    DrawUnit<NCH> d;
+    if (!load_unit<DT, ENS, NCH>(p, slot, d)) return;
+    if (tid == 0) sh.unit = d;
+  }
+  __syncthreads();
+  double* rec = p.draw_rec + static_cast<size_t>(slot) * p.draw_chunks * (2 * NCH);
+  if (PHASE != 2) {
+    const int w = part * nw + warp, W = parts * nw;
+    const int c_lo = static_cast<int>(static_cast<long long>(p.draw_chunks) * w / W);
+    const int c_hi = static_cast<int>(static_cast<long long>(p.draw_chunks) * (w + 1) / W);
+    draw_sweep<DT, ENS, NCH, AL>(p, sh.unit, p.draw_cs, c_lo, c_hi, acc, rec);
+    if (PHASE == 1) return;
+    __syncthreads();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (parts > 1) {
+      // the last block of the position to get here goes on
+      if (tid == 0) {
+        __threadfence();
+        const int prev = atomicAdd(&p.draw_arrivals[slot], 1);
+        if (prev == parts - 1) {
+          __threadfence();             // what the other blocks wrote before they reported is visible from here on
+          p.draw_arrivals[slot] = 0;   // ready for the next run (a later launch: nothing waits for this store)
+        }
+        sh.go = (prev == parts - 1) ? 1 : 0;
+      }
+      __syncthreads();
+      if (!sh.go) return;
+    }
+  }
+  locate<DT, ENS, NCH, AL>(p, sh, acc, rec);
+}
+
+// Test hook: the combined distribution of every position, token by token, from the statistics the streaming launch left.
+template <int DT>
+__global__ void __launch_bounds__(256) cos_dump_kernel(const __grid_constant__ KParams p, bool ens) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int uidx = blockIdx.y, b = uidx / p.P, j = uidx % p.P;
+  const UnitStats* st = &p.ustats[uidx];
+  if (!p.unit_res[uidx].w) return;
+  const char* base = reinterpret_cast<const char*>(p.logits) +
+                     (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
+  float* out = p.dump_r + static_cast<long long>(uidx) * p.V;
+  const long long row_step = p.s_model * Elem<DT>::bytes;
+  for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < p.V; x += gridDim.x * blockDim.x) {
+    float r = 0.f;
+    if (ens) {
+      for (int i = 0; i < p.n; ++i)
+        r = fmaf(static_cast<float>(p.w64[i] / st->s[i]), ex2_approx(fmaf(Elem<DT>::load1(base + i * row_step, x), p.cT, -st->ref[i])), r);
+    } else {
+      float cmb = 0.f;
+      bool in = true;
+      for (int i = 0; i < p.n; ++i) {
+        const float l = Elem<DT>::load1(base + i * row_step, x);
+        cmb = fmaf(p.w[i], l, cmb);
+        if (i == p.mask_model) in = l >= st->thr32;
+      }
+      r = in ? ex2_approx(fmaf(cmb, p.cT, -st->ref[1])) * static_cast<float>(1.0 / st->s[1]) : 0.f;
+    }
+    out[x] = r;
+  }
+}
+
+}  // namespace cosv
+
+#endif  // COS_DRAW_CUH
