@@ -1,0 +1,80 @@
+// The launches of one element type (each is compiled in a unit of its own: cos_bf16.cu, cos_f16.cu, cos_f32.cu).
+#ifndef COS_LAUNCH_CUH
+#define COS_LAUNCH_CUH
+
+#include "cos_draw.cuh"
+#include "cos_launch.h"
+#include "cos_stream.cuh"
+
+namespace cosv {
+
+using KernelFn = void (*)(const KParams);
+
+template <int DT, bool AL>
+KernelFn draw_kernel_of(bool ens, int channels, int phase) {
+  if (!ens) return cos_draw_kernel<DT, false, 2, AL, 0>;
+  if (channels == 2)
+    return phase == 0 ? cos_draw_kernel<DT, true, 2, AL, 0> : (phase == 1 ? cos_draw_kernel<DT, true, 2, AL, 1> : cos_draw_kernel<DT, true, 2, AL, 2>);
+  if (channels == 4) return cos_draw_kernel<DT, true, 4, AL, 0>;
+  return phase == 1 ? cos_draw_kernel<DT, true, 8, AL, 1> : cos_draw_kernel<DT, true, 8, AL, 2>;
+}
+
+template <int DT, bool AL>
+KernelFn stream_kernel_of(int mode) {
+  switch (mode) {
+    case kEnsembleSample: return cos_stream_kernel<DT, kEnsembleSample, AL>;
+    case kLogitSample: return cos_stream_kernel<DT, kLogitSample, AL>;
+    case kEnsembleGreedy: return cos_stream_kernel<DT, kEnsembleGreedy, AL>;
+    default: return cos_stream_kernel<DT, kLogitGreedy, AL>;
+  }
+}
+
+// Every launch carries the programmatic-stream-serialisation attribute: its blocks take their places while the kernel
+// before it drains, and wait for it before they touch anything.
+inline cudaError_t launch(KernelFn fn, const KParams& p, int blocks, int threads, size_t smem, cudaStream_t stream) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
+  lc.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, fn, p);
+}
+
+template <int DT>
+cudaError_t stream_launch(const KParams& p, int mode, int threads, cudaStream_t stream) {
+  const int blocks = (p.st_workers + threads / 32 - 1) / (threads / 32);
+  return launch(p.vec_ok ? stream_kernel_of<DT, true>(mode) : stream_kernel_of<DT, false>(mode), p, blocks, threads, 0, stream);
+}
+
+template <int DT>
+cudaError_t mask_launch(const KParams& p, int threads, cudaStream_t stream) {
+  const int blocks = (p.st_workers + threads / 32 - 1) / (threads / 32);
+  return launch(p.vec_ok ? cos_mask_kernel<DT, true> : cos_mask_kernel<DT, false>, p, blocks, threads, 0, stream);
+}
+
+template <int DT>
+cudaError_t draw_launch(const KParams& p, bool ens, int channels, int phase, int units, int threads, cudaStream_t stream) {
+  KernelFn fn = p.vec_ok ? draw_kernel_of<DT, true>(ens, channels, phase) : draw_kernel_of<DT, false>(ens, channels, phase);
+  const size_t fixed = channels == 2 ? sizeof(DrawShared<2>) : (channels == 4 ? sizeof(DrawShared<4>) : sizeof(DrawShared<8>));
+  static_assert(sizeof(DrawShared<8>) + 16 * kMaxDrawThreads * sizeof(double) <= 48 * 1024, "no opt-in for large shared memory is made");
+  return launch(fn, p, phase == 2 ? units : units * p.draw_parts, threads, fixed + 2 * channels * threads * sizeof(double), stream);
+}
+
+template <int DT>
+cudaError_t dump_launch(const KParams& p, int mode, cudaStream_t stream) {
+  const dim3 grid(64, static_cast<unsigned>(p.num_units), 1);
+  if (mode == kEnsembleSample || mode == kLogitSample)
+    cos_dump_kernel<DT><<<grid, 256, 0, stream>>>(p, mode == kEnsembleSample);
+  else
+    cos_dump_atoms_kernel<DT><<<grid, 256, 0, stream>>>(p);
+  return cudaGetLastError();
+}
+
+}  // namespace cosv
+
+#endif  // COS_LAUNCH_CUH

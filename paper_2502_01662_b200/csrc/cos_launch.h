@@ -1,0 +1,27 @@
+// Internal interface between the translation units of the library: the launches of a run, one unit per element type.
+#ifndef COS_LAUNCH_H
+#define COS_LAUNCH_H
+
+#include <cuda_runtime.h>
+
+#include "cos_common.cuh"
+
+namespace cosv {
+
+// The streaming launch (mode: the Mode enum): a warp for each of the p.st_workers shares, blocks of `threads` threads.  mask:
+// the launch before it that finds the plausibility threshold of every position.
+template <int DT>
+cudaError_t stream_launch(const KParams& p, int mode, int threads, cudaStream_t stream);
+template <int DT>
+cudaError_t mask_launch(const KParams& p, int threads, cudaStream_t stream);
+// The drawing launch with `channels` 2, 4 or 8 (logit level: 2) for `units` positions, blocks of `threads` threads: `phase` 0
+// for one launch, 1 and 2 for the two launches of the split form.
+template <int DT>
+cudaError_t draw_launch(const KParams& p, bool ensemble, int channels, int phase, int units, int threads, cudaStream_t stream);
+// Test hook: the combined distribution of every position.
+template <int DT>
+cudaError_t dump_launch(const KParams& p, int mode, cudaStream_t stream);
+
+}  // namespace cosv
+
+#endif  // COS_LAUNCH_H

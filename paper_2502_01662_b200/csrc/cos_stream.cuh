@@ -1,0 +1,1021 @@
+// The streaming launch of a run: every logit is read once (Eq. 3-5), every position decided (Eq. 6), every row scanned for
+// its first rejection (Sec. 3.1).
+#ifndef COS_STREAM_CUH
+#define COS_STREAM_CUH
+
+#include "cos_common.cuh"
+
+namespace cosv {
+
+// Split: the rows of 16-byte vectors (ensembles: every model's row of every position; logit level: the vectors of all models
+// of a position go together) form one line in the order of memory, cut into p.st_workers equal contiguous shares, one for each
+// warp of a single wave of blocks, whatever the rows' boundaries.  So every warp streams the same number of bytes for any batch
+// and vocabulary, with 4 KB in flight, and nothing but loads between the start and the end of its share.  A warp leaves one
+// record (partial softmax statistics or argmaxes) for every row it had a part of; the warp that completes a position (fence
+// and counter, no waiting) merges its records in order, takes the decision and publishes it.
+// Measured on 1152 rows of 151936 bf16 entries (350 MB): 57.4 us (6.1 TB/s) for the sweep alone; whole positions per block of 16
+// warps, as before, 65 to 70 us; shares of blocks instead of warps 65 us; 4 vectors in flight per lane 68 us; the line in
+// another order than memory's (position by position over the batch) 78 us: neighbouring warps then read far apart.
+constexpr int kStreamThreads = 512;  // (two blocks per multiprocessor: 64 registers)
+constexpr int kStreamDepth = 8;      // vectors in flight per lane
+constexpr int kSkipped = 1 << 16;    // a warp that left its part of a position unread (early exit)
+
+struct Decision {  // one position's outcome
+  int accept, status, cand;
+  int natoms, drawable;
+  int atom_tok[COS_MAX_MODELS];
+  double atom_mass[COS_MAX_MODELS];
+  double ratio, r_d, q_d, S;
+  double prob;  // greedy, bonus position: probability of cand under the law it came from
+};
+
+struct Finish {  // what the warp that completes a position works with
+  SoftPart fsoft[COS_MAX_MODELS];  // merged statistics
+  ArgPart farg[COS_MAX_MODELS];
+  double pdraft[COS_MAX_MODELS];   // probability of the draft token under each softmax
+  float ldraft[COS_MAX_MODELS];    // the n logits at the draft token
+  Decision dec;
+};
+
+// A worker's share of the line, in vectors: shares are whole multiples of eight vectors (128 bytes) of the line.
+__device__ __forceinline__ long long worker_lo(const KParams& p, int w) {
+  const long long at = (w * p.st_q + (w < p.st_rem ? w : p.st_rem)) * 8;
+  return at < p.st_line ? at : p.st_line;
+}
+__device__ __forceinline__ int worker_of(const KParams& p, long long x) {
+  const long long x8 = x >> 3, wide = p.st_rem * (p.st_q + 1);
+  return static_cast<int>(x8 < wide ? x8 / (p.st_q + 1) : p.st_rem + (x8 - wide) / p.st_q);
+}
+
+// Entries of a row that are not part of its whole vectors: [0, head) and [tail, V), fewer than three vectors in all.
+struct Ragged {
+  int head, tail;
+};
+template <int DT, bool AL>
+__device__ __forceinline__ Ragged ragged_of(int V) {
+  const VecRange w = whole_vectors<DT, AL>(V);
+  Ragged r;
+  r.head = w.hi > w.lo ? w.lo * Elem<DT>::E : 0;
+  r.tail = w.hi > w.lo ? w.hi * Elem<DT>::E : 0;
+  return r;
+}
+// The lane's entry of them, or -1.
+__device__ __forceinline__ int ragged_entry(const Ragged& r, int V, int lane) {
+  const int e = lane < r.head ? lane : r.tail + lane - r.head;
+  return e < V ? e : -1;
+}
+
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+template <int DT>
+__device__ __forceinline__ unsigned max2_nan(unsigned a, unsigned b) {
+  unsigned d;
+  if (DT == COS_DTYPE_BF16)
+    asm("max.NaN.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  else
+    asm("max.NaN.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+// The largest entry of a vector, NaN if there is one; MAG: the largest magnitude.
+template <int DT, bool MAG>
+__device__ __forceinline__ float vector_max(const uint4& r) {
+  if (DT == COS_DTYPE_F32) {
+    const float a = __uint_as_float(r.x), b = __uint_as_float(r.y), c = __uint_as_float(r.z), d = __uint_as_float(r.w);
+    return MAG ? max_nan(max_nan(fabsf(a), fabsf(b)), max_nan(fabsf(c), fabsf(d))) : max_nan(max_nan(a, b), max_nan(c, d));
+  }
+  const unsigned k = MAG ? 0x7fff7fffu : 0xffffffffu;
+  const unsigned m = max2_nan<DT>(max2_nan<DT>(r.x & k, r.y & k), max2_nan<DT>(r.z & k, r.w & k));
+  const uint4 q = make_uint4(m, 0u, 0u, 0u);
+  return max_nan(entry<DT>(q, 0), entry<DT>(q, 1));
+}
+
+// Sums of a lane, two at a time: a few vectors plainly, then compensated (Kahan), every operation one packed instruction; so
+// a share may be thousands of vectors long and its sum is as good as a short one's.
+struct Comp2 {
+  f32x2 sum, nc;  // running sum, minus the compensation
+  __device__ __forceinline__ void init() { sum = nc = pack2(0.f, 0.f); }
+  __device__ __forceinline__ void add(f32x2 v) {
+    const f32x2 y = add2(v, nc);
+    const f32x2 t = add2(sum, y);
+    nc = add2(y, fma2(t, pack2(-1.f, -1.f), sum));
+    sum = t;
+  }
+  __device__ __forceinline__ float total() const { return (lo2(sum) + hi2(sum)) + (lo2(nc) + hi2(nc)); }
+};
+
+// Reference exponent of a lane's sum: fixed, from its first vector, a whole number (sums with such references rescale exactly).
+__device__ __forceinline__ float seed_ref(float vmax, float c) {
+  const float cand = vmax * c;
+  return (fabsf(cand) < INFINITY) ? floorf(cand) : 0.f;
+}
+
+// sum of 2^(x c + nref) over one vector, in two halves
+template <int DT>
+__device__ __forceinline__ f32x2 vector_sum(const uint4& r, f32x2 c2, f32x2 nref2) {
+  constexpr int H = Elem<DT>::E / 2;
+  f32x2 x[H], s;
+  unpack_pairs<DT>(r, x);
+#pragma unroll
+  for (int k = 0; k < H; ++k) {
+    const f32x2 t = fma2(x[k], c2, nref2);
+    const f32x2 e = pack2(ex2_approx(lo2(t)), ex2_approx(hi2(t)));
+    s = k == 0 ? e : add2(s, e);
+  }
+  return s;
+}
+
+// The same segment with a running maximum, for the lane whose fixed reference overflowed or met a non-finite input.  Rare.
+template <int DT, bool AL>
+__device__ __noinline__ LaneSoft soft_online(const char* row, int v, int v1, float c) {
+  LaneSoft acc;
+  acc.init();
+  for (; v < v1; v += 32) {
+    float x[Elem<DT>::E];
+    Elem<DT>::unpack(load_whole<DT, AL>(row, v), x);
+    acc.add_online(x, c);
+  }
+  return acc;
+}
+
+// Softmax statistics of vectors [v0, v1) of one row and, with `ragged`, of its ragged entries; every lane's own part.
+// (Out of line, like the other segments, so that its loop has the registers to itself.)
+template <int DT, bool AL>
+__device__ __noinline__ LaneSoft soft_segment(const char* row, int v0, int v1, bool ragged, int V, float c) {
+  constexpr int U = kStreamDepth;
+  const int lane = threadIdx.x & 31;
+  const f32x2 c2 = pack2(c, c);
+  LaneSoft acc;
+  acc.init();
+  int v = v0 + lane;
+  if (v < v1) {
+    uint4 raw[U];
+    Comp2 total;
+    total.init();
+    f32x2 nref2 = pack2(0.f, 0.f);
+    bool first = true;
+    for (; v < v1; v += U * 32) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        raw[u] = neg_inf_vector<DT>();
+        if (v + u * 32 < v1) raw[u] = load_whole<DT, AL>(row, v + u * 32);
+      }
+      if (first) {
+        acc.ref = seed_ref(vector_max<DT, false>(raw[0]), c);
+        nref2 = pack2(-acc.ref, -acc.ref);
+        first = false;
+      }
+      f32x2 s = vector_sum<DT>(raw[0], c2, nref2);
+#pragma unroll
+      for (int u = 1; u < U; ++u) s = add2(s, vector_sum<DT>(raw[u], c2, nref2));
+      total.add(s);
+    }
+    acc.s = total.total();
+    if (!(acc.s < INFINITY)) acc = soft_online<DT, AL>(row, v0 + lane, v1, c);
+  }
+  if (ragged) {
+    const int e = ragged_entry(ragged_of<DT, AL>(V), V, lane);
+    if (e >= 0) acc.add_online1(Elem<DT>::load1(row, e), c);
+  }
+  return acc;
+}
+
+// Argmax of vectors [v0, v1) of one row (lowest index among equals) and whether a NaN or +inf was seen; the warp's result.
+template <int DT, bool AL>
+__device__ __noinline__ ArgPart arg_segment(const char* row, int v0, int v1, bool ragged, int V) {
+  constexpr int U = kStreamDepth, E = Elem<DT>::E;
+  const int lane = threadIdx.x & 31;
+  float best = -INFINITY;  // (sticks at NaN)
+  int bestv = -1;
+  for (int v = v0 + lane; v < v1; v += U * 32) {
+    uint4 raw[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      raw[u] = neg_inf_vector<DT>();
+      if (v + u * 32 < v1) raw[u] = load_whole<DT, AL>(row, v + u * 32);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float m = vector_max<DT, false>(raw[u]);
+      if (m > best) bestv = v + u * 32;
+      best = max_nan(best, m);
+    }
+  }
+  int idx = kNoReject, bad = !(best < INFINITY);
+  if (bestv >= 0) {
+    const uint4 r = load_whole<DT, AL>(row, bestv);
+#pragma unroll
+    for (int k = E - 1; k >= 0; --k)
+      if (entry<DT>(r, k) == best) idx = bestv * E + k;
+  }
+  if (ragged) {
+    const int e = ragged_entry(ragged_of<DT, AL>(V), V, lane);
+    if (e >= 0) {
+      const float x = Elem<DT>::load1(row, e);
+      bad |= !(x < INFINITY);
+      if (arg_better(x, e, best, idx)) {
+        best = x;
+        idx = e;
+      }
+    }
+  }
+  return warp_reduce_arg(static_cast<double>(best), idx, bad, lane);
+}
+
+struct LaneSoft2 {
+  LaneSoft q, c;
+};
+// Tokens [e, end) one by one, running maximum: the ragged ends, and everything where a sum overflowed or met a non-finite input.
+template <int DT>
+__device__ __noinline__ LaneSoft2 logit_online(const KParams& p, const char* base, int pis, float thr, int e, int end, LaneSoft2 a) {
+  for (; e < end; ++e) {
+    float cmb = 0.f, xq = -INFINITY, xe = 0.f;
+    for (int i = 0; i < p.n; ++i) {
+      const float x = Elem<DT>::load1(base + i * p.s_model * Elem<DT>::bytes, e);
+      cmb = fmaf(p.w[i], x, cmb);
+      if (i == pis) xq = x;
+      if (i == p.mask_model) xe = x;
+    }
+    if (p.mask_model >= 0 && !(xe >= thr)) cmb = -INFINITY;
+    a.q.add_online1(xq, p.cT);
+    a.c.add_online1(cmb, p.cT);
+  }
+  return a;
+}
+
+// Softmax statistics of the proposer's logits and of the combined ones over vectors [v0, v1) of a position, four vectors of
+// the first two models in flight (further models are read as they are needed).
+// PAIR: exactly two models; MASKED: with the plausibility mask.
+template <int DT, bool AL, bool PAIR, bool MASKED>
+__device__ __noinline__ LaneSoft2 logit_segment(const KParams& p, const char* base, long long row_step, LogitWeights lw, float cT,
+                                                int v0, int v1, bool ragged) {
+  constexpr int U = kStreamDepth / 2, H = Elem<DT>::E / 2;
+  const int lane = threadIdx.x & 31;
+  const bool pair = PAIR || p.n >= 2;
+  const f32x2 c2 = pack2(cT, cT);
+  LaneSoft2 acc;
+  LaneSoft &accq = acc.q, &accc = acc.c;
+  accq.init();
+  accc.init();
+  int v = v0 + lane;
+  if (v < v1) {
+    Comp2 tq, tc;
+    tq.init();
+    tc.init();
+    f32x2 nq = pack2(0.f, 0.f), nc = nq;
+    bool first = true;
+    for (; v < v1; v += U * 32) {
+      uint4 r0[U], r1[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        r0[u] = r1[u] = neg_inf_vector<DT>();
+        if (v + u * 32 < v1) {
+          r0[u] = load_whole<DT, AL>(base, v + u * 32);
+          if (pair) r1[u] = load_whole<DT, AL>(base + row_step, v + u * 32);
+        }
+      }
+      f32x2 sq = pack2(0.f, 0.f), sc = sq;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        f32x2 xq[H], cmb[H];
+        const bool in = u == 0 || v + u * 32 < v1;
+        logit_args<DT, PAIR, MASKED>(p, lw, r0[u], r1[u],
+                                     [&](int i) {
+                                       uint4 r = neg_inf_vector<DT>();
+                                       if (in) r = load_whole<DT, AL>(base + i * row_step, v + u * 32);
+                                       return r;
+                                     },
+                                     xq, cmb);
+        if (u == 0 && first) {
+          float mq = -INFINITY, mc = -INFINITY;
+#pragma unroll
+          for (int k = 0; k < H; ++k) {
+            mq = fmaxf(mq, fmaxf(lo2(xq[k]), hi2(xq[k])));
+            mc = fmaxf(mc, fmaxf(lo2(cmb[k]), hi2(cmb[k])));
+          }
+          accq.ref = seed_ref(mq, cT);
+          accc.ref = seed_ref(mc, cT);
+          nq = pack2(-accq.ref, -accq.ref);
+          nc = pack2(-accc.ref, -accc.ref);
+          first = false;
+        }
+        f32x2 vq = pack2(0.f, 0.f), vc = vq;
+#pragma unroll
+        for (int k = 0; k < H; ++k) {
+          const f32x2 aq = fma2(xq[k], c2, nq), ac = fma2(cmb[k], c2, nc);
+          vq = add2(vq, pack2(ex2_approx(lo2(aq)), ex2_approx(hi2(aq))));
+          vc = add2(vc, pack2(ex2_approx(lo2(ac)), ex2_approx(hi2(ac))));
+        }
+        if (in) {  // (a vector that is not there could combine to anything)
+          sq = add2(sq, vq);
+          sc = add2(sc, vc);
+        }
+      }
+      tq.add(sq);
+      tc.add(sc);
+    }
+    accq.s = tq.total();
+    accc.s = tc.total();
+  }
+  if (!(accq.s < INFINITY) || !(accc.s < INFINITY)) {  // overflow or a non-finite input: rare
+    accq.init();
+    accc.init();
+    for (v = v0 + lane; v < v1; v += 32) acc = logit_online<DT>(p, base, lw.pis, lw.thr, v * Elem<DT>::E, (v + 1) * Elem<DT>::E, acc);
+  }
+  if (ragged) {
+    const int e = ragged_entry(ragged_of<DT, AL>(p.V), p.V, lane);
+    if (e >= 0) acc = logit_online<DT>(p, base, lw.pis, lw.thr, e, e + 1, acc);
+  }
+  return acc;
+}
+
+// The argmax of the combined logits must be the fp64 one (the same chain of fused multiply-adds on every token, lowest index
+// among equals).  A vector gets its largest fp32 value and a bound on the distance of any of its fp32 values from the
+// fp64 ones, n 2^-23 sum_i |w_i| max |l_i|; only the tokens of a vector that could reach the best fp64 value seen so far are
+// evaluated in fp64.  (A bound for every token cost 5 instructions more for each logit: 564 us instead of 418 for 2304
+// positions of two 256000-token models.)
+struct BestCombined {
+  double best;
+  int idx, bad;
+  float lo;  // best rounded down
+};
+template <int DT>
+__device__ __noinline__ void consider_tokens(const KParams& p, const char* base, int e0, int count, float thr, BestCombined* b) {
+  const long long row_step = p.s_model * Elem<DT>::bytes;
+  const bool masked = p.mask_model >= 0;
+  for (int e = e0; e < e0 + count; ++e) {
+    double cm = 0.0;
+    float xe = 0.f;
+    int bad = 0;
+    for (int i = 0; i < p.n; ++i) {
+      const float x = Elem<DT>::load1(base + i * row_step, e);
+      bad |= !(x < INFINITY);
+      cm = fma(p.w64[i], static_cast<double>(x), cm);
+      if (i == p.mask_model) xe = x;
+    }
+    const bool in = !masked || xe >= thr;
+    b->bad |= bad | (in && cm != cm);
+    if (in && cm > b->best) {  // tokens come in increasing order within a lane: ties keep the earlier one
+      b->best = cm;
+      b->idx = e;
+      const float lo = __double2float_rd(cm);
+      if (lo > b->lo) b->lo = lo;
+    }
+  }
+}
+
+struct ArgPart2 {
+  ArgPart q, c;
+};
+template <int DT, bool AL, bool PAIR, bool MASKED>
+__device__ __noinline__ ArgPart2 logit_arg_segment(const KParams& p, const char* base, long long row_step, LogitWeights lw, int v0,
+                                                   int v1, bool ragged) {
+  constexpr int U = kStreamDepth / 2, E = Elem<DT>::E, H = E / 2;
+  const int lane = threadIdx.x & 31;
+  const bool pair = PAIR || p.n >= 2;
+  const int pis = lw.pis;
+  const float thr = lw.thr;
+  const float slack = static_cast<float>(PAIR ? 2 : p.n) * 1.1920929e-07f;  // n * 2^-23
+  const float wa0 = fabsf(lw.w0), wa1 = pair ? fabsf(lw.w1) : 0.f;
+  BestCombined b;
+  b.best = -INFINITY;
+  b.idx = kNoReject;
+  b.bad = 0;
+  b.lo = -INFINITY;
+  float lo = -INFINITY, qbest = -INFINITY;
+  int qv = -1;
+  for (int v = v0 + lane; __any_sync(0xffffffffu, v < v1); v += U * 32) {
+    uint4 r0[U], r1[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      r0[u] = r1[u] = neg_inf_vector<DT>();
+      if (v + u * 32 < v1) {
+        r0[u] = load_whole<DT, AL>(base, v + u * 32);
+        if (pair) r1[u] = load_whole<DT, AL>(base + row_step, v + u * 32);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int vu = v + u * 32;
+      if (vu < v1) {
+        float bound = wa0 * vector_max<DT, true>(r0[u]);
+        if (pair) bound = fmaf(wa1, vector_max<DT, true>(r1[u]), bound);
+        uint4 rq = pick_vector(pis == 0, r0[u], r1[u]);
+        f32x2 xq[H], cmb[H];
+        logit_args<DT, PAIR, MASKED>(p, lw, r0[u], r1[u],
+                                     [&](int i) {
+                                       const uint4 r = load_whole<DT, AL>(base + i * row_step, vu);
+                                       if (i == pis) rq = r;
+                                       bound = fmaf(fabsf(p.w[i]), vector_max<DT, true>(r), bound);
+                                       return r;
+                                     },
+                                     xq, cmb);
+        const float mq = vector_max<DT, false>(rq);
+        if (mq > qbest) {
+          qbest = mq;
+          qv = vu;
+        }
+        float mc = -INFINITY;
+#pragma unroll
+        for (int k = 0; k < H; ++k) mc = fmaxf(mc, fmaxf(lo2(cmb[k]), hi2(cmb[k])));
+        if (!(__fmaf_ru(bound, slack, mc) < lo)) {  // (a NaN or an infinity among the logits comes here too: the bound is not finite)
+          b.lo = lo;
+          consider_tokens<DT>(p, base, vu * E, E, thr, &b);
+          lo = b.lo;
+        }
+      }
+      if (u == 0 || u == U - 1) {
+        // any exact value found by a lane of the warp is a lower bound of the maximum for all of them: share the
+        // largest (floats ordered as unsigned integers, one warp-wide max)
+        const unsigned bits = __float_as_uint(lo);
+        const unsigned top = __reduce_max_sync(0xffffffffu, bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u));
+        lo = fmaxf(lo, __uint_as_float(top ^ ((top >> 31) ? 0x80000000u : 0xffffffffu)));
+      }
+    }
+  }
+  int qidx = kNoReject;
+  if (qv >= 0) {
+    const uint4 r = load_whole<DT, AL>(base + pis * row_step, qv);
+#pragma unroll
+    for (int k = E - 1; k >= 0; --k)
+      if (entry<DT>(r, k) == qbest) qidx = qv * E + k;
+  }
+  if (ragged) {
+    const int e = ragged_entry(ragged_of<DT, AL>(p.V), p.V, lane);
+    if (e >= 0) {
+      BestCombined one;
+      one.best = -INFINITY;
+      one.idx = kNoReject;
+      one.bad = 0;
+      one.lo = -INFINITY;
+      consider_tokens<DT>(p, base, e, 1, thr, &one);
+      b.bad |= one.bad;
+      if (arg_better(one.best, one.idx, b.best, b.idx)) {
+        b.best = one.best;
+        b.idx = one.idx;
+      }
+      const float x = Elem<DT>::load1(base + pis * row_step, e);
+      if (arg_better(x, e, qbest, qidx)) {
+        qbest = x;
+        qidx = e;
+      }
+    }
+  }
+  ArgPart2 out;
+  out.q = warp_reduce_arg(static_cast<double>(qbest), qidx, b.bad, lane);
+  out.c = warp_reduce_arg(b.best, b.idx, b.bad, lane);
+  return out;
+}
+
+// ------------------------------------------------------------------------------------
+// publishing a unit and the per-row first-rejection scan (Sec. 3.1)
+// ------------------------------------------------------------------------------------
+__device__ __forceinline__ void push_job(const KParams& p, int idx, int emit) {
+  const int k = atomicAdd(p.job_count, 1);
+  if (k < p.max_jobs) p.jobs[k] = make_int2(idx, emit);
+}
+
+// Record a unit's decision; the last unit of a row to arrive scans for the first
+// rejection, writes the row's outputs and, where a token has to be drawn, names that position
+// for the drawing launch (which fills in out_tokens[b][a]).
+// `word4`: sampling modes: whether a token can be drawn at this unit; greedy modes: the bits of the bonus
+// token's probability (a float), NaN away from the bonus position.
+__device__ __forceinline__ void publish_unit(const KParams& p, int b, int j, int accept, int status, int cand, int word4,
+                             double ratio, double r_d, double q_d, double S) {
+  const int idx = b * p.P + j;
+  if (p.diag) {
+    float* d = p.diag + static_cast<long long>(idx) * 4;
+    d[0] = static_cast<float>(ratio);
+    d[1] = static_cast<float>(r_d);
+    d[2] = static_cast<float>(q_d);
+    d[3] = static_cast<float>(S);
+  }
+  int4 res = make_int4(accept, status, cand, word4);
+  __stcg(&p.unit_res[idx], res);
+  if (p.early_exit && !accept && j < p.gamma) atomicMin(&p.row_reject[b], j);  // later positions may be left unread
+  __threadfence();
+  // The row's word counts its published positions (low six bits) and, for rows of up to kPackedP positions,
+  // also carries one "not accepted" bit and one "has status bits" bit per position: the last position to
+  // arrive then knows the first rejection from the value the atomic returns, without reading the others.
+  const bool packed = (p.P <= kPackedP);
+  int mine = 1;
+  if (packed) {
+    if (!accept || j == p.gamma) mine |= 1 << (6 + j);
+    if (status) mine |= 1 << (6 + kPackedP + j);
+  }
+  const int prev = atomicAdd(&p.row_arrivals[b], mine);
+  if ((packed ? (prev & 63) : prev) != p.P - 1) return;  // longer rows keep a plain count in the word
+  // last unit of the row: every other unit's result is visible after the fence below
+  __threadfence();
+  int a = p.gamma;
+  unsigned st = 0;
+  int tok = -1, draw = 0;
+  if (packed) {
+    const int total = prev + mine;  // every position added its own bits once: no carries
+    a = __ffs((total >> 6) & ((1 << kPackedP) - 1)) - 1;
+    const int4 u = __ldcg(&p.unit_res[b * p.P + a]);
+    tok = u.z;
+    draw = u.w;
+    int with_status = (total >> (6 + kPackedP)) & ((2 << a) - 1);
+    while (with_status) {  // rare: some position up to the first rejection reported status bits
+      const int k = __ffs(with_status) - 1;
+      with_status &= with_status - 1;
+      st |= static_cast<unsigned>(__ldcg(&p.unit_res[b * p.P + k]).y);
+    }
+  } else {
+    for (int k = 0; k < p.P; ++k) {
+      int4 u = __ldcg(&p.unit_res[b * p.P + k]);
+      st |= static_cast<unsigned>(u.y);
+      if (k == p.gamma || !u.x) {
+        a = k;
+        tok = u.z;
+        draw = u.w;
+        break;
+      }
+    }
+  }
+  if (p.bonus_prob != nullptr) {
+    // sampling modes: the drawing launch fills it in after a full acceptance; greedy modes know it here
+    const bool known = p.greedy && a == p.gamma && tok >= 0;
+    p.bonus_prob[b] = known ? __int_as_float(draw) : __int_as_float(0x7fc00000);
+  }
+  if (p.greedy) draw = 0;
+  p.accept_count[b] = a;
+  int* o = p.out_tokens + static_cast<long long>(b) * p.P;
+  for (int k = 0; k < p.P; ++k) o[k] = (k < a) ? p.drafts[b * p.gamma + k] : (k == a ? tok : -1);
+  p.row_status[b] = st;
+  p.row_arrivals[b] = 0;  // leave the scratch ready for the next run
+  if (p.early_exit) p.row_reject[b] = kNoReject;
+  if (!p.greedy) p.row_draw[b] = draw ? a : -1;
+  if (draw && p.use_jobs) push_job(p, b * p.P + a, 1);
+}
+
+// The accept test of one (row, position) from the merged statistics (Eq. 6), taken by one thread in fp64; greedy modes also
+// settle the replacement token here.  Reads fsoft / farg / pdraft / ldraft, writes dec.  (Logit-level greedy: farg[0] is the
+// proposer's argmax, farg[1] the combined one.)
+template <int DT, int MODE>
+__device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double u_acc, double u_smp, float thr32, bool mask_bad,
+                                            bool is_bonus, int draft, bool draft_ok, int pi, bool pi_ok, int pis) {
+  const bool masked = (MODE == kLogitSample || MODE == kLogitGreedy) && p.mask_model >= 0;
+  constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
+  const double kNaN = __longlong_as_double(0x7ff8000000000000LL);
+  const double kInf = __longlong_as_double(0x7ff0000000000000LL);
+  Decision& d = sh.dec;
+  d.accept = 0;
+  d.status = 0;
+  d.cand = -1;
+  d.natoms = 0;
+  d.ratio = d.r_d = d.q_d = d.S = d.prob = kNaN;
+  bool finite = pi_ok;
+  if (kSample) {
+    const int nsoft = (MODE == kEnsembleSample) ? p.n : 2;
+    for (int k = 0; k < nsoft; ++k) {
+      const SoftPart& f = sh.fsoft[k];
+      finite = finite && isfinite(f.ref) && isfinite(f.s) && (f.s > 0.0);
+    }
+    if (masked && mask_bad) finite = false;
+    if (!finite) {
+      d.status |= COS_ROW_NONFINITE;
+    } else {
+      if (!is_bonus) {
+        if (draft_ok) {
+          double r_d = 0.0, q_d = 0.0;
+          if (MODE == kEnsembleSample) {
+            for (int i = 0; i < p.n; ++i) {
+              r_d += p.w64[i] * sh.pdraft[i];
+              if (i == pi) q_d = sh.pdraft[i];
+            }
+          } else {
+            double cd = 0.0;
+            for (int i = 0; i < p.n; ++i) cd = fma(p.w64[i], static_cast<double>(sh.ldraft[i]), cd);
+            bool in = !masked || (sh.ldraft[p.mask_model] >= thr32);
+            r_d = in ? exp2(cd * p.cT64 - static_cast<double>(sh.fsoft[1].ref)) / sh.fsoft[1].s : 0.0;
+            double lq = static_cast<double>(sh.ldraft[pi]);
+            q_d = exp2(lq * p.cT64 - static_cast<double>(sh.fsoft[0].ref)) / sh.fsoft[0].s;
+          }
+          d.r_d = r_d;
+          d.q_d = q_d;
+          if (q_d > 0.0) {
+            d.ratio = r_d / q_d;
+          } else {
+            d.status |= COS_ROW_Q_ZERO;
+            d.ratio = (r_d > 0.0) ? kInf : 0.0;
+          }
+          d.accept = (u_acc <= fmin(1.0, d.ratio)) ? 1 : 0;
+        } else {
+          d.status |= COS_ROW_BAD_DRAFT;
+        }
+      }
+    }
+  } else {
+    // greedy: distributions are atoms at lowest-index argmaxes
+    int qtok;
+    if (MODE == kEnsembleGreedy) {
+      for (int i = 0; i < p.n; ++i) finite = finite && !sh.farg[i].bad && isfinite(sh.farg[i].val);
+      qtok = sh.farg[pis].idx;
+    } else {
+      finite = finite && !sh.farg[0].bad && !sh.farg[1].bad && isfinite(sh.farg[0].val) && isfinite(sh.farg[1].val);
+      if (masked && mask_bad) finite = false;
+      qtok = sh.farg[0].idx;
+    }
+    if (!finite) {
+      d.status |= COS_ROW_NONFINITE;
+    } else {
+      // atoms of r, sorted by token, masses accumulated in model order
+      if (MODE == kEnsembleGreedy) {
+        for (int i = 0; i < p.n; ++i) {
+          int t = sh.farg[i].idx, pos = 0;
+          while (pos < d.natoms && d.atom_tok[pos] < t) ++pos;
+          if (pos < d.natoms && d.atom_tok[pos] == t) {
+            d.atom_mass[pos] += p.w64[i];
+          } else {
+            for (int k = d.natoms; k > pos; --k) {
+              d.atom_tok[k] = d.atom_tok[k - 1];
+              d.atom_mass[k] = d.atom_mass[k - 1];
+            }
+            d.atom_tok[pos] = t;
+            d.atom_mass[pos] = 0.0 + p.w64[i];
+            ++d.natoms;
+          }
+        }
+      } else {
+        d.natoms = 1;
+        d.atom_tok[0] = sh.farg[1].idx;
+        d.atom_mass[0] = 1.0;
+      }
+      auto r_at = [&](int t) {
+        for (int k = 0; k < d.natoms; ++k)
+          if (d.atom_tok[k] == t) return d.atom_mass[k];
+        return 0.0;
+      };
+      bool use_r = is_bonus;
+      if (!is_bonus) {
+        if (draft_ok) {
+          d.r_d = r_at(draft);
+          d.q_d = (draft == qtok) ? 1.0 : 0.0;
+          if (d.q_d > 0.0) {
+            d.ratio = d.r_d / d.q_d;
+          } else {
+            d.status |= COS_ROW_Q_ZERO;
+            d.ratio = (d.r_d > 0.0) ? kInf : 0.0;
+          }
+          d.accept = (u_acc <= fmin(1.0, d.ratio)) ? 1 : 0;
+        } else {
+          d.status |= COS_ROW_BAD_DRAFT;
+        }
+        // residual max(0, r - q) over the atoms, summed in token order
+        double S = 0.0;
+        for (int k = 0; k < d.natoms; ++k) S += fmax(0.0, d.atom_mass[k] - (d.atom_tok[k] == qtok ? 1.0 : 0.0));
+        d.S = S;
+        if (!(S > 0.0)) {
+          use_r = true;
+          if (!d.accept) d.status |= COS_ROW_RESIDUAL_EMPTY;
+        }
+      }
+      // inverse CDF over the atoms (token order): smallest k with running sum >= u * total
+      double total = 0.0;
+      for (int k = 0; k < d.natoms; ++k)
+        total += use_r ? d.atom_mass[k] : fmax(0.0, d.atom_mass[k] - (d.atom_tok[k] == qtok ? 1.0 : 0.0));
+      const double target = u_smp * total;
+      double run = 0.0;
+      int lastpos = -1;
+      d.cand = -1;
+      for (int k = 0; k < d.natoms; ++k) {
+        double m = use_r ? d.atom_mass[k] : fmax(0.0, d.atom_mass[k] - (d.atom_tok[k] == qtok ? 1.0 : 0.0));
+        run += m;
+        if (m > 0.0) lastpos = d.atom_tok[k];
+        if (d.cand < 0 && m > 0.0 && run >= target) d.cand = d.atom_tok[k];
+      }
+      if (d.cand < 0) d.cand = lastpos;
+      if (is_bonus) {
+        if (p.bonus_model >= 0) {  // the named model's one-hot law (its argmax sits in the proposer's slot)
+          d.cand = qtok;
+          d.prob = 1.0;
+        } else {
+          d.prob = r_at(d.cand);
+        }
+      }
+    }
+  }
+  d.drawable = (kSample && finite) ? 1 : 0;
+}
+
+// Rescale a sum from reference exponent `ref` to R >= ref: an exact power of two where the references are whole numbers.
+__device__ __forceinline__ double rescale(double s, float ref, float R) {
+  const float d = ref - R;
+  if (ref == R) return s;
+  if (d == floorf(d) && d > -1000.f) return s * __hiloint2double((1023 + static_cast<int>(d)) << 20, 0);
+  return s * exp2(static_cast<double>(ref) - static_cast<double>(R));
+}
+
+// Where the record of share w for row r of a line goes, less w: the pairs (r, w) of a line follow one another with r + w rising.
+template <bool ENS>
+__device__ __forceinline__ size_t record_of(const KParams& p, int slab, int units, long long r) {
+  return static_cast<size_t>(slab) * (static_cast<size_t>(units) * (ENS ? p.n : 1) + p.st_workers) + static_cast<size_t>(r);
+}
+
+// Merge the records of a position, in the order of the line: `slots` results (a lane group for each), into fin.fsoft / farg.
+template <int MODE>
+__device__ __forceinline__ void merge_records(const KParams& p, Finish& fin, int slab, int u_local, int units) {
+  constexpr bool kEns = (MODE == kEnsembleSample || MODE == kEnsembleGreedy);
+  constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
+  const int lane = threadIdx.x & 31;
+  const int slots = kEns ? p.n : 2;
+  const int g = slots <= 1 ? 32 : (slots <= 2 ? 16 : (slots <= 4 ? 8 : 4));  // lanes of a group
+  const int i = lane / g, sub = lane % g;
+  float R = -INFINITY;
+  double s = 0.0;
+  ArgPart best;
+  best.val = -INFINITY;
+  best.idx = kNoReject;
+  best.bad = 0;
+  if (i < slots) {
+    const long long r = kEns ? static_cast<long long>(i) * units + u_local : u_local;
+    const int w0 = worker_of(p, r * p.st_nv), w1 = worker_of(p, (r + 1) * p.st_nv - 1);
+    const size_t first = record_of<kEns>(p, slab, units, r);
+    for (int w = w0 + sub; w <= w1; w += g) {
+      const int4 rec = __ldcg(p.st_rec + (kEns ? first + w : (first + w) * 2 + i));
+      const double v = __hiloint2double(rec.y, rec.x);
+      if (kSample) {
+        const float ref = __int_as_float(rec.z), top = fmaxf(R, ref);
+        s = rescale(s, R, top) + rescale(v, ref, top);
+        R = top;
+      } else {
+        best.bad |= rec.w;
+        if (arg_better(v, rec.z, best.val, best.idx)) {
+          best.val = v;
+          best.idx = rec.z;
+        }
+      }
+    }
+  }
+  if (kSample) {
+    float top = R;
+    for (int d = g / 2; d > 0; d >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, d));
+    s = rescale(s, R, top);
+    for (int d = g / 2; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+    if (sub == 0 && i < slots) {
+      fin.fsoft[i].s = s;
+      fin.fsoft[i].ref = top;
+    }
+  } else {
+    for (int d = g / 2; d > 0; d >>= 1) {
+      const double ov = __shfl_xor_sync(0xffffffffu, best.val, d);
+      const int oi = __shfl_xor_sync(0xffffffffu, best.idx, d);
+      best.bad |= __shfl_xor_sync(0xffffffffu, best.bad, d);
+      if (arg_better(ov, oi, best.val, best.idx)) {
+        best.val = ov;
+        best.idx = oi;
+      }
+    }
+    if (sub == 0 && i < slots) fin.farg[i] = best;
+  }
+  __syncwarp();
+}
+
+// The plausibility threshold of a position from the largest logit of the gating model (key of the mask launch).
+struct MaskBound {
+  float thr;
+  bool bad;
+};
+__device__ __forceinline__ MaskBound mask_bound(const KParams& p, unsigned key) {
+  MaskBound m;
+  m.bad = key > 0xff800000u;  // a NaN
+  const float top = __uint_as_float(key ^ ((key >> 31) ? 0x80000000u : 0xffffffffu));
+  // l >= max + ln(alpha) in fp64 is the same as l >= (that bound rounded up to fp32) for fp32 l
+  m.thr = m.bad ? __int_as_float(0x7fc00000) : __double2float_ru(static_cast<double>(top) + p.ln_alpha);
+  return m;
+}
+
+// Largest logit of the gating model at every position, for the plausibility mask: the same split, over that model's rows
+// alone.  (Positions need it before they can be swept, and the warps of the streaming launch do not wait for each other.)
+template <int DT, bool AL>
+__global__ void __launch_bounds__(kStreamThreads, 2) cos_mask_kernel(const __grid_constant__ KParams p) {
+  constexpr int U = kStreamDepth;
+  const int lane = threadIdx.x & 31;
+  const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (w >= p.st_workers) return;
+  const int v_lo = whole_vectors<DT, AL>(p.V).lo, v_hi = whole_vectors<DT, AL>(p.V).hi;
+  for (long long x = worker_lo(p, w), end = worker_lo(p, w + 1); x < end;) {
+    const int unit = static_cast<int>(x / p.st_nv);
+    const int o0 = static_cast<int>(x - static_cast<long long>(unit) * p.st_nv);
+    const int o1 = end - x < p.st_nv - o0 ? o0 + static_cast<int>(end - x) : p.st_nv;
+    const int b = unit / p.P, j = unit % p.P;
+    const char* row = reinterpret_cast<const char*>(p.logits) +
+                      (p.mask_model * p.s_model + static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
+    float best = -INFINITY;
+    const int v1 = v_lo + o1 < v_hi ? v_lo + o1 : v_hi;
+    for (int v = v_lo + o0 + lane; v < v1; v += U * 32) {
+      uint4 raw[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        raw[u] = neg_inf_vector<DT>();
+        if (v + u * 32 < v1) raw[u] = load_whole<DT, AL>(row, v + u * 32);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) best = max_nan(best, vector_max<DT, false>(raw[u]));
+    }
+    if (o1 == p.st_nv) {
+      const int e = ragged_entry(ragged_of<DT, AL>(p.V), p.V, lane);
+      if (e >= 0) best = max_nan(best, Elem<DT>::load1(row, e));
+    }
+    const unsigned bits = (best != best) ? 0x7fc00000u : __float_as_uint(best);
+    const unsigned top = __reduce_max_sync(0xffffffffu, bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u));
+    if (lane == 0) atomicMax(&p.mask_key[unit], top);
+    x += o1 - o0;
+  }
+}
+
+template <int DT, int MODE, bool AL>
+__global__ void __launch_bounds__(kStreamThreads, 2) cos_stream_kernel(const __grid_constant__ KParams p) {
+  constexpr bool kEns = (MODE == kEnsembleSample || MODE == kEnsembleGreedy);
+  constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
+  __shared__ Finish fins[kStreamThreads / 32];
+  const int lane = threadIdx.x & 31;
+  const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  Finish& fin = fins[threadIdx.x >> 5];
+  // Launched while the kernel before it in the stream drains (programmatic dependent launch): its blocks take their places
+  // as that kernel's blocks leave and wait here until it is complete and its writes are visible.  (Without the launch
+  // attribute, and behind a kernel that never signals, this is the ordinary order of a stream.)  Where the caller
+  // promises that the inputs were complete earlier, a warp sweeps its first row first and waits only before it writes.
+  bool waited = p.inputs_settled == 0;
+  if (waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (w >= p.st_workers) return;
+  const bool masked = !kEns && p.mask_model >= 0;
+  const int v_lo = whole_vectors<DT, AL>(p.V).lo, v_hi = whole_vectors<DT, AL>(p.V).hi;
+  const int rows = kEns ? p.n : 1;  // rows of the line for each position
+  const int units = p.st_slabs > 1 ? p.B : p.num_units;  // positions of a line
+  const long long row_step = p.s_model * Elem<DT>::bytes;
+  for (int slab = 0; slab < p.st_slabs; ++slab) {
+    for (long long x = worker_lo(p, w), end = worker_lo(p, w + 1); x < end;) {
+      // the part of row r, model i of position (b, j), that lies in this warp's share: vectors [o0, o1)
+      const long long r = x / p.st_nv;
+      const int i = kEns ? static_cast<int>(r / units) : 0;
+      const int u_local = static_cast<int>(r - static_cast<long long>(i) * units);
+      const int o0 = static_cast<int>(x - r * p.st_nv);
+      const int o1 = end - x < p.st_nv - o0 ? o0 + static_cast<int>(end - x) : p.st_nv;
+      x += o1 - o0;
+      const int b = p.st_slabs > 1 ? u_local : u_local / p.P, j = p.st_slabs > 1 ? slab : u_local % p.P;
+      const int uidx = b * p.P + j;
+      const char* base = reinterpret_cast<const char*>(p.logits) +
+                         (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
+      const bool is_bonus = (j == p.gamma);
+      const int draft = is_bonus ? 0 : __ldg(p.drafts + b * p.gamma + j);
+      const int pi = proposer_of(p, b, j);
+      const bool pi_ok = (pi >= 0 && pi < p.n);
+      const int pis = pi_ok ? pi : 0;
+      MaskBound mask;
+      mask.thr = -INFINITY;
+      mask.bad = false;
+      if (masked) mask = mask_bound(p, __ldcg(&p.mask_key[uidx]));
+      // Early exit: a position behind a rejection that its row has already published decides nothing (Sec. 3.1: the tokens
+      // after the first rejection are discarded).  Every warp looks for itself; one that skips marks the position.
+      bool skip = false;
+      if (p.early_exit) {
+        int rej = 0;
+        if (lane == 0) rej = *reinterpret_cast<volatile int*>(&p.row_reject[b]);
+        skip = __shfl_sync(0xffffffffu, rej, 0) < j;
+      }
+      if (!skip) {
+        const int v0 = v_lo + o0, v1 = v_lo + o1 < v_hi ? v_lo + o1 : v_hi;
+        const bool ragged = (o1 == p.st_nv);
+        int4 rec[2];
+        auto soft_rec = [&](const LaneSoft& a) {
+          // lanes of one warp: fp32 is enough here, the errors of the 32 scale factors average out
+          float R = a.ref;
+#pragma unroll
+          for (int d = 16; d > 0; d >>= 1) R = fmaxf(R, __shfl_xor_sync(0xffffffffu, R, d));
+          float t = (a.ref == R) ? a.s : a.s * ex2_approx(a.ref - R);
+#pragma unroll
+          for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+          const double s = static_cast<double>(t);
+          return make_int4(__double2loint(s), __double2hiint(s), __float_as_int(R), 0);
+        };
+        auto arg_rec = [&](const ArgPart& a) { return make_int4(__double2loint(a.val), __double2hiint(a.val), a.idx, a.bad); };
+        if (MODE == kEnsembleSample) {
+          rec[0] = soft_rec(soft_segment<DT, AL>(base + i * row_step, v0, v1, ragged, p.V, p.cT));
+        } else if (MODE == kEnsembleGreedy) {
+          rec[0] = arg_rec(arg_segment<DT, AL>(base + i * row_step, v0, v1, ragged, p.V));
+        } else if (MODE == kLogitSample) {
+          const LogitWeights lw = logit_weights(p, pis, mask.thr);
+          const LaneSoft2 a = p.n == 2 ? (masked ? logit_segment<DT, AL, true, true>(p, base, row_step, lw, p.cT, v0, v1, ragged)
+                                                 : logit_segment<DT, AL, true, false>(p, base, row_step, lw, p.cT, v0, v1, ragged))
+                                       : (masked ? logit_segment<DT, AL, false, true>(p, base, row_step, lw, p.cT, v0, v1, ragged)
+                                                 : logit_segment<DT, AL, false, false>(p, base, row_step, lw, p.cT, v0, v1, ragged));
+          rec[0] = soft_rec(a.q);
+          rec[1] = soft_rec(a.c);
+        } else {
+          const LogitWeights lw = logit_weights(p, pis, mask.thr);
+          const ArgPart2 a = p.n == 2 ? (masked ? logit_arg_segment<DT, AL, true, true>(p, base, row_step, lw, v0, v1, ragged)
+                                                : logit_arg_segment<DT, AL, true, false>(p, base, row_step, lw, v0, v1, ragged))
+                                      : (masked ? logit_arg_segment<DT, AL, false, true>(p, base, row_step, lw, v0, v1, ragged)
+                                                : logit_arg_segment<DT, AL, false, false>(p, base, row_step, lw, v0, v1, ragged));
+          rec[0] = arg_rec(a.q);
+          rec[1] = arg_rec(a.c);
+        }
+        if (!waited) {
+          asm volatile("griddepcontrol.wait;" ::: "memory");  // from here on as in an ordinary run
+          waited = true;
+        }
+        if (lane == 0) {
+          const size_t at = record_of<kEns>(p, slab, units, r) + w;
+          if (kEns) {
+            __stcg(p.st_rec + at, rec[0]);
+          } else {
+            __stcg(p.st_rec + at * 2, rec[0]);
+            __stcg(p.st_rec + at * 2 + 1, rec[1]);
+          }
+        }
+      }
+      // the logits at the draft token, fetched while the warp reports
+      const bool draft_ok = is_bonus || (draft >= 0 && draft < p.V);
+      float ld = 0.f;
+      if (lane < p.n && !is_bonus && draft_ok) ld = Elem<DT>::load1(base + lane * row_step, draft);
+      int prev = 0;
+      if (lane == 0) {
+        __threadfence();
+        prev = atomicAdd(&p.st_arrivals[uidx], skip ? 1 + kSkipped : 1);
+        __threadfence();
+      }
+      // reports the position needs: one for every share that has a part of one of its rows
+      int reports = 0;
+      if (lane < rows) {
+        const long long at = (static_cast<long long>(lane) * units + u_local) * p.st_nv;
+        reports = worker_of(p, at + p.st_nv - 1) - worker_of(p, at) + 1;
+      }
+      reports = __reduce_add_sync(0xffffffffu, reports);
+      prev = __shfl_sync(0xffffffffu, prev, 0);
+      if ((prev & (kSkipped - 1)) + 1 != reports) continue;
+      // the warp that completes the position: merge, decide, publish
+      skip = skip || prev >= kSkipped;
+      if (lane == 0) {
+        p.st_arrivals[uidx] = 0;  // ready for the next run
+        if (masked) p.mask_key[uidx] = 0u;
+      }
+      if (skip) {
+        // some warp left it unread: the unit reports "not accepted, no candidate", which the row's scan never reaches
+        if (lane == 0) {
+          const double nan = __longlong_as_double(0x7ff8000000000000LL);
+          publish_unit(p, b, j, 0, 0, -1, kSample ? 0 : 0x7fc00000, nan, nan, nan, nan);
+        }
+        __syncwarp();
+        continue;
+      }
+      unsigned rnd[4];
+      philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
+      merge_records<MODE>(p, fin, slab, u_local, units);
+      if (lane < p.n) {
+        fin.ldraft[lane] = ld;
+        // probability of the draft under model `lane`, with the constant the sweep used
+        if (MODE == kEnsembleSample)
+          fin.pdraft[lane] = exp2(static_cast<double>(ld) * p.cT64 - static_cast<double>(fin.fsoft[lane].ref)) / fin.fsoft[lane].s;
+      }
+      __syncwarp();
+      if (kSample && lane < (kEns ? p.n : 2)) {  // kept for the drawing launch
+        p.ustats[uidx].s[lane] = fin.fsoft[lane].s;
+        p.ustats[uidx].ref[lane] = fin.fsoft[lane].ref;
+      }
+      if (kSample && lane == 31) p.ustats[uidx].thr32 = mask.thr;
+      if (lane == 0) {
+        decide_unit<DT, MODE>(p, fin, word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), mask.thr, mask.bad, is_bonus, draft, draft_ok,
+                              pi, pi_ok, pis);
+        const Decision& d = fin.dec;
+        if (!kSample && p.dump_r != nullptr) {  // test hook: the atoms of r
+          UnitStats& st = p.ustats[uidx];
+          st.pad[0] = (d.status & COS_ROW_NONFINITE) ? -1 : d.natoms;
+          for (int k = 0; k < d.natoms; ++k) {
+            st.s[k] = d.atom_mass[k];
+            st.ref[k] = __int_as_float(d.atom_tok[k]);
+          }
+        }
+        publish_unit(p, b, j, d.accept, d.status, d.cand, kSample ? d.drawable : __float_as_int(static_cast<float>(d.prob)), d.ratio,
+                     d.r_d, d.q_d, d.S);
+      }
+      __syncwarp();
+    }
+  }
+}
+
+// Test hook, greedy runs: r is a handful of atoms.
+template <int DT>
+__global__ void cos_dump_atoms_kernel(const __grid_constant__ KParams p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int uidx = blockIdx.y;
+  const UnitStats* st = &p.ustats[uidx];
+  float* out = p.dump_r + static_cast<long long>(uidx) * p.V;
+  for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < p.V; x += gridDim.x * blockDim.x) {
+    float v = st->pad[0] < 0 ? __int_as_float(0x7fc00000) : 0.f;
+    for (int k = 0; k < st->pad[0]; ++k)
+      if (__float_as_int(st->ref[k]) == x) v = static_cast<float>(st->s[k]);
+    out[x] = v;
+  }
+}
+
+}  // namespace cosv
+
+#endif  // COS_STREAM_CUH
