@@ -20,22 +20,14 @@ namespace cg = cooperative_groups;
 
 namespace cosv {
 
-constexpr int kThreads = 512;
-constexpr int kWarps = kThreads / 32;
-constexpr int kMaxSlots = COS_MAX_MODELS + 2;
 constexpr int kNoReject = 0x7fffffff;
 constexpr int kPackedP = 13;  // rows of up to this many positions keep their accept flags in the arrival word
 constexpr int kDrawResidual = 0, kDrawR = 1, kDrawQ = 2;  // what a token is drawn from: max(0, r - q), r, or q
 constexpr double kBigShare = 1.0 / 256.0;  // probabilities above 2^-8 get fp64 treatment when tokens are drawn
-constexpr int kRingVecs = 8;                 // 16-byte vectors per lane staged ahead in sweep 2 (4 KB per warp)
-constexpr int kRingBytes = kWarps * kRingVecs * 32 * 16;
-constexpr int kRecG = 16;                    // running totals per warp kept in global memory between the drawing stages
-constexpr int kMaxParts = 16;                // blocks that share one unit in the drawing stages
-constexpr int kRec = 64;                     // running totals recorded per warp in sweep 2
 
 enum Mode { kEnsembleSample = 0, kLogitSample = 1, kEnsembleGreedy = 2, kLogitGreedy = 3 };
 
-struct UnitStats {  // what stage 1 needs from stage 0 about one (row, position)
+struct UnitStats {  // what the drawing launch needs to know about one (row, position)
   double s[COS_MAX_MODELS];   // normalisers sum 2^(arg - ref)
   float ref[COS_MAX_MODELS];  // reference exponents
   float thr32;                // plausibility threshold
@@ -52,15 +44,12 @@ struct KParams {
   int vec_ok;   // every row start is 16-byte aligned
   int nsteps;   // ceil(V / (32 * E))
   int flags;
-  int num_units, num_clusters;
+  int num_units;
   int per_pos;      // proposer is [B][gamma+1] (the model that proposed each draft) instead of [B]
-  int early_exit;   // positions after a row's known first rejection may be left unread (barrier-free form only)
+  int early_exit;   // positions after a row's known first rejection may be left unread
   int greedy;       // T = 0: no drawing stages; the fourth word of a unit's result carries the bonus probability
   int bonus_model;  // >= 0: the token after gamma acceptances follows this model's own distribution; -1: the combined one
-  int parts;     // blocks that share one unit in stages 1 and 2
-  int early_dependents;  // stage 0: let the next launch in the stream take places while this one runs
-  int inputs_settled;    // stage 0, barrier-free form: the inputs may be read before the kernel ahead in the stream is complete
-  int draw_cluster;      // one-sweep drawing stages: the blocks of a unit are a thread-block cluster and meet at its barrier
+  int inputs_settled;  // the inputs may be read before the kernel ahead in the stream is complete
   int max_jobs;  // capacity of the job list
   float w[COS_MAX_MODELS];
   double w64[COS_MAX_MODELS];
@@ -77,22 +66,28 @@ struct KParams {
   float* dump_r;
   float* bonus_prob;
   // scratch owned by the context
-  unsigned* work_counter;  // units are handed out from here; grows by num_units every run
-  unsigned* exit_count;    // [2]: blocks of stage 0 / stage 2 that have left; the last one clears the counters
+  unsigned* work_counter;  // (persistent kernel: cleared by a launch that only draws tokens)
   int* row_arrivals;       // [B], zero between runs
   int* row_reject;         // [B]: earliest rejected position published so far; kNoReject between runs
   int4* unit_res;          // [B*P]: x = accept flag, y = status bits, z = candidate token, w = a token can be drawn
-  int* job_count;          // units the drawing stages must process; cleared by the last block of stage 2
+  int* job_count;          // length of the job list (persistent kernel, which also clears it)
   int2* jobs;              // x = b * P + j of a unit that draws a token (y unused)
   UnitStats* ustats;       // [B*P]: merged statistics of sweep 1, read back by the later stages
-  double* zpart;           // [B*P][parts][8]: stage 1's partial normalisers
-  double* wtotg;           // [B*P][parts*16]: stage 2's mass of every warp run
-  double* srung;           // [B][parts*16][kRecG]: running totals inside the runs of the row's drawing unit
-                           // (one-sweep drawing stage: [B][nsteps], first channel sum of every step)
-  int* part_arrivals;      // [B*P]: blocks of the unit that finished stage 2; zero between runs
-  double* srungB;          // the one-sweep drawing stage: second channel of srung (null where that stage is not used)
-  double* srungC;          // ... third and fourth channel (ensembles of three or four models; null otherwise)
-  double* srungD;
+  int use_jobs;            // the list of drawing positions is kept too (tokens drawn by the persistent kernel)
+  // the streaming launch: a line of st_line vectors (st_nv for each row of it) in st_workers shares, st_rem of them of st_q + 1
+  // groups of eight vectors, the others of st_q; st_slabs lines one after another (one, or one for each position of a row)
+  int st_workers, st_slabs, st_nv;
+  long long st_line, st_q, st_rem;
+  int4* st_rec;            // records: statistics of a share's part of a row
+  int* st_arrivals;        // [B*P]: warps that have reported; zero between runs
+  unsigned* mask_key;      // [B*P]: largest logit of the gating model as an ordered integer; zero between runs
+  // the drawing launch
+  int* row_draw;           // [B]: the position of the row that draws its token, or -1
+  int draw_all;            // it visits every position (test hook, residual masses)
+  int draw_parts;          // blocks that share a position
+  int draw_cs, draw_chunks;  // steps of a chunk, chunks of a position
+  double* draw_rec;        // [positions][chunks][2 channels]: sums of every chunk
+  int* draw_arrivals;      // [positions of the launch]: blocks that have reported; zero between runs
 };
 
 // ------------------------------------------------------------------------------------
@@ -110,16 +105,6 @@ __device__ __forceinline__ uint4 ldg_stream16(const void* p) {
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                : "l"(p));
   return v;
-}
-
-__device__ __forceinline__ void cp_async16(void* smem, const void* g) {
-  unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
 template <int DT>
@@ -278,6 +263,123 @@ __device__ __forceinline__ void add2(float& d0, float& d1, float a0, float a1, f
       : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
 }
 
+// The same on values that stay packed.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float lo2(f32x2 v) { return __uint_as_float(static_cast<unsigned>(v)); }
+__device__ __forceinline__ float hi2(f32x2 v) { return __uint_as_float(static_cast<unsigned>(v >> 32)); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ void add2_if(f32x2& acc, f32x2 v, float when_positive) {
+  asm("{\n.reg .pred p;\nsetp.gt.f32 p, %2, 0f00000000;\n@p add.rn.f32x2 %0, %0, %1;\n}\n" : "+l"(acc) : "l"(v), "f"(when_positive));
+}
+
+// One entry of a 16-byte vector, and all of them in pairs of neighbours.
+template <int DT>
+__device__ __forceinline__ float entry(const uint4& r, int k) {
+  const unsigned w[4] = {r.x, r.y, r.z, r.w};
+  if (DT == COS_DTYPE_F32) return __uint_as_float(w[k & 3]);
+  const unsigned h = w[(k >> 1) & 3];
+  if (DT == COS_DTYPE_BF16) return __uint_as_float((k & 1) ? (h & 0xffff0000u) : (h << 16));
+  const __half2 hh = *reinterpret_cast<const __half2*>(&h);
+  return (k & 1) ? __high2float(hh) : __low2float(hh);
+}
+template <int DT>
+__device__ __forceinline__ void unpack_pairs(const uint4& r, f32x2 (&x)[Elem<DT>::E / 2]) {
+#pragma unroll
+  for (int k = 0; k < Elem<DT>::E / 2; ++k) x[k] = pack2(entry<DT>(r, 2 * k), entry<DT>(r, 2 * k + 1));
+}
+template <int DT>
+__device__ __forceinline__ uint4 neg_inf_vector() {
+  const unsigned w = DT == COS_DTYPE_F32 ? 0xff800000u : (DT == COS_DTYPE_BF16 ? 0xff80ff80u : 0xfc00fc00u);
+  return make_uint4(w, w, w, w);
+}
+
+// Entries [e0, e0 + E) of a row one by one; -inf beyond V.  Out of line: only the ends of a row come here.
+template <int DT>
+__device__ __noinline__ uint4 ragged_vector(const void* row, int e0, int V) {
+  uint4 r = neg_inf_vector<DT>();
+  if (DT == COS_DTYPE_F32) {
+    const unsigned* src = reinterpret_cast<const unsigned*>(row);
+    if (e0 < V) r.x = __ldg(src + e0);
+    if (e0 + 1 < V) r.y = __ldg(src + e0 + 1);
+    if (e0 + 2 < V) r.z = __ldg(src + e0 + 2);
+    if (e0 + 3 < V) r.w = __ldg(src + e0 + 3);
+    return r;
+  }
+  const unsigned short* src = reinterpret_cast<const unsigned short*>(row);
+  unsigned short h[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) h[k] = (e0 + k < V) ? __ldg(src + e0 + k) : static_cast<unsigned short>(r.x & 0xffffu);
+  return make_uint4(h[0] | (static_cast<unsigned>(h[1]) << 16), h[2] | (static_cast<unsigned>(h[3]) << 16),
+                    h[4] | (static_cast<unsigned>(h[5]) << 16), h[6] | (static_cast<unsigned>(h[7]) << 16));
+}
+
+// Vectors of a row of V entries that can be fetched with aligned 16-byte loads staying inside the row: [lo, hi).
+// AL: the rows are 16-byte aligned.  Otherwise a vector is cut out of two aligned neighbours, which leaves out the first
+// one and the last entries.
+struct VecRange {
+  int lo, hi;
+};
+template <int DT, bool AL>
+__device__ __forceinline__ VecRange whole_vectors(int V) {
+  constexpr int E = Elem<DT>::E;
+  VecRange r;
+  r.lo = AL ? 0 : 1;
+  r.hi = AL ? V / E : V / E - 1;
+  return r;
+}
+
+// One of the whole vectors of a row.  An unaligned row (its offset from a 16-byte boundary is the same for every
+// vector) costs two loads, the second one mostly a hit in L1, and a shift by whole words and by bits: about two
+// instructions per entry more, where loads of single entries cost one load for each.
+template <int DT, bool AL>
+__device__ __forceinline__ uint4 load_whole(const char* row, int v) {
+  if (AL) return ldg_stream16(row + static_cast<long long>(v) * 16);
+  const unsigned off = static_cast<unsigned>(reinterpret_cast<unsigned long long>(row)) & 15u;
+  const uint4* src = reinterpret_cast<const uint4*>(row - off) + v;
+  const uint4 a = __ldg(src);
+  if (off == 0u) return a;
+  const uint4 b = __ldg(src + 1);
+  unsigned w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  if (off & 8u) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) w[k] = w[k + 2];
+  }
+  if (off & 4u) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) w[k] = w[k + 1];
+  }
+  if (off & 2u) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[k] = __funnelshift_r(w[k], w[k + 1], 16);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+// Any vector of a row; -inf beyond V.
+template <int DT, bool AL>
+__device__ __forceinline__ uint4 load_vector(const char* row, int v, int V, const VecRange& whole) {
+  if (v >= whole.lo && v < whole.hi) return load_whole<DT, AL>(row, v);
+  return ragged_vector<DT>(row, v * Elem<DT>::E, V);
+}
+
 struct LaneSoft {
   float ref, s;
   __device__ __forceinline__ void init() {
@@ -405,11 +507,6 @@ __device__ __forceinline__ ArgPart warp_reduce_arg(double val, int idx, int bad,
   return o;
 }
 
-__device__ __forceinline__ void warp_merge_arg(double val, int idx, int bad, ArgPart* dst, int lane) {
-  ArgPart o = warp_reduce_arg(val, idx, bad, lane);
-  if (lane == 0) *dst = o;
-}
-
 // The model whose distribution is q at position j of row b: the row's proposer, or the proposer of that draft
 // when the caller gave one per position (Algorithm 2 verifies tokens of several proposers in one sequence).
 // At the bonus position of a call that names a bonus model, q is that model's distribution: the token is
@@ -439,69 +536,67 @@ struct Slice {
   int e_lo, e_hi;  // single entries [e_lo, e_hi): the ragged tail, or everything when unaligned
 };
 
-template <int DT>
-__device__ __forceinline__ Slice slice_of(int rank, int C, int V, bool vec_ok) {
-  constexpr int E = Elem<DT>::E;
-  Slice s;
-  if (vec_ok) {
-    const int nvec = V / E;
-    s.v_lo = static_cast<int>(static_cast<long long>(rank) * nvec / C);
-    s.v_hi = static_cast<int>(static_cast<long long>(rank + 1) * nvec / C);
-    s.e_lo = (rank == C - 1) ? nvec * E : V;
-    s.e_hi = V;
-  } else {
-    s.v_lo = s.v_hi = 0;
-    s.e_lo = static_cast<int>(static_cast<long long>(rank) * V / C);
-    s.e_hi = static_cast<int>(static_cast<long long>(rank + 1) * V / C);
-  }
-  return s;
+// The channel arguments of one lane's vector at logit level: the proposer's entries and the combined logits (-inf outside
+// the mask), packed in pairs of neighbouring tokens.  PAIR: exactly two models (straight code); MASKED: there is a plausibility
+// mask.  `more(i)` fetches the vector of model i >= 2.
+struct LogitWeights {
+  float w0, w1;
+  int pis, mask_model;
+  float thr;
+};
+__device__ __forceinline__ uint4 pick_vector(bool first, const uint4& a, const uint4& b) {
+  return make_uint4(first ? a.x : b.x, first ? a.y : b.y, first ? a.z : b.z, first ? a.w : b.w);
 }
-
-// Softmax normaliser of one row over the slice: fixed reference exponent (seeded from the
-// thread's first vector) with four loads in flight; overflow or a non-finite input falls
-// back to the running-maximum form.
-// U: 16-byte loads a thread issues before it consumes them
-template <int DT, int NT, int U = 4>
-__device__ __forceinline__ LaneSoft soft_slice(const void* row, const Slice& sl, int tid, float c) {
-  constexpr int E = Elem<DT>::E;
-  const char* rowb = reinterpret_cast<const char*>(row);
-  LaneSoft acc;
-  acc.init();
-  int v = sl.v_lo + tid;
-  if (v < sl.v_hi) {
-    float x[E];
-    uint4 raw[U];
-    raw[0] = ldg_stream16(rowb + static_cast<long long>(v) * 16);
-    Elem<DT>::unpack(raw[0], x);
-    acc.seed(x, c);
-    for (; v + (U - 1) * NT < sl.v_hi; v += U * NT) {
+template <int DT, bool PAIR, bool MASKED, typename F>
+__device__ __forceinline__ void logit_args(const KParams& p, const LogitWeights& lw, const uint4& r0, const uint4& r1, F more,
+                                           f32x2 (&xq)[Elem<DT>::E / 2], f32x2 (&cmb)[Elem<DT>::E / 2]) {
+  constexpr int H = Elem<DT>::E / 2;
+  uint4 rq = pick_vector(lw.pis == 0, r0, r1), rm = MASKED ? pick_vector(lw.mask_model == 0, r0, r1) : rq;
+  {
+    f32x2 x[H];
+    unpack_pairs<DT>(r0, x);
+    const f32x2 w = pack2(lw.w0, lw.w0);
 #pragma unroll
-      for (int u = 0; u < U; ++u) raw[u] = ldg_stream16(rowb + static_cast<long long>(v + u * NT) * 16);
+    for (int k = 0; k < H; ++k) cmb[k] = mul2(w, x[k]);
+  }
+  if (PAIR || p.n >= 2) {
+    f32x2 x[H];
+    unpack_pairs<DT>(r1, x);
+    const f32x2 w = pack2(lw.w1, lw.w1);
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        Elem<DT>::unpack(raw[u], x);
-        acc.add_fixed2(x, c);
-      }
-    }
-    for (; v < sl.v_hi; v += NT) {
-      raw[0] = ldg_stream16(rowb + static_cast<long long>(v) * 16);
-      Elem<DT>::unpack(raw[0], x);
-      acc.add_fixed2(x, c);
+    for (int k = 0; k < H; ++k) cmb[k] = fma2(w, x[k], cmb[k]);
+  }
+  if (!PAIR) {
+    for (int i = 2; i < p.n; ++i) {
+      const uint4 r = more(i);
+      if (i == lw.pis) rq = r;
+      if (i == lw.mask_model) rm = r;
+      f32x2 x[H];
+      unpack_pairs<DT>(r, x);
+      const f32x2 w = pack2(p.w[i], p.w[i]);
+#pragma unroll
+      for (int k = 0; k < H; ++k) cmb[k] = fma2(w, x[k], cmb[k]);
     }
   }
-  for (int e = sl.e_lo + tid; e < sl.e_hi; e += NT) acc.add_online1(Elem<DT>::load1(row, e), c);
-  if (!(acc.s < INFINITY)) {
-    acc.init();
-    for (v = sl.v_lo + tid; v < sl.v_hi; v += NT) {
-      float x[E];
-      uint4 raw = ldg_stream16(rowb + static_cast<long long>(v) * 16);
-      Elem<DT>::unpack(raw, x);
-      acc.add_online(x, c);
-    }
-    for (int e = sl.e_lo + tid; e < sl.e_hi; e += NT) acc.add_online1(Elem<DT>::load1(row, e), c);
+  unpack_pairs<DT>(rq, xq);
+  if (MASKED) {
+    f32x2 x[H];
+    unpack_pairs<DT>(rm, x);
+#pragma unroll
+    for (int k = 0; k < H; ++k)
+      cmb[k] = pack2(lo2(x[k]) >= lw.thr ? lo2(cmb[k]) : -INFINITY, hi2(x[k]) >= lw.thr ? hi2(cmb[k]) : -INFINITY);
   }
-  return acc;
 }
+__device__ __forceinline__ LogitWeights logit_weights(const KParams& p, int pis, float thr) {
+  LogitWeights lw;
+  lw.w0 = p.w[0];
+  lw.w1 = p.w[1];
+  lw.pis = pis;
+  lw.mask_model = p.mask_model;
+  lw.thr = thr;
+  return lw;
+}
+__device__ __forceinline__ float pair_at(f32x2 v, int k) { return (k & 1) ? hi2(v) : lo2(v); }
 
 // Softmax statistics of a logit-level combine over the slice `sl` of one (row, position): accq = the proposer's
 // softmax, accc = the softmax of the combined logits sum_i w_i l_i (entries outside the plausibility mask count

@@ -1,0 +1,11 @@
+// The launches for f16 logits.
+#include "cos_launch.cuh"
+
+namespace cosv {
+
+template cudaError_t stream_launch<COS_DTYPE_F16>(const KParams&, int, int, cudaStream_t);
+template cudaError_t mask_launch<COS_DTYPE_F16>(const KParams&, int, cudaStream_t);
+template cudaError_t draw_launch<COS_DTYPE_F16>(const KParams&, bool, int, int, int, int, cudaStream_t);
+template cudaError_t dump_launch<COS_DTYPE_F16>(const KParams&, int, cudaStream_t);
+
+}  // namespace cosv

@@ -1,43 +1,26 @@
 // CoS verification step for sm_100a: combine (Eq. 3-5), accept test (Eq. 6), residual / bonus sample and
 // first-rejection scan (Sec. 3.1) for every row of a batch and every one of its gamma + 1 positions.
 //
-// Work unit = one (row b, position j).  One kernel template, instantiated per stage:
-//   stage 0  every unit: stream the n logit rows once from HBM (128-bit streaming loads), keep per-lane
-//            softmax statistics (reference exponent, sum of 2^(l*c - ref)) or argmaxes, merge them, take
-//            the accept test in fp64 from the merged statistics and the logits at the draft token, publish
-//            the unit; the last unit of a row to arrive scans for the first rejection, writes the row's
-//            outputs and lists the one unit of the row that must draw a token.  Two forms of the unit loop:
-//            a barrier-free one (a block owns a unit, its warps run from unit to unit and meet through
-//            volatile words in shared memory) and a cluster form (the blocks of a thread-block cluster
-//            split the vocabulary and exchange partial results through distributed shared memory);
-//   stage 1  listed units only: the normalisers again, terms above 2^-8 of a normaliser in fp64;
-//   stage 2  listed units only: token masses max(0, r - q) (or the law of the bonus token), every warp on
-//            a contiguous run of the vocabulary so that prefix order is token order, fp64 running totals;
-//            the last block of a unit to finish locates u * S and walks to the token;
-//   stage 3  stages 1 and 2 in one sweep, for logit-level combines and two-model ensembles: there a mass is
-//            k_A e_A / Z_A + k_B e_B / Z_B clipped at zero, linear in 1/Z_A and 1/Z_B over the tokens where
-//            it is positive; that set is decided with stage 0's normalisers, the sweep records the two sums
-//            of every step (256 or 128 consecutive tokens) next to the refined normalisers, and the last
-//            block of a unit turns the sums into masses, finds the step by a prefix and walks it.
-//   stage 4  the same for ensembles of three or four models, with one sum per model and step.
-// Units are handed out from a global counter.  Between blocks there are only fences and arrival counters;
-// the launches of a run (stage 0, then 3 or 1 and 2) order the stages.  Waits exist only inside a block of the barrier-free form,
-// and they are bounded: a wait that gave up marks every row with COS_ROW_FAULT and the block leaves.
-// At T = 0 stage 0 is the whole run.
+// A run is one launch at T = 0, two at T > 0 (three for ensembles of one or of more than four models), and one more in front
+// of them for the plausibility mask:
+//   mask       the plausibility threshold of every position (cos_stream.cuh);
+//   streaming  every (row, position): stream the n logit rows once from HBM, keep softmax statistics or argmaxes, take the
+//              accept test in fp64 from the merged statistics and the logits at the draft token, publish the
+//              position; the last one of a row to arrive scans for the first rejection, writes the row's outputs and names
+//              the one position of the row that must draw a token (cos_stream.cuh);
+//   drawing    the positions that draw a token: one sweep and the token (cos_draw.cuh).
+// Between blocks there are only fences and arrival counters: nothing waits for another block.
 //
-// This file is the host side of the library (contexts, launches, the C entry points).  The device code it compiles:
-//   cos_common.cuh        constants, launch parameters, loads, Philox, softmax partials
-//   cos_stage_shared.cuh  shared-memory layout of a block, cluster merge, publishing a position and the row scan
-//   cos_stage_stream.cuh  stage 0: the sweep of a position, the accept decision, the barrier-free loop
-//   cos_stage_draw.cuh    stages 1 to 4: big tokens in fp64, the two one-sweep forms
-//   cos_stage_kernel.cuh  the kernel template
-// (cos_fused.cu holds the persistent one-launch kernel, cos_probe.cu the two streaming ceilings.)
+// This file is the host side of the library (contexts, launches, the C entry points).  The kernels are compiled in
+// cos_bf16.cu, cos_f16.cu and cos_f32.cu; cos_common.cuh holds constants, launch parameters, loads, Philox and softmax
+// partials, cos_fused.cu the persistent one-launch kernel, cos_probe.cu the two streaming ceilings.
 
 #include <mutex>
+#include <type_traits>
 
 #include "cos_common.cuh"
 #include "cos_fused.h"
-#include "cos_stage_kernel.cuh"
+#include "cos_launch.h"
 
 using namespace cosv;
 
@@ -52,13 +35,12 @@ thread_local std::string g_create_error;
 
 struct cos_verify_ctx {
   cos_verify_config cfg;
-  int parts;            // blocks per unit in the drawing stages
-  int parts_one;        // the same in the one-sweep drawing stage
-  int max_clusters[5];  // resident clusters for cluster sizes 1, 2, 4, 8, 16 (0 = not available)
-  int dense_blocks;     // resident blocks of the four-per-multiprocessor build of stage 0 (0 = there is none)
   int sm_count;
   unsigned* d_work_counter;
   bool scratch_dirty;
+  int4* d_st_rec;
+  int* d_st_arrivals;
+  unsigned* d_mask_key;
   // device scratch
   int* d_row_arrivals;
   int* d_row_reject;
@@ -66,13 +48,9 @@ struct cos_verify_ctx {
   int* d_job_count;
   int2* d_jobs;
   UnitStats* d_ustats;
-  double* d_zpart;
-  double* d_wtotg;
-  double* d_srung;
-  double* d_srungC;  // third and fourth channel of the one-sweep stage (ensembles of three or four models)
-  double* d_srungD;
-  double* d_srungB;  // second channel of d_srung, for the one-sweep drawing stage
-  int* d_part_arrivals;
+  int* d_row_draw;
+  double* d_draw_rec;
+  int* d_draw_arrivals;
   // optional per-stage timing (cos_verify_set_stage_timing)
   bool timing;
   cudaEvent_t ev[4];
@@ -100,46 +78,6 @@ struct cos_verify_ctx {
 };
 
 namespace {
-
-using KernelFn = void (*)(const KParams);
-
-KernelFn pick_kernel(int dtype, int mode, int stage, bool dense = false) {
-  // one instantiation per stage, so that each gets its own register allocation; greedy modes have stage 0 only.
-  // `dense`: stage 0 of ensemble sampling compiled for four blocks per multiprocessor; its sweep fits in 32
-  // registers, and with more units than two blocks per multiprocessor can hold the extra warps pay
-  // (measured on workload 3: 77.5 -> 74.3 us); with fewer units the 64-register build is the faster one.
-  if (dense && stage == 0 && mode == kEnsembleSample) {
-    if (dtype == COS_DTYPE_F32) return cos_verify_kernel<COS_DTYPE_F32, kEnsembleSample, 0, 4>;
-    if (dtype == COS_DTYPE_BF16) return cos_verify_kernel<COS_DTYPE_BF16, kEnsembleSample, 0, 4>;
-    if (dtype == COS_DTYPE_F16) return cos_verify_kernel<COS_DTYPE_F16, kEnsembleSample, 0, 4>;
-  }
-#define COS_CASE(DT, M, S) \
-  if (dtype == DT && mode == M && stage == S) return cos_verify_kernel<DT, M, S>;
-#define COS_SAMPLING(DT, M) COS_CASE(DT, M, 0) COS_CASE(DT, M, 1) COS_CASE(DT, M, 2) COS_CASE(DT, M, 3)
-  // (stage 4, the one-sweep drawing stage with a channel per model, exists for ensembles only)
-  // its sweep holds four vectors per lane and the next four: built for one block per multiprocessor (the
-  // 64-register build spills a kilobyte per thread and is slower than the two-stage form)
-  if (mode == kEnsembleSample && stage == 4) {
-    if (dtype == COS_DTYPE_F32) return cos_verify_kernel<COS_DTYPE_F32, kEnsembleSample, 4, 1>;
-    if (dtype == COS_DTYPE_BF16) return cos_verify_kernel<COS_DTYPE_BF16, kEnsembleSample, 4, 1>;
-    if (dtype == COS_DTYPE_F16) return cos_verify_kernel<COS_DTYPE_F16, kEnsembleSample, 4, 1>;
-  }
-  COS_SAMPLING(COS_DTYPE_F32, kEnsembleSample)
-  COS_SAMPLING(COS_DTYPE_F32, kLogitSample)
-  COS_CASE(COS_DTYPE_F32, kEnsembleGreedy, 0)
-  COS_CASE(COS_DTYPE_F32, kLogitGreedy, 0)
-  COS_SAMPLING(COS_DTYPE_BF16, kEnsembleSample)
-  COS_SAMPLING(COS_DTYPE_BF16, kLogitSample)
-  COS_CASE(COS_DTYPE_BF16, kEnsembleGreedy, 0)
-  COS_CASE(COS_DTYPE_BF16, kLogitGreedy, 0)
-  COS_SAMPLING(COS_DTYPE_F16, kEnsembleSample)
-  COS_SAMPLING(COS_DTYPE_F16, kLogitSample)
-  COS_CASE(COS_DTYPE_F16, kEnsembleGreedy, 0)
-  COS_CASE(COS_DTYPE_F16, kLogitGreedy, 0)
-#undef COS_SAMPLING
-#undef COS_CASE
-  return nullptr;
-}
 
 int mode_of(const cos_verify_config& c) {
   const bool greedy = (c.temperature == 0.0f);
@@ -192,121 +130,123 @@ bool validate_config(const cos_verify_config& c, std::string* err) {
   return true;
 }
 
-int choose_cluster(const cos_verify_config& c) {
-  if (c.cluster_size > 0) return c.cluster_size;
+// Channels of the drawing launch: two describe every mass at logit level (proposer and combined logits) and for up to
+// two models; a channel per model otherwise.
+int draw_channels(const cos_verify_config& c) {
+  if (c.combine != COS_COMBINE_PROB_ENSEMBLE || c.n <= 2) return 2;
+  return c.n <= 4 ? 4 : 8;
+}
+
+// Ensembles of one or of more than four models draw in two launches.
+bool draw_split(const cos_verify_config& c) { return c.combine == COS_COMBINE_PROB_ENSEMBLE && (c.n == 1 || c.n > 4); }
+
+// How the drawing launch shares a position out.  The device holds 32 warps per multiprocessor (two channels) or 16;
+// every position gets as many blocks as all of them fit at once, blocks of 128 threads where that is eight or more, of 64
+// where the rounding down would leave more of the device idle.  A chunk (one record of sums) has one step at least for
+// each warp, about eight at most, so that the token is searched in few steps, as far as the scratch holds `records` of them.
+struct DrawPlan {
+  int threads, parts, cs, chunks;
+};
+DrawPlan draw_plan(const cos_verify_config& c, long long units, int sm_count, long long records) {
+  DrawPlan d;
   const int nsteps = (c.vocab + 32 * entries_per_vec(c.dtype) - 1) / (32 * entries_per_vec(c.dtype));
-  int cs = 8;
-  // keep a step per warp (small vocabularies are a chain of latencies: workload 1 went from 25.3 to 24.1 us per call
-  // and workload 2 from 35.3 to 34.2 when this asked for one step instead of two)
-  while (cs > 1 && nsteps / (cs * kWarps) < 1) cs >>= 1;
-  return cs;
+  const long long warps = static_cast<long long>(sm_count) * (draw_channels(c) == 2 ? 32 : 16);
+  d.threads = draw_split(c) ? 256 : (warps / 4 >= 8 * units ? 128 : 64);
+  const int nw = d.threads / 32;
+  long long parts = warps / nw / units;
+  if (parts > (nsteps + nw - 1) / nw) parts = (nsteps + nw - 1) / nw;
+  d.parts = parts < 1 ? 1 : static_cast<int>(parts);
+  const int mine = (nsteps + d.parts * nw - 1) / (d.parts * nw);  // steps of a warp
+  const int k = (mine + 7) / 8;
+  d.cs = (mine + k - 1) / k;
+  const long long most = records / units;  // chunks of a position
+  if (static_cast<long long>(d.cs) * most < nsteps) d.cs = static_cast<int>((nsteps + most - 1) / most);
+  d.chunks = (nsteps + d.cs - 1) / d.cs;
+  return d;
 }
 
-// Blocks per unit in the drawing stages: as many as fit on the device in one wave (two blocks per
-// multiprocessor), at least two steps per warp.
-// The stage that draws the tokens in one sweep: 3 where two channel sums describe every mass (the combine is at
-// logit level: proposer and combined logits; or it mixes two models), 4 for ensembles of three or four models (a
-// channel per model); 0: the two-stage form (more models, one model, greedy decoding).
-int one_sweep_stage(const cos_verify_config& c) {
-  if (c.temperature == 0.0f) return 0;
-  if (c.combine != COS_COMBINE_PROB_ENSEMBLE) return 3;
-  return c.n == 2 ? 3 : ((c.n == 3 || c.n == 4) ? 4 : 0);
+// Records the scratch of a context holds: chunks of four steps for a position of every row, of sixteen for all positions.
+long long draw_records(const cos_verify_config& c, int sm_count) {
+  const long long nsteps = (c.vocab + 32 * entries_per_vec(c.dtype) - 1) / (32 * entries_per_vec(c.dtype));
+  const long long rows = c.max_batch, one = rows * ((nsteps + 3) / 4), all = rows * (c.gamma + 1) * ((nsteps + 15) / 16);
+  return (one > all ? one : all) + 64LL * sm_count;
 }
 
-int choose_parts(const cos_verify_config& c, int rows, int sm_count) {
-  int parts = 1;
-  while (parts < kMaxParts && rows * parts * 2 <= 2 * sm_count) parts <<= 1;
-  const int E = entries_per_vec(c.dtype);
-  const int nsteps = (c.vocab + 32 * E - 1) / (32 * E);
-  while (parts > 1 && nsteps / (parts * kWarps) < 2) parts >>= 1;
-  return parts;
+constexpr int kStreamBlock = 512;   // threads of a block of a full streaming launch, two blocks per multiprocessor
+constexpr int kMinShare = 128;      // vectors a warp should have at least: four loads for each lane
+
+// Rows of whole 16-byte vectors in the line of the streaming launch: every model's row of every position, or (logit level)
+// the vectors of all models of a position together.
+int line_rows(const cos_verify_config& c) { return c.combine == COS_COMBINE_PROB_ENSEMBLE ? c.n : 1; }
+
+// Cut the line of `rows` rows into shares for at most `workers` warps (see cos_stream.cuh).  Small runs take fewer warps, so
+// that each has a few loads in flight, in small blocks, so that they spread over the device.  Returns the block size.
+int plan_line(KParams& p, const cos_verify_config& c, long long rows, long long workers, int sm_count) {
+  const int E = entries_per_vec(c.dtype), nvec = c.vocab / E;
+  p.st_nv = p.vec_ok ? nvec : nvec - 2;  // (unaligned rows: the first vector and the last one go entry by entry)
+  if (p.st_nv < 1) p.st_nv = 1;          // nothing but ragged entries
+  p.st_line = rows * p.st_nv;
+  const long long groups = (p.st_line + 7) / 8;
+  if (workers > p.st_line / kMinShare) workers = p.st_line / kMinShare;
+  if (workers < 1) workers = 1;
+  p.st_workers = static_cast<int>(workers);
+  p.st_q = groups / workers;
+  p.st_rem = groups % workers;
+  return workers <= 16LL * sm_count ? 128 : kStreamBlock;
 }
 
-// Blocks per unit in the one-sweep drawing stage.  Where a block still has enough to do (eight steps per
-// warp), several times more blocks than the device holds at once, so that it hands them out as slots come
-// free: one wave of whole units leaves some multiprocessors with twice the work of others.  Small units
-// stay at one wave: their blocks are bound by latency, not by throughput.
-int choose_parts_one(const cos_verify_config& c, int rows, int sm_count) {
-  const bool channels = (one_sweep_stage(c) == 4);
-  const long long slots = (channels ? 1LL : 2LL) * sm_count;  // blocks the device holds at once
-  const int E = entries_per_vec(c.dtype);
-  const int nsteps = (c.vocab + 32 * E - 1) / (32 * E);
-  // (choose_parts counts two blocks per multiprocessor; the stage with a channel per model holds one, so it is
-  // asked for half the device: one wave of blocks instead of two.  Workload 4: 96.1 -> 90.1 us per call with 128
-  // blocks instead of 256; 64 blocks: 104.8 us)
-  int parts = choose_parts(c, rows, channels ? sm_count / 2 : sm_count);
-  while (parts < 8 && static_cast<long long>(rows) * parts < 3 * slots && nsteps / (2 * parts * kWarps) >= 8) parts <<= 1;
-  // few rows of a small vocabulary: the stage is a chain of latencies, and more blocks per row (one cluster, down
-  // to a step per warp) shorten the sweep in it (workload 1: 26.5 -> 25.3 us per call, workload 2: 41.7 -> 36.0 us)
-  while (parts < 8 && static_cast<long long>(rows) * parts * 2 <= slots && nsteps / (2 * parts) >= kWarps / 2) parts <<= 1;
-  return parts;
+// Warps of the streaming launch: what the device holds at once, or the cluster size's worth of blocks for every position.
+long long stream_workers(const cos_verify_config& c, long long units, int sm_count) {
+  const long long most = static_cast<long long>(sm_count) * 2 * (kStreamBlock / 32);
+  const long long asked = units * c.cluster_size * (kStreamBlock / 32);
+  return c.cluster_size > 0 && asked < most ? asked : most;
 }
 
-int log2i(int c) { return c >= 16 ? 4 : (c >= 8 ? 3 : (c >= 4 ? 2 : (c >= 2 ? 1 : 0))); }
-
-// Stage 0 streams best with one block per unit (long contiguous reads, no cluster barrier);
-// more blocks per unit only when there are too few units to occupy the device.
-int choose_stream_cluster(const cos_verify_config& c, int units, int sm_count) {
-  if (c.cluster_size > 0) return c.cluster_size;
-  const int cap = choose_cluster(c);
-  int cs = 1;
-  while (cs < cap && units * cs < sm_count) cs <<= 1;
-  return cs;
+template <typename F>
+cudaError_t by_dtype(int dtype, F f) {
+  if (dtype == COS_DTYPE_F32) return f(std::integral_constant<int, COS_DTYPE_F32>());
+  if (dtype == COS_DTYPE_BF16) return f(std::integral_constant<int, COS_DTYPE_BF16>());
+  return f(std::integral_constant<int, COS_DTYPE_F16>());
 }
 
-cudaError_t query_clusters(KernelFn fn, int cluster, int sm_count, int* out) {
-  cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3(cluster * sm_count, 1, 1);
-  lc.blockDim = dim3(kThreads, 1, 1);
-  lc.dynamicSmemBytes = 0;  // only stage 0 runs in clusters, and it stages nothing
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cluster;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  lc.attrs = at;
-  lc.numAttrs = 1;
-  return cudaOccupancyMaxActiveClusters(out, reinterpret_cast<const void*>(fn), &lc);
+// The streaming launch, and before it the one that finds the plausibility thresholds.
+cudaError_t launch_stream(const cos_verify_config& c, int mode, KParams& p, long long workers, int sm_count, cudaStream_t stream) {
+  return by_dtype(c.dtype, [&](auto dt) {
+    constexpr int DT = decltype(dt)::value;
+    cudaError_t e = cudaSuccess;
+    p.st_slabs = 1;
+    if (p.mask_model >= 0) {
+      const int threads = plan_line(p, c, p.num_units, workers, sm_count);
+      e = mask_launch<DT>(p, threads, stream);
+    }
+    // Early exit: position by position, so that a row's rejection is known before its later positions are begun; where a
+    // warp's part of a position is short, every position is under way at once anyway and the hint is not taken.
+    const long long nv = c.vocab / entries_per_vec(c.dtype), part = static_cast<long long>(p.B) * line_rows(c) * nv / workers;
+    if (part < 1024) p.early_exit = 0;
+    if (p.early_exit) p.st_slabs = p.P;
+    const int threads = plan_line(p, c, static_cast<long long>(p.num_units / p.st_slabs) * line_rows(c), workers, sm_count);
+    if (e == cudaSuccess) e = stream_launch<DT>(p, mode, threads, stream);
+    if (e == cudaSuccess && p.dump_r != nullptr) e = dump_launch<DT>(p, mode, stream);
+    return e;
+  });
 }
 
-// attributes the kernels of one (dtype, mode) need before their first launch
-cudaError_t prepare_kernels(int dtype, int mode, int cluster_size);
-
-int stage_smem(int stage) { return stage >= 2 ? kRingBytes : 0; }  // the staging ring of the token-mass sweep
-
-cudaError_t launch_stage(int dtype, int mode, int stage, const KParams& p, int cluster, cudaStream_t stream,
-                         bool overlap_prev = false, bool dense = false) {
-  KernelFn fn = pick_kernel(dtype, mode, stage, dense);
-  if (fn == nullptr) return cudaErrorInvalidDeviceFunction;
-  cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3(static_cast<unsigned>(p.num_clusters) * cluster, 1, 1);
-  lc.blockDim = dim3(kThreads, 1, 1);
-  lc.dynamicSmemBytes = stage_smem(stage);
-  lc.stream = stream;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cluster;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  lc.attrs = at;
-  lc.numAttrs = overlap_prev ? 2 : 1;
-  return cudaLaunchKernelEx(&lc, fn, p);
-}
-
-cudaError_t prepare_kernels(int dtype, int mode, int cluster_size) {
-  const bool draws = (mode == kEnsembleSample || mode == kLogitSample);
-  cudaError_t e = cudaSuccess;
-  for (int st = 2; draws && st <= 4 && e == cudaSuccess; ++st) {
-    KernelFn fn = pick_kernel(dtype, mode, st);
-    if (fn != nullptr)
-      e = cudaFuncSetAttribute(reinterpret_cast<const void*>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize, stage_smem(st));
-  }
-  if (e == cudaSuccess && cluster_size > 8)
-    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(pick_kernel(dtype, mode, 0)),
-                             cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  return e;
+// The launches that draw the tokens: of every position (`all`: test hook, residual masses) or of one per row.
+cudaError_t launch_draw(const cos_verify_config& c, KParams& p, bool all, int sm_count, long long records, cudaStream_t stream) {
+  const bool ens = c.combine == COS_COMBINE_PROB_ENSEMBLE;
+  const int units = all ? p.num_units : p.B;
+  const DrawPlan d = draw_plan(c, units, sm_count, records);
+  p.draw_all = all ? 1 : 0;
+  p.draw_parts = d.parts;
+  p.draw_cs = d.cs;
+  p.draw_chunks = d.chunks;
+  return by_dtype(c.dtype, [&](auto dt) {
+    constexpr int DT = decltype(dt)::value;
+    cudaError_t e = cudaSuccess;
+    if (!draw_split(c)) return draw_launch<DT>(p, ens, draw_channels(c), 0, units, d.threads, stream);
+    for (int phase = 1; phase <= 2 && e == cudaSuccess; ++phase) e = draw_launch<DT>(p, ens, draw_channels(c), phase, units, d.threads, stream);
+    return e;
+  });
 }
 
 cos_status cuda_fail(cos_verify_ctx* ctx, const char* what, cudaError_t e) {
@@ -369,12 +309,14 @@ void fill_params(const cos_verify_config& c, const cos_verify_args* a, KParams& 
 
 cos_status init_scratch(cos_verify_ctx* ctx, cudaStream_t stream) {
   const size_t rows = static_cast<size_t>(ctx->cfg.max_batch);
-  cudaError_t e = cudaMemsetAsync(ctx->d_work_counter, 0, 4 * sizeof(unsigned), stream);  // counter and the two exit counts
+  const size_t units = rows * (static_cast<size_t>(ctx->cfg.gamma) + 1);
+  cudaError_t e = cudaMemsetAsync(ctx->d_work_counter, 0, 4 * sizeof(unsigned), stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_st_arrivals, 0, units * sizeof(int), stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_mask_key, 0, units * sizeof(unsigned), stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_draw_arrivals, 0, units * sizeof(int), stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_row_arrivals, 0, rows * sizeof(int), stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_row_reject, 0x7f, rows * sizeof(int), stream);  // "none yet"
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_job_count, 0, 2 * sizeof(int), stream);
-  if (e == cudaSuccess)
-    e = cudaMemsetAsync(ctx->d_part_arrivals, 0, rows * (static_cast<size_t>(ctx->cfg.gamma) + 1) * sizeof(int), stream);
   if (ctx->fused) {
     // counters, row words, arrival counters and the queue start at zero; the rest is written before it is read
     static const int kClear[] = {0, 1, 2, 4, 5, 6};
@@ -410,45 +352,6 @@ extern "C" cos_status cos_verify_create(const cos_verify_config* config, cos_ver
     return cuda_fail(nullptr, "cudaGetDeviceProperties", e);
   }
   ctx->sm_count = prop.multiProcessorCount;
-  ctx->parts = choose_parts(*config, config->max_batch, ctx->sm_count);
-  ctx->parts_one = choose_parts_one(*config, config->max_batch, ctx->sm_count);
-  const size_t pmax = static_cast<size_t>(ctx->parts > ctx->parts_one ? ctx->parts : ctx->parts_one);
-  KernelFn fn = pick_kernel(config->dtype, mode_of(*config), 0);
-  e = prepare_kernels(config->dtype, mode_of(*config), config->cluster_size);
-  if (e != cudaSuccess) {
-    delete ctx;
-    return cuda_fail(nullptr, "cudaFuncSetAttribute (shared memory or cluster size)", e);
-  }
-  for (int k = 0; k < 5; ++k) {
-    const int cs = 1 << k;
-    ctx->max_clusters[k] = 0;
-    if (cs == 16 && config->cluster_size != 16) continue;
-    int nc = 0;
-    e = query_clusters(fn, cs, ctx->sm_count, &nc);
-    if (e != cudaSuccess) {
-      (void)cudaGetLastError();
-      nc = 0;
-    }
-    ctx->max_clusters[k] = nc;
-  }
-  ctx->dense_blocks = 0;
-  if (mode_of(*config) == kEnsembleSample) {
-    int nc = 0;
-    e = query_clusters(pick_kernel(config->dtype, kEnsembleSample, 0, true), 1, ctx->sm_count, &nc);
-    if (e != cudaSuccess) {
-      (void)cudaGetLastError();
-      nc = 0;
-    }
-    ctx->dense_blocks = nc;
-  }
-  {
-    const int need = config->cluster_size > 0 ? config->cluster_size : 1;
-    if (ctx->max_clusters[log2i(need)] < 1 || ctx->max_clusters[0] < 1) {
-      delete ctx;
-      g_create_error = "no cluster of the requested size fits on the device";
-      return COS_ERR_UNSUPPORTED;
-    }
-  }
   const size_t rows = static_cast<size_t>(config->max_batch), P = static_cast<size_t>(config->gamma) + 1;
   bool ok = true;
   ok = ok && cudaMalloc(&ctx->d_work_counter, 256) == cudaSuccess;
@@ -458,17 +361,18 @@ extern "C" cos_status cos_verify_create(const cos_verify_config* config, cos_ver
   ok = ok && cudaMalloc(&ctx->d_job_count, 256) == cudaSuccess;
   ok = ok && cudaMalloc(&ctx->d_jobs, (rows * P + rows) * sizeof(int2)) == cudaSuccess;
   ok = ok && cudaMalloc(&ctx->d_ustats, rows * P * sizeof(UnitStats)) == cudaSuccess;
-  ok = ok && cudaMalloc(&ctx->d_zpart, rows * P * pmax * 8 * sizeof(double)) == cudaSuccess;
-  ok = ok && cudaMalloc(&ctx->d_wtotg, rows * P * pmax * kWarps * sizeof(double)) == cudaSuccess;
-  const size_t steps = (static_cast<size_t>(config->vocab) + 32 * entries_per_vec(config->dtype) - 1) / (32 * entries_per_vec(config->dtype));
-  const size_t rec_per_row = steps > pmax * kWarps * kRecG ? steps : pmax * kWarps * kRecG;  // one record per step, or per group of a run
-  ok = ok && cudaMalloc(&ctx->d_srung, rows * rec_per_row * sizeof(double)) == cudaSuccess;
-  ok = ok && cudaMalloc(&ctx->d_srungB, rows * rec_per_row * sizeof(double)) == cudaSuccess;
-  if (one_sweep_stage(*config) == 4) {
-    ok = ok && cudaMalloc(&ctx->d_srungC, rows * rec_per_row * sizeof(double)) == cudaSuccess;
-    ok = ok && cudaMalloc(&ctx->d_srungD, rows * rec_per_row * sizeof(double)) == cudaSuccess;
+  {
+    // a record (logit level: two) for every row of the line and one for every warp and slab
+    const size_t warps = static_cast<size_t>(ctx->sm_count) * 2 * (kStreamBlock / 32) * P;
+    const size_t recs = config->combine == COS_COMBINE_PROB_ENSEMBLE ? rows * P * config->n + warps : 2 * (rows * P + warps);
+    ok = ok && cudaMalloc(&ctx->d_st_rec, recs * sizeof(int4)) == cudaSuccess;
   }
-  ok = ok && cudaMalloc(&ctx->d_part_arrivals, rows * P * sizeof(int)) == cudaSuccess;
+  ok = ok && cudaMalloc(&ctx->d_st_arrivals, rows * P * sizeof(int)) == cudaSuccess;
+  ok = ok && cudaMalloc(&ctx->d_mask_key, rows * P * sizeof(unsigned)) == cudaSuccess;
+  ok = ok && cudaMalloc(&ctx->d_row_draw, rows * sizeof(int)) == cudaSuccess;
+  ok = ok && cudaMalloc(&ctx->d_draw_arrivals, rows * P * sizeof(int)) == cudaSuccess;
+  if (ok && config->temperature > 0.0f)
+    ok = cudaMalloc(&ctx->d_draw_rec, static_cast<size_t>(draw_records(*config, ctx->sm_count)) * 2 * draw_channels(*config) * sizeof(double)) == cudaSuccess;
   ctx->wait_limit = 1u << 20;
   ctx->test_drop = 0;
   ctx->fused = false;
@@ -583,7 +487,6 @@ cos_status run_launches(cos_verify_ctx* ctx, const cos_verify_args* a, void* cud
   KParams p;
   fill_params(c, a, p);
   p.work_counter = ctx->d_work_counter;
-  p.exit_count = ctx->d_work_counter + 1;
   p.row_arrivals = ctx->d_row_arrivals;
   p.row_reject = ctx->d_row_reject;
   p.early_exit = (a->flags & COS_RUN_EARLY_EXIT) ? 1 : 0;
@@ -591,14 +494,12 @@ cos_status run_launches(cos_verify_ctx* ctx, const cos_verify_args* a, void* cud
   p.job_count = ctx->d_job_count;
   p.jobs = ctx->d_jobs;
   p.ustats = ctx->d_ustats;
-  p.zpart = ctx->d_zpart;
-  p.wtotg = ctx->d_wtotg;
-  p.srung = ctx->d_srung;
-  p.part_arrivals = ctx->d_part_arrivals;
-  p.srungB = ctx->d_srungB;
-  p.srungC = ctx->d_srungC;
-  p.srungD = ctx->d_srungD;
-  p.parts = ctx->parts;
+  p.st_rec = ctx->d_st_rec;
+  p.st_arrivals = ctx->d_st_arrivals;
+  p.mask_key = ctx->d_mask_key;
+  p.row_draw = ctx->d_row_draw;
+  p.draw_rec = ctx->d_draw_rec;
+  p.draw_arrivals = ctx->d_draw_arrivals;
   p.max_jobs = p.num_units + a->batch;
 
   const int mode = mode_of(c);
@@ -616,96 +517,57 @@ cos_status run_launches(cos_verify_ctx* ctx, const cos_verify_args* a, void* cud
     ctx->scratch_dirty = (ctx->test_drop != 0);  // a run that was made to give up leaves its counters behind
     return COS_OK;
   }
-  // stage 0: every unit once (statistics, accept tests, row scans)
-  const int c0 = choose_stream_cluster(c, p.num_units, ctx->sm_count);
-  const int mc0 = ctx->max_clusters[log2i(c0)];
-  if (mc0 < 1) {
-    ctx->err = "no cluster of the chosen size fits on the device";
-    return COS_ERR_UNSUPPORTED;
-  }
-  p.num_clusters = p.num_units < mc0 ? p.num_units : mc0;
-  // more units than the 64-register build keeps resident, in the barrier-free form: the dense build
-  const bool dense = (mode == kEnsembleSample) && c0 == 1 && p.num_units > mc0 && ctx->dense_blocks > mc0;
-  if (dense) p.num_clusters = p.num_units < ctx->dense_blocks ? p.num_units : ctx->dense_blocks;
   ctx->scratch_dirty = true;  // cleared below once the launches are known to be queued
   if (ctx->timing) cudaEventRecord(ctx->ev[0], stream);
-  p.early_dependents = (c0 == 1 && p.num_units >= ctx->sm_count) ? 1 : 0;
-  {
-    const bool masked = (c.combine != COS_COMBINE_PROB_ENSEMBLE) && c.mask_model >= 0;
-    const bool hooks = (a->dump_r != nullptr) || (a->flags & COS_RUN_ALL_RESIDUALS);
-    // what it overlaps with is the end of the previous call's drawing stage, where one block per row goes on alone;
-    // a drawing stage of several waves of blocks leaves nothing to fill (workload 5 was 12 us slower with it), and
-    // greedy runs have no drawing stage
-    const int sweep_stage = one_sweep_stage(c);
-    const long long slots = (sweep_stage == 4 ? 1LL : 2LL) * ctx->sm_count;
-    const bool one_wave = draws && sweep_stage != 0 && static_cast<long long>(a->batch) * ctx->parts_one <= slots;
-    p.inputs_settled =
-        ((a->flags & COS_RUN_INPUTS_SETTLED) && p.early_dependents && one_wave && !masked && !hooks && !p.early_exit) ? 1 : 0;
-  }
-  e = launch_stage(c.dtype, mode, 0, p, c0, stream, true, dense);
-  if (e != cudaSuccess) return cuda_fail(ctx, "kernel launch (stage 0)", e);
+  const bool all = draws && ((a->dump_r != nullptr) || (a->flags & COS_RUN_ALL_RESIDUALS));
+  // what it overlaps with is the end of the previous call's drawing launch, where one block per row goes on alone; a
+  // drawing launch of more rows than the device has multiprocessors leaves nothing to fill (workload 5 was 12 us slower with
+  // it), and greedy runs have no drawing launch
+  p.inputs_settled = ((a->flags & COS_RUN_INPUTS_SETTLED) && draws && !all && !p.early_exit && p.mask_model < 0 &&
+                      p.num_units >= ctx->sm_count && a->batch <= ctx->sm_count)
+                         ? 1
+                         : 0;
+  const bool by_items = draws && !all && ctx->fused && ctx->draw_fused && p.vec_ok;
+  p.use_jobs = by_items ? 1 : 0;
+  e = launch_stream(c, mode, p, stream_workers(c, p.num_units, ctx->sm_count), ctx->sm_count, stream);
+  if (e != cudaSuccess) return cuda_fail(ctx, "kernel launch (streaming)", e);
   if (ctx->timing) cudaEventRecord(ctx->ev[1], stream);
   ctx->ev_used = 2;
   if (draws) {
-    // stages 1 and 2: the units listed by stage 0 (one per row, or all of them under the test hooks);
-    // blocks of a launch are independent, the launches themselves order the steps
-    const bool all = (a->dump_r != nullptr) || (a->flags & COS_RUN_ALL_RESIDUALS);
-    const int most = all ? p.max_jobs : a->batch;
-    const int cap = 4096;  // a block walks the job list with a stride, so the grid may be smaller than the list
-    p.num_clusters = (most < cap ? most : cap) * p.parts;  // blocks of a drawing launch
-    // Two channel sums describe every mass when the combine is at logit level (proposer, combined logits) or
-    // mixes two models: then one sweep does the work of stages 1 and 2.  The test hooks keep the two-stage form.
-    const int sweep_stage = one_sweep_stage(c);
-    const bool one_sweep = !all && sweep_stage != 0;
-    if (!all && ctx->fused && ctx->draw_fused && p.vec_ok) {
-      // the tokens are drawn by the persistent kernel's drawing items (one sweep with a channel sum per model, any
-      // block takes any chunk of any row) instead of the drawing stages
+    if (by_items) {
+      // the tokens are drawn by the persistent kernel's drawing items (any block takes any chunk of any row)
       e = fused_launch(c.dtype, mode, p, ctx->fplan, ctx->fscr, ctx->wait_limit, 0, true, stream);
       if (e != cudaSuccess) return cuda_fail(ctx, "kernel launch (drawing items)", e);
-      if (ctx->timing) cudaEventRecord(ctx->ev[2], stream);
-      ctx->ev_used = 3;
-      ctx->scratch_dirty = false;
-      return COS_OK;
+    } else {
+      e = launch_draw(c, p, all, ctx->sm_count, draw_records(c, ctx->sm_count), stream);
+      if (e != cudaSuccess) return cuda_fail(ctx, "kernel launch (drawing)", e);
     }
-    if (one_sweep) {
-      p.parts = ctx->parts_one;
-      p.num_clusters = (most < cap ? most : cap) * p.parts;
-      int draw_cs = 1;
-      // the blocks of a unit as one cluster (portable sizes), where the launch is a single wave of blocks: with
-      // several waves the clusters wait for four free places at once (workload 5: +17 us per call), with one the
-      // barrier is cheaper than fence and counter (workloads 1 to 4: -1.4 to -1.7 us)
-      const long long draw_slots = (sweep_stage == 4 ? 1LL : 2LL) * ctx->sm_count;
-      if (p.parts > 1 && p.parts <= 8 && static_cast<long long>(most) * p.parts <= draw_slots) {
-        draw_cs = p.parts;
-        p.draw_cluster = 1;
-        p.num_clusters = (most < cap ? most : cap);
-      }
-      e = launch_stage(c.dtype, mode, sweep_stage, p, draw_cs, stream, true);
-      if (e != cudaSuccess) return cuda_fail(ctx, "kernel launch (drawing stage)", e);
-      if (ctx->timing) cudaEventRecord(ctx->ev[2], stream);
-      ctx->ev_used = 3;
-    }
-    for (int st = 1; st <= 2 && !one_sweep; ++st) {
-      e = launch_stage(c.dtype, mode, st, p, 1, stream, true);
-      if (e != cudaSuccess) return cuda_fail(ctx, "kernel launch (drawing stages)", e);
-      if (ctx->timing) cudaEventRecord(ctx->ev[st + 1], stream);
-      ctx->ev_used = st + 2;
-    }
+    if (ctx->timing) cudaEventRecord(ctx->ev[2], stream);
+    ctx->ev_used = 3;
   }
-  // the last block of stage 0 to leave clears the work counter, the last of stage 2 the job counter: every
-  // run starts from the same scratch state with the same arguments, whatever ran before it
+  // (the kernels leave the scratch as they found it: every run starts from the same state with the same arguments)
   ctx->scratch_dirty = false;
   return COS_OK;
 }
 
 }  // namespace
 
-#ifdef COS_STAGE_PROFILE
-extern "C" int cos_stage_profile_read(unsigned long long* out, int blocks) {  // 8 words per block
-  const size_t n = static_cast<size_t>(blocks < kSprofBlocks ? blocks : kSprofBlocks) * 8 * sizeof(unsigned long long);
-  return cudaMemcpyFromSymbol(out, g_sprof, n) == cudaSuccess ? 0 : -1;
+namespace {
+// The log-sum-exp behind every softmax of a position, from the merged statistics a run leaves per position:
+// ln sum_x exp(l(x) / T) = (ref + log2 s) ln 2.  One thread per (position, slot).
+__global__ void export_lse_kernel(const UnitStats* ustats, const int4* unit_res, float* lse, int units, int slots, int sampling) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= units * slots) return;
+  const int u = t / slots, k = t % slots;
+  float v = __int_as_float(0x7fc00000);
+  if (sampling && !(__ldcg(&unit_res[u]).y & COS_ROW_NONFINITE)) {
+    const double sum = ustats[u].s[k];
+    v = static_cast<float>((static_cast<double>(ustats[u].ref[k]) + log2(sum)) * 0.6931471805599453);
+  }
+  lse[t] = v;
 }
-#endif
+
+}  // namespace
 
 extern "C" cos_status cos_verify_run(cos_verify_ctx* ctx, const cos_verify_args* a, void* cuda_stream) {
   if (ctx && a && a->lse && reinterpret_cast<uintptr_t>(a->lse) % 4) {
@@ -846,19 +708,25 @@ extern "C" cos_status cos_verify_set_wait_limit(cos_verify_ctx* ctx, uint32_t po
 extern "C" cos_status cos_verify_get_info(const cos_verify_ctx* ctx, cos_verify_info* info) {
   if (!ctx || !info) return COS_ERR_INVALID_ARG;
   memset(info, 0, sizeof(*info));
-  info->cluster_size = choose_stream_cluster(ctx->cfg, ctx->cfg.max_batch * (ctx->cfg.gamma + 1), ctx->sm_count);
-  info->threads_per_block = kThreads;
-  info->max_clusters = ctx->max_clusters[log2i(info->cluster_size)];
+  {
+    // blocks of the streaming launch that share a position, and how many positions they share at once
+    const long long units = static_cast<long long>(ctx->cfg.max_batch) * (ctx->cfg.gamma + 1);
+    const long long blocks = stream_workers(ctx->cfg, units, ctx->sm_count) / (kStreamBlock / 32);
+    const long long each = ctx->cfg.cluster_size > 0 ? ctx->cfg.cluster_size : (blocks + units - 1) / units;
+    info->cluster_size = static_cast<int32_t>(each);
+    info->max_clusters = static_cast<int32_t>((2LL * ctx->sm_count + each - 1) / each);
+  }
+  info->threads_per_block = kStreamBlock;
   info->sm_count = ctx->sm_count;
   {
-    // ordinary runs (no test hook): one launch at T = 0; else stage 0 and the one-sweep drawing stage where it
-    // applies (see one_sweep_stage), stages 0, 1 and 2 otherwise
-    const int mode = mode_of(ctx->cfg);
-    const bool one_sweep = one_sweep_stage(ctx->cfg) != 0 || (ctx->fused && ctx->draw_fused);
-    info->launches_per_run = (ctx->cfg.temperature > 0.0f && !(ctx->fused && ctx->use_fused)) ? (one_sweep ? 2 : 3) : 1;
+    // ordinary runs (no test hook): one launch at T = 0; else the streaming launch and one or two that draw; one more for
+    // the mask
+    const bool one_draw = !draw_split(ctx->cfg) || (ctx->fused && ctx->draw_fused);
+    info->launches_per_run = (ctx->cfg.temperature > 0.0f && !(ctx->fused && ctx->use_fused)) ? (one_draw ? 2 : 3) : 1;
+    if (ctx->cfg.combine == COS_COMBINE_LOGIT_LINEAR && ctx->cfg.mask_model >= 0) ++info->launches_per_run;
   }
-  info->reserved[0] = ctx->fused ? ctx->fplan.chunks : ctx->parts;
-  info->reserved[1] = ctx->fused ? ctx->fplan.dchunks : ctx->parts_one;
+  info->reserved[0] = ctx->fused ? ctx->fplan.chunks : 1;
+  info->reserved[1] = ctx->fused ? ctx->fplan.dchunks : 1;
   info->reserved[2] = ((ctx->fused && ctx->use_fused) ? 1 : 0) | ((ctx->fused && ctx->draw_fused) ? 2 : 0);
   return COS_OK;
 }
@@ -873,13 +741,12 @@ extern "C" cos_status cos_verify_destroy(cos_verify_ctx* ctx) {
   cudaFree(ctx->d_job_count);
   cudaFree(ctx->d_jobs);
   cudaFree(ctx->d_ustats);
-  cudaFree(ctx->d_zpart);
-  cudaFree(ctx->d_wtotg);
-  cudaFree(ctx->d_srung);
-  cudaFree(ctx->d_srungB);
-  cudaFree(ctx->d_srungC);
-  cudaFree(ctx->d_srungD);
-  cudaFree(ctx->d_part_arrivals);
+  cudaFree(ctx->d_st_rec);
+  cudaFree(ctx->d_st_arrivals);
+  cudaFree(ctx->d_mask_key);
+  cudaFree(ctx->d_row_draw);
+  cudaFree(ctx->d_draw_rec);
+  cudaFree(ctx->d_draw_arrivals);
   for (int k = 0; k < 4; ++k)
     if (ctx->ev[k]) cudaEventDestroy(ctx->ev[k]);
   cudaFree(ctx->d_unit_res);
@@ -908,10 +775,12 @@ namespace {
 
 // Scratch of the context-free entry point.  It is part of the library image: every device
 // that loads the library holds these COS_STATIC_SCRATCH_BYTES until the process exits.
-// Layout: [0, 256) work and job counters | row arrival counters | unit results | job list | unit statistics |
-// partial normalisers | run masses | running totals of the drawing unit of each row.
+// Layout: [0, 256) unused | arrival counters and mask keys | unit results | records of the streaming launch | unit
+// statistics | drawing positions | records of the drawing launch (kStaticDrawDoubles numbers).
 static __device__ __align__(256) unsigned char g_static_scratch[COS_STATIC_SCRATCH_BYTES];
 
+constexpr long long kStaticDrawDoubles = 16LL * (COS_STATIC_MAX_POSITIONS + 8 * COS_STATIC_MAX_BATCH);
+constexpr int kStaticWorkers = 5120;  // warps of a streaming launch there is room for
 constexpr int kStaticMaxDevices = 64;
 // Device address of g_static_scratch per device.  In host code the symbol itself is only a
 // stand-in, never an address a kernel may use, so the address is asked for once per device.
@@ -963,7 +832,6 @@ extern "C" cos_status cos_verify_run_static(const cos_verify_config* config, con
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   cudaError_t e = cudaSetDevice(c.device);
   if (e != cudaSuccess) return cuda_fail(nullptr, "cudaSetDevice", e);
-  KernelFn fn = pick_kernel(c.dtype, mode_of(c), 0);
   {
     std::lock_guard<std::mutex> guard(g_static_mutex);
     if (!g_static_ready[c.device]) {
@@ -975,68 +843,51 @@ extern "C" cos_status cos_verify_run_static(const cos_verify_config* config, con
       g_static_ready[c.device] = true;
     }
   }
-  e = prepare_kernels(c.dtype, mode_of(c), c.cluster_size);
-  if (e != cudaSuccess) return cuda_fail(nullptr, "cudaFuncSetAttribute", e);
   int sm_count = 0;
   e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, c.device);
   if (e != cudaSuccess) return cuda_fail(nullptr, "cudaDeviceGetAttribute", e);
-  const int c0 = choose_stream_cluster(c, static_cast<int>(units), sm_count);
-  int mc0 = 0;
-  e = query_clusters(fn, c0, sm_count, &mc0);
-  if (e != cudaSuccess) return cuda_fail(nullptr, "cudaOccupancyMaxActiveClusters", e);
-  if (mc0 < 1) return static_fail(COS_ERR_UNSUPPORTED, "no cluster of the requested size fits on the device");
 
-  // carve the array; what must start clean is cleared on the caller's stream before the kernels
+  // carve the array; what must start clean comes first and is cleared on the caller's stream before the kernels
+  const bool draws = c.temperature > 0.0f;
+  const bool all = draws && ((a->dump_r != nullptr) || (a->flags & COS_RUN_ALL_RESIDUALS));
+  const bool masked = c.combine == COS_COMBINE_LOGIT_LINEAR && c.mask_model >= 0;
+  const size_t n_units = static_cast<size_t>(units), n_rows = static_cast<size_t>(a->batch);
   unsigned char* basep = g_static_addr[c.device];
-  unsigned* d_counter = reinterpret_cast<unsigned*>(basep);
-  int* d_job_count = reinterpret_cast<int*>(basep + 16);
   int* d_arrivals = reinterpret_cast<int*>(basep + 256);
-  int4* d_unit_res = reinterpret_cast<int4*>(basep + 256 + 4 * COS_STATIC_MAX_BATCH);
-  int2* d_jobs = reinterpret_cast<int2*>(reinterpret_cast<unsigned char*>(d_unit_res) + 16 * COS_STATIC_MAX_POSITIONS);
-  UnitStats* d_ustats = reinterpret_cast<UnitStats*>(reinterpret_cast<unsigned char*>(d_jobs) +
-                                                      8 * (COS_STATIC_MAX_POSITIONS + COS_STATIC_MAX_BATCH));
-  static_assert(sizeof(UnitStats) == 112, "COS_STATIC_SCRATCH_BYTES assumes 112 bytes of statistics per position");
-  // one block per unit in the drawing stages here (parts = 1), which keeps the built-in array small
-  double* d_zpart = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(d_ustats) + 112 * COS_STATIC_MAX_POSITIONS);
-  double* d_wtotg = d_zpart + 8 * COS_STATIC_MAX_POSITIONS;
-  double* d_srung = d_wtotg + 16 * COS_STATIC_MAX_POSITIONS;
-  int* d_part_arrivals = reinterpret_cast<int*>(d_srung + 16 * 16 * COS_STATIC_MAX_BATCH);
-  static_assert(kWarps == 16 && kRecG == 16, "COS_STATIC_SCRATCH_BYTES assumes 16 runs and 16 recorded totals per run");
-  e = cudaMemsetAsync(basep, 0, 256, stream);  // work counter and both job counters
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_arrivals, 0, static_cast<size_t>(a->batch) * sizeof(int), stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_part_arrivals, 0, static_cast<size_t>(units) * sizeof(int), stream);
+  int* d_st_arrivals = d_arrivals + n_rows;
+  int* d_draw_arrivals = d_st_arrivals + n_units;
+  unsigned* d_mask_key = reinterpret_cast<unsigned*>(d_draw_arrivals + (draws ? (all ? n_units : n_rows) : 0));
+  e = cudaMemsetAsync(basep, 0, reinterpret_cast<unsigned char*>(d_mask_key + (masked ? n_units : 0)) - basep, stream);
   if (e != cudaSuccess) return cuda_fail(nullptr, "clearing the built-in scratch", e);
+  int4* d_unit_res = reinterpret_cast<int4*>(basep + 256 + 4 * (COS_STATIC_MAX_BATCH + 3 * COS_STATIC_MAX_POSITIONS));
+  int4* d_st_rec = d_unit_res + COS_STATIC_MAX_POSITIONS;
+  UnitStats* d_ustats = reinterpret_cast<UnitStats*>(d_st_rec + COS_MAX_MODELS * COS_STATIC_MAX_POSITIONS + kStaticWorkers);
+  static_assert(sizeof(UnitStats) == 112, "COS_STATIC_SCRATCH_BYTES assumes 112 bytes of statistics per position");
+  int* d_row_draw = reinterpret_cast<int*>(d_ustats + COS_STATIC_MAX_POSITIONS);
+  double* d_draw_rec = reinterpret_cast<double*>(d_row_draw + COS_STATIC_MAX_BATCH);
 
   KParams p;
   fill_params(c, a, p);
   p.num_units = static_cast<int>(units);
-  p.work_counter = d_counter;
-  p.exit_count = d_counter + 1;
   p.row_arrivals = d_arrivals;
   p.row_reject = nullptr;  // the hint to leave positions unread is not taken here
   p.early_exit = 0;
   p.unit_res = d_unit_res;
-  p.job_count = d_job_count;
-  p.jobs = d_jobs;
   p.ustats = d_ustats;
-  p.zpart = d_zpart;
-  p.wtotg = d_wtotg;
-  p.srung = d_srung;
-  p.part_arrivals = d_part_arrivals;
-  p.parts = 1;
-  p.max_jobs = p.num_units + a->batch;
+  p.st_rec = d_st_rec;
+  p.st_arrivals = d_st_arrivals;
+  p.mask_key = d_mask_key;
+  p.row_draw = d_row_draw;
+  p.draw_rec = d_draw_rec;
+  p.draw_arrivals = d_draw_arrivals;
 
-  p.num_clusters = p.num_units < mc0 ? p.num_units : mc0;
-  e = launch_stage(c.dtype, mode_of(c), 0, p, c0, stream);
-  if (e != cudaSuccess) return cuda_fail(nullptr, "kernel launch (stage 0)", e);
-  if (mode_of(c) == kEnsembleSample || mode_of(c) == kLogitSample) {
-    const bool all = (a->dump_r != nullptr) || (a->flags & COS_RUN_ALL_RESIDUALS);
-    const int most = all ? p.max_jobs : a->batch;
-    for (int st = 1; st <= 2; ++st) {
-      p.num_clusters = most < 4096 ? most : 4096;
-      e = launch_stage(c.dtype, mode_of(c), st, p, 1, stream);
-      if (e != cudaSuccess) return cuda_fail(nullptr, "kernel launch (drawing stages)", e);
-    }
+  long long workers = stream_workers(c, units, sm_count);
+  if (workers > kStaticWorkers) workers = kStaticWorkers;
+  e = launch_stream(c, mode_of(c), p, workers, sm_count, stream);
+  if (e != cudaSuccess) return cuda_fail(nullptr, "kernel launch (streaming)", e);
+  if (draws) {
+    e = launch_draw(c, p, all, sm_count, kStaticDrawDoubles / (2 * draw_channels(c)), stream);
+    if (e != cudaSuccess) return cuda_fail(nullptr, "kernel launch (drawing)", e);
   }
   return COS_OK;
 }
