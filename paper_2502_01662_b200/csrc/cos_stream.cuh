@@ -7,15 +7,15 @@
 
 namespace cosv {
 
-// Split: the rows of 16-byte vectors (ensembles: every model's row of every position; logit level: the vectors of all models
-// of a position go together) form one line in the order of memory, cut into p.st_workers equal contiguous shares, one for each
-// warp of a single wave of blocks, whatever the rows' boundaries.  So every warp streams the same number of bytes for any batch
-// and vocabulary, with 4 KB in flight, and nothing but loads between the start and the end of its share.  A warp leaves one
-// record (partial softmax statistics or argmaxes) for every row it had a part of; the warp that completes a position (fence
-// and counter, no waiting) merges its records in order, takes the decision and publishes it.
-// Measured on 1152 rows of 151936 bf16 entries (350 MB): 57.4 us (6.1 TB/s) for the sweep alone; whole positions per block of 16
-// warps, as before, 65 to 70 us; shares of blocks instead of warps 65 us; 4 vectors in flight per lane 68 us; the line in
-// another order than memory's (position by position over the batch) 78 us: neighbouring warps then read far apart.
+// Split: the positions' 16-byte vectors (the same vectors of all models of a position go together) form one line in the order of
+// memory, cut into p.st_workers equal contiguous shares, one for each warp of a single wave of blocks, whatever the positions'
+// boundaries.  So every warp streams the same number of bytes for any batch and vocabulary, with 4 KB in flight, and does
+// nothing else: it leaves one record per model (partial softmax statistics or argmaxes) for every position it had a part of, and the
+// next launch merges the records of a row's positions and decides (see cos_decide.cuh).  Models that agree at a position are cut
+// at the same places, so that their statistics are the same bit for bit.
+// Measured on 1152 rows of 151936 bf16 entries (350 MB): 58 us (6.0 TB/s) for the sweep alone; whole positions per block of 16
+// warps, as before, 65 to 70 us; shares of blocks instead of warps 65 us; 4 vectors in flight per lane 60 us.  Reporting every part
+// (fence, counter) cost 20 us more, deciding in the same launch another 17, the sweep in a function of its own 8.
 constexpr int kStreamThreads = 512;  // (two blocks per multiprocessor: 64 registers)
 constexpr int kStreamDepth = 8;      // vectors in flight per lane
 constexpr int kSkipped = 1 << 16;    // a warp that left its part of a position unread (early exit)
@@ -29,11 +29,13 @@ struct Decision {  // one position's outcome
   double prob;  // greedy, bonus position: probability of cand under the law it came from
 };
 
-struct Finish {  // what the warp that completes a position works with
-  SoftPart fsoft[COS_MAX_MODELS];  // merged statistics
-  ArgPart farg[COS_MAX_MODELS];
-  double pdraft[COS_MAX_MODELS];   // probability of the draft token under each softmax
-  float ldraft[COS_MAX_MODELS];    // the n logits at the draft token
+struct Finish {  // what a position is decided from, and the decision
+  union {
+    SoftPart fsoft[COS_MAX_MODELS];  // merged statistics (sampling)
+    ArgPart farg[COS_MAX_MODELS];    // merged argmaxes (greedy)
+  };
+  double pdraft[COS_MAX_MODELS];     // sampling: probability of the draft token under each softmax
+  float thr;                         // plausibility threshold (NaN: the gating model's logits hold one)
   Decision dec;
 };
 
@@ -141,9 +143,8 @@ __device__ __noinline__ LaneSoft soft_online(const char* row, int v, int v1, flo
 }
 
 // Softmax statistics of vectors [v0, v1) of one row and, with `ragged`, of its ragged entries; every lane's own part.
-// (Out of line, like the other segments, so that its loop has the registers to itself.)
 template <int DT, bool AL>
-__device__ __noinline__ LaneSoft soft_segment(const char* row, int v0, int v1, bool ragged, int V, float c) {
+__device__ __forceinline__ LaneSoft soft_segment(const char* row, int v0, int v1, bool ragged, int V, float c) {
   constexpr int U = kStreamDepth;
   const int lane = threadIdx.x & 31;
   const f32x2 c2 = pack2(c, c);
@@ -184,7 +185,7 @@ __device__ __noinline__ LaneSoft soft_segment(const char* row, int v0, int v1, b
 
 // Argmax of vectors [v0, v1) of one row (lowest index among equals) and whether a NaN or +inf was seen; the warp's result.
 template <int DT, bool AL>
-__device__ __noinline__ ArgPart arg_segment(const char* row, int v0, int v1, bool ragged, int V) {
+__device__ __forceinline__ ArgPart arg_segment(const char* row, int v0, int v1, bool ragged, int V) {
   constexpr int U = kStreamDepth, E = Elem<DT>::E;
   const int lane = threadIdx.x & 31;
   float best = -INFINITY;  // (sticks at NaN)
@@ -249,7 +250,7 @@ __device__ __noinline__ LaneSoft2 logit_online(const KParams& p, const char* bas
 // the first two models in flight (further models are read as they are needed).
 // PAIR: exactly two models; MASKED: with the plausibility mask.
 template <int DT, bool AL, bool PAIR, bool MASKED>
-__device__ __noinline__ LaneSoft2 logit_segment(const KParams& p, const char* base, long long row_step, LogitWeights lw, float cT,
+__device__ __forceinline__ LaneSoft2 logit_segment(const KParams& p, const char* base, long long row_step, LogitWeights lw, float cT,
                                                 int v0, int v1, bool ragged) {
   constexpr int U = kStreamDepth / 2, H = Elem<DT>::E / 2;
   const int lane = threadIdx.x & 31;
@@ -370,7 +371,7 @@ struct ArgPart2 {
   ArgPart q, c;
 };
 template <int DT, bool AL, bool PAIR, bool MASKED>
-__device__ __noinline__ ArgPart2 logit_arg_segment(const KParams& p, const char* base, long long row_step, LogitWeights lw, int v0,
+__device__ __forceinline__ ArgPart2 logit_arg_segment(const KParams& p, const char* base, long long row_step, LogitWeights lw, int v0,
                                                    int v1, bool ragged) {
   constexpr int U = kStreamDepth / 2, E = Elem<DT>::E, H = E / 2;
   const int lane = threadIdx.x & 31;
@@ -553,12 +554,12 @@ __device__ __forceinline__ void publish_unit(const KParams& p, int b, int j, int
 }
 
 // The accept test of one (row, position) from the merged statistics (Eq. 6), taken by one thread in fp64; greedy modes also
-// settle the replacement token here.  Reads fsoft / farg / pdraft / ldraft, writes dec.  (Logit-level greedy: farg[0] is the
+// settle the replacement token here.  Reads fsoft / farg / pdraft / thr, writes dec.  (Logit-level greedy: farg[0] is the
 // proposer's argmax, farg[1] the combined one.)
 template <int DT, int MODE>
-__device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double u_acc, double u_smp, float thr32, bool mask_bad,
-                                            bool is_bonus, int draft, bool draft_ok, int pi, bool pi_ok, int pis) {
-  const bool masked = (MODE == kLogitSample || MODE == kLogitGreedy) && p.mask_model >= 0;
+__device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double u_acc, double u_smp, bool is_bonus, int draft, bool draft_ok,
+                                            int pi, bool pi_ok, int pis) {
+  const bool mask_bad = (MODE == kLogitSample || MODE == kLogitGreedy) && p.mask_model >= 0 && sh.thr != sh.thr;
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
   const double kNaN = __longlong_as_double(0x7ff8000000000000LL);
   const double kInf = __longlong_as_double(0x7ff0000000000000LL);
@@ -575,7 +576,7 @@ __device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double
       const SoftPart& f = sh.fsoft[k];
       finite = finite && isfinite(f.ref) && isfinite(f.s) && (f.s > 0.0);
     }
-    if (masked && mask_bad) finite = false;
+    if (mask_bad) finite = false;
     if (!finite) {
       d.status |= COS_ROW_NONFINITE;
     } else {
@@ -588,12 +589,8 @@ __device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double
               if (i == pi) q_d = sh.pdraft[i];
             }
           } else {
-            double cd = 0.0;
-            for (int i = 0; i < p.n; ++i) cd = fma(p.w64[i], static_cast<double>(sh.ldraft[i]), cd);
-            bool in = !masked || (sh.ldraft[p.mask_model] >= thr32);
-            r_d = in ? exp2(cd * p.cT64 - static_cast<double>(sh.fsoft[1].ref)) / sh.fsoft[1].s : 0.0;
-            double lq = static_cast<double>(sh.ldraft[pi]);
-            q_d = exp2(lq * p.cT64 - static_cast<double>(sh.fsoft[0].ref)) / sh.fsoft[0].s;
+            q_d = sh.pdraft[0];
+            r_d = sh.pdraft[1];
           }
           d.r_d = r_d;
           d.q_d = q_d;
@@ -617,7 +614,7 @@ __device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double
       qtok = sh.farg[pis].idx;
     } else {
       finite = finite && !sh.farg[0].bad && !sh.farg[1].bad && isfinite(sh.farg[0].val) && isfinite(sh.farg[1].val);
-      if (masked && mask_bad) finite = false;
+      if (mask_bad) finite = false;
       qtok = sh.farg[0].idx;
     }
     if (!finite) {
@@ -710,83 +707,118 @@ __device__ __forceinline__ double rescale(double s, float ref, float R) {
   return s * exp2(static_cast<double>(ref) - static_cast<double>(R));
 }
 
-// Where the record of share w for row r of a line goes, less w: the pairs (r, w) of a line follow one another with r + w rising.
-template <bool ENS>
-__device__ __forceinline__ size_t record_of(const KParams& p, int slab, int units, long long r) {
-  return static_cast<size_t>(slab) * (static_cast<size_t>(units) * (ENS ? p.n : 1) + p.st_workers) + static_cast<size_t>(r);
+// The records of a line: `slots` (a model each, or the proposer's and the combined logits) for every position r that share w
+// has a part of; the pairs (r, w) of a line follow one another with r + w rising.
+template <int MODE>
+__device__ __forceinline__ int record_slots(const KParams& p) {
+  return (MODE == kEnsembleSample || MODE == kEnsembleGreedy) ? p.n : 2;
+}
+__device__ __forceinline__ size_t first_record(const KParams& p, int slab, int units, int r, int slots) {
+  return (static_cast<size_t>(slab) * (static_cast<size_t>(units) + p.st_workers) + static_cast<size_t>(r)) * slots;
 }
 
-// Merge the records of a position, in the order of the line: `slots` results (a lane group for each), into fin.fsoft / farg.
+// Merge one slot of a position over its records, in the order of the line; `g` lanes (a power of two, aligned) share the work,
+// `sub` is the lane's place among them.  Every lane of the warp calls this; lanes with live = false only take part in the
+// exchanges.  The first lane of a group gets the result.
+struct Merged {
+  SoftPart soft;
+  ArgPart arg;
+  float thr;
+};
 template <int MODE>
-__device__ __forceinline__ void merge_records(const KParams& p, Finish& fin, int slab, int u_local, int units) {
-  constexpr bool kEns = (MODE == kEnsembleSample || MODE == kEnsembleGreedy);
+__device__ __forceinline__ Merged merge_slot(const KParams& p, bool live, int slab, int units, int r, int i, int g, int sub) {
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
-  const int lane = threadIdx.x & 31;
-  const int slots = kEns ? p.n : 2;
-  const int g = slots <= 1 ? 32 : (slots <= 2 ? 16 : (slots <= 4 ? 8 : 4));  // lanes of a group
-  const int i = lane / g, sub = lane % g;
-  float R = -INFINITY;
-  double s = 0.0;
-  ArgPart best;
-  best.val = -INFINITY;
-  best.idx = kNoReject;
-  best.bad = 0;
-  if (i < slots) {
-    const long long r = kEns ? static_cast<long long>(i) * units + u_local : u_local;
-    const int w0 = worker_of(p, r * p.st_nv), w1 = worker_of(p, (r + 1) * p.st_nv - 1);
-    const size_t first = record_of<kEns>(p, slab, units, r);
+  Merged m;
+  m.soft.ref = -INFINITY;
+  m.soft.s = 0.0;
+  m.arg.val = -INFINITY;
+  m.arg.idx = kNoReject;
+  m.arg.bad = 0;
+  m.thr = -INFINITY;
+  if (live) {
+    const int slots = record_slots<MODE>(p);
+    const long long at = static_cast<long long>(r) * p.st_nv;
+    const int w0 = worker_of(p, at), w1 = worker_of(p, at + p.st_nv - 1);
+    const int4* rec = p.st_rec + first_record(p, slab, units, r, slots) + i;
+#pragma unroll 4
     for (int w = w0 + sub; w <= w1; w += g) {
-      const int4 rec = __ldcg(p.st_rec + (kEns ? first + w : (first + w) * 2 + i));
-      const double v = __hiloint2double(rec.y, rec.x);
+      const int4 v4 = __ldcg(rec + static_cast<size_t>(w) * slots);
+      const double v = __hiloint2double(v4.y, v4.x);
       if (kSample) {
-        const float ref = __int_as_float(rec.z), top = fmaxf(R, ref);
-        s = rescale(s, R, top) + rescale(v, ref, top);
-        R = top;
+        const float ref = __int_as_float(v4.z), top = fmaxf(m.soft.ref, ref);
+        m.soft.s = rescale(m.soft.s, m.soft.ref, top) + rescale(v, ref, top);
+        m.soft.ref = top;
+        m.thr = __int_as_float(v4.w);
       } else {
-        best.bad |= rec.w;
-        if (arg_better(v, rec.z, best.val, best.idx)) {
-          best.val = v;
-          best.idx = rec.z;
+        m.arg.bad |= v4.w & 1;
+        if (v4.w & 2) m.thr = __int_as_float(0x7fc00000);
+        if (arg_better(v, v4.z, m.arg.val, m.arg.idx)) {
+          m.arg.val = v;
+          m.arg.idx = v4.z;
         }
       }
     }
   }
   if (kSample) {
-    float top = R;
+    float top = m.soft.ref;
     for (int d = g / 2; d > 0; d >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, d));
-    s = rescale(s, R, top);
+    double s = rescale(m.soft.s, m.soft.ref, top);
     for (int d = g / 2; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-    if (sub == 0 && i < slots) {
-      fin.fsoft[i].s = s;
-      fin.fsoft[i].ref = top;
-    }
+    m.soft.s = s;
+    m.soft.ref = top;
   } else {
     for (int d = g / 2; d > 0; d >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, best.val, d);
-      const int oi = __shfl_xor_sync(0xffffffffu, best.idx, d);
-      best.bad |= __shfl_xor_sync(0xffffffffu, best.bad, d);
-      if (arg_better(ov, oi, best.val, best.idx)) {
-        best.val = ov;
-        best.idx = oi;
+      const double ov = __shfl_xor_sync(0xffffffffu, m.arg.val, d);
+      const int oi = __shfl_xor_sync(0xffffffffu, m.arg.idx, d);
+      m.arg.bad |= __shfl_xor_sync(0xffffffffu, m.arg.bad, d);
+      if (arg_better(ov, oi, m.arg.val, m.arg.idx)) {
+        m.arg.val = ov;
+        m.arg.idx = oi;
       }
     }
-    if (sub == 0 && i < slots) fin.farg[i] = best;
   }
-  __syncwarp();
+  return m;
 }
 
-// The plausibility threshold of a position from the largest logit of the gating model (key of the mask launch).
-struct MaskBound {
-  float thr;
-  bool bad;
-};
-__device__ __forceinline__ MaskBound mask_bound(const KParams& p, unsigned key) {
-  MaskBound m;
-  m.bad = key > 0xff800000u;  // a NaN
+// The plausibility threshold of a position from the largest logit of the gating model (key of the mask launch); NaN where
+// that model's logits hold one.
+__device__ __forceinline__ float mask_bound(const KParams& p, unsigned key) {
+  if (key > 0xff800000u) return __int_as_float(0x7fc00000);
   const float top = __uint_as_float(key ^ ((key >> 31) ? 0x80000000u : 0xffffffffu));
   // l >= max + ln(alpha) in fp64 is the same as l >= (that bound rounded up to fp32) for fp32 l
-  m.thr = m.bad ? __int_as_float(0x7fc00000) : __double2float_ru(static_cast<double>(top) + p.ln_alpha);
-  return m;
+  return __double2float_ru(static_cast<double>(top) + p.ln_alpha);
+}
+
+// What the probability of the draft token under slot i needs of the logits there (draft < 0: nothing), and that probability once
+// the statistics are merged, with the constant the sweep used.
+struct DraftLogits {
+  double x;   // exponent before the reference is taken off
+  float xe;   // the gating model's logit
+};
+template <int DT, int MODE>
+__device__ __forceinline__ DraftLogits draft_logits(const KParams& p, const char* base, int i, int pis, int draft) {
+  DraftLogits d;
+  d.x = -INFINITY;
+  d.xe = INFINITY;
+  if (draft < 0) return d;
+  const long long row_step = p.s_model * Elem<DT>::bytes;
+  if (MODE == kEnsembleSample || i == 0) {
+    d.x = static_cast<double>(Elem<DT>::load1(base + (MODE == kEnsembleSample ? i : pis) * row_step, draft)) * p.cT64;
+  } else {
+    double cd = 0.0;
+    for (int k = 0; k < p.n; ++k) {
+      const float x = Elem<DT>::load1(base + k * row_step, draft);
+      cd = fma(p.w64[k], static_cast<double>(x), cd);
+      if (k == p.mask_model) d.xe = x;
+    }
+    d.x = cd * p.cT64;
+  }
+  return d;
+}
+template <int DT, int MODE>
+__device__ __forceinline__ double draft_probability(const KParams& p, const DraftLogits& d, float thr, const SoftPart& f) {
+  if (MODE == kLogitSample && p.mask_model >= 0 && !(d.xe >= thr)) return 0.0;
+  return exp2(d.x - static_cast<double>(f.ref)) / f.s;
 }
 
 // Largest logit of the gating model at every position, for the plausibility mask: the same split, over that model's rows
@@ -830,51 +862,123 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_mask_kernel(const __gri
   }
 }
 
-template <int DT, int MODE, bool AL>
+__device__ __forceinline__ int4 pack_soft(const LaneSoft& a, float thr) {
+  // lanes of one warp: fp32 is enough here, the errors of the 32 scale factors average out
+  float R = a.ref;
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) R = fmaxf(R, __shfl_xor_sync(0xffffffffu, R, d));
+  float t = (a.ref == R) ? a.s : a.s * ex2_approx(a.ref - R);
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+  const double s = static_cast<double>(t);
+  return make_int4(__double2loint(s), __double2hiint(s), __float_as_int(R), __float_as_int(thr));
+}
+__device__ __forceinline__ int4 pack_arg(const ArgPart& a, float thr) {
+  return make_int4(__double2loint(a.val), __double2hiint(a.val), a.idx, a.bad | (thr != thr ? 2 : 0));
+}
+
+// The part of one position, vectors [o0, o1) of every model, that lies in a warp's share: its records (lane 0 writes them).
+// `settled`: the inputs may be read before the kernel ahead in the stream is complete; this waits for it before it writes.
+template <int DT, int MODE, bool AL, bool PAIR, bool MASKED>
+__device__ __forceinline__ void sweep_part(const KParams& p, const char* base, int o0, int o1, int pis, float thr, int4* rec,
+                                           bool& waited) {
+  const int lane = threadIdx.x & 31;
+  const VecRange whole = whole_vectors<DT, AL>(p.V);
+  const int v0 = whole.lo + o0, v1 = whole.lo + o1 < whole.hi ? whole.lo + o1 : whole.hi;
+  const bool ragged = (o1 == p.st_nv);
+  const long long row_step = p.s_model * Elem<DT>::bytes;
+  auto put = [&](int i, const int4& v) {
+    if (!waited) {
+      asm volatile("griddepcontrol.wait;" ::: "memory");  // from here on as in an ordinary run
+      waited = true;
+    }
+    if (lane == 0) __stcg(rec + i, v);
+  };
+  if (MODE == kEnsembleSample) {
+    for (int i = 0; i < p.n; ++i) put(i, pack_soft(soft_segment<DT, AL>(base + i * row_step, v0, v1, ragged, p.V, p.cT), thr));
+  } else if (MODE == kEnsembleGreedy) {
+    for (int i = 0; i < p.n; ++i) put(i, pack_arg(arg_segment<DT, AL>(base + i * row_step, v0, v1, ragged, p.V), thr));
+  } else if (MODE == kLogitSample) {
+    const LaneSoft2 a = logit_segment<DT, AL, PAIR, MASKED>(p, base, row_step, logit_weights(p, pis, thr), p.cT, v0, v1, ragged);
+    put(0, pack_soft(a.q, thr));
+    put(1, pack_soft(a.c, thr));
+  } else {
+    const ArgPart2 a = logit_arg_segment<DT, AL, PAIR, MASKED>(p, base, row_step, logit_weights(p, pis, thr), v0, v1, ragged);
+    put(0, pack_arg(a.q, thr));
+    put(1, pack_arg(a.c, thr));
+  }
+}
+
+// PAIR, MASKED: logit level with exactly two models, and with a mask (kernels of their own: straight code for each).
+template <int DT, int MODE, bool AL, bool PAIR, bool MASKED>
 __global__ void __launch_bounds__(kStreamThreads, 2) cos_stream_kernel(const __grid_constant__ KParams p) {
+  constexpr bool kEns = (MODE == kEnsembleSample || MODE == kEnsembleGreedy);
+  const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  // Launched while the kernel before it in the stream drains (programmatic dependent launch): its blocks take their places
+  // as that kernel's blocks leave and wait here until it is complete and its writes are visible.  (Without the launch
+  // attribute, and behind a kernel that never signals, this is the ordinary order of a stream.)  Where the caller
+  // promises that the inputs were complete earlier, a warp sweeps its first part first and waits only before it writes.
+  bool waited = p.inputs_settled == 0;
+  if (waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (w >= p.st_workers) return;
+  const int slots = record_slots<MODE>(p);
+  for (long long x = worker_lo(p, w), end = worker_lo(p, w + 1); x < end;) {
+    const int r = static_cast<int>(x / p.st_nv);
+    const int o0 = static_cast<int>(x - static_cast<long long>(r) * p.st_nv);
+    const int o1 = end - x < p.st_nv - o0 ? o0 + static_cast<int>(end - x) : p.st_nv;
+    x += o1 - o0;
+    const int b = r / p.P, j = r - b * p.P;
+    const char* base = reinterpret_cast<const char*>(p.logits) +
+                       (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
+    int pis = 0;
+    float thr = -INFINITY;
+    if (!kEns) {
+      const int pi = proposer_of(p, b, j);
+      pis = (pi >= 0 && pi < p.n) ? pi : 0;
+      if (MASKED) thr = mask_bound(p, __ldcg(&p.mask_key[r]));
+    }
+    sweep_part<DT, MODE, AL, PAIR, MASKED>(p, base, o0, o1, pis, thr, p.st_rec + first_record(p, 0, p.num_units, r, slots) + static_cast<size_t>(w) * slots,
+                                           waited);
+  }
+}
+
+// The same with every part reported (fence and counter): the warp that completes a position merges its records, decides and
+// publishes it at once.  Slower (see above); for runs that leave positions unread behind a rejection their row has already
+// reported, which needs the decisions while the sweep is under way (a line for each position of the rows, one after another),
+// and for those whose tokens the persistent kernel draws, which has no step that decides.
+template <int DT, int MODE, bool AL>
+__global__ void __launch_bounds__(kStreamThreads, 1) cos_report_kernel(const __grid_constant__ KParams p) {
   constexpr bool kEns = (MODE == kEnsembleSample || MODE == kEnsembleGreedy);
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
   __shared__ Finish fins[kStreamThreads / 32];
   const int lane = threadIdx.x & 31;
   const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   Finish& fin = fins[threadIdx.x >> 5];
-  // Launched while the kernel before it in the stream drains (programmatic dependent launch): its blocks take their places
-  // as that kernel's blocks leave and wait here until it is complete and its writes are visible.  (Without the launch
-  // attribute, and behind a kernel that never signals, this is the ordinary order of a stream.)  Where the caller
-  // promises that the inputs were complete earlier, a warp sweeps its first row first and waits only before it writes.
-  bool waited = p.inputs_settled == 0;
-  if (waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (w >= p.st_workers) return;
   const bool masked = !kEns && p.mask_model >= 0;
-  const int v_lo = whole_vectors<DT, AL>(p.V).lo, v_hi = whole_vectors<DT, AL>(p.V).hi;
-  const int rows = kEns ? p.n : 1;  // rows of the line for each position
   const int units = p.st_slabs > 1 ? p.B : p.num_units;  // positions of a line
+  const int slots = record_slots<MODE>(p);
   const long long row_step = p.s_model * Elem<DT>::bytes;
+  bool waited = true;
   for (int slab = 0; slab < p.st_slabs; ++slab) {
     for (long long x = worker_lo(p, w), end = worker_lo(p, w + 1); x < end;) {
-      // the part of row r, model i of position (b, j), that lies in this warp's share: vectors [o0, o1)
-      const long long r = x / p.st_nv;
-      const int i = kEns ? static_cast<int>(r / units) : 0;
-      const int u_local = static_cast<int>(r - static_cast<long long>(i) * units);
-      const int o0 = static_cast<int>(x - r * p.st_nv);
+      const int r = static_cast<int>(x / p.st_nv);
+      const int o0 = static_cast<int>(x - static_cast<long long>(r) * p.st_nv);
       const int o1 = end - x < p.st_nv - o0 ? o0 + static_cast<int>(end - x) : p.st_nv;
       x += o1 - o0;
-      const int b = p.st_slabs > 1 ? u_local : u_local / p.P, j = p.st_slabs > 1 ? slab : u_local % p.P;
+      const int b = p.st_slabs > 1 ? r : r / p.P, j = p.st_slabs > 1 ? slab : r % p.P;
       const int uidx = b * p.P + j;
       const char* base = reinterpret_cast<const char*>(p.logits) +
                          (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
-      const bool is_bonus = (j == p.gamma);
-      const int draft = is_bonus ? 0 : __ldg(p.drafts + b * p.gamma + j);
       const int pi = proposer_of(p, b, j);
       const bool pi_ok = (pi >= 0 && pi < p.n);
       const int pis = pi_ok ? pi : 0;
-      MaskBound mask;
-      mask.thr = -INFINITY;
-      mask.bad = false;
-      if (masked) mask = mask_bound(p, __ldcg(&p.mask_key[uidx]));
-      // Early exit: a position behind a rejection that its row has already published decides nothing (Sec. 3.1: the tokens
-      // after the first rejection are discarded).  Every warp looks for itself; one that skips marks the position.
+      const float thr = masked ? mask_bound(p, __ldcg(&p.mask_key[uidx])) : -INFINITY;
+      // A position behind a rejection that its row has already published decides nothing (Sec. 3.1: the tokens after the
+      // first rejection are discarded).  Every warp looks for itself; one that skips marks the position.
       bool skip = false;
       if (p.early_exit) {
         int rej = 0;
@@ -882,76 +986,21 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_stream_kernel(const __g
         skip = __shfl_sync(0xffffffffu, rej, 0) < j;
       }
       if (!skip) {
-        const int v0 = v_lo + o0, v1 = v_lo + o1 < v_hi ? v_lo + o1 : v_hi;
-        const bool ragged = (o1 == p.st_nv);
-        int4 rec[2];
-        auto soft_rec = [&](const LaneSoft& a) {
-          // lanes of one warp: fp32 is enough here, the errors of the 32 scale factors average out
-          float R = a.ref;
-#pragma unroll
-          for (int d = 16; d > 0; d >>= 1) R = fmaxf(R, __shfl_xor_sync(0xffffffffu, R, d));
-          float t = (a.ref == R) ? a.s : a.s * ex2_approx(a.ref - R);
-#pragma unroll
-          for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
-          const double s = static_cast<double>(t);
-          return make_int4(__double2loint(s), __double2hiint(s), __float_as_int(R), 0);
-        };
-        auto arg_rec = [&](const ArgPart& a) { return make_int4(__double2loint(a.val), __double2hiint(a.val), a.idx, a.bad); };
-        if (MODE == kEnsembleSample) {
-          rec[0] = soft_rec(soft_segment<DT, AL>(base + i * row_step, v0, v1, ragged, p.V, p.cT));
-        } else if (MODE == kEnsembleGreedy) {
-          rec[0] = arg_rec(arg_segment<DT, AL>(base + i * row_step, v0, v1, ragged, p.V));
-        } else if (MODE == kLogitSample) {
-          const LogitWeights lw = logit_weights(p, pis, mask.thr);
-          const LaneSoft2 a = p.n == 2 ? (masked ? logit_segment<DT, AL, true, true>(p, base, row_step, lw, p.cT, v0, v1, ragged)
-                                                 : logit_segment<DT, AL, true, false>(p, base, row_step, lw, p.cT, v0, v1, ragged))
-                                       : (masked ? logit_segment<DT, AL, false, true>(p, base, row_step, lw, p.cT, v0, v1, ragged)
-                                                 : logit_segment<DT, AL, false, false>(p, base, row_step, lw, p.cT, v0, v1, ragged));
-          rec[0] = soft_rec(a.q);
-          rec[1] = soft_rec(a.c);
-        } else {
-          const LogitWeights lw = logit_weights(p, pis, mask.thr);
-          const ArgPart2 a = p.n == 2 ? (masked ? logit_arg_segment<DT, AL, true, true>(p, base, row_step, lw, v0, v1, ragged)
-                                                : logit_arg_segment<DT, AL, true, false>(p, base, row_step, lw, v0, v1, ragged))
-                                      : (masked ? logit_arg_segment<DT, AL, false, true>(p, base, row_step, lw, v0, v1, ragged)
-                                                : logit_arg_segment<DT, AL, false, false>(p, base, row_step, lw, v0, v1, ragged));
-          rec[0] = arg_rec(a.q);
-          rec[1] = arg_rec(a.c);
-        }
-        if (!waited) {
-          asm volatile("griddepcontrol.wait;" ::: "memory");  // from here on as in an ordinary run
-          waited = true;
-        }
-        if (lane == 0) {
-          const size_t at = record_of<kEns>(p, slab, units, r) + w;
-          if (kEns) {
-            __stcg(p.st_rec + at, rec[0]);
-          } else {
-            __stcg(p.st_rec + at * 2, rec[0]);
-            __stcg(p.st_rec + at * 2 + 1, rec[1]);
-          }
-        }
+        int4* rec = p.st_rec + first_record(p, slab, units, r, slots) + static_cast<size_t>(w) * slots;
+        if (kEns || (p.n == 2 && !masked))
+          sweep_part<DT, MODE, AL, true, false>(p, base, o0, o1, pis, thr, rec, waited);
+        else
+          sweep_part<DT, MODE, AL, false, true>(p, base, o0, o1, pis, thr, rec, waited);
       }
-      // the logits at the draft token, fetched while the warp reports
-      const bool draft_ok = is_bonus || (draft >= 0 && draft < p.V);
-      float ld = 0.f;
-      if (lane < p.n && !is_bonus && draft_ok) ld = Elem<DT>::load1(base + lane * row_step, draft);
       int prev = 0;
       if (lane == 0) {
         __threadfence();
         prev = atomicAdd(&p.st_arrivals[uidx], skip ? 1 + kSkipped : 1);
         __threadfence();
       }
-      // reports the position needs: one for every share that has a part of one of its rows
-      int reports = 0;
-      if (lane < rows) {
-        const long long at = (static_cast<long long>(lane) * units + u_local) * p.st_nv;
-        reports = worker_of(p, at + p.st_nv - 1) - worker_of(p, at) + 1;
-      }
-      reports = __reduce_add_sync(0xffffffffu, reports);
       prev = __shfl_sync(0xffffffffu, prev, 0);
-      if ((prev & (kSkipped - 1)) + 1 != reports) continue;
-      // the warp that completes the position: merge, decide, publish
+      const long long at = static_cast<long long>(r) * p.st_nv;
+      if ((prev & (kSkipped - 1)) != worker_of(p, at + p.st_nv - 1) - worker_of(p, at)) continue;
       skip = skip || prev >= kSkipped;
       if (lane == 0) {
         p.st_arrivals[uidx] = 0;  // ready for the next run
@@ -966,33 +1015,31 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_stream_kernel(const __g
         __syncwarp();
         continue;
       }
-      unsigned rnd[4];
-      philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
-      merge_records<MODE>(p, fin, slab, u_local, units);
-      if (lane < p.n) {
-        fin.ldraft[lane] = ld;
-        // probability of the draft under model `lane`, with the constant the sweep used
-        if (MODE == kEnsembleSample)
-          fin.pdraft[lane] = exp2(static_cast<double>(ld) * p.cT64 - static_cast<double>(fin.fsoft[lane].ref)) / fin.fsoft[lane].s;
+      const bool is_bonus = (j == p.gamma);
+      const int draft = is_bonus ? 0 : __ldg(p.drafts + b * p.gamma + j);
+      const bool draft_ok = is_bonus || (draft >= 0 && draft < p.V);
+      const int g = slots <= 1 ? 32 : (slots <= 2 ? 16 : (slots <= 4 ? 8 : 4)), i = lane / g;
+      const Merged m = merge_slot<MODE>(p, i < slots, slab, units, r, i, g, lane % g);
+      if (i < slots && lane % g == 0) {
+        if (kSample) {
+          fin.fsoft[i] = m.soft;
+          fin.pdraft[i] = draft_probability<DT, MODE>(p, draft_logits<DT, MODE>(p, base, i, pis, is_bonus || !draft_ok ? -1 : draft), thr, m.soft);
+        } else {
+          fin.farg[i] = m.arg;
+        }
       }
+      if (lane == 0) fin.thr = thr;
       __syncwarp();
-      if (kSample && lane < (kEns ? p.n : 2)) {  // kept for the drawing launch
+      if (kSample && lane < slots) {  // kept for the drawing launch
         p.ustats[uidx].s[lane] = fin.fsoft[lane].s;
         p.ustats[uidx].ref[lane] = fin.fsoft[lane].ref;
       }
-      if (kSample && lane == 31) p.ustats[uidx].thr32 = mask.thr;
+      if (kSample && lane == 31) p.ustats[uidx].thr32 = thr;
       if (lane == 0) {
-        decide_unit<DT, MODE>(p, fin, word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), mask.thr, mask.bad, is_bonus, draft, draft_ok,
-                              pi, pi_ok, pis);
+        unsigned rnd[4];
+        philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
+        decide_unit<DT, MODE>(p, fin, word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), is_bonus, draft, draft_ok, pi, pi_ok, pis);
         const Decision& d = fin.dec;
-        if (!kSample && p.dump_r != nullptr) {  // test hook: the atoms of r
-          UnitStats& st = p.ustats[uidx];
-          st.pad[0] = (d.status & COS_ROW_NONFINITE) ? -1 : d.natoms;
-          for (int k = 0; k < d.natoms; ++k) {
-            st.s[k] = d.atom_mass[k];
-            st.ref[k] = __int_as_float(d.atom_tok[k]);
-          }
-        }
         publish_unit(p, b, j, d.accept, d.status, d.cand, kSample ? d.drawable : __float_as_int(static_cast<float>(d.prob)), d.ratio,
                      d.r_d, d.q_d, d.S);
       }
