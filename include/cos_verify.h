@@ -156,12 +156,12 @@ typedef struct {
   int32_t threads_per_block;
   int32_t max_clusters;      /* clusters that can be resident at once on the device                   */
   int32_t sm_count;
-  int32_t launches_per_run;  /* kernels an ordinary cos_verify_run enqueues: 1 at T = 0 and where the     */
-                             /* one-launch form was chosen (reserved[2] bit 0); else 2 for logit-level */
-                             /* combines and ensembles of two to four models, 3 otherwise.  Every      */
+  int32_t launches_per_run;  /* kernels an ordinary cos_verify_run enqueues: 1 where the one-launch form was    */
+                             /* chosen (reserved[2] bit 0); else 2, 3 for ensembles of one or of more than     */
+                             /* four models at T > 0, and one more with a plausibility mask.  Every            */
                              /* launch takes its places on the device while the kernel before it in    */
-                             /* the stream drains, and reads or writes nothing until that kernel is    */
-                             /* complete (unless COS_RUN_INPUTS_SETTLED says the inputs may be read)   */
+                             /* the stream drains, and reads or writes nothing that kernel may still write     */
+                             /* until it is complete (unless COS_RUN_INPUTS_SETTLED says the inputs may be read) */
   int32_t reserved[3];       /* [0], [1]: work items per position when streaming / drawing; [2]: bit  */
                              /* 0: an ordinary run is one launch; bit 1: the tokens of a staged run   */
                              /* are drawn by the persistent kernel's drawing items                    */
@@ -230,7 +230,7 @@ cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_args* args,
 #define COS_STATIC_MAX_POSITIONS 8192
 #define COS_STATIC_SCRATCH_BYTES                                                                          \
   (256 + 4 * (COS_STATIC_MAX_BATCH + 3 * COS_STATIC_MAX_POSITIONS) + 16 * COS_STATIC_MAX_POSITIONS +     \
-   16 * (COS_MAX_MODELS * COS_STATIC_MAX_POSITIONS + 5120) + 112 * COS_STATIC_MAX_POSITIONS +            \
+   16 * COS_MAX_MODELS * (COS_STATIC_MAX_POSITIONS + 5120) + 112 * COS_STATIC_MAX_POSITIONS +            \
    4 * COS_STATIC_MAX_BATCH + 8 * 16 * (COS_STATIC_MAX_POSITIONS + 8 * COS_STATIC_MAX_BATCH))
 cos_status cos_verify_run_static(const cos_verify_config* config, const cos_verify_args* args, void* cuda_stream);
 

@@ -74,16 +74,18 @@ struct KParams {
   int2* jobs;              // x = b * P + j of a unit that draws a token (y unused)
   UnitStats* ustats;       // [B*P]: merged statistics of sweep 1, read back by the later stages
   int use_jobs;            // the list of drawing positions is kept too (tokens drawn by the persistent kernel)
-  // the streaming launch: a line of st_line vectors (st_nv for each row of it) in st_workers shares, st_rem of them of st_q + 1
+  // the streaming launch: a line of st_line vectors (st_nv for each position) in st_workers shares, st_rem of them of st_q + 1
   // groups of eight vectors, the others of st_q; st_slabs lines one after another (one, or one for each position of a row)
   int st_workers, st_slabs, st_nv;
   long long st_line, st_q, st_rem;
-  int4* st_rec;            // records: statistics of a share's part of a row
+  int4* st_rec;            // records: statistics of a share's part of a position
   int* st_arrivals;        // [B*P]: warps that have reported; zero between runs
   unsigned* mask_key;      // [B*P]: largest logit of the gating model as an ordered integer; zero between runs
   // the drawing launch
   int* row_draw;           // [B]: the position of the row that draws its token, or -1
   int draw_all;            // it visits every position (test hook, residual masses)
+  int decide;              // it also merges the records of the streaming launch and decides (else that is done)
+  int keep_stats;          // ustats, unit_res and row_draw are wanted afterwards
   int draw_parts;          // blocks that share a position
   int draw_cs, draw_chunks;  // steps of a chunk, chunks of a position
   double* draw_rec;        // [positions][chunks][2 channels]: sums of every chunk

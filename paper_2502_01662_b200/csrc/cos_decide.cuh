@@ -1,0 +1,175 @@
+// Decisions from the records of a streaming launch: accept tests of a row's positions (Eq. 6), the first rejection and the
+// row's outputs (Sec. 3.1).
+#ifndef COS_DECIDE_CUH
+#define COS_DECIDE_CUH
+
+#include "cos_stream.cuh"
+
+namespace cosv {
+
+// A block decides a whole row: a few lanes merge the records of one (position, slot) pair each, one thread takes the accept test
+// of a position, a ballot finds the first rejection.  Every block of a row does it for itself (the records of a row are a
+// few KB, read from L2), which costs the device nothing that it would use otherwise and no word has to travel between blocks;
+// one of them writes the outputs.  It is a chain of latencies: what it needs of the inputs (drafts, proposers, the logits at the
+// drafts) is fetched before the launch waits for the streaming launch to end.
+constexpr int kTile = 16;  // positions decided at a time
+
+struct RowShared {
+  Finish fin[kTile];
+  int a;            // the row's first rejected position, or gamma; -1 until it is known
+  int drawable;     // whether a token can be drawn there
+  int cand;         // greedy: the token there
+  float prob;       // greedy: the bonus token's probability
+  unsigned status;  // status bits up to there
+};
+
+// Decide row b.  `want` >= 0: a position whose statistics the block needs, whatever the first rejection; otherwise the first
+// rejected position is what it needs.  `keep(fin, j)` is called by every thread, between two barriers, with that
+// position's merged statistics.  `writes_row(a)` / `writes_unit(j)`: whether this block writes the row's outputs and a
+// position's optional ones.
+template <int DT, int MODE, typename K, typename WR, typename WU>
+__device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int b, int want, K keep, WR writes_row, WU writes_unit) {
+  constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
+  const int tid = threadIdx.x, lane = tid & 31, T = blockDim.x;
+  const int slots = record_slots<MODE>(p);
+  const bool optional = p.diag != nullptr || p.keep_stats;
+  // lanes that share a pair: as many as the block has to spare
+  const int pairs0 = (p.P < kTile ? p.P : kTile) * slots;
+  int g = 32;
+  while (g > 1 && pairs0 * g > T) g >>= 1;
+  const int per = T / g, mine = tid / g, sub = tid % g;
+  const char* row = reinterpret_cast<const char*>(p.logits) + static_cast<long long>(b) * p.s_row * Elem<DT>::bytes;
+  auto fetch = [&](int j0, int q) {  // the logits at the draft of pair q of the tile at j0
+    const int j = j0 + q / slots, i = q % slots;
+    DraftLogits d;
+    d.x = -INFINITY;
+    d.xe = INFINITY;
+    if (kSample && sub == 0 && j < p.gamma) {
+      const int draft = __ldg(p.drafts + b * p.gamma + j);
+      const int pi = (MODE == kLogitSample) ? proposer_of(p, b, j) : 0;
+      const int pis = (pi >= 0 && pi < p.n) ? pi : 0;
+      d = draft_logits<DT, MODE>(p, row + static_cast<long long>(j) * p.s_pos * Elem<DT>::bytes, i, pis,
+                                 draft >= 0 && draft < p.V ? draft : -1);
+    }
+    return d;
+  };
+  DraftLogits first = fetch(0, mine);
+  if (tid == 0) {
+    sh.a = -1;
+    sh.status = 0u;
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  for (int j0 = 0; j0 < p.P; j0 += kTile) {
+    const int count = p.P - j0 < kTile ? p.P - j0 : kTile;
+    for (int q0 = 0; q0 < count * slots; q0 += per) {  // (the same number of times for every lane of a warp)
+      const int q = q0 + mine, pos = q / slots, i = q % slots;
+      const bool live = q < count * slots;
+      const DraftLogits d = (j0 == 0 && q0 == 0) ? first : (live ? fetch(j0, q) : first);
+      const Merged m = merge_slot<MODE>(p, live, 0, p.num_units, b * p.P + j0 + pos, i, g, sub);
+      if (live && sub == 0) {
+        Finish& f = sh.fin[pos];
+        if (kSample) {
+          f.fsoft[i] = m.soft;
+          f.pdraft[i] = draft_probability<DT, MODE>(p, d, m.thr, m.soft);
+        } else {
+          f.farg[i] = m.arg;
+        }
+        if (i == slots - 1) f.thr = m.thr;
+      }
+    }
+    __syncthreads();
+    if (tid < count) {
+      const int j = j0 + tid;
+      const bool is_bonus = (j == p.gamma);
+      const int draft = is_bonus ? 0 : __ldg(p.drafts + b * p.gamma + j);
+      const bool draft_ok = is_bonus || (draft >= 0 && draft < p.V);
+      const int pi = proposer_of(p, b, j);
+      const bool pi_ok = (pi >= 0 && pi < p.n);
+      unsigned rnd[4];
+      philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
+      decide_unit<DT, MODE>(p, sh.fin[tid], word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), is_bonus, draft, draft_ok, pi, pi_ok, pi_ok ? pi : 0);
+    }
+    __syncthreads();
+    if (tid < 32 && sh.a < 0) {
+      const bool stop = lane < count && (!sh.fin[lane].dec.accept || j0 + lane == p.gamma);
+      const unsigned stops = __ballot_sync(0xffffffffu, stop);
+      const int k = stops ? __ffs(stops) - 1 : count - 1;
+      const unsigned st = __reduce_or_sync(0xffffffffu, lane <= k ? static_cast<unsigned>(sh.fin[lane].dec.status) : 0u);
+      if (lane == 0) {
+        sh.status |= st;
+        if (stops) {
+          const Decision& d = sh.fin[k].dec;
+          sh.a = j0 + k;
+          sh.drawable = d.drawable;
+          sh.cand = d.cand;
+          sh.prob = static_cast<float>(d.prob);
+        }
+      }
+    }
+    __syncthreads();
+    const int a = sh.a;
+    const int asked = want >= 0 ? want : a;
+    if (asked >= j0 && asked < j0 + count) keep(sh.fin[asked - j0], asked);
+    if (optional) {
+      for (int k = tid; k < count; k += T) {
+        const int j = j0 + k, uidx = b * p.P + j;
+        if (!writes_unit(j)) continue;
+        const Finish& f = sh.fin[k];
+        if (p.diag) {
+          float* d = p.diag + static_cast<long long>(uidx) * 4;
+          d[0] = static_cast<float>(f.dec.ratio);
+          d[1] = static_cast<float>(f.dec.r_d);
+          d[2] = static_cast<float>(f.dec.q_d);
+          d[3] = static_cast<float>(f.dec.S);
+        }
+        if (p.keep_stats) {
+          UnitStats& st = p.ustats[uidx];
+          if (kSample) {
+            for (int i = 0; i < slots; ++i) {
+              st.s[i] = f.fsoft[i].s;
+              st.ref[i] = f.fsoft[i].ref;
+            }
+            st.thr32 = f.thr;
+          } else {  // the atoms of r, for the test hook
+            st.pad[0] = (f.dec.status & COS_ROW_NONFINITE) ? -1 : f.dec.natoms;
+            for (int i = 0; i < f.dec.natoms; ++i) {
+              st.s[i] = f.dec.atom_mass[i];
+              st.ref[i] = __int_as_float(f.dec.atom_tok[i]);
+            }
+          }
+          p.unit_res[uidx] = make_int4(f.dec.accept, f.dec.status, f.dec.cand, f.dec.drawable);
+        }
+      }
+    }
+    if (MODE == kLogitSample || MODE == kLogitGreedy) {
+      if (p.mask_model >= 0)
+        for (int k = tid; k < count; k += T)
+          if (writes_unit(j0 + k)) p.mask_key[b * p.P + j0 + k] = 0u;  // ready for the next run
+    }
+    if (a >= 0 && asked < j0 + count && !optional && p.mask_model < 0) break;
+    __syncthreads();  // the tile is about to be overwritten
+  }
+  const int a = sh.a;
+  if (writes_row(a)) {
+    for (int k = tid; k < p.P; k += T)
+      p.out_tokens[static_cast<long long>(b) * p.P + k] = k < a ? p.drafts[b * p.gamma + k] : (k == a && !kSample ? sh.cand : -1);
+    if (tid == 0) {
+      p.accept_count[b] = a;
+      p.row_status[b] = sh.status;
+      if (p.bonus_prob != nullptr) p.bonus_prob[b] = (!kSample && a == p.gamma && sh.cand >= 0) ? sh.prob : __int_as_float(0x7fc00000);
+      if (kSample && p.keep_stats) p.row_draw[b] = sh.drawable ? a : -1;
+    }
+  }
+}
+
+// A greedy run has nothing to draw: its decisions are the rest of it.  One block per row.
+template <int DT, int MODE>
+__global__ void __launch_bounds__(128) cos_decide_kernel(const __grid_constant__ KParams p) {
+  __shared__ RowShared sh;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  decide_row<DT, MODE>(p, sh, blockIdx.x, -1, [](const Finish&, int) {}, [](int) { return true; }, [](int) { return true; });
+}
+
+}  // namespace cosv
+
+#endif  // COS_DECIDE_CUH

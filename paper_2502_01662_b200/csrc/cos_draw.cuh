@@ -3,7 +3,7 @@
 #ifndef COS_DRAW_CUH
 #define COS_DRAW_CUH
 
-#include "cos_common.cuh"
+#include "cos_decide.cuh"
 
 namespace cosv {
 
@@ -55,7 +55,7 @@ struct DrawUnit {
   int pis;               // model whose distribution is q
   int law;               // kDrawResidual, kDrawR or kDrawQ
   int emit;              // the token drawn here is the row's output (else only the residual mass is wanted)
-  int accepted;
+  int accepted, drawable;
   float thr;             // plausibility threshold
   float nref[NCH], bt[NCH], ct[NCH];  // minus the reference exponents, "big" bounds, k / Z in fp32
 };
@@ -89,6 +89,7 @@ __device__ __forceinline__ bool load_unit(const KParams& p, int u, DrawUnit<NCH>
   const int4 res = __ldcg(&p.unit_res[d.uidx]);
   if (!res.w) return false;
   d.accepted = res.x;
+  d.drawable = 1;
   const int pi = proposer_of(p, d.b, d.j);
   d.pis = (pi >= 0 && pi < p.n) ? pi : 0;
   d.law = (d.j == p.gamma) ? (p.bonus_model >= 0 ? kDrawQ : kDrawR) : kDrawResidual;
@@ -560,7 +561,7 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
         u.law = kDrawR;
 #pragma unroll
         for (int i = 0; i < NCH; ++i)
-          u.ct[i] = static_cast<float>(coefficient<ENS>(p, i, u.pis, kDrawR) / (i < live ? __ldcg(&p.ustats[u.uidx].s[i]) : 1.0));
+          u.ct[i] = static_cast<float>(coefficient<ENS>(p, i, u.pis, kDrawR) / (i < live ? static_cast<double>(u.bt[i]) / kBigShare : 1.0));
       }
       __syncthreads();
       draw_sweep_again<DT, ENS, NCH, AL>(p, u, acc, rec);
@@ -642,6 +643,51 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
   }
 }
 
+// The block's position from the records of the streaming launch (and the row's outputs, see decide_row): every block decides
+// its row for itself.  False when there is nothing to draw.
+template <int DT, bool ENS, int NCH>
+__device__ __noinline__ bool decide_unit_to_draw(const KParams& p, DrawShared<NCH>& sh, RowShared& rs, int slot, int part) {
+  const int tid = threadIdx.x;
+  int b = slot, want = -1;
+  if (p.draw_all) {
+    const int drafts = p.B * p.gamma;  // every draft position, then the bonus positions
+    b = slot < drafts ? slot / p.gamma : slot - drafts;
+    want = slot < drafts ? slot % p.gamma : p.gamma;
+  }
+  DrawUnit<NCH>& u = sh.unit;
+  decide_row<DT, ENS ? kEnsembleSample : kLogitSample>(
+      p, rs, b, want,
+      [&](const Finish& f, int j) {
+        const int pi = proposer_of(p, b, j);
+        const int pis = (pi >= 0 && pi < p.n) ? pi : 0;
+        const int law = (j == p.gamma) ? (p.bonus_model >= 0 ? kDrawQ : kDrawR) : kDrawResidual;
+        if (tid < NCH) {
+          const bool live = tid < (ENS ? p.n : 2);
+          const double z = live ? f.fsoft[tid].s : 1.0;
+          u.nref[tid] = live ? -f.fsoft[tid].ref : 0.f;
+          u.bt[tid] = live ? static_cast<float>(z * kBigShare) : INFINITY;
+          u.ct[tid] = static_cast<float>(coefficient<ENS>(p, tid, pis, law) / z);
+        }
+        if (tid == 0) {
+          u.b = b;
+          u.j = j;
+          u.uidx = b * p.P + j;
+          u.pis = pis;
+          u.law = law;
+          u.accepted = f.dec.accept;
+          u.drawable = f.dec.drawable;
+          u.thr = (!ENS && p.mask_model >= 0) ? f.thr : -INFINITY;
+          u.base = reinterpret_cast<const char*>(p.logits) +
+                   (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
+        }
+      },
+      [&](int a) { return part == 0 && (want < 0 || want == a); }, [&](int j) { return part == 0 && (want < 0 || want == j); });
+  __syncthreads();
+  const bool emit = (rs.a == u.j);
+  if (tid == 0) u.emit = emit ? 1 : 0;
+  return u.drawable && (emit || u.j != p.gamma);
+}
+
 // PHASE 0: everything in one launch.  1 and 2: the sweep and the rest as two launches (one block per position in the second).
 template <int DT, bool ENS, int NCH, bool AL, int PHASE>
 __global__ void __launch_bounds__(kMaxDrawThreads, NCH == 2 ? 4 : 2) cos_draw_kernel(const __grid_constant__ KParams p) {
@@ -651,10 +697,13 @@ __global__ void __launch_bounds__(kMaxDrawThreads, NCH == 2 ? 4 : 2) cos_draw_ke
   const int tid = threadIdx.x, warp = tid >> 5, nw = blockDim.x >> 5;
   const int parts = PHASE == 2 ? 1 : p.draw_parts;
   const int slot = blockIdx.x / parts, part = blockIdx.x % parts;
-  // launched while the kernel before it drains; nothing is read or written before that one is complete
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (PHASE == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  {
+  // launched while the kernel before it drains; nothing but inputs is read before that one is complete
+  if (PHASE != 2 && p.decide) {
+    if (!decide_unit_to_draw<DT, ENS, NCH>(p, sh, *reinterpret_cast<RowShared*>(draw_smem_raw + sizeof(DrawShared<NCH>)), slot, part)) return;
+    if (PHASE == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  } else {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (PHASE == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     DrawUnit<NCH> d;
     if (!load_unit<DT, ENS, NCH>(p, slot, d)) return;
     if (tid == 0) sh.unit = d;

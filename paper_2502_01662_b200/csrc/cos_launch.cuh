@@ -19,13 +19,19 @@ KernelFn draw_kernel_of(bool ens, int channels, int phase) {
   return phase == 1 ? cos_draw_kernel<DT, true, 8, AL, 1> : cos_draw_kernel<DT, true, 8, AL, 2>;
 }
 
+template <int DT, int MODE, bool AL>
+KernelFn logit_kernel_of(bool pair, bool masked) {
+  if (pair) return masked ? cos_stream_kernel<DT, MODE, AL, true, true> : cos_stream_kernel<DT, MODE, AL, true, false>;
+  return masked ? cos_stream_kernel<DT, MODE, AL, false, true> : cos_stream_kernel<DT, MODE, AL, false, false>;
+}
+
 template <int DT, bool AL>
-KernelFn stream_kernel_of(int mode) {
+KernelFn stream_kernel_of(int mode, bool report, bool pair, bool masked) {
   switch (mode) {
-    case kEnsembleSample: return cos_stream_kernel<DT, kEnsembleSample, AL>;
-    case kLogitSample: return cos_stream_kernel<DT, kLogitSample, AL>;
-    case kEnsembleGreedy: return cos_stream_kernel<DT, kEnsembleGreedy, AL>;
-    default: return cos_stream_kernel<DT, kLogitGreedy, AL>;
+    case kEnsembleSample: return report ? cos_report_kernel<DT, kEnsembleSample, AL> : cos_stream_kernel<DT, kEnsembleSample, AL, true, false>;
+    case kEnsembleGreedy: return report ? cos_report_kernel<DT, kEnsembleGreedy, AL> : cos_stream_kernel<DT, kEnsembleGreedy, AL, true, false>;
+    case kLogitSample: return report ? cos_report_kernel<DT, kLogitSample, AL> : logit_kernel_of<DT, kLogitSample, AL>(pair, masked);
+    default: return report ? cos_report_kernel<DT, kLogitGreedy, AL> : logit_kernel_of<DT, kLogitGreedy, AL>(pair, masked);
   }
 }
 
@@ -46,9 +52,16 @@ inline cudaError_t launch(KernelFn fn, const KParams& p, int blocks, int threads
 }
 
 template <int DT>
-cudaError_t stream_launch(const KParams& p, int mode, int threads, cudaStream_t stream) {
+cudaError_t stream_launch(const KParams& p, int mode, bool report, int threads, cudaStream_t stream) {
   const int blocks = (p.st_workers + threads / 32 - 1) / (threads / 32);
-  return launch(p.vec_ok ? stream_kernel_of<DT, true>(mode) : stream_kernel_of<DT, false>(mode), p, blocks, threads, 0, stream);
+  const bool pair = p.n == 2, masked = p.mask_model >= 0;
+  return launch(p.vec_ok ? stream_kernel_of<DT, true>(mode, report, pair, masked) : stream_kernel_of<DT, false>(mode, report, pair, masked), p,
+                blocks, threads, 0, stream);
+}
+
+template <int DT>
+cudaError_t decide_launch(const KParams& p, int mode, cudaStream_t stream) {
+  return launch(mode == kEnsembleGreedy ? cos_decide_kernel<DT, kEnsembleGreedy> : cos_decide_kernel<DT, kLogitGreedy>, p, p.B, 128, 0, stream);
 }
 
 template <int DT>
@@ -62,7 +75,8 @@ cudaError_t draw_launch(const KParams& p, bool ens, int channels, int phase, int
   KernelFn fn = p.vec_ok ? draw_kernel_of<DT, true>(ens, channels, phase) : draw_kernel_of<DT, false>(ens, channels, phase);
   const size_t fixed = channels == 2 ? sizeof(DrawShared<2>) : (channels == 4 ? sizeof(DrawShared<4>) : sizeof(DrawShared<8>));
   static_assert(sizeof(DrawShared<8>) + 16 * kMaxDrawThreads * sizeof(double) <= 48 * 1024, "no opt-in for large shared memory is made");
-  return launch(fn, p, phase == 2 ? units : units * p.draw_parts, threads, fixed + 2 * channels * threads * sizeof(double), stream);
+  const size_t slow = 2 * channels * threads * sizeof(double);  // (the decisions come first, in the same place)
+  return launch(fn, p, phase == 2 ? units : units * p.draw_parts, threads, fixed + (slow > sizeof(RowShared) ? slow : sizeof(RowShared)), stream);
 }
 
 template <int DT>

@@ -8,10 +8,13 @@
 
 namespace cosv {
 
-// The streaming launch (mode: the Mode enum): a warp for each of the p.st_workers shares, blocks of `threads` threads.  mask:
-// the launch before it that finds the plausibility threshold of every position.
+// The streaming launch (mode: the Mode enum): a warp for each of the p.st_workers shares, blocks of `threads` threads; `report`:
+// the form that also decides and publishes.  mask: the launch before it that finds the plausibility threshold of every
+// position.  decide: the launch after it that decides the rows of a greedy run.
 template <int DT>
-cudaError_t stream_launch(const KParams& p, int mode, int threads, cudaStream_t stream);
+cudaError_t stream_launch(const KParams& p, int mode, bool report, int threads, cudaStream_t stream);
+template <int DT>
+cudaError_t decide_launch(const KParams& p, int mode, cudaStream_t stream);
 template <int DT>
 cudaError_t mask_launch(const KParams& p, int threads, cudaStream_t stream);
 // The drawing launch with `channels` 2, 4 or 8 (logit level: 2) for `units` positions, blocks of `threads` threads: `phase` 0

@@ -948,7 +948,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_stream_kernel(const __g
 // reported, which needs the decisions while the sweep is under way (a line for each position of the rows, one after another),
 // and for those whose tokens the persistent kernel draws, which has no step that decides.
 template <int DT, int MODE, bool AL>
-__global__ void __launch_bounds__(kStreamThreads, 1) cos_report_kernel(const __grid_constant__ KParams p) {
+__global__ void __launch_bounds__(kStreamThreads, 2) cos_report_kernel(const __grid_constant__ KParams p) {
   constexpr bool kEns = (MODE == kEnsembleSample || MODE == kEnsembleGreedy);
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
   __shared__ Finish fins[kStreamThreads / 32];
@@ -989,8 +989,10 @@ __global__ void __launch_bounds__(kStreamThreads, 1) cos_report_kernel(const __g
         int4* rec = p.st_rec + first_record(p, slab, units, r, slots) + static_cast<size_t>(w) * slots;
         if (kEns || (p.n == 2 && !masked))
           sweep_part<DT, MODE, AL, true, false>(p, base, o0, o1, pis, thr, rec, waited);
-        else
+        else if (masked)
           sweep_part<DT, MODE, AL, false, true>(p, base, o0, o1, pis, thr, rec, waited);
+        else
+          sweep_part<DT, MODE, AL, false, false>(p, base, o0, o1, pis, thr, rec, waited);
       }
       int prev = 0;
       if (lane == 0) {

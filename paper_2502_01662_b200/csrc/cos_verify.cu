@@ -1,14 +1,14 @@
 // CoS verification step for sm_100a: combine (Eq. 3-5), accept test (Eq. 6), residual / bonus sample and
 // first-rejection scan (Sec. 3.1) for every row of a batch and every one of its gamma + 1 positions.
 //
-// A run is one launch at T = 0, two at T > 0 (three for ensembles of one or of more than four models), and one more in front
-// of them for the plausibility mask:
+// A run is two launches (three for ensembles of one or of more than four models at T > 0), and one more in front of them for
+// the plausibility mask:
 //   mask       the plausibility threshold of every position (cos_stream.cuh);
-//   streaming  every (row, position): stream the n logit rows once from HBM, keep softmax statistics or argmaxes, take the
-//              accept test in fp64 from the merged statistics and the logits at the draft token, publish the
-//              position; the last one of a row to arrive scans for the first rejection, writes the row's outputs and names
-//              the one position of the row that must draw a token (cos_stream.cuh);
-//   drawing    the positions that draw a token: one sweep and the token (cos_draw.cuh).
+//   streaming  stream the n logit rows of every (row, position) once from HBM: partial softmax statistics or argmaxes
+//              (cos_stream.cuh);
+//   drawing    merge them, take the accept tests in fp64, find every row's first rejection, write the row's outputs
+//              (cos_decide.cuh; at T = 0 that is all), and draw the row's token: one more sweep of the one position that
+//              needs it (cos_draw.cuh).
 // Between blocks there are only fences and arrival counters: nothing waits for another block.
 //
 // This file is the host side of the library (contexts, launches, the C entry points).  The kernels are compiled in
@@ -175,17 +175,13 @@ long long draw_records(const cos_verify_config& c, int sm_count) {
 constexpr int kStreamBlock = 512;   // threads of a block of a full streaming launch, two blocks per multiprocessor
 constexpr int kMinShare = 128;      // vectors a warp should have at least: four loads for each lane
 
-// Rows of whole 16-byte vectors in the line of the streaming launch: every model's row of every position, or (logit level)
-// the vectors of all models of a position together.
-int line_rows(const cos_verify_config& c) { return c.combine == COS_COMBINE_PROB_ENSEMBLE ? c.n : 1; }
-
-// Cut the line of `rows` rows into shares for at most `workers` warps (see cos_stream.cuh).  Small runs take fewer warps, so
+// Cut the line of `units` positions into shares for at most `workers` warps (see cos_stream.cuh).  Small runs take fewer warps, so
 // that each has a few loads in flight, in small blocks, so that they spread over the device.  Returns the block size.
-int plan_line(KParams& p, const cos_verify_config& c, long long rows, long long workers, int sm_count) {
+int plan_line(KParams& p, const cos_verify_config& c, long long units, long long workers, int sm_count) {
   const int E = entries_per_vec(c.dtype), nvec = c.vocab / E;
   p.st_nv = p.vec_ok ? nvec : nvec - 2;  // (unaligned rows: the first vector and the last one go entry by entry)
   if (p.st_nv < 1) p.st_nv = 1;          // nothing but ragged entries
-  p.st_line = rows * p.st_nv;
+  p.st_line = units * p.st_nv;
   const long long groups = (p.st_line + 7) / 8;
   if (workers > p.st_line / kMinShare) workers = p.st_line / kMinShare;
   if (workers < 1) workers = 1;
@@ -209,8 +205,9 @@ cudaError_t by_dtype(int dtype, F f) {
   return f(std::integral_constant<int, COS_DTYPE_F16>());
 }
 
-// The streaming launch, and before it the one that finds the plausibility thresholds.
-cudaError_t launch_stream(const cos_verify_config& c, int mode, KParams& p, long long workers, int sm_count, cudaStream_t stream) {
+// The streaming launch, before it the one that finds the plausibility thresholds, and after it, at T = 0, the one that
+// decides.  `report`: the streaming launch decides itself (see cos_report_kernel).
+cudaError_t launch_stream(const cos_verify_config& c, int mode, KParams& p, bool report, long long workers, int sm_count, cudaStream_t stream) {
   return by_dtype(c.dtype, [&](auto dt) {
     constexpr int DT = decltype(dt)::value;
     cudaError_t e = cudaSuccess;
@@ -219,14 +216,13 @@ cudaError_t launch_stream(const cos_verify_config& c, int mode, KParams& p, long
       const int threads = plan_line(p, c, p.num_units, workers, sm_count);
       e = mask_launch<DT>(p, threads, stream);
     }
-    // Early exit: position by position, so that a row's rejection is known before its later positions are begun; where a
-    // warp's part of a position is short, every position is under way at once anyway and the hint is not taken.
-    const long long nv = c.vocab / entries_per_vec(c.dtype), part = static_cast<long long>(p.B) * line_rows(c) * nv / workers;
-    if (part < 1024) p.early_exit = 0;
-    if (p.early_exit) p.st_slabs = p.P;
-    const int threads = plan_line(p, c, static_cast<long long>(p.num_units / p.st_slabs) * line_rows(c), workers, sm_count);
-    if (e == cudaSuccess) e = stream_launch<DT>(p, mode, threads, stream);
-    if (e == cudaSuccess && p.dump_r != nullptr) e = dump_launch<DT>(p, mode, stream);
+    // early exit: position by position, so that a row's rejection is known before its later positions are begun
+    if (report && p.early_exit) p.st_slabs = p.P;
+    const int threads = plan_line(p, c, p.num_units / p.st_slabs, workers, sm_count);
+    if (e == cudaSuccess) e = stream_launch<DT>(p, mode, report, threads, stream);
+    p.decide = report ? 0 : 1;
+    if (e == cudaSuccess && !report && p.greedy) e = decide_launch<DT>(p, mode, stream);
+    if (e == cudaSuccess && p.greedy && p.dump_r != nullptr) e = dump_launch<DT>(p, mode, stream);
     return e;
   });
 }
@@ -243,8 +239,9 @@ cudaError_t launch_draw(const cos_verify_config& c, KParams& p, bool all, int sm
   return by_dtype(c.dtype, [&](auto dt) {
     constexpr int DT = decltype(dt)::value;
     cudaError_t e = cudaSuccess;
-    if (!draw_split(c)) return draw_launch<DT>(p, ens, draw_channels(c), 0, units, d.threads, stream);
-    for (int phase = 1; phase <= 2 && e == cudaSuccess; ++phase) e = draw_launch<DT>(p, ens, draw_channels(c), phase, units, d.threads, stream);
+    for (int phase = draw_split(c) ? 1 : 0; phase <= (draw_split(c) ? 2 : 0) && e == cudaSuccess; ++phase)
+      e = draw_launch<DT>(p, ens, draw_channels(c), phase, units, d.threads, stream);
+    if (e == cudaSuccess && p.dump_r != nullptr) e = dump_launch<DT>(p, mode_of(c), stream);
     return e;
   });
 }
@@ -362,9 +359,9 @@ extern "C" cos_status cos_verify_create(const cos_verify_config* config, cos_ver
   ok = ok && cudaMalloc(&ctx->d_jobs, (rows * P + rows) * sizeof(int2)) == cudaSuccess;
   ok = ok && cudaMalloc(&ctx->d_ustats, rows * P * sizeof(UnitStats)) == cudaSuccess;
   {
-    // a record (logit level: two) for every row of the line and one for every warp and slab
+    // records of a slot for each model (logit level: two) for every position of the line and for every warp and slab
     const size_t warps = static_cast<size_t>(ctx->sm_count) * 2 * (kStreamBlock / 32) * P;
-    const size_t recs = config->combine == COS_COMBINE_PROB_ENSEMBLE ? rows * P * config->n + warps : 2 * (rows * P + warps);
+    const size_t recs = (rows * P + warps) * (config->combine == COS_COMBINE_PROB_ENSEMBLE ? config->n : 2);
     ok = ok && cudaMalloc(&ctx->d_st_rec, recs * sizeof(int4)) == cudaSuccess;
   }
   ok = ok && cudaMalloc(&ctx->d_st_arrivals, rows * P * sizeof(int)) == cudaSuccess;
@@ -527,9 +524,14 @@ cos_status run_launches(cos_verify_ctx* ctx, const cos_verify_args* a, void* cud
                       p.num_units >= ctx->sm_count && a->batch <= ctx->sm_count)
                          ? 1
                          : 0;
-  const bool by_items = draws && !all && ctx->fused && ctx->draw_fused && p.vec_ok;
+  const bool by_items = draws && !all && ctx->fused && ctx->draw_fused && p.vec_ok && a->lse == nullptr;
   p.use_jobs = by_items ? 1 : 0;
-  e = launch_stream(c, mode, p, stream_workers(c, p.num_units, ctx->sm_count), ctx->sm_count, stream);
+  // Early exit needs the decisions while the sweep is under way; where a warp's part of a position is short, every position is
+  // under way at once anyway and the hint is not taken.
+  const long long workers = stream_workers(c, p.num_units, ctx->sm_count);
+  if (static_cast<long long>(p.B) * c.n * (c.vocab / entries_per_vec(c.dtype)) / workers < 1024 || a->dump_r != nullptr) p.early_exit = 0;
+  p.keep_stats = (a->lse != nullptr || a->dump_r != nullptr || draw_split(c)) ? 1 : 0;
+  e = launch_stream(c, mode, p, p.early_exit || by_items, workers, ctx->sm_count, stream);
   if (e != cudaSuccess) return cuda_fail(ctx, "kernel launch (streaming)", e);
   if (ctx->timing) cudaEventRecord(ctx->ev[1], stream);
   ctx->ev_used = 2;
@@ -719,10 +721,10 @@ extern "C" cos_status cos_verify_get_info(const cos_verify_ctx* ctx, cos_verify_
   info->threads_per_block = kStreamBlock;
   info->sm_count = ctx->sm_count;
   {
-    // ordinary runs (no test hook): one launch at T = 0; else the streaming launch and one or two that draw; one more for
-    // the mask
+    // ordinary runs (no test hook): the streaming launch and one that decides, or one or two that decide and draw; one
+    // more for the mask
     const bool one_draw = !draw_split(ctx->cfg) || (ctx->fused && ctx->draw_fused);
-    info->launches_per_run = (ctx->cfg.temperature > 0.0f && !(ctx->fused && ctx->use_fused)) ? (one_draw ? 2 : 3) : 1;
+    info->launches_per_run = (ctx->fused && ctx->use_fused) ? 1 : (ctx->cfg.temperature == 0.0f || one_draw ? 2 : 3);
     if (ctx->cfg.combine == COS_COMBINE_LOGIT_LINEAR && ctx->cfg.mask_model >= 0) ++info->launches_per_run;
   }
   info->reserved[0] = ctx->fused ? ctx->fplan.chunks : 1;
@@ -861,7 +863,7 @@ extern "C" cos_status cos_verify_run_static(const cos_verify_config* config, con
   if (e != cudaSuccess) return cuda_fail(nullptr, "clearing the built-in scratch", e);
   int4* d_unit_res = reinterpret_cast<int4*>(basep + 256 + 4 * (COS_STATIC_MAX_BATCH + 3 * COS_STATIC_MAX_POSITIONS));
   int4* d_st_rec = d_unit_res + COS_STATIC_MAX_POSITIONS;
-  UnitStats* d_ustats = reinterpret_cast<UnitStats*>(d_st_rec + COS_MAX_MODELS * COS_STATIC_MAX_POSITIONS + kStaticWorkers);
+  UnitStats* d_ustats = reinterpret_cast<UnitStats*>(d_st_rec + COS_MAX_MODELS * (COS_STATIC_MAX_POSITIONS + kStaticWorkers));
   static_assert(sizeof(UnitStats) == 112, "COS_STATIC_SCRATCH_BYTES assumes 112 bytes of statistics per position");
   int* d_row_draw = reinterpret_cast<int*>(d_ustats + COS_STATIC_MAX_POSITIONS);
   double* d_draw_rec = reinterpret_cast<double*>(d_row_draw + COS_STATIC_MAX_BATCH);
@@ -883,7 +885,8 @@ extern "C" cos_status cos_verify_run_static(const cos_verify_config* config, con
 
   long long workers = stream_workers(c, units, sm_count);
   if (workers > kStaticWorkers) workers = kStaticWorkers;
-  e = launch_stream(c, mode_of(c), p, workers, sm_count, stream);
+  p.keep_stats = (a->dump_r != nullptr || draw_split(c)) ? 1 : 0;
+  e = launch_stream(c, mode_of(c), p, false, workers, sm_count, stream);
   if (e != cudaSuccess) return cuda_fail(nullptr, "kernel launch (streaming)", e);
   if (draws) {
     e = launch_draw(c, p, all, sm_count, kStaticDrawDoubles / (2 * draw_channels(c)), stream);
