@@ -53,7 +53,12 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
     }
     return d;
   };
-  DraftLogits first = fetch(0, mine);
+  auto range = [&](int j0, int q, bool live) {
+    const RecordRange none = {nullptr, 0};
+    return live ? records_of<MODE>(p, 0, p.num_units, b * p.P + j0 + q / slots) : none;
+  };
+  const DraftLogits first = fetch(0, mine);
+  const RecordRange first_range = range(0, mine, mine < pairs0);
   if (tid == 0) {
     sh.a = -1;
     sh.status = 0u;
@@ -63,9 +68,9 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
     const int count = p.P - j0 < kTile ? p.P - j0 : kTile;
     for (int q0 = 0; q0 < count * slots; q0 += per) {  // (the same number of times for every lane of a warp)
       const int q = q0 + mine, pos = q / slots, i = q % slots;
-      const bool live = q < count * slots;
-      const DraftLogits d = (j0 == 0 && q0 == 0) ? first : (live ? fetch(j0, q) : first);
-      const Merged m = merge_slot<MODE>(p, live, 0, p.num_units, b * p.P + j0 + pos, i, g, sub);
+      const bool live = q < count * slots, ready = j0 == 0 && q0 == 0;
+      const DraftLogits d = ready ? first : (live ? fetch(j0, q) : first);
+      const Merged m = merge_slot<MODE>(p, ready ? first_range : range(j0, q, live), i, g, sub);
       if (live && sub == 0) {
         Finish& f = sh.fin[pos];
         if (kSample) {
