@@ -231,7 +231,7 @@ cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_args* args,
 #define COS_STATIC_SCRATCH_BYTES                                                                          \
   (256 + 4 * (COS_STATIC_MAX_BATCH + 3 * COS_STATIC_MAX_POSITIONS) + 16 * COS_STATIC_MAX_POSITIONS +     \
    16 * COS_MAX_MODELS * (COS_STATIC_MAX_POSITIONS + 5120) + 112 * COS_STATIC_MAX_POSITIONS +            \
-   4 * COS_STATIC_MAX_BATCH + 8 * 16 * (COS_STATIC_MAX_POSITIONS + 8 * COS_STATIC_MAX_BATCH))
+   4 * COS_STATIC_MAX_BATCH)
 cos_status cos_verify_run_static(const cos_verify_config* config, const cos_verify_args* args, void* cuda_stream);
 
 /*

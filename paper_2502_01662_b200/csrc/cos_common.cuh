@@ -86,10 +86,8 @@ struct KParams {
   int draw_all;            // it visits every position (test hook, residual masses)
   int decide;              // it also merges the records of the streaming launch and decides (else that is done)
   int keep_stats;          // ustats, unit_res and row_draw are wanted afterwards
-  int draw_parts;          // blocks that share a position
-  int draw_cs, draw_chunks;  // steps of a chunk, chunks of a position
-  double* draw_rec;        // [positions][chunks][2 channels]: sums of every chunk
-  int* draw_arrivals;      // [positions of the launch]: blocks that have reported; zero between runs
+  int draw_parts;          // blocks of a position's cluster
+  int draw_cs, draw_chunks;  // steps of a chunk, chunks of a warp
 };
 
 // ------------------------------------------------------------------------------------
@@ -190,7 +188,7 @@ __device__ __forceinline__ void load_chunk(const void* row, int entry0, int V, b
 // Weyl key schedule.
 __device__ __forceinline__ void philox4x32_10(unsigned c0, unsigned c1, unsigned c2, unsigned c3, unsigned k0,
                                               unsigned k1, unsigned (&out)[4]) {
-#pragma unroll
+#pragma unroll 1  // (a chain of latencies either way; ten copies of it are a kilobyte of instructions to fetch)
   for (int r = 0; r < 10; ++r) {
     if (r > 0) {
       k0 += 0x9E3779B9u;

@@ -7,8 +7,8 @@
 
 namespace cosv {
 
-// A block decides a whole row: a few lanes merge the records of one (position, slot) pair each, one thread takes the accept test
-// of a position, a ballot finds the first rejection.  Every block of a row does it for itself (the records of a row are a
+// A block decides a whole row: a few lanes merge the records of one (position, slot) pair each, then one warp goes on, a lane taking the accept
+// test of a position, a ballot finding the first rejection.  Every block of a row does it for itself (the records of a row are a
 // few KB, read from L2), which costs the device nothing that it would use otherwise and no word has to travel between blocks;
 // one of them writes the outputs.  It is a chain of latencies: what it needs of the inputs (drafts, proposers, the logits at the
 // drafts) is fetched before the launch waits for the streaming launch to end.
@@ -16,6 +16,7 @@ constexpr int kTile = 16;  // positions decided at a time
 
 struct RowShared {
   Finish fin[kTile];
+  unsigned word[kTile];
   int a;            // the row's first rejected position, or gamma; -1 until it is known
   int drawable;     // whether a token can be drawn there
   int cand;         // greedy: the token there
@@ -24,8 +25,8 @@ struct RowShared {
 };
 
 // Decide row b.  `want` >= 0: a position whose statistics the block needs, whatever the first rejection; otherwise the first
-// rejected position is what it needs.  `keep(fin, j)` is called by every thread, between two barriers, with that
-// position's merged statistics.  `writes_row(a)` / `writes_unit(j)`: whether this block writes the row's outputs and a
+// rejected position is what it needs.  `keep(fin, j, word)` is called by the first warp with that
+// position's merged statistics and the random word its token is drawn with.  `writes_row(a)` / `writes_unit(j)`: whether this block writes the row's outputs and a
 // position's optional ones.
 template <int DT, int MODE, typename K, typename WR, typename WU>
 __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int b, int want, K keep, WR writes_row, WU writes_unit) {
@@ -83,38 +84,44 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
       }
     }
     __syncthreads();
-    if (tid < count) {
-      const int j = j0 + tid;
-      const bool is_bonus = (j == p.gamma);
-      const int draft = is_bonus ? 0 : __ldg(p.drafts + b * p.gamma + j);
-      const bool draft_ok = is_bonus || (draft >= 0 && draft < p.V);
-      const int pi = proposer_of(p, b, j);
-      const bool pi_ok = (pi >= 0 && pi < p.n);
-      unsigned rnd[4];
-      philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
-      decide_unit<DT, MODE>(p, sh.fin[tid], word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), is_bonus, draft, draft_ok, pi, pi_ok, pi_ok ? pi : 0);
-    }
-    __syncthreads();
-    if (tid < 32 && sh.a < 0) {
-      const bool stop = lane < count && (!sh.fin[lane].dec.accept || j0 + lane == p.gamma);
-      const unsigned stops = __ballot_sync(0xffffffffu, stop);
-      const int k = stops ? __ffs(stops) - 1 : count - 1;
-      const unsigned st = __reduce_or_sync(0xffffffffu, lane <= k ? static_cast<unsigned>(sh.fin[lane].dec.status) : 0u);
-      if (lane == 0) {
-        sh.status |= st;
-        if (stops) {
-          const Decision& d = sh.fin[k].dec;
-          sh.a = j0 + k;
-          sh.drawable = d.drawable;
-          sh.cand = d.cand;
-          sh.prob = static_cast<float>(d.prob);
-        }
+    if (tid < 32) {
+      if (lane < count) {
+        const int j = j0 + lane;
+        const bool is_bonus = (j == p.gamma);
+        const int draft = is_bonus ? 0 : __ldg(p.drafts + b * p.gamma + j);
+        const bool draft_ok = is_bonus || (draft >= 0 && draft < p.V);
+        const int pi = proposer_of(p, b, j);
+        const bool pi_ok = (pi >= 0 && pi < p.n);
+        unsigned rnd[4];
+        philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
+        sh.word[lane] = rnd[1];
+        decide_unit<DT, MODE>(p, sh.fin[lane], word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), is_bonus, draft, draft_ok, pi, pi_ok, pi_ok ? pi : 0);
       }
+      __syncwarp();
+      if (sh.a < 0) {
+        const bool stop = lane < count && (!sh.fin[lane].dec.accept || j0 + lane == p.gamma);
+        const unsigned stops = __ballot_sync(0xffffffffu, stop);
+        const int k = stops ? __ffs(stops) - 1 : count - 1;
+        const unsigned st = __reduce_or_sync(0xffffffffu, lane <= k ? static_cast<unsigned>(sh.fin[lane].dec.status) : 0u);
+        __syncwarp();
+        if (lane == 0) {
+          sh.status |= st;
+          if (stops) {
+            const Decision& d = sh.fin[k].dec;
+            sh.a = j0 + k;
+            sh.drawable = d.drawable;
+            sh.cand = d.cand;
+            sh.prob = static_cast<float>(d.prob);
+          }
+        }
+        __syncwarp();
+      }
+      const int asked = want >= 0 ? want : sh.a;
+      if (asked >= j0 && asked < j0 + count) keep(sh.fin[asked - j0], asked, sh.word[asked - j0]);
     }
     __syncthreads();
     const int a = sh.a;
     const int asked = want >= 0 ? want : a;
-    if (asked >= j0 && asked < j0 + count) keep(sh.fin[asked - j0], asked);
     if (optional) {
       for (int k = tid; k < count; k += T) {
         const int j = j0 + k, uidx = b * p.P + j;
@@ -167,12 +174,13 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
   }
 }
 
-// A greedy run has nothing to draw: its decisions are the rest of it.  One block per row.
+// The decisions in a launch of their own, one block per row: greedy runs have nothing to draw; ensembles of one or of more than four
+// models draw in the launch after it.
 template <int DT, int MODE>
 __global__ void __launch_bounds__(128) cos_decide_kernel(const __grid_constant__ KParams p) {
   __shared__ RowShared sh;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  decide_row<DT, MODE>(p, sh, blockIdx.x, -1, [](const Finish&, int) {}, [](int) { return true; }, [](int) { return true; });
+  decide_row<DT, MODE>(p, sh, blockIdx.x, -1, [](const Finish&, int, unsigned) {}, [](int) { return true; }, [](int) { return true; });
 }
 
 }  // namespace cosv

@@ -13,12 +13,37 @@ namespace cosv {
 // sign that could change carries no mass to speak of), products rounded one by one so that equal terms cancel exactly.
 // Over that set the mass is linear in the 1/Z_i, so the sweep only adds up e_i over it, next to the refined normalisers.
 //
-// Split: a position is shared by p.draw_parts blocks, its steps (32 lanes x one 16-byte vector of every model) cut into
-// chunks of p.draw_cs; a warp takes consecutive chunks and leaves one record of sums for each, nothing per step.  The host
-// picks block size and parts so that the launch fills the device in one wave (see draw_plan).  The block that completes a
-// position (fence and counter, no waiting) adds its records up, finds the chunk that holds the token, then the step, then the token.
-constexpr int kMaxDrawThreads = 256;
-constexpr int kChunksKept = 4;  // chunks of a thread of the locating block whose masses it keeps in registers
+// Split: a position is shared by one cluster of p.draw_parts blocks, its steps (32 lanes x one 16-byte vector of every model)
+// dealt out in equal consecutive runs to the cluster's warps; a warp sends one record of sums for each chunk of p.draw_cs steps to
+// the shared memory of the cluster's first block, nothing per step.  After one barrier of the cluster that block alone
+// adds the records up, finds the chunk that holds the token, then the step, then the token.  The host picks block size and parts so
+// that the launch fills the device in one wave (see draw_plan).
+// The part behind the sweep is a chain of latencies, issue slots and instruction fetches (counted on one row of 151936 tokens: most
+// stalls are for instructions), so what can be done by one warp is, and nothing is unrolled that need not be.
+// Records in global memory and the last block to report (fence and counter) took 5 us longer.
+constexpr int kMaxDrawThreads = 512;
+constexpr int kMaxDrawWarps = kMaxDrawThreads / 32;
+constexpr int kMaxParts = 8;       // blocks of a cluster
+constexpr int kMaxSums = 768;      // chunks of a position times channels
+
+// Every thread of the cluster arrives and waits; what was written before, to a peer's shared memory too, is visible after.
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The address of a place in this block's shared memory, in the cluster's first block.
+__device__ __forceinline__ unsigned at_first(const double* mine) {
+  unsigned r;
+  asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(static_cast<unsigned>(__cvta_generic_to_shared(mine))));
+  return r;
+}
+__device__ __forceinline__ void store_cluster(unsigned a, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
 
 __device__ __forceinline__ double warp_sum(double t) {
 #pragma unroll
@@ -54,6 +79,7 @@ struct DrawUnit {
   int b, j, uidx;
   int pis;               // model whose distribution is q
   int law;               // kDrawResidual, kDrawR or kDrawQ
+  unsigned word;         // the random word the token is drawn with
   int emit;              // the token drawn here is the row's output (else only the residual mass is wanted)
   int accepted, drawable;
   float thr;             // plausibility threshold
@@ -93,6 +119,9 @@ __device__ __forceinline__ bool load_unit(const KParams& p, int u, DrawUnit<NCH>
   const int pi = proposer_of(p, d.b, d.j);
   d.pis = (pi >= 0 && pi < p.n) ? pi : 0;
   d.law = (d.j == p.gamma) ? (p.bonus_model >= 0 ? kDrawQ : kDrawR) : kDrawResidual;
+  unsigned rnd[4];
+  philox4x32_10(static_cast<unsigned>(p.row_base + d.b), static_cast<unsigned>(d.j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
+  d.word = rnd[1];
   d.base = reinterpret_cast<const char*>(p.logits) +
            (static_cast<long long>(d.b) * p.s_row + static_cast<long long>(d.j) * p.s_pos) * Elem<DT>::bytes;
   d.thr = (!ENS && p.mask_model >= 0) ? __ldcg(&st->thr32) : -INFINITY;
@@ -225,14 +254,15 @@ __device__ __noinline__ void slow_vector(const KParams& p, const DrawUnit<NCH>& 
   }
 }
 
-// The chunks [c_lo, c_hi) of a position by one warp: per channel the normaliser's share and the sum over the tokens with a
-// positive mass, 2 NCH sums for every chunk at rec[chunk * 2 NCH].  The fast loop adds vectors up in fp32; vectors that need the
+// The steps [s_lo, s_hi) of a position by one warp, in chunks of cs steps: per channel the sum over the tokens with a positive mass,
+// for every chunk NCH sums to rec, and to part the normaliser's share, of all chunks together (both in the cluster's first block).
+// The fast loop adds vectors up in fp32; vectors that need the
 // slow path it only remembers until the end of the strip (their sums, in fp64, in the thread's slots of `acc`).
 // What bounds it: loads in flight (two steps of every model at a time) and issue (about 17 instructions per pair of terms).
 // PAIR, MASKED: logit level with exactly two models, and with a mask.
 template <int DT, bool ENS, int NCH, bool AL, bool PAIR, bool MASKED>
-__device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawUnit<NCH>& u, int cs, int c_lo, int c_hi, double* acc,
-                                              double* rec) {
+__device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawUnit<NCH>& u, int cs, int s_lo, int s_hi, double* acc,
+                                              unsigned rec, unsigned part) {
   constexpr int E = Elem<DT>::E;
   constexpr int NP = NCH / 2;
   constexpr int NR = ENS ? NCH : 2;         // vectors of a step kept in registers
@@ -252,11 +282,13 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawUnit<N
     bt[2 * q + 1] = u.bt[2 * q + 1];
   }
   const LogitWeights lw = logit_weights(p, u.pis, u.thr);
-  for (int chunk = c_lo; chunk < c_hi; ++chunk) {
-    const int end = (chunk + 1) * cs < p.nsteps ? (chunk + 1) * cs : p.nsteps;
+  double all = 0.0;
+#pragma unroll 1
+  for (int begin = s_lo; begin < s_hi; begin += cs, rec += NCH * 8) {
+    const int end = begin + cs < s_hi ? begin + cs : s_hi;
     double sums[2 * NCH];
     // in strips of 32 steps: a bit each in the slow-path mask
-    for (int c = chunk * cs; c < end; c += 32) {
+    for (int c = begin; c < end; c += 32) {
       const int ce = c + 32 < end ? c + 32 : end;
       unsigned slow = 0u;
       f32x2 zc[NP], ac[NP];
@@ -350,7 +382,7 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawUnit<N
         }
       }
       const int T = blockDim.x;
-      const bool more = c > chunk * cs;
+      const bool more = c > begin;
 #pragma unroll
       for (int q = 0; q < NP; ++q) {
         sums[2 * q] = static_cast<double>(lo2(zc[q])) + (more ? acc[(2 * q) * T] : 0.0);
@@ -372,18 +404,40 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawUnit<N
     }
     __syncwarp();
     const double mine = warp_sums<2 * NCH>(sums, lane);
-    if (lane % (32 / (2 * NCH)) == 0) rec[static_cast<size_t>(chunk) * (2 * NCH) + lane / (32 / (2 * NCH))] = mine;
+    if (lane >= 16 && lane % (16 / NCH) == 0) store_cluster(rec + (lane - 16) / (16 / NCH) * 8, mine);
+    all += mine;
   }
+  if (lane < 16 && lane % (16 / NCH) == 0) store_cluster(part + lane / (16 / NCH) * 8, all);
 }
 
+// Shared memory of a block, in front of every thread's 2 NCH slots of the slow path.
+template <int NCH>
+struct DrawShared {
+  DrawUnit<NCH> unit;
+  // (of the cluster's first block)
+  double recs[kMaxSums];                         // sums of the chunks
+  double part[kMaxParts * kMaxDrawWarps][NCH];   // shares of the normalisers, of every warp
+  double step_mass[32];
+  double inv[NCH];      // one over the normalisers
+  double base, target;  // mass before the winning chunk; the running total to be reached
+  float cf[NCH];        // k / Z
+  int win;              // the winning chunk; -1: nothing to draw, -2: no mass
+};
+
+// The share of warp w of W; chunks without steps get sums of zero.
 template <int DT, bool ENS, int NCH, bool AL>
-__device__ __forceinline__ void draw_sweep(const KParams& p, const DrawUnit<NCH>& u, int cs, int c_lo, int c_hi, double* acc,
-                                           double* rec) {
-  if (ENS) return draw_sweep_as<DT, ENS, NCH, AL, true, false>(p, u, cs, c_lo, c_hi, acc, rec);
-  if (p.n == 2 && p.mask_model < 0) return draw_sweep_as<DT, ENS, NCH, AL, true, false>(p, u, cs, c_lo, c_hi, acc, rec);
-  if (p.n == 2) return draw_sweep_as<DT, ENS, NCH, AL, true, true>(p, u, cs, c_lo, c_hi, acc, rec);
-  if (p.mask_model < 0) return draw_sweep_as<DT, ENS, NCH, AL, false, false>(p, u, cs, c_lo, c_hi, acc, rec);
-  draw_sweep_as<DT, ENS, NCH, AL, false, true>(p, u, cs, c_lo, c_hi, acc, rec);
+__device__ __forceinline__ void draw_sweep(const KParams& p, DrawShared<NCH>& sh, int w, int W, double* acc) {
+  const int s_lo = static_cast<int>(static_cast<long long>(p.nsteps) * w / W);
+  const int s_hi = static_cast<int>(static_cast<long long>(p.nsteps) * (w + 1) / W);
+  const unsigned rec = at_first(&sh.recs[w * p.draw_chunks * NCH]), part = at_first(sh.part[w]);
+  const int cs = p.draw_cs, used = (s_hi - s_lo + cs - 1) / cs;
+  for (int k = used * NCH + (threadIdx.x & 31); k < p.draw_chunks * NCH; k += 32) store_cluster(rec + k * 8, 0.0);
+  const DrawUnit<NCH>& u = sh.unit;
+  if (ENS) return draw_sweep_as<DT, ENS, NCH, AL, true, false>(p, u, cs, s_lo, s_hi, acc, rec, part);
+  if (p.n == 2 && p.mask_model < 0) return draw_sweep_as<DT, ENS, NCH, AL, true, false>(p, u, cs, s_lo, s_hi, acc, rec, part);
+  if (p.n == 2) return draw_sweep_as<DT, ENS, NCH, AL, true, true>(p, u, cs, s_lo, s_hi, acc, rec, part);
+  if (p.mask_model < 0) return draw_sweep_as<DT, ENS, NCH, AL, false, false>(p, u, cs, s_lo, s_hi, acc, rec, part);
+  draw_sweep_as<DT, ENS, NCH, AL, false, true>(p, u, cs, s_lo, s_hi, acc, rec, part);
 }
 
 // Masses of one lane's tokens of step s under the refined normalisers (coefficients cf = k / Z): small ones in fp32, big
@@ -428,131 +482,92 @@ __device__ __forceinline__ double step_masses(const KParams& p, const DrawUnit<N
   return own;
 }
 
-// The whole position again by one block, for another law.  Rare; out of line.
+// The whole position again by the cluster's first block, for another law.  Rare; out of line.
 template <int DT, bool ENS, int NCH, bool AL>
-__device__ __noinline__ void draw_sweep_again(const KParams& p, const DrawUnit<NCH>& u, double* acc, double* rec) {
-  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int c_lo = static_cast<int>(static_cast<long long>(p.draw_chunks) * warp / nw);
-  const int c_hi = static_cast<int>(static_cast<long long>(p.draw_chunks) * (warp + 1) / nw);
-  draw_sweep<DT, ENS, NCH, AL>(p, u, p.draw_cs, c_lo, c_hi, acc, rec);
+__device__ __noinline__ void draw_sweep_again(const KParams& p, DrawShared<NCH>& sh, int W, double* acc) {
+  for (int w = threadIdx.x >> 5; w < W; w += blockDim.x >> 5) draw_sweep<DT, ENS, NCH, AL>(p, sh, w, W, acc);
 }
 
-// Shared memory of a block, in front of every thread's 2 NCH slots of the slow path.
-template <int NCH>
-struct DrawShared {
-  DrawUnit<NCH> unit;
-  double part[NCH][kMaxDrawThreads / 32];
-  double wmass[kMaxDrawThreads / 32];
-  double step_mass[32];
-  double base;      // mass before the winning chunk
-  int first, last;  // the winning chunk; the last chunk with mass
-  int go;
-};
-
-// A position whose records are all in: add them up, find the chunk, the step and the token.  Whole block.
-template <int DT, bool ENS, int NCH, bool AL>
-__device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, double* acc, double* rec) {
-  constexpr int E = Elem<DT>::E;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const int live = ENS ? p.n : 2;
-  DrawUnit<NCH>& u = sh.unit;
-  const int nch = p.draw_chunks, cs = p.draw_cs;
-  const int per = (nch + blockDim.x - 1) / blockDim.x;  // consecutive chunks of a thread
-  unsigned rnd[4];
-  philox4x32_10(static_cast<unsigned>(p.row_base + u.b), static_cast<unsigned>(u.j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
-  for (int pass = 0; pass < 2; ++pass) {
-    double z[NCH], a[kChunksKept][NCH];
+// The normalisers from the shares of all W warps, and the chunk that holds the token.  One warp.
+template <bool ENS, int NCH>
+__device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh, int W) {
+  constexpr int G = 32 / NCH;  // lanes of a channel
+  const int lane = threadIdx.x & 31, i = lane / G, live = ENS ? p.n : 2;
+  const DrawUnit<NCH>& u = sh.unit;
+  double z = 0.0;
+  for (int w = lane % G; w < W; w += G) z += sh.part[w][i];
 #pragma unroll
-    for (int i = 0; i < NCH; ++i) z[i] = 0.0;
-    const int c_lo = tid * per, c_hi = c_lo + per < nch ? c_lo + per : nch;
+  for (int d = G / 2; d > 0; d >>= 1) z += __shfl_xor_sync(0xffffffffu, z, d);
+  const double inv = i < live ? 1.0 / z : 0.0, k = i < live ? coefficient<ENS>(p, i, u.pis, u.law) * inv : 0.0;
+  if (lane % G == 0) {
+    sh.inv[i] = inv;
+    sh.cf[i] = static_cast<float>(k);
+  }
+  double c64[NCH];
 #pragma unroll
-    for (int q = 0; q < kChunksKept; ++q) {
-      const double* r = rec + static_cast<size_t>(c_lo + q) * (2 * NCH);
+  for (int q = 0; q < NCH; ++q) c64[q] = __shfl_sync(0xffffffffu, k, q * G);
+  auto mass_of = [&](int c) -> double {  // (products rounded one by one: equal sums under opposite coefficients cancel)
+    const double* a = &sh.recs[c * NCH];
+    double m = __dmul_rn(c64[0], a[0]);
 #pragma unroll
-      for (int i = 0; i < NCH; ++i) {
-        a[q][i] = 0.0;
-        if (c_lo + q < c_hi) {
-          z[i] += __ldcg(r + i);
-          a[q][i] = __ldcg(r + NCH + i);
-        }
-      }
-    }
-    for (int c = c_lo + kChunksKept; c < c_hi; ++c)
-      for (int i = 0; i < NCH; ++i) z[i] += __ldcg(rec + static_cast<size_t>(c) * (2 * NCH) + i);
-    {
-      double t[NCH];
-#pragma unroll
-      for (int i = 0; i < NCH; ++i) t[i] = z[i];
-      const double mine = warp_sums<NCH>(t, lane);
-      if (lane % (32 / NCH) == 0) sh.part[lane / (32 / NCH)][warp] = mine;
-    }
-    if (tid == 0) {
-      sh.first = 0x7fffffff;
-      sh.last = -1;
-    }
-    __syncthreads();
-    double inv[NCH], c64[NCH], mass[kChunksKept], mine = 0.0;
-    float cf[NCH];
-#pragma unroll
-    for (int i = 0; i < NCH; ++i) {
-      double t = 0.0;
-      for (int w = 0; w < nw; ++w) t += sh.part[i][w];
-      inv[i] = i < live ? 1.0 / t : 0.0;
-      c64[i] = i < live ? coefficient<ENS>(p, i, u.pis, u.law) * inv[i] : 0.0;
-      cf[i] = static_cast<float>(c64[i]);
-    }
-    auto mass_of = [&](const double* w) -> double {  // (products rounded one by one: equal sums under opposite coefficients cancel)
-      double m = __dmul_rn(c64[0], w[0]);
-#pragma unroll
-      for (int i = 1; i < NCH; ++i) m = __dadd_rn(m, __dmul_rn(c64[i], w[i]));
-      return fmax(0.0, m);
-    };
-#pragma unroll
-    for (int q = 0; q < kChunksKept; ++q) {
-      mass[q] = mass_of(a[q]);
-      mine += mass[q];
-    }
-    for (int c = c_lo + kChunksKept; c < c_hi; ++c) mine += mass_of(rec + static_cast<size_t>(c) * (2 * NCH) + NCH);
-    double incl = mine;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const double o = __shfl_up_sync(0xffffffffu, incl, d);
-      if (lane >= d) incl += o;
-    }
-    if (lane == 31) sh.wmass[warp] = incl;
-    __syncthreads();
-    double before = 0.0, S = 0.0;
-    for (int w = 0; w < nw; ++w) {
-      if (w == warp) before = S;
-      S += sh.wmass[w];
-    }
-    before += incl - mine;
-    const double target = word_to_uniform(rnd[1]) * S;
-    if (pass == 0 && tid == 0 && p.diag && u.j != p.gamma) p.diag[static_cast<long long>(u.uidx) * 4 + 3] = static_cast<float>(S);
-    if (!u.emit) return;
-    // the first chunk whose running total reaches the target; where rounding leaves none, the last chunk with mass
-    int first = -1, last = -1;
-    double first_base = 0.0, last_base = 0.0;
-    auto look = [&](int c, double m) {
-      if (m > 0.0) {
+    for (int q = 1; q < NCH; ++q) m = __dadd_rn(m, __dmul_rn(c64[q], a[q]));
+    return fmax(0.0, m);
+  };
+  // consecutive chunks to a lane, their masses in the place of their first sums
+  const int chunks = W * p.draw_chunks, per = (chunks + 31) / 32;
+  const int c_lo = lane * per, c_hi = c_lo + per < chunks ? c_lo + per : chunks;
+  double mine = 0.0;
+#pragma unroll 2
+  for (int c = c_lo; c < c_hi; ++c) {
+    const double m = mass_of(c);
+    sh.recs[c * NCH] = m;
+    mine += m;
+  }
+  double incl = mine;
+#pragma unroll 1
+  for (int d = 1; d < 32; d <<= 1) {
+    const double o = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += o;
+  }
+  const double S = __shfl_sync(0xffffffffu, incl, 31), target = word_to_uniform(u.word) * S;
+  // the first chunk whose running total reaches the target; where rounding leaves none, the last chunk with mass
+  double before = incl - mine, base = 0.0;
+  int first = -1, last = -1;
+  if (mine > 0.0)
+    for (int c = c_lo; c < c_hi; ++c) {
+      const double m = sh.recs[c * NCH];
+      if (m > 0.0 && first < 0) {
         last = c;
-        last_base = before;
-        if (first < 0 && before + m >= target) {
-          first = c;
-          first_base = before;
-        }
+        base = before;
+        if (before + m >= target) first = c;
       }
       before += m;
-    };
-#pragma unroll
-    for (int q = 0; q < kChunksKept; ++q) look(c_lo + q, mass[q]);
-    for (int c = c_lo + kChunksKept; c < c_hi; ++c) look(c, mass_of(rec + static_cast<size_t>(c) * (2 * NCH) + NCH));
-    if (first >= 0) atomicMin(&sh.first, first);
-    if (last >= 0) atomicMax(&sh.last, last);
+    }
+  const unsigned hit = __ballot_sync(0xffffffffu, first >= 0), some = __ballot_sync(0xffffffffu, last >= 0);
+  const int winner = hit ? __ffs(hit) - 1 : 31 - __clz(some);
+  if (some != 0u ? lane == winner : lane == 0) {
+    sh.win = some != 0u && S > 0.0 ? last : -2;
+    sh.base = base;
+    sh.target = target;
+    if (!u.emit) sh.win = -1;
+    if (p.diag && u.j != p.gamma && u.law == kDrawResidual) p.diag[static_cast<long long>(u.uidx) * 4 + 3] = static_cast<float>(S);
+  }
+}
+
+// The rest of a position, after the sweep: the block that has the sums finds the chunk, the step and the token.
+template <int DT, bool ENS, int NCH, bool AL>
+__device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, double* acc) {
+  constexpr int E = Elem<DT>::E;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int live = ENS ? p.n : 2, W = p.draw_parts * nw;
+  DrawUnit<NCH>& u = sh.unit;
+  const int cs = p.draw_cs;
+  for (int pass = 0; pass < 2; ++pass) {
+    if (warp == 0) find_chunk<ENS, NCH>(p, sh, W);
     __syncthreads();
-    const bool hit = sh.first != 0x7fffffff;
-    const int win = hit ? sh.first : sh.last;
-    if (win < 0 || !(S > 0.0)) {
+    const int win = sh.win;
+    if (win == -1) return;
+    if (win < 0) {
       // no residual mass although a token is needed: this block draws from r instead, over the whole position
       if (u.law != kDrawResidual) return;
       __syncthreads();
@@ -564,13 +579,18 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
           u.ct[i] = static_cast<float>(coefficient<ENS>(p, i, u.pis, kDrawR) / (i < live ? static_cast<double>(u.bt[i]) / kBigShare : 1.0));
       }
       __syncthreads();
-      draw_sweep_again<DT, ENS, NCH, AL>(p, u, acc, rec);
+      draw_sweep_again<DT, ENS, NCH, AL>(p, sh, W, acc);
       __syncthreads();
       continue;
     }
-    if ((hit ? first : last) == win) sh.base = hit ? first_base : last_base;
+    const double* inv = sh.inv;
+    const float* cf = sh.cf;
+    const double target = sh.target;
     // the steps of that chunk, dealt out over the warps in up to 32 records of `gsz` steps (one step, nearly always)
-    const int s0 = win * cs, s1 = s0 + cs < p.nsteps ? s0 + cs : p.nsteps, gsz = (cs + 31) / 32;
+    const int ww = win / p.draw_chunks;
+    const int s0 = static_cast<int>(static_cast<long long>(p.nsteps) * ww / W) + win % p.draw_chunks * cs;
+    const int end = static_cast<int>(static_cast<long long>(p.nsteps) * (ww + 1) / W);
+    const int s1 = s0 + cs < end ? s0 + cs : end, gsz = (cs + 31) / 32;
     float m32[E];
     unsigned bigbits = 0u;
     double mbig[E], own = 0.0;
@@ -587,19 +607,20 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
       if (lane == 0) sh.step_mass[t] = rm;
     }
     __syncthreads();
+    if (held < 0) return;  // (no step of the chunk is this warp's)
     const double v = (s0 + lane * gsz < s1) ? sh.step_mass[lane] : 0.0;
     double inc = v;
-#pragma unroll
+#pragma unroll 1
     for (int d = 1; d < 32; d <<= 1) {
       const double o = __shfl_up_sync(0xffffffffu, inc, d);
       if (lane >= d) inc += o;
     }
-    const double base = sh.base;
-    const unsigned ok = __ballot_sync(0xffffffffu, v > 0.0 && base + inc >= target), pos = __ballot_sync(0xffffffffu, v > 0.0);
+    const double from = sh.base;
+    const unsigned ok = __ballot_sync(0xffffffffu, v > 0.0 && from + inc >= target), pos = __ballot_sync(0xffffffffu, v > 0.0);
     if (pos == 0u) return;
     const int k = ok ? __ffs(ok) - 1 : 31 - __clz(pos);  // rounding corner: the last record with mass
     if (k % nw != warp) return;
-    double at = base + __shfl_sync(0xffffffffu, inc - v, k);
+    double at = from + __shfl_sync(0xffffffffu, inc - v, k);
     // one warp goes on: the record's steps in order, an fp64 prefix over the lanes, then the lane's tokens
     int token = -1, last_tok = -1;
 #pragma unroll 1
@@ -607,7 +628,7 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
       if (s != held) own = step_masses<DT, ENS, NCH, AL>(p, u, cf, inv, s, m32, bigbits, mbig);
       held = s;
       double in = own;
-#pragma unroll
+#pragma unroll 1
       for (int d = 1; d < 32; d <<= 1) {
         const double o = __shfl_up_sync(0xffffffffu, in, d);
         if (lane >= d) in += o;
@@ -657,7 +678,7 @@ __device__ __noinline__ bool decide_unit_to_draw(const KParams& p, DrawShared<NC
   DrawUnit<NCH>& u = sh.unit;
   decide_row<DT, ENS ? kEnsembleSample : kLogitSample>(
       p, rs, b, want,
-      [&](const Finish& f, int j) {
+      [&](const Finish& f, int j, unsigned word) {
         const int pi = proposer_of(p, b, j);
         const int pis = (pi >= 0 && pi < p.n) ? pi : 0;
         const int law = (j == p.gamma) ? (p.bonus_model >= 0 ? kDrawQ : kDrawR) : kDrawResidual;
@@ -674,6 +695,7 @@ __device__ __noinline__ bool decide_unit_to_draw(const KParams& p, DrawShared<NC
           u.uidx = b * p.P + j;
           u.pis = pis;
           u.law = law;
+          u.word = word;
           u.accepted = f.dec.accept;
           u.drawable = f.dec.drawable;
           u.thr = (!ENS && p.mask_model >= 0) ? f.thr : -INFINITY;
@@ -682,58 +704,38 @@ __device__ __noinline__ bool decide_unit_to_draw(const KParams& p, DrawShared<NC
         }
       },
       [&](int a) { return part == 0 && (want < 0 || want == a); }, [&](int j) { return part == 0 && (want < 0 || want == j); });
-  __syncthreads();
   const bool emit = (rs.a == u.j);
   if (tid == 0) u.emit = emit ? 1 : 0;
   return u.drawable && (emit || u.j != p.gamma);
 }
 
-// PHASE 0: everything in one launch.  1 and 2: the sweep and the rest as two launches (one block per position in the second).
-template <int DT, bool ENS, int NCH, bool AL, int PHASE>
-__global__ void __launch_bounds__(kMaxDrawThreads, NCH == 2 ? 4 : 2) cos_draw_kernel(const __grid_constant__ KParams p) {
+// One cluster of p.draw_parts blocks for each position.  All blocks of a cluster take the same way, and so meet at its barriers.
+template <int DT, bool ENS, int NCH, bool AL>
+__global__ void __launch_bounds__(NCH == 8 ? 256 : kMaxDrawThreads, NCH == 2 ? 2 : (NCH == 4 ? 1 : 2)) cos_draw_kernel(const __grid_constant__ KParams p) {
   extern __shared__ __align__(16) unsigned char draw_smem_raw[];
   DrawShared<NCH>& sh = *reinterpret_cast<DrawShared<NCH>*>(draw_smem_raw);
-  double* acc = reinterpret_cast<double*>(draw_smem_raw + sizeof(DrawShared<NCH>)) + threadIdx.x;
-  const int tid = threadIdx.x, warp = tid >> 5, nw = blockDim.x >> 5;
-  const int parts = PHASE == 2 ? 1 : p.draw_parts;
-  const int slot = blockIdx.x / parts, part = blockIdx.x % parts;
+  double* slots = reinterpret_cast<double*>(draw_smem_raw + sizeof(DrawShared<NCH>));
+  double* acc = slots + threadIdx.x;
+  const int slot = blockIdx.x / p.draw_parts, rank = blockIdx.x % p.draw_parts, nw = blockDim.x >> 5;
+  cluster_arrive();  // (the first block has begun: its shared memory may be written to)
   // launched while the kernel before it drains; nothing but inputs is read before that one is complete
-  if (PHASE != 2 && p.decide) {
-    if (!decide_unit_to_draw<DT, ENS, NCH>(p, sh, *reinterpret_cast<RowShared*>(draw_smem_raw + sizeof(DrawShared<NCH>)), slot, part)) return;
-    if (PHASE == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  bool draws;
+  if (NCH != 8 && p.decide) {
+    draws = decide_unit_to_draw<DT, ENS, NCH>(p, sh, *reinterpret_cast<RowShared*>(slots), slot, rank);
   } else {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (PHASE == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     DrawUnit<NCH> d;
-    if (!load_unit<DT, ENS, NCH>(p, slot, d)) return;
-    if (tid == 0) sh.unit = d;
+    draws = load_unit<DT, ENS, NCH>(p, slot, d);
+    if (threadIdx.x == 0) sh.unit = d;
   }
+  cluster_wait();
+  if (!draws) return;
   __syncthreads();
-  double* rec = p.draw_rec + static_cast<size_t>(slot) * p.draw_chunks * (2 * NCH);
-  if (PHASE != 2) {
-    const int w = part * nw + warp, W = parts * nw;
-    const int c_lo = static_cast<int>(static_cast<long long>(p.draw_chunks) * w / W);
-    const int c_hi = static_cast<int>(static_cast<long long>(p.draw_chunks) * (w + 1) / W);
-    draw_sweep<DT, ENS, NCH, AL>(p, sh.unit, p.draw_cs, c_lo, c_hi, acc, rec);
-    if (PHASE == 1) return;
-    __syncthreads();
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (parts > 1) {
-      // the last block of the position to get here goes on
-      if (tid == 0) {
-        __threadfence();
-        const int prev = atomicAdd(&p.draw_arrivals[slot], 1);
-        if (prev == parts - 1) {
-          __threadfence();             // what the other blocks wrote before they reported is visible from here on
-          p.draw_arrivals[slot] = 0;   // ready for the next run (a later launch: nothing waits for this store)
-        }
-        sh.go = (prev == parts - 1) ? 1 : 0;
-      }
-      __syncthreads();
-      if (!sh.go) return;
-    }
-  }
-  locate<DT, ENS, NCH, AL>(p, sh, acc, rec);
+  draw_sweep<DT, ENS, NCH, AL>(p, sh, rank * nw + (threadIdx.x >> 5), p.draw_parts * nw, acc);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
+  if (rank == 0) locate<DT, ENS, NCH, AL>(p, sh, acc);
 }
 
 // Test hook: the combined distribution of every position, token by token, from the statistics the streaming launch left.

@@ -11,12 +11,10 @@ namespace cosv {
 using KernelFn = void (*)(const KParams);
 
 template <int DT, bool AL>
-KernelFn draw_kernel_of(bool ens, int channels, int phase) {
-  if (!ens) return cos_draw_kernel<DT, false, 2, AL, 0>;
-  if (channels == 2)
-    return phase == 0 ? cos_draw_kernel<DT, true, 2, AL, 0> : (phase == 1 ? cos_draw_kernel<DT, true, 2, AL, 1> : cos_draw_kernel<DT, true, 2, AL, 2>);
-  if (channels == 4) return cos_draw_kernel<DT, true, 4, AL, 0>;
-  return phase == 1 ? cos_draw_kernel<DT, true, 8, AL, 1> : cos_draw_kernel<DT, true, 8, AL, 2>;
+KernelFn draw_kernel_of(bool ens, int channels) {
+  if (!ens) return cos_draw_kernel<DT, false, 2, AL>;
+  if (channels == 2) return cos_draw_kernel<DT, true, 2, AL>;
+  return channels == 4 ? cos_draw_kernel<DT, true, 4, AL> : cos_draw_kernel<DT, true, 8, AL>;
 }
 
 template <int DT, int MODE, bool AL>
@@ -37,17 +35,20 @@ KernelFn stream_kernel_of(int mode, bool report, bool pair, bool masked) {
 
 // Every launch carries the programmatic-stream-serialisation attribute: its blocks take their places while the kernel
 // before it drains, and wait for it before they touch anything.
-inline cudaError_t launch(KernelFn fn, const KParams& p, int blocks, int threads, size_t smem, cudaStream_t stream) {
+inline cudaError_t launch(KernelFn fn, const KParams& p, int blocks, int threads, size_t smem, cudaStream_t stream, int cluster = 1) {
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
   lc.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
   lc.dynamicSmemBytes = smem;
   lc.stream = stream;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = static_cast<unsigned>(cluster);
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   lc.attrs = at;
-  lc.numAttrs = 1;
+  lc.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&lc, fn, p);
 }
 
@@ -61,7 +62,9 @@ cudaError_t stream_launch(const KParams& p, int mode, bool report, int threads, 
 
 template <int DT>
 cudaError_t decide_launch(const KParams& p, int mode, cudaStream_t stream) {
-  return launch(mode == kEnsembleGreedy ? cos_decide_kernel<DT, kEnsembleGreedy> : cos_decide_kernel<DT, kLogitGreedy>, p, p.B, 128, 0, stream);
+  KernelFn fn = mode == kEnsembleGreedy ? cos_decide_kernel<DT, kEnsembleGreedy>
+                                        : (mode == kLogitGreedy ? cos_decide_kernel<DT, kLogitGreedy> : cos_decide_kernel<DT, kEnsembleSample>);
+  return launch(fn, p, p.B, 128, 0, stream);
 }
 
 template <int DT>
@@ -71,12 +74,13 @@ cudaError_t mask_launch(const KParams& p, int threads, cudaStream_t stream) {
 }
 
 template <int DT>
-cudaError_t draw_launch(const KParams& p, bool ens, int channels, int phase, int units, int threads, cudaStream_t stream) {
-  KernelFn fn = p.vec_ok ? draw_kernel_of<DT, true>(ens, channels, phase) : draw_kernel_of<DT, false>(ens, channels, phase);
+cudaError_t draw_launch(const KParams& p, bool ens, int channels, int units, int threads, cudaStream_t stream) {
+  KernelFn fn = p.vec_ok ? draw_kernel_of<DT, true>(ens, channels) : draw_kernel_of<DT, false>(ens, channels);
   const size_t fixed = channels == 2 ? sizeof(DrawShared<2>) : (channels == 4 ? sizeof(DrawShared<4>) : sizeof(DrawShared<8>));
-  static_assert(sizeof(DrawShared<8>) + 16 * kMaxDrawThreads * sizeof(double) <= 48 * 1024, "no opt-in for large shared memory is made");
+  static_assert(sizeof(DrawShared<4>) + 8 * 8 * kMaxDrawThreads <= 48 * 1024 && sizeof(DrawShared<8>) + 8 * 16 * 256 <= 48 * 1024,
+                "no opt-in for large shared memory is made");
   const size_t slow = 2 * channels * threads * sizeof(double);  // (the decisions come first, in the same place)
-  return launch(fn, p, phase == 2 ? units : units * p.draw_parts, threads, fixed + (slow > sizeof(RowShared) ? slow : sizeof(RowShared)), stream);
+  return launch(fn, p, units * p.draw_parts, threads, fixed + (slow > sizeof(RowShared) ? slow : sizeof(RowShared)), stream, p.draw_parts);
 }
 
 template <int DT>

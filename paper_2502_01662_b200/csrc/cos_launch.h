@@ -10,17 +10,18 @@ namespace cosv {
 
 // The streaming launch (mode: the Mode enum): a warp for each of the p.st_workers shares, blocks of `threads` threads; `report`:
 // the form that also decides and publishes.  mask: the launch before it that finds the plausibility threshold of every
-// position.  decide: the launch after it that decides the rows of a greedy run.
+// position.  decide: a launch after it that decides the rows (greedy runs, and
+// ensembles of one or of more than four models).
 template <int DT>
 cudaError_t stream_launch(const KParams& p, int mode, bool report, int threads, cudaStream_t stream);
 template <int DT>
 cudaError_t decide_launch(const KParams& p, int mode, cudaStream_t stream);
 template <int DT>
 cudaError_t mask_launch(const KParams& p, int threads, cudaStream_t stream);
-// The drawing launch with `channels` 2, 4 or 8 (logit level: 2) for `units` positions, blocks of `threads` threads: `phase` 0
-// for one launch, 1 and 2 for the two launches of the split form.
+// The drawing launch with `channels` 2, 4 or 8 (logit level: 2) for `units` positions: a cluster of p.draw_parts blocks of `threads`
+// threads for each.
 template <int DT>
-cudaError_t draw_launch(const KParams& p, bool ensemble, int channels, int phase, int units, int threads, cudaStream_t stream);
+cudaError_t draw_launch(const KParams& p, bool ensemble, int channels, int units, int threads, cudaStream_t stream);
 // Test hook: the combined distribution of every position.
 template <int DT>
 cudaError_t dump_launch(const KParams& p, int mode, cudaStream_t stream);

@@ -705,10 +705,9 @@ static __device__ __noinline__ double rescale_any(double s, float ref, float R) 
   return s == 0.0 ? 0.0 : s * exp2(static_cast<double>(ref) - static_cast<double>(R));
 }
 __device__ __forceinline__ double rescale(double s, float ref, float R) {
-  const float d = ref - R;
-  if (ref == R) return s;
-  if (d == floorf(d) && d > -1000.f) return s * __hiloint2double((1023 + static_cast<int>(d)) << 20, 0);
-  return rescale_any(s, ref, R);
+  const float d = fmaxf(ref - R, -1000.f);  // (a sum that far below is nothing; the empty sum's reference is minus infinity)
+  if (d != floorf(d)) return rescale_any(s, ref, R);
+  return s * __hiloint2double((1023 + static_cast<int>(d)) << 20, 0);
 }
 
 // The records of a line: `slots` (a model each, or the proposer's and the combined logits) for every position r that share w

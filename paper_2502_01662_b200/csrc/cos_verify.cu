@@ -49,8 +49,6 @@ struct cos_verify_ctx {
   int2* d_jobs;
   UnitStats* d_ustats;
   int* d_row_draw;
-  double* d_draw_rec;
-  int* d_draw_arrivals;
   // optional per-stage timing (cos_verify_set_stage_timing)
   bool timing;
   cudaEvent_t ev[4];
@@ -137,39 +135,43 @@ int draw_channels(const cos_verify_config& c) {
   return c.n <= 4 ? 4 : 8;
 }
 
-// Ensembles of one or of more than four models draw in two launches.
-bool draw_split(const cos_verify_config& c) { return c.combine == COS_COMBINE_PROB_ENSEMBLE && (c.n == 1 || c.n > 4); }
+// Ensembles of one or of more than four models decide in a launch of their own.
+bool decides_first(const cos_verify_config& c) { return c.combine == COS_COMBINE_PROB_ENSEMBLE && (c.n == 1 || c.n > 4); }
 
-// How the drawing launch shares a position out.  The device holds 32 warps per multiprocessor (two channels) or 16;
-// every position gets as many blocks as all of them fit at once, blocks of 128 threads where that is eight or more, of 64
-// where the rounding down would leave more of the device idle.  A chunk (one record of sums) has one step at least for
-// each warp, about eight at most, so that the token is searched in few steps, as far as the scratch holds `records` of them.
+// How the drawing launch shares a position out.  The device holds 32 warps per multiprocessor (two channels) or 16; a
+// position gets a cluster of blocks of 16, 8 or 4 warps, whichever leaves least of the device idle.  Clusters of more than four
+// blocks are taken only where they need no more than two thirds of the device: they do not pack (32 clusters of 8 blocks
+// of 16 warps, on paper a fit, ran in two waves: 51 us instead of 37 for 32 rows of 32000 tokens; 64 of 8 blocks of 8 warps
+// 109 instead of 92 for 64 rows of 151936).
+// A warp has a few chunks (one record of sums each), of eight steps where there is room for the records, so that the token is
+// searched in few steps.
 struct DrawPlan {
   int threads, parts, cs, chunks;
 };
-DrawPlan draw_plan(const cos_verify_config& c, long long units, int sm_count, long long records) {
+DrawPlan draw_plan(const cos_verify_config& c, long long units, int sm_count) {
   DrawPlan d;
   const int nsteps = (c.vocab + 32 * entries_per_vec(c.dtype) - 1) / (32 * entries_per_vec(c.dtype));
-  const long long warps = static_cast<long long>(sm_count) * (draw_channels(c) == 2 ? 32 : 16);
-  d.threads = draw_split(c) ? 256 : (warps / 4 >= 8 * units ? 128 : 64);
-  const int nw = d.threads / 32;
-  long long parts = warps / nw / units;
-  if (parts > (nsteps + nw - 1) / nw) parts = (nsteps + nw - 1) / nw;
-  d.parts = parts < 1 ? 1 : static_cast<int>(parts);
-  const int mine = (nsteps + d.parts * nw - 1) / (d.parts * nw);  // steps of a warp
-  const int k = (mine + 7) / 8;
-  d.cs = (mine + k - 1) / k;
-  const long long most = records / units;  // chunks of a position
-  if (static_cast<long long>(d.cs) * most < nsteps) d.cs = static_cast<int>((nsteps + most - 1) / most);
-  d.chunks = (nsteps + d.cs - 1) / d.cs;
+  const int ch = draw_channels(c), most = ch == 2 ? 32 : 16;
+  int best = 0;
+  for (int nw = ch == 8 ? 8 : 16; nw >= 4; nw /= 2) {
+    const long long blocks = static_cast<long long>(sm_count) * (most / nw);
+    long long parts = blocks / units;
+    if (parts > 4) {
+      const long long loose = blocks * 2 / 3 / units;
+      parts = loose < 4 ? 4 : (loose > 8 ? 8 : loose);
+    }
+    if (parts > (nsteps + nw - 1) / nw) parts = (nsteps + nw - 1) / nw;
+    if (parts < 1 && nw == 4) parts = 1;
+    if (parts * nw > best) {
+      best = static_cast<int>(parts) * nw;
+      d.threads = nw * 32;
+      d.parts = static_cast<int>(parts);
+    }
+  }
+  const int mine = (nsteps + best - 1) / best, room = 768 / ch / best;  // steps and records of a warp
+  d.chunks = (mine + 7) / 8 < room ? (mine + 7) / 8 : room;
+  d.cs = (mine + d.chunks - 1) / d.chunks;
   return d;
-}
-
-// Records the scratch of a context holds: chunks of four steps for a position of every row, of sixteen for all positions.
-long long draw_records(const cos_verify_config& c, int sm_count) {
-  const long long nsteps = (c.vocab + 32 * entries_per_vec(c.dtype) - 1) / (32 * entries_per_vec(c.dtype));
-  const long long rows = c.max_batch, one = rows * ((nsteps + 3) / 4), all = rows * (c.gamma + 1) * ((nsteps + 15) / 16);
-  return (one > all ? one : all) + 64LL * sm_count;
 }
 
 constexpr int kStreamBlock = 512;   // threads of a block of a full streaming launch, two blocks per multiprocessor
@@ -220,27 +222,26 @@ cudaError_t launch_stream(const cos_verify_config& c, int mode, KParams& p, bool
     if (report && p.early_exit) p.st_slabs = p.P;
     const int threads = plan_line(p, c, p.num_units / p.st_slabs, workers, sm_count);
     if (e == cudaSuccess) e = stream_launch<DT>(p, mode, report, threads, stream);
-    p.decide = report ? 0 : 1;
-    if (e == cudaSuccess && !report && p.greedy) e = decide_launch<DT>(p, mode, stream);
+    p.decide = report || decides_first(c) ? 0 : 1;
+    const bool first = p.greedy || decides_first(c);
+    if (e == cudaSuccess && !report && first) e = decide_launch<DT>(p, mode, stream);
     if (e == cudaSuccess && p.greedy && p.dump_r != nullptr) e = dump_launch<DT>(p, mode, stream);
     return e;
   });
 }
 
 // The launches that draw the tokens: of every position (`all`: test hook, residual masses) or of one per row.
-cudaError_t launch_draw(const cos_verify_config& c, KParams& p, bool all, int sm_count, long long records, cudaStream_t stream) {
+cudaError_t launch_draw(const cos_verify_config& c, KParams& p, bool all, int sm_count, cudaStream_t stream) {
   const bool ens = c.combine == COS_COMBINE_PROB_ENSEMBLE;
   const int units = all ? p.num_units : p.B;
-  const DrawPlan d = draw_plan(c, units, sm_count, records);
+  const DrawPlan d = draw_plan(c, units, sm_count);
   p.draw_all = all ? 1 : 0;
   p.draw_parts = d.parts;
   p.draw_cs = d.cs;
   p.draw_chunks = d.chunks;
   return by_dtype(c.dtype, [&](auto dt) {
     constexpr int DT = decltype(dt)::value;
-    cudaError_t e = cudaSuccess;
-    for (int phase = draw_split(c) ? 1 : 0; phase <= (draw_split(c) ? 2 : 0) && e == cudaSuccess; ++phase)
-      e = draw_launch<DT>(p, ens, draw_channels(c), phase, units, d.threads, stream);
+    cudaError_t e = draw_launch<DT>(p, ens, draw_channels(c), units, d.threads, stream);
     if (e == cudaSuccess && p.dump_r != nullptr) e = dump_launch<DT>(p, mode_of(c), stream);
     return e;
   });
@@ -310,7 +311,6 @@ cos_status init_scratch(cos_verify_ctx* ctx, cudaStream_t stream) {
   cudaError_t e = cudaMemsetAsync(ctx->d_work_counter, 0, 4 * sizeof(unsigned), stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_st_arrivals, 0, units * sizeof(int), stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_mask_key, 0, units * sizeof(unsigned), stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_draw_arrivals, 0, units * sizeof(int), stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_row_arrivals, 0, rows * sizeof(int), stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_row_reject, 0x7f, rows * sizeof(int), stream);  // "none yet"
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_job_count, 0, 2 * sizeof(int), stream);
@@ -367,9 +367,6 @@ extern "C" cos_status cos_verify_create(const cos_verify_config* config, cos_ver
   ok = ok && cudaMalloc(&ctx->d_st_arrivals, rows * P * sizeof(int)) == cudaSuccess;
   ok = ok && cudaMalloc(&ctx->d_mask_key, rows * P * sizeof(unsigned)) == cudaSuccess;
   ok = ok && cudaMalloc(&ctx->d_row_draw, rows * sizeof(int)) == cudaSuccess;
-  ok = ok && cudaMalloc(&ctx->d_draw_arrivals, rows * P * sizeof(int)) == cudaSuccess;
-  if (ok && config->temperature > 0.0f)
-    ok = cudaMalloc(&ctx->d_draw_rec, static_cast<size_t>(draw_records(*config, ctx->sm_count)) * 2 * draw_channels(*config) * sizeof(double)) == cudaSuccess;
   ctx->wait_limit = 1u << 20;
   ctx->test_drop = 0;
   ctx->fused = false;
@@ -495,8 +492,6 @@ cos_status run_launches(cos_verify_ctx* ctx, const cos_verify_args* a, void* cud
   p.st_arrivals = ctx->d_st_arrivals;
   p.mask_key = ctx->d_mask_key;
   p.row_draw = ctx->d_row_draw;
-  p.draw_rec = ctx->d_draw_rec;
-  p.draw_arrivals = ctx->d_draw_arrivals;
   p.max_jobs = p.num_units + a->batch;
 
   const int mode = mode_of(c);
@@ -530,7 +525,7 @@ cos_status run_launches(cos_verify_ctx* ctx, const cos_verify_args* a, void* cud
   // under way at once anyway and the hint is not taken.
   const long long workers = stream_workers(c, p.num_units, ctx->sm_count);
   if (static_cast<long long>(p.B) * c.n * (c.vocab / entries_per_vec(c.dtype)) / workers < 1024 || a->dump_r != nullptr) p.early_exit = 0;
-  p.keep_stats = (a->lse != nullptr || a->dump_r != nullptr || draw_split(c)) ? 1 : 0;
+  p.keep_stats = (a->lse != nullptr || a->dump_r != nullptr || decides_first(c)) ? 1 : 0;
   e = launch_stream(c, mode, p, p.early_exit || by_items, workers, ctx->sm_count, stream);
   if (e != cudaSuccess) return cuda_fail(ctx, "kernel launch (streaming)", e);
   if (ctx->timing) cudaEventRecord(ctx->ev[1], stream);
@@ -541,7 +536,7 @@ cos_status run_launches(cos_verify_ctx* ctx, const cos_verify_args* a, void* cud
       e = fused_launch(c.dtype, mode, p, ctx->fplan, ctx->fscr, ctx->wait_limit, 0, true, stream);
       if (e != cudaSuccess) return cuda_fail(ctx, "kernel launch (drawing items)", e);
     } else {
-      e = launch_draw(c, p, all, ctx->sm_count, draw_records(c, ctx->sm_count), stream);
+      e = launch_draw(c, p, all, ctx->sm_count, stream);
       if (e != cudaSuccess) return cuda_fail(ctx, "kernel launch (drawing)", e);
     }
     if (ctx->timing) cudaEventRecord(ctx->ev[2], stream);
@@ -723,7 +718,7 @@ extern "C" cos_status cos_verify_get_info(const cos_verify_ctx* ctx, cos_verify_
   {
     // ordinary runs (no test hook): the streaming launch and one that decides, or one or two that decide and draw; one
     // more for the mask
-    const bool one_draw = !draw_split(ctx->cfg) || (ctx->fused && ctx->draw_fused);
+    const bool one_draw = !decides_first(ctx->cfg) || (ctx->fused && ctx->draw_fused);
     info->launches_per_run = (ctx->fused && ctx->use_fused) ? 1 : (ctx->cfg.temperature == 0.0f || one_draw ? 2 : 3);
     if (ctx->cfg.combine == COS_COMBINE_LOGIT_LINEAR && ctx->cfg.mask_model >= 0) ++info->launches_per_run;
   }
@@ -747,8 +742,6 @@ extern "C" cos_status cos_verify_destroy(cos_verify_ctx* ctx) {
   cudaFree(ctx->d_st_arrivals);
   cudaFree(ctx->d_mask_key);
   cudaFree(ctx->d_row_draw);
-  cudaFree(ctx->d_draw_rec);
-  cudaFree(ctx->d_draw_arrivals);
   for (int k = 0; k < 4; ++k)
     if (ctx->ev[k]) cudaEventDestroy(ctx->ev[k]);
   cudaFree(ctx->d_unit_res);
@@ -778,10 +771,9 @@ namespace {
 // Scratch of the context-free entry point.  It is part of the library image: every device
 // that loads the library holds these COS_STATIC_SCRATCH_BYTES until the process exits.
 // Layout: [0, 256) unused | arrival counters and mask keys | unit results | records of the streaming launch | unit
-// statistics | drawing positions | records of the drawing launch (kStaticDrawDoubles numbers).
+// statistics | drawing positions.
 static __device__ __align__(256) unsigned char g_static_scratch[COS_STATIC_SCRATCH_BYTES];
 
-constexpr long long kStaticDrawDoubles = 16LL * (COS_STATIC_MAX_POSITIONS + 8 * COS_STATIC_MAX_BATCH);
 constexpr int kStaticWorkers = 5120;  // warps of a streaming launch there is room for
 constexpr int kStaticMaxDevices = 64;
 // Device address of g_static_scratch per device.  In host code the symbol itself is only a
@@ -857,8 +849,7 @@ extern "C" cos_status cos_verify_run_static(const cos_verify_config* config, con
   unsigned char* basep = g_static_addr[c.device];
   int* d_arrivals = reinterpret_cast<int*>(basep + 256);
   int* d_st_arrivals = d_arrivals + n_rows;
-  int* d_draw_arrivals = d_st_arrivals + n_units;
-  unsigned* d_mask_key = reinterpret_cast<unsigned*>(d_draw_arrivals + (draws ? (all ? n_units : n_rows) : 0));
+  unsigned* d_mask_key = reinterpret_cast<unsigned*>(d_st_arrivals + n_units);
   e = cudaMemsetAsync(basep, 0, reinterpret_cast<unsigned char*>(d_mask_key + (masked ? n_units : 0)) - basep, stream);
   if (e != cudaSuccess) return cuda_fail(nullptr, "clearing the built-in scratch", e);
   int4* d_unit_res = reinterpret_cast<int4*>(basep + 256 + 4 * (COS_STATIC_MAX_BATCH + 3 * COS_STATIC_MAX_POSITIONS));
@@ -866,7 +857,6 @@ extern "C" cos_status cos_verify_run_static(const cos_verify_config* config, con
   UnitStats* d_ustats = reinterpret_cast<UnitStats*>(d_st_rec + COS_MAX_MODELS * (COS_STATIC_MAX_POSITIONS + kStaticWorkers));
   static_assert(sizeof(UnitStats) == 112, "COS_STATIC_SCRATCH_BYTES assumes 112 bytes of statistics per position");
   int* d_row_draw = reinterpret_cast<int*>(d_ustats + COS_STATIC_MAX_POSITIONS);
-  double* d_draw_rec = reinterpret_cast<double*>(d_row_draw + COS_STATIC_MAX_BATCH);
 
   KParams p;
   fill_params(c, a, p);
@@ -880,16 +870,14 @@ extern "C" cos_status cos_verify_run_static(const cos_verify_config* config, con
   p.st_arrivals = d_st_arrivals;
   p.mask_key = d_mask_key;
   p.row_draw = d_row_draw;
-  p.draw_rec = d_draw_rec;
-  p.draw_arrivals = d_draw_arrivals;
 
   long long workers = stream_workers(c, units, sm_count);
   if (workers > kStaticWorkers) workers = kStaticWorkers;
-  p.keep_stats = (a->dump_r != nullptr || draw_split(c)) ? 1 : 0;
+  p.keep_stats = (a->dump_r != nullptr || decides_first(c)) ? 1 : 0;
   e = launch_stream(c, mode_of(c), p, false, workers, sm_count, stream);
   if (e != cudaSuccess) return cuda_fail(nullptr, "kernel launch (streaming)", e);
   if (draws) {
-    e = launch_draw(c, p, all, sm_count, kStaticDrawDoubles / (2 * draw_channels(c)), stream);
+    e = launch_draw(c, p, all, sm_count, stream);
     if (e != cudaSuccess) return cuda_fail(nullptr, "kernel launch (drawing)", e);
   }
   return COS_OK;
