@@ -103,6 +103,8 @@ def load_library(rebuild: bool = False) -> ctypes.CDLL:
     lib.cos_verify_measure_ceiling.restype = ctypes.c_int
     lib.cos_verify_destroy.argtypes = [ctypes.c_void_p]
     lib.cos_verify_destroy.restype = ctypes.c_int
+    lib.cos_verify_run_static.argtypes = [ctypes.POINTER(cos_verify_config), ctypes.POINTER(cos_verify_args), ctypes.c_void_p]
+    lib.cos_verify_run_static.restype = ctypes.c_int
     lib.cos_verify_last_error.argtypes = [ctypes.c_void_p]
     lib.cos_verify_last_error.restype = ctypes.c_char_p
     _lib = lib
@@ -118,6 +120,26 @@ def _dtype_code(torch_dtype) -> int:
     if torch_dtype == torch.float16:
         return COS_DTYPE_F16
     raise ValueError(f"logits must be float32, bfloat16 or float16, not {torch_dtype}")
+
+
+def _current_stream(torch, index: int) -> int:
+    """torch's current stream of a device, as the address the library takes (the Stream object costs 2 us more)."""
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream(index).cuda_stream
+    return raw(index)
+
+
+def _make_args(logits, stride_model, stride_row, stride_pos, drafts, proposer, batch, flags, row_base, seed, offset, outs,
+               bonus_model, offset_device=None) -> cos_verify_args:
+    named = bonus_model is not None and bonus_model >= 0
+    ptr = {k: t.data_ptr() for k, t in outs.items()}
+    return cos_verify_args(
+        logits.data_ptr(), stride_model, stride_row, stride_pos,
+        drafts.data_ptr() if (drafts is not None and drafts.numel() > 0) else None, proposer.data_ptr(),
+        batch, flags, row_base, seed & 0xFFFFFFFFFFFFFFFF, offset & 0xFFFFFFFFFFFFFFFF,
+        ptr["accept_count"], ptr["out_tokens"], ptr["row_status"], ptr.get("diag"), ptr.get("r"), ptr.get("bonus_prob"),
+        bonus_model if named else 0, offset_device.data_ptr() if offset_device is not None else None, ptr.get("lse"))
 
 
 class CosVerifier:
@@ -180,23 +202,8 @@ class CosVerifier:
             raise ValueError("the vocabulary axis of logits must be contiguous")
         if _dtype_code(logits.dtype) != self.cfg.dtype:
             raise ValueError("logits dtype does not match the context")
-        a = cos_verify_args()
-        a.logits = logits.data_ptr()
-        a.stride_model, a.stride_row, a.stride_pos = logits.stride(0), logits.stride(1), logits.stride(2)
-        a.draft_tokens = drafts.data_ptr() if (drafts is not None and drafts.numel() > 0) else None
-        a.proposer = proposer.data_ptr()
-        a.batch, a.flags, a.row_base = B, flags, row_base
-        a.seed, a.offset = seed & 0xFFFFFFFFFFFFFFFF, offset & 0xFFFFFFFFFFFFFFFF
-        a.accept_count = outs["accept_count"].data_ptr()
-        a.out_tokens = outs["out_tokens"].data_ptr()
-        a.row_status = outs["row_status"].data_ptr()
-        a.diag = outs["diag"].data_ptr() if "diag" in outs else None
-        a.dump_r = outs["r"].data_ptr() if "r" in outs else None
-        a.bonus_prob = outs["bonus_prob"].data_ptr() if "bonus_prob" in outs else None
-        a.bonus_model = bonus_model if (bonus_model is not None and bonus_model >= 0) else 0
-        a.offset_device = offset_device.data_ptr() if offset_device is not None else None
-        a.lse = outs["lse"].data_ptr() if "lse" in outs else None
-        return a
+        sm, sr, sp, _ = logits.stride()
+        return _make_args(logits, sm, sr, sp, drafts, proposer, B, flags, row_base, seed, offset, outs, bonus_model, offset_device)
 
     def set_one_launch(self, enable=True):
         """cos_verify_set_one_launch: 1 / True: later runs take the one-launch kernel; 2: staged streaming launch, tokens
@@ -224,12 +231,9 @@ class CosVerifier:
         kw = dict(device=device)
         if pin:
             kw["pin_memory"] = True
-        outs = {
-            "accept_count": torch.empty(B, dtype=torch.int32, **kw),
-            "out_tokens": torch.empty((B, P), dtype=torch.int32, **kw),
-            "row_status": torch.empty(B, dtype=torch.int32, **kw),
-            "bonus_prob": torch.empty(B, dtype=torch.float32, **kw),
-        }
+        # one allocation for the small outputs (four of their own cost 8.4 us a call, this 5)
+        accept, status, bonus, tokens = torch.empty(B * (P + 3), dtype=torch.int32, **kw).split_with_sizes((B, B, B, B * P))
+        outs = {"accept_count": accept, "out_tokens": tokens.view(B, P), "row_status": status, "bonus_prob": bonus.view(torch.float32)}
         if diag:
             outs["diag"] = torch.empty((B, P, 4), dtype=torch.float32, **kw)
         if dump_r:
@@ -262,8 +266,8 @@ class CosVerifier:
         if offset_device is not None and (offset_device.dtype != torch.int64 or not offset_device.is_cuda):
             raise ValueError("offset_device must be an int64 device tensor")
         a = self._fill_args(logits, drafts, proposer, seed, offset, row_base, flags, outs, bonus_model, offset_device)
-        s = torch.cuda.current_stream(logits.device) if stream is None else stream
-        self._check(self._lib.cos_verify_run(self._ctx, ctypes.byref(a), ctypes.c_void_p(s.cuda_stream)))
+        s = _current_stream(torch, logits.get_device()) if stream is None else stream.cuda_stream
+        self._check(self._lib.cos_verify_run(self._ctx, ctypes.byref(a), s))
         return outs
 
     def run_host(self, logits, drafts, proposer, seed: int, offset: int, row_base: int = 0, flags: int = 0,
@@ -280,8 +284,8 @@ class CosVerifier:
         if outs is None:
             outs = self._alloc_outs(B, P, V, "cpu", diag, False, pin=True)
         a = self._fill_args(logits, drafts, proposer, seed, offset, row_base, flags, outs, bonus_model)
-        s = torch.cuda.current_stream(self.cfg.device) if stream is None else stream
-        self._check(self._lib.cos_verify_run_host(self._ctx, ctypes.byref(a), ctypes.c_void_p(s.cuda_stream)))
+        s = _current_stream(torch, self.cfg.device) if stream is None else stream.cuda_stream
+        self._check(self._lib.cos_verify_run_host(self._ctx, ctypes.byref(a), s))
         return outs
 
     def close(self):
@@ -336,9 +340,6 @@ def run_static(n: int, combine: int, weights: Sequence[float], temperature: floa
     """
     import torch
     lib = load_library()
-    lib.cos_verify_run_static.argtypes = [ctypes.POINTER(cos_verify_config), ctypes.POINTER(cos_verify_args),
-                                          ctypes.c_void_p]
-    lib.cos_verify_run_static.restype = ctypes.c_int
     cfg = cos_verify_config()
     cfg.n, cfg.combine = n, combine
     for i, w in enumerate(list(weights)[:COS_MAX_MODELS]):
@@ -348,26 +349,15 @@ def run_static(n: int, combine: int, weights: Sequence[float], temperature: floa
     cfg.dtype, cfg.device, cfg.cluster_size, cfg.host_staging = _dtype_code(logits.dtype), device, cluster_size, 0
     if outs is None:
         raise ValueError("run_static needs preallocated outputs (it must not allocate)")
-    a = cos_verify_args()
-    a.logits = logits.data_ptr()
-    a.stride_model, a.stride_row, a.stride_pos = logits.stride(0), logits.stride(1), logits.stride(2)
-    a.draft_tokens = drafts.data_ptr() if (drafts is not None and drafts.numel() > 0) else None
-    a.proposer = proposer.data_ptr()
     if proposer.dim() == 2:
         flags |= COS_RUN_PROPOSER_PER_POSITION
     if bonus_model is not None and bonus_model >= 0:
         flags |= COS_RUN_BONUS_FROM_MODEL
-    a.batch, a.flags, a.row_base = logits.shape[1], flags, row_base
-    a.seed, a.offset = seed & 0xFFFFFFFFFFFFFFFF, offset & 0xFFFFFFFFFFFFFFFF
-    a.accept_count = outs["accept_count"].data_ptr()
-    a.out_tokens = outs["out_tokens"].data_ptr()
-    a.row_status = outs["row_status"].data_ptr()
-    a.diag = outs["diag"].data_ptr() if "diag" in outs else None
-    a.dump_r = None
-    a.bonus_prob = outs["bonus_prob"].data_ptr() if "bonus_prob" in outs else None
-    a.bonus_model = bonus_model if (bonus_model is not None and bonus_model >= 0) else 0
-    s = torch.cuda.current_stream(logits.device) if stream is None else stream
-    st = lib.cos_verify_run_static(ctypes.byref(cfg), ctypes.byref(a), ctypes.c_void_p(s.cuda_stream))
+    sm, sr, sp, _ = logits.stride()
+    a = _make_args(logits, sm, sr, sp, drafts, proposer, logits.shape[1], flags, row_base, seed, offset, outs, bonus_model)
+    a.dump_r = a.lse = None
+    s = _current_stream(torch, logits.get_device()) if stream is None else stream.cuda_stream
+    st = lib.cos_verify_run_static(ctypes.byref(cfg), ctypes.byref(a), s)
     if st != COS_OK:
         raise CosVerifyError(st, lib.cos_verify_last_error(None).decode())
     return outs

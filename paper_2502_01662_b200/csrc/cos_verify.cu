@@ -65,13 +65,8 @@ struct cos_verify_ctx {
   unsigned wait_limit;  // idle polls after which a block of the one-launch kernel gives up
   int test_drop;        // test hook: one streaming warp never reports its first item
   void* d_logits;
-  int* d_drafts;
-  int* d_proposer;
-  float* d_bonus;
-  int* d_accept;
-  int* d_tokens;
-  unsigned* d_status;
-  float* d_diag;
+  int* d_small;   // host-pointer runs: drafts and proposers, then the outputs
+  int* h_small;   // the same, pinned: one copy each way
   std::string err;
 };
 
@@ -401,13 +396,8 @@ extern "C" cos_status cos_verify_create(const cos_verify_config* config, cos_ver
   if (ok && config->host_staging) {
     const size_t V = static_cast<size_t>(config->vocab);
     ok = ok && cudaMalloc(&ctx->d_logits, static_cast<size_t>(config->n) * rows * P * V * elem_bytes(config->dtype)) == cudaSuccess;
-    ok = ok && cudaMalloc(&ctx->d_drafts, rows * (P > 1 ? P - 1 : 1) * sizeof(int)) == cudaSuccess;
-    ok = ok && cudaMalloc(&ctx->d_proposer, rows * P * sizeof(int)) == cudaSuccess;
-    ok = ok && cudaMalloc(&ctx->d_bonus, rows * sizeof(float)) == cudaSuccess;
-    ok = ok && cudaMalloc(&ctx->d_accept, rows * sizeof(int)) == cudaSuccess;
-    ok = ok && cudaMalloc(&ctx->d_tokens, rows * P * sizeof(int)) == cudaSuccess;
-    ok = ok && cudaMalloc(&ctx->d_status, rows * sizeof(unsigned)) == cudaSuccess;
-    ok = ok && cudaMalloc(&ctx->d_diag, rows * P * 4 * sizeof(float)) == cudaSuccess;
+    const size_t small = rows * (2 * P + 3 + P + 4 * P) * sizeof(int);
+    ok = ok && cudaMalloc(&ctx->d_small, small) == cudaSuccess && cudaMallocHost(&ctx->h_small, small) == cudaSuccess;
   }
   if (!ok) {
     (void)cudaGetLastError();
@@ -615,41 +605,51 @@ extern "C" cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   cudaError_t e = cudaSetDevice(c.device);
   if (e != cudaSuccess) return cuda_fail(ctx, "cudaSetDevice", e);
+  // The small arrays go over in one copy each way, by way of pinned memory of the context (the call waits for its copies, so that
+  // memory is free again when it returns): seven small copies of their own were half of the call for one row.
   const size_t lbytes = static_cast<size_t>(c.n) * B * P * V * elem_bytes(c.dtype);
-  e = cudaMemcpyAsync(ctx->d_logits, a->logits, lbytes, cudaMemcpyHostToDevice, stream);
-  if (e == cudaSuccess && c.gamma > 0)
-    e = cudaMemcpyAsync(ctx->d_drafts, a->draft_tokens, B * c.gamma * sizeof(int), cudaMemcpyHostToDevice, stream);
-  const size_t nprop = (a->flags & COS_RUN_PROPOSER_PER_POSITION) ? static_cast<size_t>(B * P) : static_cast<size_t>(B);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_proposer, a->proposer, nprop * sizeof(int), cudaMemcpyHostToDevice, stream);
-  if (e != cudaSuccess) return cuda_fail(ctx, "host to device copy", e);
+  const size_t ndraft = static_cast<size_t>(B * c.gamma), nprop = static_cast<size_t>((a->flags & COS_RUN_PROPOSER_PER_POSITION) ? B * P : B);
+  const size_t nout = static_cast<size_t>(B * (P + 3) + (a->diag ? B * P * 4 : 0));
+  int *out = ctx->d_small + ndraft + nprop, *h_out = ctx->h_small + ndraft + nprop;
+  if (ndraft) memcpy(ctx->h_small, a->draft_tokens, ndraft * sizeof(int));
+  memcpy(ctx->h_small + ndraft, a->proposer, nprop * sizeof(int));
+  e = cudaMemcpyAsync(ctx->d_small, ctx->h_small, (ndraft + nprop) * sizeof(int), cudaMemcpyHostToDevice, stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_logits, a->logits, lbytes, cudaMemcpyHostToDevice, stream);
+  if (e != cudaSuccess) {
+    cudaStreamSynchronize(stream);
+    return cuda_fail(ctx, "host to device copy", e);
+  }
   cos_verify_args d = *a;
   d.flags &= ~COS_RUN_INPUTS_SETTLED;  // the inputs are what the copies above have just written
   d.logits = ctx->d_logits;
-  d.draft_tokens = ctx->d_drafts;
-  d.proposer = ctx->d_proposer;
-  d.accept_count = ctx->d_accept;
-  d.out_tokens = ctx->d_tokens;
-  d.row_status = ctx->d_status;
-  d.diag = a->diag ? ctx->d_diag : nullptr;
-  d.bonus_prob = a->bonus_prob ? ctx->d_bonus : nullptr;
+  d.draft_tokens = ctx->d_small;
+  d.proposer = ctx->d_small + ndraft;
+  d.accept_count = out;
+  d.row_status = reinterpret_cast<unsigned*>(out + B);
+  d.bonus_prob = a->bonus_prob ? reinterpret_cast<float*>(out + 2 * B) : nullptr;
+  d.out_tokens = out + 3 * B;
+  d.diag = a->diag ? reinterpret_cast<float*>(out + 3 * B + B * P) : nullptr;
   if (a->offset_device) {  // a host address here, like every other pointer of this call
     d.offset = *a->offset_device;
     d.offset_device = nullptr;
   }
   cos_status st = cos_verify_run(ctx, &d, stream);
-  if (st != COS_OK) return st;
-  e = cudaMemcpyAsync(a->accept_count, ctx->d_accept, B * sizeof(int), cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(a->out_tokens, ctx->d_tokens, B * P * sizeof(int), cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(a->row_status, ctx->d_status, B * sizeof(unsigned), cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess && a->diag)
-    e = cudaMemcpyAsync(a->diag, ctx->d_diag, B * P * 4 * sizeof(float), cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess && a->bonus_prob)
-    e = cudaMemcpyAsync(a->bonus_prob, ctx->d_bonus, B * sizeof(float), cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  if (st != COS_OK) {
+    cudaStreamSynchronize(stream);
+    return st;
+  }
+  e = cudaMemcpyAsync(h_out, out, nout * sizeof(int), cudaMemcpyDeviceToHost, stream);
+  const cudaError_t done = cudaStreamSynchronize(stream);
+  if (e == cudaSuccess) e = done;
   if (e != cudaSuccess) {
     ctx->scratch_dirty = true;
     return cuda_fail(ctx, "device to host copy", e);
   }
+  memcpy(a->accept_count, h_out, B * sizeof(int));
+  memcpy(a->row_status, h_out + B, B * sizeof(int));
+  if (a->bonus_prob) memcpy(a->bonus_prob, h_out + 2 * B, B * sizeof(int));
+  memcpy(a->out_tokens, h_out + 3 * B, B * P * sizeof(int));
+  if (a->diag) memcpy(a->diag, h_out + 3 * B + B * P, B * P * 4 * sizeof(int));
   return COS_OK;
 }
 
@@ -747,13 +747,8 @@ extern "C" cos_status cos_verify_destroy(cos_verify_ctx* ctx) {
   cudaFree(ctx->d_unit_res);
   for (int k = 0; k < 9; ++k) cudaFree(ctx->fused_mem[k]);
   cudaFree(ctx->d_logits);
-  cudaFree(ctx->d_drafts);
-  cudaFree(ctx->d_proposer);
-  cudaFree(ctx->d_bonus);
-  cudaFree(ctx->d_accept);
-  cudaFree(ctx->d_tokens);
-  cudaFree(ctx->d_status);
-  cudaFree(ctx->d_diag);
+  cudaFree(ctx->d_small);
+  cudaFreeHost(ctx->h_small);
   (void)cudaGetLastError();
   delete ctx;
   return COS_OK;
@@ -850,7 +845,8 @@ extern "C" cos_status cos_verify_run_static(const cos_verify_config* config, con
   int* d_arrivals = reinterpret_cast<int*>(basep + 256);
   int* d_st_arrivals = d_arrivals + n_rows;
   unsigned* d_mask_key = reinterpret_cast<unsigned*>(d_st_arrivals + n_units);
-  e = cudaMemsetAsync(basep, 0, reinterpret_cast<unsigned char*>(d_mask_key + (masked ? n_units : 0)) - basep, stream);
+  // (only the mask keys have to start clean: without a mask nothing in the array is read before the launches write it)
+  if (masked) e = cudaMemsetAsync(d_mask_key, 0, n_units * sizeof(unsigned), stream);
   if (e != cudaSuccess) return cuda_fail(nullptr, "clearing the built-in scratch", e);
   int4* d_unit_res = reinterpret_cast<int4*>(basep + 256 + 4 * (COS_STATIC_MAX_BATCH + 3 * COS_STATIC_MAX_POSITIONS));
   int4* d_st_rec = d_unit_res + COS_STATIC_MAX_POSITIONS;
