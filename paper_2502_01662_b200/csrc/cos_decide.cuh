@@ -14,6 +14,11 @@ namespace cosv {
 // drafts) is fetched before the launch waits for the streaming launch to end.
 constexpr int kTile = 16;  // positions decided at a time
 
+struct TestInputs {
+  int draft, pi;
+  unsigned word[2];
+};
+
 struct RowShared {
   Finish fin[kTile];
   unsigned word[kTile];
@@ -60,11 +65,24 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
   };
   const DraftLogits first = fetch(0, mine);
   const RecordRange first_range = range(0, mine, mine < pairs0);
+  auto ahead = [&](int j) {  // what the accept test of position j needs of the inputs
+    TestInputs t;
+    t.draft = j < p.gamma ? __ldg(p.drafts + b * p.gamma + j) : 0;
+    t.pi = proposer_of(p, b, j);
+    unsigned rnd[4];
+    philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
+    t.word[0] = rnd[0];
+    t.word[1] = rnd[1];
+    return t;
+  };
+  TestInputs first_test = {0, 0, {0u, 0u}};
+  if (tid < p.P && tid < kTile) first_test = ahead(tid);
   if (tid == 0) {
     sh.a = -1;
     sh.status = 0u;
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
+#pragma unroll 1
   for (int j0 = 0; j0 < p.P; j0 += kTile) {
     const int count = p.P - j0 < kTile ? p.P - j0 : kTile;
     for (int q0 = 0; q0 < count * slots; q0 += per) {  // (the same number of times for every lane of a warp)
@@ -87,15 +105,13 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
     if (tid < 32) {
       if (lane < count) {
         const int j = j0 + lane;
+        const TestInputs t = j0 == 0 ? first_test : ahead(j);
         const bool is_bonus = (j == p.gamma);
-        const int draft = is_bonus ? 0 : __ldg(p.drafts + b * p.gamma + j);
-        const bool draft_ok = is_bonus || (draft >= 0 && draft < p.V);
-        const int pi = proposer_of(p, b, j);
-        const bool pi_ok = (pi >= 0 && pi < p.n);
-        unsigned rnd[4];
-        philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
-        sh.word[lane] = rnd[1];
-        decide_unit<DT, MODE>(p, sh.fin[lane], word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), is_bonus, draft, draft_ok, pi, pi_ok, pi_ok ? pi : 0);
+        const bool draft_ok = is_bonus || (t.draft >= 0 && t.draft < p.V);
+        const bool pi_ok = (t.pi >= 0 && t.pi < p.n);
+        sh.word[lane] = t.word[1];
+        decide_unit<DT, MODE>(p, sh.fin[lane], word_to_uniform(t.word[0]), word_to_uniform(t.word[1]), is_bonus, t.draft, draft_ok, t.pi, pi_ok,
+                              pi_ok ? t.pi : 0);
       }
       __syncwarp();
       if (sh.a < 0) {

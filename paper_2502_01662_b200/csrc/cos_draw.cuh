@@ -136,22 +136,55 @@ __device__ __forceinline__ bool load_unit(const KParams& p, int u, DrawUnit<NCH>
   return true;
 }
 
-// fp64 terms of one token from the stored logits: e_i of every channel.  Rare ("big" tokens, more than 2^-8 of a
-// normaliser, and the bonus token's probability); out of line.
+// The arguments of the channels for one token.
 template <int DT, bool ENS, int NCH>
-__device__ __noinline__ void exact_terms(const KParams& p, const DrawUnit<NCH>& u, int e, double* out) {
-  float lv[COS_MAX_MODELS];
-  for (int i = 0; i < p.n; ++i) lv[i] = Elem<DT>::load1(u.base + i * p.s_model * Elem<DT>::bytes, e);
+__device__ __forceinline__ void entry_args(const KParams& p, const DrawUnit<NCH>& u, int e, float (&x)[NCH]) {
+  const long long row_step = p.s_model * Elem<DT>::bytes;
   if (ENS) {
 #pragma unroll
-    for (int i = 0; i < NCH; ++i)
-      out[i] = (i < p.n) ? exp2(static_cast<double>(lv[i]) * p.cT64 + static_cast<double>(u.nref[i])) : 0.0;
+    for (int i = 0; i < NCH; ++i) {
+      x[i] = -INFINITY;
+      if (i < p.n) x[i] = Elem<DT>::load1(u.base + i * row_step, e);
+    }
   } else {
-    double cd = 0.0;
-    for (int i = 0; i < p.n; ++i) cd = fma(p.w64[i], static_cast<double>(lv[i]), cd);
-    const bool in = p.mask_model < 0 || (lv[p.mask_model] >= u.thr);
-    out[0] = exp2(static_cast<double>(lv[u.pis]) * p.cT64 + static_cast<double>(u.nref[0]));
-    out[1] = in ? exp2(cd * p.cT64 + static_cast<double>(u.nref[1])) : 0.0;
+    const float l0 = Elem<DT>::load1(u.base, e);
+    float l1 = 0.f, gate = l0;
+    if (p.n >= 2) l1 = Elem<DT>::load1(u.base + row_step, e);
+    x[0] = u.pis == 0 ? l0 : l1;
+    if (p.mask_model == 1) gate = l1;
+    x[1] = __fmul_rn(p.w[0], l0);
+    if (p.n >= 2) x[1] = fmaf(p.w[1], l1, x[1]);
+    for (int i = 2; i < p.n; ++i) {
+      const float l = Elem<DT>::load1(u.base + i * row_step, e);
+      if (i == u.pis) x[0] = l;
+      if (i == p.mask_model) gate = l;
+      x[1] = fmaf(p.w[i], l, x[1]);
+    }
+    if (p.mask_model >= 0 && !(gate >= u.thr)) x[1] = -INFINITY;
+  }
+}
+
+// fp64 terms of one token (its arguments: x): e_i of every channel.  For "big" tokens (more than 2^-8 of a normaliser) and the
+// bonus token's probability.
+template <int DT, bool ENS, int NCH>
+__device__ __forceinline__ void exact_terms(const KParams& p, const DrawUnit<NCH>& u, int e, const float (&x)[NCH], double (&out)[NCH]) {
+  double t[NCH];
+#pragma unroll
+  for (int i = 0; i < NCH; ++i) t[i] = static_cast<double>(x[i]);
+  if (!ENS && !(x[1] == -INFINITY)) {  // (the combination again, in fp64)
+    t[1] = 0.0;
+    for (int i = 0; i < p.n; ++i) t[1] = fma(p.w64[i], static_cast<double>(Elem<DT>::load1(u.base + i * p.s_model * Elem<DT>::bytes, e)), t[1]);
+  }
+#pragma unroll 1
+  for (int k = 0; k < NCH; ++k) {  // (one copy of the exponential)
+    double v = 0.0;
+#pragma unroll
+    for (int i = 0; i < NCH; ++i)
+      if (i == k) v = t[i] * p.cT64 + static_cast<double>(u.nref[i]);
+    v = exp2(v);
+#pragma unroll
+    for (int i = 0; i < NCH; ++i)
+      if (i == k) out[i] = v;
   }
 }
 
@@ -207,50 +240,63 @@ __device__ __forceinline__ void vector_args(const KParams& p, const DrawUnit<NCH
   }
 }
 
-// One vector the fast loop left out, entry by entry: it holds a big entry (in fp64 then), or it is one of the ragged ends
-// of the row.  Its sums go to the thread's slots of `acc`.  Rare; out of line.
-template <int DT, bool ENS, int NCH, bool AL>
-__device__ __noinline__ void slow_vector(const KParams& p, const DrawUnit<NCH>& u, int v, double* acc) {
-  constexpr int E = Elem<DT>::E;
-  const int T = blockDim.x;
-  if (v * E >= p.V) return;
-  float x[NCH][E];
-  vector_args<DT, ENS, NCH, AL>(p, u, v, x);
-  float z[NCH], a[NCH];
+// The mass of one big token.  Out of line.
+template <int DT, bool ENS, int NCH>
+__device__ __noinline__ double big_mass(const KParams& p, const DrawUnit<NCH>& u, const double* inv, int e) {
+  float x[NCH];
+  double d[NCH];
+  entry_args<DT, ENS, NCH>(p, u, e, x);
+  exact_terms<DT, ENS, NCH>(p, u, e, x, d);
+  return exact_mass<ENS, NCH>(p, d, inv, u.pis, u.law);
+}
+
+// The vectors the fast loop left out (bit k of a lane's `slow`: its vector of step c + k): those with a big entry, which is summed in
+// fp64 then, and the ragged ends of the row.  The warp takes 32 entries at a time, one a lane; the sums go to the lanes'
+// slots of `acc`.  Out of line.  (One lane going through its vector while the others waited took 2 us a vector, and the warp that
+// happened on most big tokens was the last of its cluster by 5 to 8 us.)
+template <int DT, bool ENS, int NCH>
+__device__ __noinline__ void slow_vectors(const KParams& p, const DrawUnit<NCH>& u, int c, unsigned slow, double* acc) {
+  constexpr int E = Elem<DT>::E, G = 32 / E;
+  const int T = blockDim.x, lane = threadIdx.x & 31;
+  for (unsigned any = __reduce_or_sync(0xffffffffu, slow); any; any &= any - 1) {
+    const int k = __ffs(any) - 1;
+    unsigned m = __ballot_sync(0xffffffffu, (slow >> k) & 1u);
+    while (m) {
+      unsigned t = m;
 #pragma unroll
-  for (int i = 0; i < NCH; ++i) z[i] = a[i] = 0.f;
-#pragma unroll
-  for (int k = 0; k < E; ++k) {
-    float e[NCH], tot = 0.f;
-    bool big = false;
-#pragma unroll
-    for (int i = 0; i < NCH; ++i) {
-      e[i] = ex2_approx(fmaf(x[i][k], p.cT, u.nref[i]));
-      big = big || e[i] > u.bt[i];
-      tot = __fadd_rn(tot, __fmul_rn(u.ct[i], e[i]));
-    }
-    if (big) {
-      double d[NCH], t64 = 0.0;
-      exact_terms<DT, ENS, NCH>(p, u, v * E + k, d);
-#pragma unroll
-      for (int i = 0; i < NCH; ++i) t64 += static_cast<double>(u.ct[i]) * d[i];
-#pragma unroll
-      for (int i = 0; i < NCH; ++i) {
-        acc[i * T] += d[i];
-        if (t64 > 0.0) acc[(NCH + i) * T] += d[i];
+      for (int q = 0; q < G; ++q) {
+        if (q < lane / E) t &= t - 1;
+        m &= m - 1;
       }
-    } else {
+      const int e = t ? ((c + k) * 32 + __ffs(t) - 1) * E + lane % E : p.V;
+      if (e < p.V) {
+        float x[NCH], f[NCH], tot = 0.f;
+        bool big = false;
+        entry_args<DT, ENS, NCH>(p, u, e, x);
 #pragma unroll
-      for (int i = 0; i < NCH; ++i) {
-        z[i] += e[i];
-        if (tot > 0.f) a[i] += e[i];
+        for (int i = 0; i < NCH; ++i) {
+          f[i] = ex2_approx(fmaf(x[i], p.cT, u.nref[i]));
+          big = big || f[i] > u.bt[i];
+          tot = __fadd_rn(tot, __fmul_rn(u.ct[i], f[i]));
+        }
+        double d[NCH];
+#pragma unroll
+        for (int i = 0; i < NCH; ++i) d[i] = static_cast<double>(f[i]);
+        bool counts = tot > 0.f;
+        if (big) {
+          exact_terms<DT, ENS, NCH>(p, u, e, x, d);
+          double t64 = 0.0;
+#pragma unroll
+          for (int i = 0; i < NCH; ++i) t64 += static_cast<double>(u.ct[i]) * d[i];
+          counts = t64 > 0.0;
+        }
+#pragma unroll
+        for (int i = 0; i < NCH; ++i) {
+          acc[i * T] += d[i];
+          if (counts) acc[(NCH + i) * T] += d[i];
+        }
       }
     }
-  }
-#pragma unroll
-  for (int i = 0; i < NCH; ++i) {
-    acc[i * T] += static_cast<double>(z[i]);
-    acc[(NCH + i) * T] += static_cast<double>(a[i]);
   }
 }
 
@@ -390,14 +436,10 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawUnit<N
         sums[NCH + 2 * q] = static_cast<double>(lo2(ac[q])) + (more ? acc[(NCH + 2 * q) * T] : 0.0);
         sums[NCH + 2 * q + 1] = static_cast<double>(hi2(ac[q])) + (more ? acc[(NCH + 2 * q + 1) * T] : 0.0);
       }
-      if (slow || ce < end) {
+      if (ce < end || __any_sync(0xffffffffu, slow != 0u)) {
 #pragma unroll
         for (int q = 0; q < 2 * NCH; ++q) acc[q * T] = sums[q];
-        while (slow) {
-          const int k = __ffs(slow) - 1;
-          slow &= slow - 1;
-          slow_vector<DT, ENS, NCH, AL>(p, u, (c + k) * 32 + lane, acc);
-        }
+        slow_vectors<DT, ENS, NCH>(p, u, c, slow, acc);
 #pragma unroll
         for (int q = 0; q < 2 * NCH; ++q) sums[q] = acc[q * T];
       }
@@ -440,17 +482,16 @@ __device__ __forceinline__ void draw_sweep(const KParams& p, DrawShared<NCH>& sh
   draw_sweep_as<DT, ENS, NCH, AL, false, true>(p, u, cs, s_lo, s_hi, acc, rec, part);
 }
 
-// Masses of one lane's tokens of step s under the refined normalisers (coefficients cf = k / Z): small ones in fp32, big
-// ones in fp64; returns the lane's total (fp32 sum of the small ones in token order, then the big ones).
+// The mass of one lane's tokens of step s under the refined normalisers (coefficients cf = k / Z): small ones in fp32, big
+// ones in fp64.
 template <int DT, bool ENS, int NCH, bool AL>
-__device__ __forceinline__ double step_masses(const KParams& p, const DrawUnit<NCH>& u, const float* cf, const double* inv,
-                                              int s, float (&m32)[Elem<DT>::E], unsigned& bigbits,
-                                              double (&mbig)[Elem<DT>::E]) {
+__device__ __forceinline__ double step_mass(const KParams& p, const DrawUnit<NCH>& u, const float* cf, const double* inv, int s) {
   constexpr int E = Elem<DT>::E;
   const int v = s * 32 + (threadIdx.x & 31);
   float x[NCH][E];
   vector_args<DT, ENS, NCH, AL>(p, u, v, x);
-  bigbits = 0u;
+  unsigned bigbits = 0u;
+  float ls = 0.f;
 #pragma unroll
   for (int k = 0; k < E; ++k) {
     float tot = 0.f;
@@ -461,25 +502,25 @@ __device__ __forceinline__ double step_masses(const KParams& p, const DrawUnit<N
       big = big || e > u.bt[i];
       tot = __fadd_rn(tot, __fmul_rn(cf[i], e));
     }
-    m32[k] = big ? 0.f : fmaxf(0.f, tot);
+    ls += big ? 0.f : fmaxf(0.f, tot);
     bigbits |= big ? (1u << k) : 0u;
-    mbig[k] = 0.0;
   }
-  float ls = 0.f;
-#pragma unroll
-  for (int k = 0; k < E; ++k) ls += m32[k];
   double own = static_cast<double>(ls);
-  if (bigbits) {
-#pragma unroll
-    for (int k = 0; k < E; ++k)
-      if (bigbits & (1u << k)) {
-        double d[NCH];
-        exact_terms<DT, ENS, NCH>(p, u, v * E + k, d);
-        mbig[k] = exact_mass<ENS, NCH>(p, d, inv, u.pis, u.law);
-        own += mbig[k];
-      }
-  }
+  for (; bigbits; bigbits &= bigbits - 1) own += big_mass<DT, ENS, NCH>(p, u, inv, v * E + __ffs(bigbits) - 1);
   return own;
+}
+template <int DT, bool ENS, int NCH>
+__device__ __forceinline__ double token_mass(const KParams& p, const DrawUnit<NCH>& u, const float* cf, const double* inv, int e) {
+  float x[NCH], tot = 0.f;
+  bool big = false;
+  entry_args<DT, ENS, NCH>(p, u, e, x);
+#pragma unroll
+  for (int i = 0; i < NCH; ++i) {
+    const float f = ex2_approx(fmaf(x[i], p.cT, u.nref[i]));
+    big = big || f > u.bt[i];
+    tot = __fadd_rn(tot, __fmul_rn(cf[i], f));
+  }
+  return big ? big_mass<DT, ENS, NCH>(p, u, inv, e) : static_cast<double>(fmaxf(0.f, tot));
 }
 
 // The whole position again by the cluster's first block, for another law.  Rare; out of line.
@@ -591,16 +632,14 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
     const int s0 = static_cast<int>(static_cast<long long>(p.nsteps) * ww / W) + win % p.draw_chunks * cs;
     const int end = static_cast<int>(static_cast<long long>(p.nsteps) * (ww + 1) / W);
     const int s1 = s0 + cs < end ? s0 + cs : end, gsz = (cs + 31) / 32;
-    float m32[E];
-    unsigned bigbits = 0u;
-    double mbig[E], own = 0.0;
-    int held = -1;  // the step whose masses the lanes of this warp hold
+    double own = 0.0;
+    int held = -1;  // the step whose mass the lanes of this warp hold
 #pragma unroll 1
     for (int t = warp; s0 + t * gsz < s1; t += nw) {
       double rm = 0.0;
 #pragma unroll 1
       for (int s = s0 + t * gsz; s < s0 + (t + 1) * gsz && s < s1; ++s) {
-        own = step_masses<DT, ENS, NCH, AL>(p, u, cf, inv, s, m32, bigbits, mbig);
+        own = step_mass<DT, ENS, NCH, AL>(p, u, cf, inv, s);
         rm += warp_sum(own);
         held = s;
       }
@@ -608,57 +647,51 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
     }
     __syncthreads();
     if (held < 0) return;  // (no step of the chunk is this warp's)
-    const double v = (s0 + lane * gsz < s1) ? sh.step_mass[lane] : 0.0;
-    double inc = v;
-#pragma unroll 1
-    for (int d = 1; d < 32; d <<= 1) {
-      const double o = __shfl_up_sync(0xffffffffu, inc, d);
-      if (lane >= d) inc += o;
-    }
-    const double from = sh.base;
-    const unsigned ok = __ballot_sync(0xffffffffu, v > 0.0 && from + inc >= target), pos = __ballot_sync(0xffffffffu, v > 0.0);
-    if (pos == 0u) return;
-    const int k = ok ? __ffs(ok) - 1 : 31 - __clz(pos);  // rounding corner: the last record with mass
-    if (k % nw != warp) return;
-    double at = from + __shfl_sync(0xffffffffu, inc - v, k);
-    // one warp goes on: the record's steps in order, an fp64 prefix over the lanes, then the lane's tokens
-    int token = -1, last_tok = -1;
-#pragma unroll 1
-    for (int s = s0 + k * gsz; s < s0 + (k + 1) * gsz && s < s1 && token < 0; ++s) {
-      if (s != held) own = step_masses<DT, ENS, NCH, AL>(p, u, cf, inv, s, m32, bigbits, mbig);
-      held = s;
-      double in = own;
+    // running total over the lanes; the first that reaches the target, or the last with mass where rounding leaves none
+    auto first_reach = [&](double m, double from, double& upto) -> int {
+      double in = m;
 #pragma unroll 1
       for (int d = 1; d < 32; d <<= 1) {
         const double o = __shfl_up_sync(0xffffffffu, in, d);
         if (lane >= d) in += o;
       }
-      const unsigned lok = __ballot_sync(0xffffffffu, own > 0.0 && at + in >= target), lpos = __ballot_sync(0xffffffffu, own > 0.0);
-      double part = at + (in - own);
-      int found = -1, lastk = -1;
-#pragma unroll
-      for (int q = 0; q < E; ++q) {
-        const double mk = (bigbits & (1u << q)) ? mbig[q] : static_cast<double>(m32[q]);
-        part += mk;
-        if (mk > 0.0) {
-          lastk = (s * 32 + lane) * E + q;
-          if (found < 0 && part >= target) found = lastk;
-        }
+      const unsigned some = __ballot_sync(0xffffffffu, m > 0.0), ok = __ballot_sync(0xffffffffu, m > 0.0 && from + in >= target);
+      const int k = ok ? __ffs(ok) - 1 : 31 - __clz(some);
+      upto = from + __shfl_sync(0xffffffffu, in - m, k & 31);
+      return ok ? k : k - 32;  // (negative: not reached; -33: no mass at all)
+    };
+    double at;
+    int k = first_reach((s0 + lane * gsz < s1) ? sh.step_mass[lane] : 0.0, sh.base, at);
+    if (k == -33) return;
+    if ((k & 31) % nw != warp) return;
+    // one warp goes on: the record's steps in order, the lanes of a step, the tokens of a lane's vector
+    const int g0 = s0 + (k & 31) * gsz, g1 = g0 + gsz < s1 ? g0 + gsz : s1;
+    int step = -1, who = 0;
+    double before = 0.0;
+#pragma unroll 1
+    for (int s = g0; s < g1; ++s) {
+      if (s != held) own = step_mass<DT, ENS, NCH, AL>(p, u, cf, inv, s);
+      double upto;
+      const int l = first_reach(own, at, upto);
+      if (l != -33) {
+        step = s;
+        who = l & 31;
+        before = upto;
       }
-      if (found < 0) found = lastk;
-      if (lok) token = __shfl_sync(0xffffffffu, found, __ffs(lok) - 1);
-      if (lpos) last_tok = __shfl_sync(0xffffffffu, lastk, 31 - __clz(lpos));
-      at += __shfl_sync(0xffffffffu, in, 31);
+      if (l >= 0) break;
+      held = s;
+      if (s + 1 < g1) at += warp_sum(own);
     }
-    if (token < 0) token = last_tok;
-    if (lane == 0 && token >= 0) {
+    if (step < 0) return;
+    const int e = (step * 32 + who) * E + lane;
+    double m = 0.0;
+    if (lane < E && e < p.V) m = token_mass<DT, ENS, NCH>(p, u, cf, inv, e);
+    k = first_reach(m, before, at);
+    const int token = (step * 32 + who) * E + (k & 31);
+    if (lane == 0 && k != -33) {
       p.out_tokens[u.uidx] = token;
       // Algorithm 2's Score returns the bonus token with its probability under the law it came from
-      if (u.j == p.gamma && p.bonus_prob != nullptr) {
-        double d[NCH];
-        exact_terms<DT, ENS, NCH>(p, u, token, d);
-        p.bonus_prob[u.b] = static_cast<float>(exact_mass<ENS, NCH>(p, d, inv, u.pis, u.law));
-      }
+      if (u.j == p.gamma && p.bonus_prob != nullptr) p.bonus_prob[u.b] = static_cast<float>(big_mass<DT, ENS, NCH>(p, u, inv, token));
     }
     return;
   }
@@ -721,7 +754,8 @@ __global__ void __launch_bounds__(NCH == 8 ? 256 : kMaxDrawThreads, NCH == 2 ? 2
   // launched while the kernel before it drains; nothing but inputs is read before that one is complete
   bool draws;
   if (NCH != 8 && p.decide) {
-    draws = decide_unit_to_draw<DT, ENS, NCH>(p, sh, *reinterpret_cast<RowShared*>(slots), slot, rank);
+    RowShared& rs = *reinterpret_cast<RowShared*>(slots);
+    draws = decide_unit_to_draw<DT, ENS, NCH>(p, sh, rs, slot, rank);
   } else {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     DrawUnit<NCH> d;
@@ -735,7 +769,10 @@ __global__ void __launch_bounds__(NCH == 8 ? 256 : kMaxDrawThreads, NCH == 2 ? 2
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   cluster_arrive();
   cluster_wait();
-  if (rank == 0) locate<DT, ENS, NCH, AL>(p, sh, acc);
+  if (rank == 0) {
+    __syncthreads();
+    locate<DT, ENS, NCH, AL>(p, sh, acc);
+  }
 }
 
 // Test hook: the combined distribution of every position, token by token, from the statistics the streaming launch left.
