@@ -74,10 +74,12 @@ struct KParams {
   int2* jobs;              // x = b * P + j of a unit that draws a token (y unused)
   UnitStats* ustats;       // [B*P]: merged statistics of sweep 1, read back by the later stages
   int use_jobs;            // the list of drawing positions is kept too (tokens drawn by the persistent kernel)
-  // the streaming launch: a line of st_line vectors (st_nv for each position) in st_workers shares, st_rem of them of st_q + 1
-  // groups of eight vectors, the others of st_q; st_slabs lines one after another (one, or one for each position of a row)
-  int st_workers, st_slabs, st_nv;
-  long long st_line, st_q, st_rem;
+  // the streaming launch: a line of st_line vectors (st_nv for each position) in st_workers shares of st_share vectors (the last may
+  // be shorter); st_slabs lines one after another (one, or one for each position of a row)
+  int st_workers, st_slabs, st_nv, st_share;
+  long long st_line;
+  double st_inv_nv, st_inv_share;  // one over them, for divisions
+  int slot_inv;            // 65536 over the records of a (share, position) pair, rounded up: likewise
   int4* st_rec;            // records: statistics of a share's part of a position
   int* st_arrivals;        // [B*P]: warps that have reported; zero between runs
   unsigned* mask_key;      // [B*P]: largest logit of the gating model as an ordered integer; zero between runs

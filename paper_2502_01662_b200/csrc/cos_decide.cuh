@@ -14,11 +14,6 @@ namespace cosv {
 // drafts) is fetched before the launch waits for the streaming launch to end.
 constexpr int kTile = 16;  // positions decided at a time
 
-struct TestInputs {
-  int draft, pi;
-  unsigned word[2];
-};
-
 struct RowShared {
   Finish fin[kTile];
   unsigned word[kTile];
@@ -39,57 +34,48 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
   const int tid = threadIdx.x, lane = tid & 31, T = blockDim.x;
   const int slots = record_slots<MODE>(p);
   const bool optional = p.diag != nullptr || p.keep_stats;
-  // lanes that share a pair: as many as the block has to spare
-  const int pairs0 = (p.P < kTile ? p.P : kTile) * slots;
-  int g = 32;
-  while (g > 1 && pairs0 * g > T) g >>= 1;
-  const int per = T / g, mine = tid / g, sub = tid % g;
+  // lanes that share a pair: as many as the block has to spare (it has a thread for each at least)
+  const int pairs = (p.P < kTile ? p.P : kTile) * slots;
+  int lg = 5;
+#pragma unroll 1
+  while (pairs << lg > T) --lg;
+  const int mine = tid >> lg, sub = tid & ((1 << lg) - 1);
+  const int pos = (mine * p.slot_inv) >> 16, i = mine - pos * slots;
   const char* row = reinterpret_cast<const char*>(p.logits) + static_cast<long long>(b) * p.s_row * Elem<DT>::bytes;
-  auto fetch = [&](int j0, int q) {  // the logits at the draft of pair q of the tile at j0
-    const int j = j0 + q / slots, i = q % slots;
-    DraftLogits d;
-    d.x = -INFINITY;
-    d.xe = INFINITY;
-    if (kSample && sub == 0 && j < p.gamma) {
-      const int draft = __ldg(p.drafts + b * p.gamma + j);
-      const int pi = (MODE == kLogitSample) ? proposer_of(p, b, j) : 0;
-      const int pis = (pi >= 0 && pi < p.n) ? pi : 0;
-      d = draft_logits<DT, MODE>(p, row + static_cast<long long>(j) * p.s_pos * Elem<DT>::bytes, i, pis,
-                                 draft >= 0 && draft < p.V ? draft : -1);
-    }
-    return d;
-  };
-  auto range = [&](int j0, int q, bool live) {
-    const RecordRange none = {nullptr, 0};
-    return live ? records_of<MODE>(p, 0, p.num_units, b * p.P + j0 + q / slots) : none;
-  };
-  const DraftLogits first = fetch(0, mine);
-  const RecordRange first_range = range(0, mine, mine < pairs0);
-  auto ahead = [&](int j) {  // what the accept test of position j needs of the inputs
-    TestInputs t;
-    t.draft = j < p.gamma ? __ldg(p.drafts + b * p.gamma + j) : 0;
-    t.pi = proposer_of(p, b, j);
-    unsigned rnd[4];
-    philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
-    t.word[0] = rnd[0];
-    t.word[1] = rnd[1];
-    return t;
-  };
-  TestInputs first_test = {0, 0, {0u, 0u}};
-  if (tid < p.P && tid < kTile) first_test = ahead(tid);
   if (tid == 0) {
     sh.a = -1;
     sh.status = 0u;
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");
 #pragma unroll 1
   for (int j0 = 0; j0 < p.P; j0 += kTile) {
     const int count = p.P - j0 < kTile ? p.P - j0 : kTile;
-    for (int q0 = 0; q0 < count * slots; q0 += per) {  // (the same number of times for every lane of a warp)
-      const int q = q0 + mine, pos = q / slots, i = q % slots;
-      const bool live = q < count * slots, ready = j0 == 0 && q0 == 0;
-      const DraftLogits d = ready ? first : (live ? fetch(j0, q) : first);
-      const Merged m = merge_slot<MODE>(p, ready ? first_range : range(j0, q, live), i, g, sub);
+    const bool live = pos < count;
+    // what the merge and the accept test need of the inputs
+    DraftLogits d;
+    d.x = -INFINITY;
+    d.xe = INFINITY;
+    RecordRange range = {nullptr, 0};
+    if (live) {
+      const int j = j0 + pos;
+      range = records_of<MODE>(p, 0, p.num_units, b * p.P + j);
+      if (kSample && sub == 0 && j < p.gamma) {
+        const int draft = __ldg(p.drafts + b * p.gamma + j);
+        const int pi = (MODE == kLogitSample) ? proposer_of(p, b, j) : 0;
+        d = draft_logits<DT, MODE>(p, row + static_cast<long long>(j) * p.s_pos * Elem<DT>::bytes, i, (pi >= 0 && pi < p.n) ? pi : 0,
+                                   draft >= 0 && draft < p.V ? draft : -1);
+      }
+    }
+    int draft = 0, pi = 0;
+    unsigned rnd[4] = {0u, 0u, 0u, 0u};
+    if (tid < count) {
+      const int j = j0 + tid;
+      if (j < p.gamma) draft = __ldg(p.drafts + b * p.gamma + j);
+      pi = proposer_of(p, b, j);
+      philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
+    }
+    if (j0 == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+    {
+      const Merged m = merge_slot<MODE>(p, range, i, 1 << lg, sub);
       if (live && sub == 0) {
         Finish& f = sh.fin[pos];
         if (kSample) {
@@ -104,14 +90,12 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
     __syncthreads();
     if (tid < 32) {
       if (lane < count) {
-        const int j = j0 + lane;
-        const TestInputs t = j0 == 0 ? first_test : ahead(j);
-        const bool is_bonus = (j == p.gamma);
-        const bool draft_ok = is_bonus || (t.draft >= 0 && t.draft < p.V);
-        const bool pi_ok = (t.pi >= 0 && t.pi < p.n);
-        sh.word[lane] = t.word[1];
-        decide_unit<DT, MODE>(p, sh.fin[lane], word_to_uniform(t.word[0]), word_to_uniform(t.word[1]), is_bonus, t.draft, draft_ok, t.pi, pi_ok,
-                              pi_ok ? t.pi : 0);
+        const bool is_bonus = (j0 + lane == p.gamma);
+        const bool draft_ok = is_bonus || (draft >= 0 && draft < p.V);
+        const bool pi_ok = (pi >= 0 && pi < p.n);
+        sh.word[lane] = rnd[1];
+        decide_unit<DT, MODE>(p, sh.fin[lane], word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), is_bonus, draft, draft_ok, pi, pi_ok,
+                              pi_ok ? pi : 0);
       }
       __syncwarp();
       if (sh.a < 0) {
@@ -139,6 +123,7 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
     const int a = sh.a;
     const int asked = want >= 0 ? want : a;
     if (optional) {
+#pragma unroll 1
       for (int k = tid; k < count; k += T) {
         const int j = j0 + k, uidx = b * p.P + j;
         if (!writes_unit(j)) continue;
@@ -153,6 +138,7 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
         if (p.keep_stats) {
           UnitStats& st = p.ustats[uidx];
           if (kSample) {
+#pragma unroll 1
             for (int i = 0; i < slots; ++i) {
               st.s[i] = f.fsoft[i].s;
               st.ref[i] = f.fsoft[i].ref;
@@ -160,6 +146,7 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
             st.thr32 = f.thr;
           } else {  // the atoms of r, for the test hook
             st.pad[0] = (f.dec.status & COS_ROW_NONFINITE) ? -1 : f.dec.natoms;
+#pragma unroll 1
             for (int i = 0; i < f.dec.natoms; ++i) {
               st.s[i] = f.dec.atom_mass[i];
               st.ref[i] = __int_as_float(f.dec.atom_tok[i]);
@@ -170,15 +157,16 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
       }
     }
     if (MODE == kLogitSample || MODE == kLogitGreedy) {
-      if (p.mask_model >= 0)
-        for (int k = tid; k < count; k += T)
-          if (writes_unit(j0 + k)) p.mask_key[b * p.P + j0 + k] = 0u;  // ready for the next run
+#pragma unroll 1
+      for (int k = p.mask_model >= 0 ? tid : count; k < count; k += T)
+        if (writes_unit(j0 + k)) p.mask_key[b * p.P + j0 + k] = 0u;  // ready for the next run
     }
     if (a >= 0 && asked < j0 + count && !optional && p.mask_model < 0) break;
     __syncthreads();  // the tile is about to be overwritten
   }
   const int a = sh.a;
   if (writes_row(a)) {
+#pragma unroll 1
     for (int k = tid; k < p.P; k += T)
       p.out_tokens[static_cast<long long>(b) * p.P + k] = k < a ? p.drafts[b * p.gamma + k] : (k == a && !kSample ? sh.cand : -1);
     if (tid == 0) {

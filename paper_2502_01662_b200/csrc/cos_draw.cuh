@@ -536,6 +536,7 @@ __device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh
   const int lane = threadIdx.x & 31, i = lane / G, live = ENS ? p.n : 2;
   const DrawUnit<NCH>& u = sh.unit;
   double z = 0.0;
+#pragma unroll 1
   for (int w = lane % G; w < W; w += G) z += sh.part[w][i];
 #pragma unroll
   for (int d = G / 2; d > 0; d >>= 1) z += __shfl_xor_sync(0xffffffffu, z, d);
@@ -558,7 +559,7 @@ __device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh
   const int chunks = W * p.draw_chunks, per = (chunks + 31) / 32;
   const int c_lo = lane * per, c_hi = c_lo + per < chunks ? c_lo + per : chunks;
   double mine = 0.0;
-#pragma unroll 2
+#pragma unroll 1
   for (int c = c_lo; c < c_hi; ++c) {
     const double m = mass_of(c);
     sh.recs[c * NCH] = m;
@@ -575,6 +576,7 @@ __device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh
   double before = incl - mine, base = 0.0;
   int first = -1, last = -1;
   if (mine > 0.0)
+#pragma unroll 1
     for (int c = c_lo; c < c_hi; ++c) {
       const double m = sh.recs[c * NCH];
       if (m > 0.0 && first < 0) {
@@ -603,6 +605,7 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
   const int live = ENS ? p.n : 2, W = p.draw_parts * nw;
   DrawUnit<NCH>& u = sh.unit;
   const int cs = p.draw_cs;
+#pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {
     if (warp == 0) find_chunk<ENS, NCH>(p, sh, W);
     __syncthreads();

@@ -39,14 +39,19 @@ struct Finish {  // what a position is decided from, and the decision
   Decision dec;
 };
 
-// A worker's share of the line, in vectors: shares are whole multiples of eight vectors (128 bytes) of the line.
-__device__ __forceinline__ long long worker_lo(const KParams& p, int w) {
-  const long long at = (w * p.st_q + (w < p.st_rem ? w : p.st_rem)) * 8;
-  return at < p.st_line ? at : p.st_line;
+// x / d for places in the line (x < 2^53, quotient an int): a multiplication and a correction; the compiler's 64-bit division
+// is 100 instructions long, and code is what the short launches spend their time on.
+__device__ __forceinline__ int line_div(long long x, int d, double inv) {
+  int q = static_cast<int>(static_cast<double>(x) * inv);
+  const long long r = x - static_cast<long long>(q) * d;
+  if (r < 0) --q;
+  if (r >= d) ++q;
+  return q;
 }
-__device__ __forceinline__ int worker_of(const KParams& p, long long x) {
-  const long long x8 = x >> 3, wide = p.st_rem * (p.st_q + 1);
-  return static_cast<int>(x8 < wide ? x8 / (p.st_q + 1) : p.st_rem + (x8 - wide) / p.st_q);
+__device__ __forceinline__ int worker_of(const KParams& p, long long x) { return line_div(x, p.st_share, p.st_inv_share); }
+__device__ __forceinline__ long long worker_lo(const KParams& p, int w) {
+  const long long x = static_cast<long long>(w) * p.st_share;
+  return x < p.st_line ? x : p.st_line;
 }
 
 // Entries of a row that are not part of its whole vectors: [0, head) and [tail, V), fewer than three vectors in all.
@@ -572,6 +577,7 @@ __device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double
   bool finite = pi_ok;
   if (kSample) {
     const int nsoft = (MODE == kEnsembleSample) ? p.n : 2;
+#pragma unroll 1
     for (int k = 0; k < nsoft; ++k) {
       const SoftPart& f = sh.fsoft[k];
       finite = finite && isfinite(f.ref) && isfinite(f.s) && (f.s > 0.0);
@@ -584,6 +590,7 @@ __device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double
         if (draft_ok) {
           double r_d = 0.0, q_d = 0.0;
           if (MODE == kEnsembleSample) {
+#pragma unroll 1
             for (int i = 0; i < p.n; ++i) {
               r_d += p.w64[i] * sh.pdraft[i];
               if (i == pi) q_d = sh.pdraft[i];
@@ -610,6 +617,7 @@ __device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double
     // greedy: distributions are atoms at lowest-index argmaxes
     int qtok;
     if (MODE == kEnsembleGreedy) {
+#pragma unroll 1
       for (int i = 0; i < p.n; ++i) finite = finite && !sh.farg[i].bad && isfinite(sh.farg[i].val);
       qtok = sh.farg[pis].idx;
     } else {
@@ -622,12 +630,15 @@ __device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double
     } else {
       // atoms of r, sorted by token, masses accumulated in model order
       if (MODE == kEnsembleGreedy) {
+#pragma unroll 1
         for (int i = 0; i < p.n; ++i) {
           int t = sh.farg[i].idx, pos = 0;
+#pragma unroll 1
           while (pos < d.natoms && d.atom_tok[pos] < t) ++pos;
           if (pos < d.natoms && d.atom_tok[pos] == t) {
             d.atom_mass[pos] += p.w64[i];
           } else {
+#pragma unroll 1
             for (int k = d.natoms; k > pos; --k) {
               d.atom_tok[k] = d.atom_tok[k - 1];
               d.atom_mass[k] = d.atom_mass[k - 1];
@@ -643,6 +654,7 @@ __device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double
         d.atom_mass[0] = 1.0;
       }
       auto r_at = [&](int t) {
+#pragma unroll 1
         for (int k = 0; k < d.natoms; ++k)
           if (d.atom_tok[k] == t) return d.atom_mass[k];
         return 0.0;
@@ -664,6 +676,7 @@ __device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double
         }
         // residual max(0, r - q) over the atoms, summed in token order
         double S = 0.0;
+#pragma unroll 1
         for (int k = 0; k < d.natoms; ++k) S += fmax(0.0, d.atom_mass[k] - (d.atom_tok[k] == qtok ? 1.0 : 0.0));
         d.S = S;
         if (!(S > 0.0)) {
@@ -673,12 +686,14 @@ __device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double
       }
       // inverse CDF over the atoms (token order): smallest k with running sum >= u * total
       double total = 0.0;
+#pragma unroll 1
       for (int k = 0; k < d.natoms; ++k)
         total += use_r ? d.atom_mass[k] : fmax(0.0, d.atom_mass[k] - (d.atom_tok[k] == qtok ? 1.0 : 0.0));
       const double target = u_smp * total;
       double run = 0.0;
       int lastpos = -1;
       d.cand = -1;
+#pragma unroll 1
       for (int k = 0; k < d.natoms; ++k) {
         double m = use_r ? d.atom_mass[k] : fmax(0.0, d.atom_mass[k] - (d.atom_tok[k] == qtok ? 1.0 : 0.0));
         run += m;
@@ -862,7 +877,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_mask_kernel(const __gri
   if (w >= p.st_workers) return;
   const int v_lo = whole_vectors<DT, AL>(p.V).lo, v_hi = whole_vectors<DT, AL>(p.V).hi;
   for (long long x = worker_lo(p, w), end = worker_lo(p, w + 1); x < end;) {
-    const int unit = static_cast<int>(x / p.st_nv);
+    const int unit = line_div(x, p.st_nv, p.st_inv_nv);
     const int o0 = static_cast<int>(x - static_cast<long long>(unit) * p.st_nv);
     const int o1 = end - x < p.st_nv - o0 ? o0 + static_cast<int>(end - x) : p.st_nv;
     const int b = unit / p.P, j = unit % p.P;
@@ -953,7 +968,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_stream_kernel(const __g
   if (w >= p.st_workers) return;
   const int slots = record_slots<MODE>(p);
   for (long long x = worker_lo(p, w), end = worker_lo(p, w + 1); x < end;) {
-    const int r = static_cast<int>(x / p.st_nv);
+    const int r = line_div(x, p.st_nv, p.st_inv_nv);
     const int o0 = static_cast<int>(x - static_cast<long long>(r) * p.st_nv);
     const int o1 = end - x < p.st_nv - o0 ? o0 + static_cast<int>(end - x) : p.st_nv;
     x += o1 - o0;
@@ -994,7 +1009,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_report_kernel(const __g
   bool waited = true;
   for (int slab = 0; slab < p.st_slabs; ++slab) {
     for (long long x = worker_lo(p, w), end = worker_lo(p, w + 1); x < end;) {
-      const int r = static_cast<int>(x / p.st_nv);
+      const int r = line_div(x, p.st_nv, p.st_inv_nv);
       const int o0 = static_cast<int>(x - static_cast<long long>(r) * p.st_nv);
       const int o1 = end - x < p.st_nv - o0 ? o0 + static_cast<int>(end - x) : p.st_nv;
       x += o1 - o0;

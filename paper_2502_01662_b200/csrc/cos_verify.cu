@@ -170,7 +170,7 @@ DrawPlan draw_plan(const cos_verify_config& c, long long units, int sm_count) {
 }
 
 constexpr int kStreamBlock = 512;   // threads of a block of a full streaming launch, two blocks per multiprocessor
-constexpr int kMinShare = 128;      // vectors a warp should have at least: four loads for each lane
+constexpr int kMinShare = 256;      // vectors a warp should have at least: eight loads for each lane, all on their way at once
 
 // Cut the line of `units` positions into shares for at most `workers` warps (see cos_stream.cuh).  Small runs take fewer warps, so
 // that each has a few loads in flight, in small blocks, so that they spread over the device.  Returns the block size.
@@ -179,12 +179,14 @@ int plan_line(KParams& p, const cos_verify_config& c, long long units, long long
   p.st_nv = p.vec_ok ? nvec : nvec - 2;  // (unaligned rows: the first vector and the last one go entry by entry)
   if (p.st_nv < 1) p.st_nv = 1;          // nothing but ragged entries
   p.st_line = units * p.st_nv;
-  const long long groups = (p.st_line + 7) / 8;
   if (workers > p.st_line / kMinShare) workers = p.st_line / kMinShare;
   if (workers < 1) workers = 1;
-  p.st_workers = static_cast<int>(workers);
-  p.st_q = groups / workers;
-  p.st_rem = groups % workers;
+  p.st_share = static_cast<int>(((p.st_line + workers - 1) / workers + 7) / 8 * 8);
+  p.st_workers = static_cast<int>((p.st_line + p.st_share - 1) / p.st_share);
+  p.st_inv_nv = 1.0 / p.st_nv;
+  p.st_inv_share = 1.0 / p.st_share;
+  const int slots = c.combine == COS_COMBINE_PROB_ENSEMBLE ? c.n : 2;
+  p.slot_inv = (65536 + slots - 1) / slots;
   return workers <= 16LL * sm_count ? 128 : kStreamBlock;
 }
 
