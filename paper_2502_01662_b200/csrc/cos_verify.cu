@@ -170,7 +170,7 @@ DrawPlan draw_plan(const cos_verify_config& c, long long units, int sm_count) {
 }
 
 constexpr int kStreamBlock = 512;   // threads of a block of a full streaming launch, two blocks per multiprocessor
-constexpr int kMinShare = 256;      // vectors a warp should have at least: eight loads for each lane, all on their way at once
+constexpr int kMinShare = 128;      // vectors a warp should have at least: four loads for each lane
 
 // Cut the line of `units` positions into shares for at most `workers` warps (see cos_stream.cuh).  Small runs take fewer warps, so
 // that each has a few loads in flight, in small blocks, so that they spread over the device.  Returns the block size.
@@ -179,7 +179,9 @@ int plan_line(KParams& p, const cos_verify_config& c, long long units, long long
   p.st_nv = p.vec_ok ? nvec : nvec - 2;  // (unaligned rows: the first vector and the last one go entry by entry)
   if (p.st_nv < 1) p.st_nv = 1;          // nothing but ragged entries
   p.st_line = units * p.st_nv;
-  if (workers > p.st_line / kMinShare) workers = p.st_line / kMinShare;
+  long long most = p.st_line / kMinShare;
+  if (most < 8LL * sm_count) most /= 2;  // (where that leaves most of the device idle anyway: fewer records to merge)
+  if (workers > most) workers = most;
   if (workers < 1) workers = 1;
   p.st_share = static_cast<int>(((p.st_line + workers - 1) / workers + 7) / 8 * 8);
   p.st_workers = static_cast<int>((p.st_line + p.st_share - 1) / p.st_share);
