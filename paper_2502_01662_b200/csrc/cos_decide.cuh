@@ -51,18 +51,18 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
     const int count = p.P - j0 < kTile ? p.P - j0 : kTile;
     const bool live = pos < count;
     // what the merge and the accept test need of the inputs
-    DraftLogits d;
-    d.x = -INFINITY;
-    d.xe = INFINITY;
+    DraftLogits d = {0.f, 0.f};
     RecordRange range = {nullptr, 0};
+    int at = -1;  // the pair's draft token
+    const char* base = row + static_cast<long long>(j0 + pos) * p.s_pos * Elem<DT>::bytes;
     if (live) {
       const int j = j0 + pos;
       range = records_of<MODE>(p, 0, p.num_units, b * p.P + j);
       if (kSample && sub == 0 && j < p.gamma) {
-        const int draft = __ldg(p.drafts + b * p.gamma + j);
+        at = __ldg(p.drafts + b * p.gamma + j);
+        if (at >= p.V) at = -1;
         const int pi = (MODE == kLogitSample) ? proposer_of(p, b, j) : 0;
-        d = draft_logits<DT, MODE>(p, row + static_cast<long long>(j) * p.s_pos * Elem<DT>::bytes, i, (pi >= 0 && pi < p.n) ? pi : 0,
-                                   draft >= 0 && draft < p.V ? draft : -1);
+        d = draft_logits<DT, MODE>(p, base, i, (pi >= 0 && pi < p.n) ? pi : 0, at);
       }
     }
     int draft = 0, pi = 0;
@@ -80,7 +80,7 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
         Finish& f = sh.fin[pos];
         if (kSample) {
           f.fsoft[i] = m.soft;
-          f.pdraft[i] = draft_probability<DT, MODE>(p, d, m.thr, m.soft);
+          f.pdraft[i] = draft_probability<DT, MODE>(p, d, base, i, at, m.thr, m.soft);
         } else {
           f.farg[i] = m.arg;
         }

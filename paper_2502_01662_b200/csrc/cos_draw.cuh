@@ -72,6 +72,15 @@ __device__ __forceinline__ double warp_sums(double (&v)[N], int lane) {
   return v[0];
 }
 
+// What the functions that are not inlined need of the parameters, in shared memory: behind a call the parameters are no longer
+// operands from the constant bank but loads through a generic address, a trip to L2 for each line of them the first time.
+struct DrawConst {
+  long long row_step;  // bytes from one model's row to the next
+  double cT64, w64[COS_MAX_MODELS];
+  float cT, w[COS_MAX_MODELS];
+  int n, V, mask_model;
+};
+
 // What a block knows about its position.
 template <int NCH>
 struct DrawUnit {
@@ -138,24 +147,23 @@ __device__ __forceinline__ bool load_unit(const KParams& p, int u, DrawUnit<NCH>
 
 // The arguments of the channels for one token.
 template <int DT, bool ENS, int NCH>
-__device__ __forceinline__ void entry_args(const KParams& p, const DrawUnit<NCH>& u, int e, float (&x)[NCH]) {
-  const long long row_step = p.s_model * Elem<DT>::bytes;
+__device__ __forceinline__ void entry_args(const DrawConst& p, const DrawUnit<NCH>& u, int e, float (&x)[NCH]) {
   if (ENS) {
 #pragma unroll
     for (int i = 0; i < NCH; ++i) {
       x[i] = -INFINITY;
-      if (i < p.n) x[i] = Elem<DT>::load1(u.base + i * row_step, e);
+      if (i < p.n) x[i] = Elem<DT>::load1(u.base + i * p.row_step, e);
     }
   } else {
     const float l0 = Elem<DT>::load1(u.base, e);
     float l1 = 0.f, gate = l0;
-    if (p.n >= 2) l1 = Elem<DT>::load1(u.base + row_step, e);
+    if (p.n >= 2) l1 = Elem<DT>::load1(u.base + p.row_step, e);
     x[0] = u.pis == 0 ? l0 : l1;
     if (p.mask_model == 1) gate = l1;
     x[1] = __fmul_rn(p.w[0], l0);
     if (p.n >= 2) x[1] = fmaf(p.w[1], l1, x[1]);
     for (int i = 2; i < p.n; ++i) {
-      const float l = Elem<DT>::load1(u.base + i * row_step, e);
+      const float l = Elem<DT>::load1(u.base + i * p.row_step, e);
       if (i == u.pis) x[0] = l;
       if (i == p.mask_model) gate = l;
       x[1] = fmaf(p.w[i], l, x[1]);
@@ -167,13 +175,13 @@ __device__ __forceinline__ void entry_args(const KParams& p, const DrawUnit<NCH>
 // fp64 terms of one token (its arguments: x): e_i of every channel.  For "big" tokens (more than 2^-8 of a normaliser) and the
 // bonus token's probability.
 template <int DT, bool ENS, int NCH>
-__device__ __forceinline__ void exact_terms(const KParams& p, const DrawUnit<NCH>& u, int e, const float (&x)[NCH], double (&out)[NCH]) {
+__device__ __forceinline__ void exact_terms(const DrawConst& p, const DrawUnit<NCH>& u, int e, const float (&x)[NCH], double (&out)[NCH]) {
   double t[NCH];
 #pragma unroll
   for (int i = 0; i < NCH; ++i) t[i] = static_cast<double>(x[i]);
   if (!ENS && !(x[1] == -INFINITY)) {  // (the combination again, in fp64)
     t[1] = 0.0;
-    for (int i = 0; i < p.n; ++i) t[1] = fma(p.w64[i], static_cast<double>(Elem<DT>::load1(u.base + i * p.s_model * Elem<DT>::bytes, e)), t[1]);
+    for (int i = 0; i < p.n; ++i) t[1] = fma(p.w64[i], static_cast<double>(Elem<DT>::load1(u.base + i * p.row_step, e)), t[1]);
   }
 #pragma unroll 1
   for (int k = 0; k < NCH; ++k) {  // (one copy of the exponential)
@@ -190,7 +198,7 @@ __device__ __forceinline__ void exact_terms(const KParams& p, const DrawUnit<NCH
 
 // Mass of one token from its fp64 terms under the refined normalisers `inv` = 1 / Z_i.
 template <bool ENS, int NCH>
-__device__ __forceinline__ double exact_mass(const KParams& p, const double* e, const double* inv, int pis, int law) {
+__device__ __forceinline__ double exact_mass(const DrawConst& p, const double* e, const double* inv, int pis, int law) {
   double r = 0.0, q = 0.0;
   if (ENS) {
 #pragma unroll
@@ -242,7 +250,7 @@ __device__ __forceinline__ void vector_args(const KParams& p, const DrawUnit<NCH
 
 // The mass of one big token.  Out of line.
 template <int DT, bool ENS, int NCH>
-__device__ __noinline__ double big_mass(const KParams& p, const DrawUnit<NCH>& u, const double* inv, int e) {
+__device__ __noinline__ double big_mass(const DrawConst& p, const DrawUnit<NCH>& u, const double* inv, int e) {
   float x[NCH];
   double d[NCH];
   entry_args<DT, ENS, NCH>(p, u, e, x);
@@ -255,7 +263,7 @@ __device__ __noinline__ double big_mass(const KParams& p, const DrawUnit<NCH>& u
 // slots of `acc`.  Out of line.  (One lane going through its vector while the others waited took 2 us a vector, and the warp that
 // happened on most big tokens was the last of its cluster by 5 to 8 us.)
 template <int DT, bool ENS, int NCH>
-__device__ __noinline__ void slow_vectors(const KParams& p, const DrawUnit<NCH>& u, int c, unsigned slow, double* acc) {
+__device__ __noinline__ void slow_vectors(const DrawConst& p, const DrawUnit<NCH>& u, int c, unsigned slow, double* acc) {
   constexpr int E = Elem<DT>::E, G = 32 / E;
   const int T = blockDim.x, lane = threadIdx.x & 31;
   for (unsigned any = __reduce_or_sync(0xffffffffu, slow); any; any &= any - 1) {
@@ -307,7 +315,7 @@ __device__ __noinline__ void slow_vectors(const KParams& p, const DrawUnit<NCH>&
 // What bounds it: loads in flight (two steps of every model at a time) and issue (about 17 instructions per pair of terms).
 // PAIR, MASKED: logit level with exactly two models, and with a mask.
 template <int DT, bool ENS, int NCH, bool AL, bool PAIR, bool MASKED>
-__device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawUnit<NCH>& u, int cs, int s_lo, int s_hi, double* acc,
+__device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst& kc, const DrawUnit<NCH>& u, int cs, int s_lo, int s_hi, double* acc,
                                               unsigned rec, unsigned part) {
   constexpr int E = Elem<DT>::E;
   constexpr int NP = NCH / 2;
@@ -439,7 +447,7 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawUnit<N
       if (ce < end || __any_sync(0xffffffffu, slow != 0u)) {
 #pragma unroll
         for (int q = 0; q < 2 * NCH; ++q) acc[q * T] = sums[q];
-        slow_vectors<DT, ENS, NCH>(p, u, c, slow, acc);
+        slow_vectors<DT, ENS, NCH>(kc, u, c, slow, acc);
 #pragma unroll
         for (int q = 0; q < 2 * NCH; ++q) sums[q] = acc[q * T];
       }
@@ -455,6 +463,7 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawUnit<N
 // Shared memory of a block, in front of every thread's 2 NCH slots of the slow path.
 template <int NCH>
 struct DrawShared {
+  DrawConst kc;
   DrawUnit<NCH> unit;
   // (of the cluster's first block)
   double recs[kMaxSums];                         // sums of the chunks
@@ -475,17 +484,17 @@ __device__ __forceinline__ void draw_sweep(const KParams& p, DrawShared<NCH>& sh
   const int cs = p.draw_cs, used = (s_hi - s_lo + cs - 1) / cs;
   for (int k = used * NCH + (threadIdx.x & 31); k < p.draw_chunks * NCH; k += 32) store_cluster(rec + k * 8, 0.0);
   const DrawUnit<NCH>& u = sh.unit;
-  if (ENS) return draw_sweep_as<DT, ENS, NCH, AL, true, false>(p, u, cs, s_lo, s_hi, acc, rec, part);
-  if (p.n == 2 && p.mask_model < 0) return draw_sweep_as<DT, ENS, NCH, AL, true, false>(p, u, cs, s_lo, s_hi, acc, rec, part);
-  if (p.n == 2) return draw_sweep_as<DT, ENS, NCH, AL, true, true>(p, u, cs, s_lo, s_hi, acc, rec, part);
-  if (p.mask_model < 0) return draw_sweep_as<DT, ENS, NCH, AL, false, false>(p, u, cs, s_lo, s_hi, acc, rec, part);
-  draw_sweep_as<DT, ENS, NCH, AL, false, true>(p, u, cs, s_lo, s_hi, acc, rec, part);
+  if (ENS) return draw_sweep_as<DT, ENS, NCH, AL, true, false>(p, sh.kc, u, cs, s_lo, s_hi, acc, rec, part);
+  if (p.n == 2 && p.mask_model < 0) return draw_sweep_as<DT, ENS, NCH, AL, true, false>(p, sh.kc, u, cs, s_lo, s_hi, acc, rec, part);
+  if (p.n == 2) return draw_sweep_as<DT, ENS, NCH, AL, true, true>(p, sh.kc, u, cs, s_lo, s_hi, acc, rec, part);
+  if (p.mask_model < 0) return draw_sweep_as<DT, ENS, NCH, AL, false, false>(p, sh.kc, u, cs, s_lo, s_hi, acc, rec, part);
+  draw_sweep_as<DT, ENS, NCH, AL, false, true>(p, sh.kc, u, cs, s_lo, s_hi, acc, rec, part);
 }
 
 // The mass of one lane's tokens of step s under the refined normalisers (coefficients cf = k / Z): small ones in fp32, big
 // ones in fp64.
 template <int DT, bool ENS, int NCH, bool AL>
-__device__ __forceinline__ double step_mass(const KParams& p, const DrawUnit<NCH>& u, const float* cf, const double* inv, int s) {
+__device__ __forceinline__ double step_mass(const KParams& p, const DrawConst& kc, const DrawUnit<NCH>& u, const float* cf, const double* inv, int s) {
   constexpr int E = Elem<DT>::E;
   const int v = s * 32 + (threadIdx.x & 31);
   float x[NCH][E];
@@ -506,11 +515,11 @@ __device__ __forceinline__ double step_mass(const KParams& p, const DrawUnit<NCH
     bigbits |= big ? (1u << k) : 0u;
   }
   double own = static_cast<double>(ls);
-  for (; bigbits; bigbits &= bigbits - 1) own += big_mass<DT, ENS, NCH>(p, u, inv, v * E + __ffs(bigbits) - 1);
+  for (; bigbits; bigbits &= bigbits - 1) own += big_mass<DT, ENS, NCH>(kc, u, inv, v * E + __ffs(bigbits) - 1);
   return own;
 }
 template <int DT, bool ENS, int NCH>
-__device__ __forceinline__ double token_mass(const KParams& p, const DrawUnit<NCH>& u, const float* cf, const double* inv, int e) {
+__device__ __forceinline__ double token_mass(const DrawConst& p, const DrawUnit<NCH>& u, const float* cf, const double* inv, int e) {
   float x[NCH], tot = 0.f;
   bool big = false;
   entry_args<DT, ENS, NCH>(p, u, e, x);
@@ -642,7 +651,7 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
       double rm = 0.0;
 #pragma unroll 1
       for (int s = s0 + t * gsz; s < s0 + (t + 1) * gsz && s < s1; ++s) {
-        own = step_mass<DT, ENS, NCH, AL>(p, u, cf, inv, s);
+        own = step_mass<DT, ENS, NCH, AL>(p, sh.kc, u, cf, inv, s);
         rm += warp_sum(own);
         held = s;
       }
@@ -673,7 +682,7 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
     double before = 0.0;
 #pragma unroll 1
     for (int s = g0; s < g1; ++s) {
-      if (s != held) own = step_mass<DT, ENS, NCH, AL>(p, u, cf, inv, s);
+      if (s != held) own = step_mass<DT, ENS, NCH, AL>(p, sh.kc, u, cf, inv, s);
       double upto;
       const int l = first_reach(own, at, upto);
       if (l != -33) {
@@ -688,13 +697,13 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
     if (step < 0) return;
     const int e = (step * 32 + who) * E + lane;
     double m = 0.0;
-    if (lane < E && e < p.V) m = token_mass<DT, ENS, NCH>(p, u, cf, inv, e);
+    if (lane < E && e < p.V) m = token_mass<DT, ENS, NCH>(sh.kc, u, cf, inv, e);
     k = first_reach(m, before, at);
     const int token = (step * 32 + who) * E + (k & 31);
     if (lane == 0 && k != -33) {
       p.out_tokens[u.uidx] = token;
       // Algorithm 2's Score returns the bonus token with its probability under the law it came from
-      if (u.j == p.gamma && p.bonus_prob != nullptr) p.bonus_prob[u.b] = static_cast<float>(big_mass<DT, ENS, NCH>(p, u, inv, token));
+      if (u.j == p.gamma && p.bonus_prob != nullptr) p.bonus_prob[u.b] = static_cast<float>(big_mass<DT, ENS, NCH>(sh.kc, u, inv, token));
     }
     return;
   }
@@ -703,7 +712,7 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
 // The block's position from the records of the streaming launch (and the row's outputs, see decide_row): every block decides
 // its row for itself.  False when there is nothing to draw.
 template <int DT, bool ENS, int NCH>
-__device__ __noinline__ bool decide_unit_to_draw(const KParams& p, DrawShared<NCH>& sh, RowShared& rs, int slot, int part) {
+__device__ __forceinline__ bool decide_unit_to_draw(const KParams& p, DrawShared<NCH>& sh, RowShared& rs, int slot, int part) {
   const int tid = threadIdx.x;
   int b = slot, want = -1;
   if (p.draw_all) {
@@ -753,6 +762,19 @@ __global__ void __launch_bounds__(NCH == 8 ? 256 : kMaxDrawThreads, NCH == 2 ? 2
   double* slots = reinterpret_cast<double*>(draw_smem_raw + sizeof(DrawShared<NCH>));
   double* acc = slots + threadIdx.x;
   const int slot = blockIdx.x / p.draw_parts, rank = blockIdx.x % p.draw_parts, nw = blockDim.x >> 5;
+  if (threadIdx.x < COS_MAX_MODELS) {
+    DrawConst& kc = sh.kc;
+    kc.w[threadIdx.x] = p.w[threadIdx.x];
+    kc.w64[threadIdx.x] = p.w64[threadIdx.x];
+    if (threadIdx.x == 0) {
+      kc.row_step = p.s_model * Elem<DT>::bytes;
+      kc.cT64 = p.cT64;
+      kc.cT = p.cT;
+      kc.n = p.n;
+      kc.V = p.V;
+      kc.mask_model = p.mask_model;
+    }
+  }
   cluster_arrive();  // (the first block has begun: its shared memory may be written to)
   // launched while the kernel before it drains; nothing but inputs is read before that one is complete
   bool draws;

@@ -835,34 +835,38 @@ __device__ __forceinline__ float mask_bound(const KParams& p, unsigned key) {
 
 // What the probability of the draft token under slot i needs of the logits there (draft < 0: nothing), and that probability once
 // the statistics are merged, with the constant the sweep used.
+// Probability of the draft token under softmax i: what it needs of the logits (fetched early), and the rest (whose first use of them it is).
 struct DraftLogits {
-  double x;   // exponent before the reference is taken off
-  float xe;   // the gating model's logit
+  float a, b;  // the slot's logit; combined logits: those of models 0 and 1
 };
 template <int DT, int MODE>
 __device__ __forceinline__ DraftLogits draft_logits(const KParams& p, const char* base, int i, int pis, int draft) {
   DraftLogits d;
-  d.x = -INFINITY;
-  d.xe = INFINITY;
+  d.a = d.b = -INFINITY;
   if (draft < 0) return d;
   const long long row_step = p.s_model * Elem<DT>::bytes;
-  if (MODE == kEnsembleSample || i == 0) {
-    d.x = static_cast<double>(Elem<DT>::load1(base + (MODE == kEnsembleSample ? i : pis) * row_step, draft)) * p.cT64;
-  } else {
-    double cd = 0.0;
-    for (int k = 0; k < p.n; ++k) {
-      const float x = Elem<DT>::load1(base + k * row_step, draft);
-      cd = fma(p.w64[k], static_cast<double>(x), cd);
-      if (k == p.mask_model) d.xe = x;
-    }
-    d.x = cd * p.cT64;
-  }
+  const int first = MODE == kEnsembleSample ? i : (i == 0 ? pis : 0);
+  d.a = Elem<DT>::load1(base + first * row_step, draft);
+  if (MODE == kLogitSample && i == 1 && p.n >= 2) d.b = Elem<DT>::load1(base + row_step, draft);
   return d;
 }
 template <int DT, int MODE>
-__device__ __forceinline__ double draft_probability(const KParams& p, const DraftLogits& d, float thr, const SoftPart& f) {
-  if (MODE == kLogitSample && p.mask_model >= 0 && !(d.xe >= thr)) return 0.0;
-  return exp2(d.x - static_cast<double>(f.ref)) / f.s;
+__device__ __forceinline__ double draft_probability(const KParams& p, const DraftLogits& d, const char* base, int i, int draft, float thr,
+                                                    const SoftPart& f) {
+  if (draft < 0) return 0.0;
+  double x = static_cast<double>(d.a);
+  if (MODE == kLogitSample && i == 1) {
+    float gate = p.mask_model == 1 ? d.b : d.a;
+    x = p.w64[0] * x;
+    if (p.n >= 2) x = fma(p.w64[1], static_cast<double>(d.b), x);
+    for (int k = 2; k < p.n; ++k) {
+      const float l = Elem<DT>::load1(base + k * p.s_model * Elem<DT>::bytes, draft);
+      x = fma(p.w64[k], static_cast<double>(l), x);
+      if (k == p.mask_model) gate = l;
+    }
+    if (p.mask_model >= 0 && !(gate >= thr)) return 0.0;
+  }
+  return exp2(x * p.cT64 - static_cast<double>(f.ref)) / f.s;
 }
 
 // Largest logit of the gating model at every position, for the plausibility mask: the same split, over that model's rows
@@ -1071,7 +1075,8 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_report_kernel(const __g
       if (i < slots && lane % g == 0) {
         if (kSample) {
           fin.fsoft[i] = m.soft;
-          fin.pdraft[i] = draft_probability<DT, MODE>(p, draft_logits<DT, MODE>(p, base, i, pis, is_bonus || !draft_ok ? -1 : draft), thr, m.soft);
+          const int at = is_bonus || !draft_ok ? -1 : draft;
+          fin.pdraft[i] = draft_probability<DT, MODE>(p, draft_logits<DT, MODE>(p, base, i, pis, at), base, i, at, thr, m.soft);
         } else {
           fin.farg[i] = m.arg;
         }
