@@ -16,7 +16,6 @@ constexpr int kTile = 16;  // positions decided at a time
 
 struct RowShared {
   Finish fin[kTile];
-  unsigned word[kTile];
   int a;            // the row's first rejected position, or gamma; -1 until it is known
   int drawable;     // whether a token can be drawn there
   int cand;         // greedy: the token there
@@ -25,7 +24,7 @@ struct RowShared {
 };
 
 // Decide row b.  `want` >= 0: a position whose statistics the block needs, whatever the first rejection; otherwise the first
-// rejected position is what it needs.  `keep(fin, j, word)` is called by the first warp with that
+// rejected position is what it needs.  `keep(fin, j, word, accepted, drawable)` is called by the first warp with that
 // position's merged statistics and the random word its token is drawn with.  `writes_row(a)` / `writes_unit(j)`: whether this block writes the row's outputs and a
 // position's optional ones.
 template <int DT, int MODE, typename K, typename WR, typename WU>
@@ -80,7 +79,8 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
         Finish& f = sh.fin[pos];
         if (kSample) {
           f.fsoft[i] = m.soft;
-          f.pdraft[i] = draft_probability<DT, MODE>(p, d, base, i, at, m.thr, m.soft);
+          f.inv[i] = 1.0 / m.soft.s;
+          f.pdraft[i] = draft_probability<DT, MODE>(p, d, base, i, at, m.thr, m.soft, f.inv[i]);
         } else {
           f.farg[i] = m.arg;
         }
@@ -89,35 +89,40 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
     }
     __syncthreads();
     if (tid < 32) {
+      // (sampling: the decision stays in registers but where somebody asked to see it)
+      Decision own;
+      own.accept = own.status = own.drawable = 0;
+      Decision& dec = kSample || lane >= count ? own : sh.fin[lane].dec;
       if (lane < count) {
         const bool is_bonus = (j0 + lane == p.gamma);
         const bool draft_ok = is_bonus || (draft >= 0 && draft < p.V);
         const bool pi_ok = (pi >= 0 && pi < p.n);
-        sh.word[lane] = rnd[1];
-        decide_unit<DT, MODE>(p, sh.fin[lane], word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), is_bonus, draft, draft_ok, pi, pi_ok,
+        decide_unit<DT, MODE>(p, sh.fin[lane], dec, word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), is_bonus, draft, draft_ok, pi, pi_ok,
                               pi_ok ? pi : 0);
+        if (kSample && optional) sh.fin[lane].dec = dec;
       }
+      int a = sh.a;
       __syncwarp();
-      if (sh.a < 0) {
-        const bool stop = lane < count && (!sh.fin[lane].dec.accept || j0 + lane == p.gamma);
-        const unsigned stops = __ballot_sync(0xffffffffu, stop);
+      if (a < 0) {
+        const unsigned stops = __ballot_sync(0xffffffffu, lane < count && (!dec.accept || j0 + lane == p.gamma));
         const int k = stops ? __ffs(stops) - 1 : count - 1;
-        const unsigned st = __reduce_or_sync(0xffffffffu, lane <= k ? static_cast<unsigned>(sh.fin[lane].dec.status) : 0u);
-        __syncwarp();
-        if (lane == 0) {
+        const unsigned st = __reduce_or_sync(0xffffffffu, lane <= k && lane < count ? static_cast<unsigned>(dec.status) : 0u);
+        if (stops) a = j0 + k;
+        if (lane == k) {
           sh.status |= st;
-          if (stops) {
-            const Decision& d = sh.fin[k].dec;
-            sh.a = j0 + k;
-            sh.drawable = d.drawable;
-            sh.cand = d.cand;
-            sh.prob = static_cast<float>(d.prob);
+          sh.a = a;
+          sh.drawable = dec.drawable;
+          if (!kSample) {
+            sh.cand = dec.cand;
+            sh.prob = static_cast<float>(dec.prob);
           }
         }
-        __syncwarp();
       }
-      const int asked = want >= 0 ? want : sh.a;
-      if (asked >= j0 && asked < j0 + count) keep(sh.fin[asked - j0], asked, sh.word[asked - j0]);
+      const int asked = want >= 0 ? want : a;
+      const int k = asked >= j0 && asked < j0 + count ? asked - j0 : 0;
+      const int accepted = __shfl_sync(0xffffffffu, dec.accept, k), drawable = __shfl_sync(0xffffffffu, dec.drawable, k);
+      const unsigned word = __shfl_sync(0xffffffffu, rnd[1], k);
+      if (asked >= j0 && asked < j0 + count) keep(sh.fin[k], asked, word, accepted, drawable);
     }
     __syncthreads();
     const int a = sh.a;
@@ -184,7 +189,7 @@ template <int DT, int MODE>
 __global__ void __launch_bounds__(128) cos_decide_kernel(const __grid_constant__ KParams p) {
   __shared__ RowShared sh;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  decide_row<DT, MODE>(p, sh, blockIdx.x, -1, [](const Finish&, int, unsigned) {}, [](int) { return true; }, [](int) { return true; });
+  decide_row<DT, MODE>(p, sh, blockIdx.x, -1, [](const Finish&, int, unsigned, int, int) {}, [](int) { return true; }, [](int) { return true; });
 }
 
 }  // namespace cosv

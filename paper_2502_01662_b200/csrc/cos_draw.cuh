@@ -545,7 +545,7 @@ __device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh
   const int lane = threadIdx.x & 31, i = lane / G, live = ENS ? p.n : 2;
   const DrawUnit<NCH>& u = sh.unit;
   double z = 0.0;
-#pragma unroll 1
+#pragma unroll 4
   for (int w = lane % G; w < W; w += G) z += sh.part[w][i];
 #pragma unroll
   for (int d = G / 2; d > 0; d >>= 1) z += __shfl_xor_sync(0xffffffffu, z, d);
@@ -568,7 +568,7 @@ __device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh
   const int chunks = W * p.draw_chunks, per = (chunks + 31) / 32;
   const int c_lo = lane * per, c_hi = c_lo + per < chunks ? c_lo + per : chunks;
   double mine = 0.0;
-#pragma unroll 1
+#pragma unroll 4
   for (int c = c_lo; c < c_hi; ++c) {
     const double m = mass_of(c);
     sh.recs[c * NCH] = m;
@@ -659,11 +659,11 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
     }
     __syncthreads();
     if (held < 0) return;  // (no step of the chunk is this warp's)
-    // running total over the lanes; the first that reaches the target, or the last with mass where rounding leaves none
-    auto first_reach = [&](double m, double from, double& upto) -> int {
+    // running total over the first `lanes` lanes; the first that reaches the target, or the last with mass where rounding leaves none
+    auto first_reach = [&](double m, int lanes, double from, double& upto) -> int {
       double in = m;
 #pragma unroll 1
-      for (int d = 1; d < 32; d <<= 1) {
+      for (int d = 1; d < lanes; d <<= 1) {
         const double o = __shfl_up_sync(0xffffffffu, in, d);
         if (lane >= d) in += o;
       }
@@ -673,7 +673,7 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
       return ok ? k : k - 32;  // (negative: not reached; -33: no mass at all)
     };
     double at;
-    int k = first_reach((s0 + lane * gsz < s1) ? sh.step_mass[lane] : 0.0, sh.base, at);
+    int k = first_reach((s0 + lane * gsz < s1) ? sh.step_mass[lane] : 0.0, (s1 - s0 + gsz - 1) / gsz, sh.base, at);
     if (k == -33) return;
     if ((k & 31) % nw != warp) return;
     // one warp goes on: the record's steps in order, the lanes of a step, the tokens of a lane's vector
@@ -684,7 +684,7 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
     for (int s = g0; s < g1; ++s) {
       if (s != held) own = step_mass<DT, ENS, NCH, AL>(p, sh.kc, u, cf, inv, s);
       double upto;
-      const int l = first_reach(own, at, upto);
+      const int l = first_reach(own, 32, at, upto);
       if (l != -33) {
         step = s;
         who = l & 31;
@@ -698,7 +698,7 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
     const int e = (step * 32 + who) * E + lane;
     double m = 0.0;
     if (lane < E && e < p.V) m = token_mass<DT, ENS, NCH>(sh.kc, u, cf, inv, e);
-    k = first_reach(m, before, at);
+    k = first_reach(m, E, before, at);
     const int token = (step * 32 + who) * E + (k & 31);
     if (lane == 0 && k != -33) {
       p.out_tokens[u.uidx] = token;
@@ -723,16 +723,15 @@ __device__ __forceinline__ bool decide_unit_to_draw(const KParams& p, DrawShared
   DrawUnit<NCH>& u = sh.unit;
   decide_row<DT, ENS ? kEnsembleSample : kLogitSample>(
       p, rs, b, want,
-      [&](const Finish& f, int j, unsigned word) {
+      [&](const Finish& f, int j, unsigned word, int accepted, int drawable) {
         const int pi = proposer_of(p, b, j);
         const int pis = (pi >= 0 && pi < p.n) ? pi : 0;
         const int law = (j == p.gamma) ? (p.bonus_model >= 0 ? kDrawQ : kDrawR) : kDrawResidual;
         if (tid < NCH) {
           const bool live = tid < (ENS ? p.n : 2);
-          const double z = live ? f.fsoft[tid].s : 1.0;
           u.nref[tid] = live ? -f.fsoft[tid].ref : 0.f;
-          u.bt[tid] = live ? static_cast<float>(z * kBigShare) : INFINITY;
-          u.ct[tid] = static_cast<float>(coefficient<ENS>(p, tid, pis, law) / z);
+          u.bt[tid] = live ? static_cast<float>(f.fsoft[tid].s * kBigShare) : INFINITY;
+          u.ct[tid] = live ? static_cast<float>(coefficient<ENS>(p, tid, pis, law) * f.inv[tid]) : 0.f;
         }
         if (tid == 0) {
           u.b = b;
@@ -741,8 +740,8 @@ __device__ __forceinline__ bool decide_unit_to_draw(const KParams& p, DrawShared
           u.pis = pis;
           u.law = law;
           u.word = word;
-          u.accepted = f.dec.accept;
-          u.drawable = f.dec.drawable;
+          u.accepted = accepted;
+          u.drawable = drawable;
           u.thr = (!ENS && p.mask_model >= 0) ? f.thr : -INFINITY;
           u.base = reinterpret_cast<const char*>(p.logits) +
                    (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;

@@ -35,6 +35,7 @@ struct Finish {  // what a position is decided from, and the decision
     ArgPart farg[COS_MAX_MODELS];    // merged argmaxes (greedy)
   };
   double pdraft[COS_MAX_MODELS];     // sampling: probability of the draft token under each softmax
+  double inv[COS_MAX_MODELS];        // sampling: one over each normaliser
   float thr;                         // plausibility threshold (NaN: the gating model's logits hold one)
   Decision dec;
 };
@@ -559,16 +560,15 @@ __device__ __forceinline__ void publish_unit(const KParams& p, int b, int j, int
 }
 
 // The accept test of one (row, position) from the merged statistics (Eq. 6), taken by one thread in fp64; greedy modes also
-// settle the replacement token here.  Reads fsoft / farg / pdraft / thr, writes dec.  (Logit-level greedy: farg[0] is the
+// settle the replacement token here.  Reads fsoft / farg / pdraft / thr, writes d.  (Logit-level greedy: farg[0] is the
 // proposer's argmax, farg[1] the combined one.)
 template <int DT, int MODE>
-__device__ __forceinline__ void decide_unit(const KParams& p, Finish& sh, double u_acc, double u_smp, bool is_bonus, int draft, bool draft_ok,
+__device__ __forceinline__ void decide_unit(const KParams& p, const Finish& sh, Decision& d, double u_acc, double u_smp, bool is_bonus, int draft, bool draft_ok,
                                             int pi, bool pi_ok, int pis) {
   const bool mask_bad = (MODE == kLogitSample || MODE == kLogitGreedy) && p.mask_model >= 0 && sh.thr != sh.thr;
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
   const double kNaN = __longlong_as_double(0x7ff8000000000000LL);
   const double kInf = __longlong_as_double(0x7ff0000000000000LL);
-  Decision& d = sh.dec;
   d.accept = 0;
   d.status = 0;
   d.cand = -1;
@@ -852,7 +852,7 @@ __device__ __forceinline__ DraftLogits draft_logits(const KParams& p, const char
 }
 template <int DT, int MODE>
 __device__ __forceinline__ double draft_probability(const KParams& p, const DraftLogits& d, const char* base, int i, int draft, float thr,
-                                                    const SoftPart& f) {
+                                                    const SoftPart& f, double inv) {
   if (draft < 0) return 0.0;
   double x = static_cast<double>(d.a);
   if (MODE == kLogitSample && i == 1) {
@@ -866,7 +866,7 @@ __device__ __forceinline__ double draft_probability(const KParams& p, const Draf
     }
     if (p.mask_model >= 0 && !(gate >= thr)) return 0.0;
   }
-  return exp2(x * p.cT64 - static_cast<double>(f.ref)) / f.s;
+  return exp2(x * p.cT64 - static_cast<double>(f.ref)) * inv;
 }
 
 // Largest logit of the gating model at every position, for the plausibility mask: the same split, over that model's rows
@@ -1076,7 +1076,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_report_kernel(const __g
         if (kSample) {
           fin.fsoft[i] = m.soft;
           const int at = is_bonus || !draft_ok ? -1 : draft;
-          fin.pdraft[i] = draft_probability<DT, MODE>(p, draft_logits<DT, MODE>(p, base, i, pis, at), base, i, at, thr, m.soft);
+          fin.pdraft[i] = draft_probability<DT, MODE>(p, draft_logits<DT, MODE>(p, base, i, pis, at), base, i, at, thr, m.soft, 1.0 / m.soft.s);
         } else {
           fin.farg[i] = m.arg;
         }
@@ -1091,7 +1091,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_report_kernel(const __g
       if (lane == 0) {
         unsigned rnd[4];
         philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
-        decide_unit<DT, MODE>(p, fin, word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), is_bonus, draft, draft_ok, pi, pi_ok, pis);
+        decide_unit<DT, MODE>(p, fin, fin.dec, word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), is_bonus, draft, draft_ok, pi, pi_ok, pis);
         const Decision& d = fin.dec;
         publish_unit(p, b, j, d.accept, d.status, d.cand, kSample ? d.drawable : __float_as_int(static_cast<float>(d.prob)), d.ratio,
                      d.r_d, d.q_d, d.S);

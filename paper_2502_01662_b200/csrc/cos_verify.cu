@@ -173,23 +173,36 @@ constexpr int kStreamBlock = 512;   // threads of a block of a full streaming la
 constexpr int kMinShare = 128;      // vectors a warp should have at least: four loads for each lane
 
 // Cut the line of `units` positions into shares for at most `workers` warps (see cos_stream.cuh).  Small runs take fewer warps, so
-// that each has a few loads in flight, in small blocks, so that they spread over the device.  Returns the block size.
+// that each has a few loads in flight, in small blocks, so that they spread over the device.  Where nine tenths of the warps are
+// busy that way, every position is a whole number of shares (its end padded): a warp then has one part, not the end of one and
+// the beginning of the next, one after the other (16 rows of 50001 tokens and three models: the last warp ended after 17 us, the
+// average one after 10).  Returns the block size.
 int plan_line(KParams& p, const cos_verify_config& c, long long units, long long workers, int sm_count) {
   const int E = entries_per_vec(c.dtype), nvec = c.vocab / E;
-  p.st_nv = p.vec_ok ? nvec : nvec - 2;  // (unaligned rows: the first vector and the last one go entry by entry)
-  if (p.st_nv < 1) p.st_nv = 1;          // nothing but ragged entries
-  p.st_line = units * p.st_nv;
-  long long most = p.st_line / kMinShare;
+  int nv = p.vec_ok ? nvec : nvec - 2;  // (unaligned rows: the first vector and the last one go entry by entry)
+  if (nv < 1) nv = 1;                   // nothing but ragged entries
+  long long most = units * nv / kMinShare;
   if (most < 8LL * sm_count) most /= 2;  // (where that leaves most of the device idle anyway: fewer records to merge)
-  if (workers > most) workers = most;
+  const bool small = workers > most;
+  if (small) workers = most;
   if (workers < 1) workers = 1;
-  p.st_share = static_cast<int>(((p.st_line + workers - 1) / workers + 7) / 8 * 8);
+  long long each = workers / units;  // shares of a position
+  if (small && each < 1 && units <= static_cast<long long>(sm_count) * 32) each = 1;
+  if (each >= 1 && (small || units * each * 10 >= workers * 9)) {
+    p.st_share = static_cast<int>(((nv + each - 1) / each + 7) / 8 * 8);
+    p.st_nv = (nv + p.st_share - 1) / p.st_share * p.st_share;
+    p.st_line = units * p.st_nv;
+  } else {
+    p.st_nv = nv;
+    p.st_line = units * nv;
+    p.st_share = static_cast<int>(((p.st_line + workers - 1) / workers + 7) / 8 * 8);
+  }
   p.st_workers = static_cast<int>((p.st_line + p.st_share - 1) / p.st_share);
   p.st_inv_nv = 1.0 / p.st_nv;
   p.st_inv_share = 1.0 / p.st_share;
   const int slots = c.combine == COS_COMBINE_PROB_ENSEMBLE ? c.n : 2;
   p.slot_inv = (65536 + slots - 1) / slots;
-  return workers <= 16LL * sm_count ? 128 : kStreamBlock;
+  return p.st_workers <= 16LL * sm_count ? 128 : kStreamBlock;
 }
 
 // Warps of the streaming launch: what the device holds at once, or the cluster size's worth of blocks for every position.
