@@ -130,18 +130,6 @@ def _current_stream(torch, index: int) -> int:
     return raw(index)
 
 
-def _make_args(logits, stride_model, stride_row, stride_pos, drafts, proposer, batch, flags, row_base, seed, offset, outs,
-               bonus_model, offset_device=None) -> cos_verify_args:
-    named = bonus_model is not None and bonus_model >= 0
-    ptr = {k: t.data_ptr() for k, t in outs.items()}
-    return cos_verify_args(
-        logits.data_ptr(), stride_model, stride_row, stride_pos,
-        drafts.data_ptr() if (drafts is not None and drafts.numel() > 0) else None, proposer.data_ptr(),
-        batch, flags, row_base, seed & 0xFFFFFFFFFFFFFFFF, offset & 0xFFFFFFFFFFFFFFFF,
-        ptr["accept_count"], ptr["out_tokens"], ptr["row_status"], ptr.get("diag"), ptr.get("r"), ptr.get("bonus_prob"),
-        bonus_model if named else 0, offset_device.data_ptr() if offset_device is not None else None, ptr.get("lse"))
-
-
 class CosVerifier:
     """One verification context (cos_verify_create ... cos_verify_destroy).
 
@@ -163,6 +151,7 @@ class CosVerifier:
         cfg.dtype = dtype if isinstance(dtype, int) else _dtype_code(dtype)
         cfg.device, cfg.cluster_size, cfg.host_staging = device, cluster_size, int(host_staging)
         self.cfg = cfg
+        self._dims, self._dtype = (n, gamma + 1, vocab), cfg.dtype
         st = self._lib.cos_verify_create(ctypes.byref(cfg), ctypes.byref(self._ctx))
         if st != COS_OK:
             msg = self._lib.cos_verify_last_error(None).decode()
@@ -185,7 +174,7 @@ class CosVerifier:
         return out
 
     def _fill_args(self, logits, drafts, proposer, seed, offset, row_base, flags, outs,
-                   bonus_model=None, offset_device=None) -> cos_verify_args:
+                   bonus_model=None, offset_device=None, ptr=None) -> cos_verify_args:
         n, B, P, V = logits.shape
         # a [B, gamma+1] proposer table selects the per-position form; a bonus model selects its flag
         if proposer.dim() == 2:
@@ -194,16 +183,24 @@ class CosVerifier:
             flags |= COS_RUN_PROPOSER_PER_POSITION
         elif proposer.numel() != B:
             raise ValueError("proposer must be [B] or [B, gamma+1]")
-        if bonus_model is not None and bonus_model >= 0:
+        named = bonus_model is not None and bonus_model >= 0
+        if named:
             flags |= COS_RUN_BONUS_FROM_MODEL
-        if n != self.cfg.n or P != self.cfg.gamma + 1 or V != self.cfg.vocab:
+        if (n, P, V) != self._dims:
             raise ValueError(f"logits shape {tuple(logits.shape)} does not match the context")
-        if logits.stride(3) != 1:
+        sm, sr, sp, sv = logits.stride()
+        if sv != 1:
             raise ValueError("the vocabulary axis of logits must be contiguous")
-        if _dtype_code(logits.dtype) != self.cfg.dtype:
+        if _dtype_code(logits.dtype) != self._dtype:
             raise ValueError("logits dtype does not match the context")
-        sm, sr, sp, _ = logits.stride()
-        return _make_args(logits, sm, sr, sp, drafts, proposer, B, flags, row_base, seed, offset, outs, bonus_model, offset_device)
+        if ptr is None:
+            ptr = {k: t.data_ptr() for k, t in outs.items()}
+        get = ptr.get
+        return cos_verify_args(
+            logits.data_ptr(), sm, sr, sp, drafts.data_ptr() if (drafts is not None and drafts.numel() > 0) else None,
+            proposer.data_ptr(), B, flags, row_base, seed & 0xFFFFFFFFFFFFFFFF, offset & 0xFFFFFFFFFFFFFFFF,
+            ptr["accept_count"], ptr["out_tokens"], ptr["row_status"], get("diag"), get("r"), get("bonus_prob"),
+            bonus_model if named else 0, offset_device.data_ptr() if offset_device is not None else None, get("lse"))
 
     def set_one_launch(self, enable=True):
         """cos_verify_set_one_launch: 1 / True: later runs take the one-launch kernel; 2: staged streaming launch, tokens
@@ -226,14 +223,19 @@ class CosVerifier:
         return [float(ms[k]) for k in range(count.value)]
 
     @staticmethod
+    def _small_outs(buf, B, P):
+        # one allocation for the small outputs: four of their own cost 8.4 us a call, this 5
+        import torch
+        accept, status, bonus, tokens = buf.split_with_sizes((B, B, B, B * P))
+        return {"accept_count": accept, "out_tokens": tokens.view(B, P), "row_status": status, "bonus_prob": bonus.view(torch.float32)}
+
+    @staticmethod
     def _alloc_outs(B, P, V, device, diag, dump_r, pin=False):
         import torch
         kw = dict(device=device)
         if pin:
             kw["pin_memory"] = True
-        # one allocation for the small outputs (four of their own cost 8.4 us a call, this 5)
-        accept, status, bonus, tokens = torch.empty(B * (P + 3), dtype=torch.int32, **kw).split_with_sizes((B, B, B, B * P))
-        outs = {"accept_count": accept, "out_tokens": tokens.view(B, P), "row_status": status, "bonus_prob": bonus.view(torch.float32)}
+        outs = CosVerifier._small_outs(torch.empty(B * (P + 3), dtype=torch.int32, **kw), B, P)
         if diag:
             outs["diag"] = torch.empty((B, P, 4), dtype=torch.float32, **kw)
         if dump_r:
@@ -254,20 +256,33 @@ class CosVerifier:
         import torch
         if not logits.is_cuda:
             raise ValueError("run() needs device tensors; use run_host() for host tensors")
-        for t, name in ((drafts, "drafts"), (proposer, "proposer")):
-            if t is not None and t.numel() > 0 and (t.dtype != torch.int32 or not t.is_contiguous() or not t.is_cuda):
-                raise ValueError(f"{name} must be a contiguous int32 device tensor")
-        n, B, P, V = logits.shape
+        i32 = torch.int32
+        if (drafts is not None and drafts.numel() > 0 and
+                (drafts.dtype is not i32 or not drafts.is_contiguous() or not drafts.is_cuda)):
+            raise ValueError("drafts must be a contiguous int32 device tensor")
+        if (proposer is not None and proposer.numel() > 0 and
+                (proposer.dtype is not i32 or not proposer.is_contiguous() or not proposer.is_cuda)):
+            raise ValueError("proposer must be a contiguous int32 device tensor")
+        ptr = None
         if outs is None:
-            outs = self._alloc_outs(B, P, V, logits.device, diag, dump_r)
-            if lse:     # log-sum-exp behind every softmax of a position: [B, gamma+1, n] (ensemble) or [B, gamma+1, 2]
-                slots = self.cfg.n if self.cfg.combine == COS_COMBINE_PROB_ENSEMBLE else 2
-                outs["lse"] = torch.empty((B, P, slots), dtype=torch.float32, device=logits.device)
+            n, B, P, V = logits.shape
+            if diag or dump_r or lse:
+                outs = self._alloc_outs(B, P, V, logits.device, diag, dump_r)
+                if lse:     # log-sum-exp behind every softmax of a position: [B, gamma+1, n] (ensemble) or [B, gamma+1, 2]
+                    slots = self.cfg.n if self.cfg.combine == COS_COMBINE_PROB_ENSEMBLE else 2
+                    outs["lse"] = torch.empty((B, P, slots), dtype=torch.float32, device=logits.device)
+            else:
+                buf = logits.new_empty(B * (P + 3), dtype=i32)
+                outs = self._small_outs(buf, B, P)
+                at, b4 = buf.data_ptr(), 4 * B
+                ptr = {"accept_count": at, "row_status": at + b4, "bonus_prob": at + 2 * b4, "out_tokens": at + 3 * b4}
         if offset_device is not None and (offset_device.dtype != torch.int64 or not offset_device.is_cuda):
             raise ValueError("offset_device must be an int64 device tensor")
-        a = self._fill_args(logits, drafts, proposer, seed, offset, row_base, flags, outs, bonus_model, offset_device)
+        a = self._fill_args(logits, drafts, proposer, seed, offset, row_base, flags, outs, bonus_model, offset_device, ptr)
         s = _current_stream(torch, logits.get_device()) if stream is None else stream.cuda_stream
-        self._check(self._lib.cos_verify_run(self._ctx, ctypes.byref(a), s))
+        st = self._lib.cos_verify_run(self._ctx, ctypes.byref(a), s)
+        if st != COS_OK:
+            self._check(st)
         return outs
 
     def run_host(self, logits, drafts, proposer, seed: int, offset: int, row_base: int = 0, flags: int = 0,
@@ -354,8 +369,13 @@ def run_static(n: int, combine: int, weights: Sequence[float], temperature: floa
     if bonus_model is not None and bonus_model >= 0:
         flags |= COS_RUN_BONUS_FROM_MODEL
     sm, sr, sp, _ = logits.stride()
-    a = _make_args(logits, sm, sr, sp, drafts, proposer, logits.shape[1], flags, row_base, seed, offset, outs, bonus_model)
-    a.dump_r = a.lse = None
+    named = bonus_model is not None and bonus_model >= 0
+    a = cos_verify_args(
+        logits.data_ptr(), sm, sr, sp, drafts.data_ptr() if (drafts is not None and drafts.numel() > 0) else None,
+        proposer.data_ptr(), logits.shape[1], flags, row_base, seed & 0xFFFFFFFFFFFFFFFF, offset & 0xFFFFFFFFFFFFFFFF,
+        outs["accept_count"].data_ptr(), outs["out_tokens"].data_ptr(), outs["row_status"].data_ptr(),
+        outs["diag"].data_ptr() if "diag" in outs else None, None,
+        outs["bonus_prob"].data_ptr() if "bonus_prob" in outs else None, bonus_model if named else 0, None, None)
     s = _current_stream(torch, logits.get_device()) if stream is None else stream.cuda_stream
     st = lib.cos_verify_run_static(ctypes.byref(cfg), ctypes.byref(a), s)
     if st != COS_OK:
