@@ -77,6 +77,8 @@ struct KParams {
   // the streaming launch: a line of st_line vectors (st_nv for each position) in st_workers shares of st_share vectors (the last may
   // be shorter); st_slabs lines one after another (one, or one for each position of a row)
   int st_workers, st_slabs, st_nv, st_share;
+  int st_split;            // ensembles: shares of a position, each model's a warp of its own; 0: a warp sweeps all models of its share
+  int st_warps;            // warps of the launch
   long long st_line;
   double st_inv_nv, st_inv_share;  // one over them, for divisions
   int slot_inv;            // 65536 over the records of a (share, position) pair, rounded up: likewise

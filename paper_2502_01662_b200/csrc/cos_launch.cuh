@@ -54,7 +54,7 @@ inline cudaError_t launch(KernelFn fn, const KParams& p, int blocks, int threads
 
 template <int DT>
 cudaError_t stream_launch(const KParams& p, int mode, bool report, int threads, cudaStream_t stream) {
-  const int blocks = (p.st_workers + threads / 32 - 1) / (threads / 32);
+  const int blocks = (p.st_warps + threads / 32 - 1) / (threads / 32);
   const bool pair = p.n == 2, masked = p.mask_model >= 0;
   return launch(p.vec_ok ? stream_kernel_of<DT, true>(mode, report, pair, masked) : stream_kernel_of<DT, false>(mode, report, pair, masked), p,
                 blocks, threads, 0, stream);
@@ -69,7 +69,7 @@ cudaError_t decide_launch(const KParams& p, int mode, cudaStream_t stream) {
 
 template <int DT>
 cudaError_t mask_launch(const KParams& p, int threads, cudaStream_t stream) {
-  const int blocks = (p.st_workers + threads / 32 - 1) / (threads / 32);
+  const int blocks = (p.st_warps + threads / 32 - 1) / (threads / 32);
   return launch(p.vec_ok ? cos_mask_kernel<DT, true> : cos_mask_kernel<DT, false>, p, blocks, threads, 0, stream);
 }
 

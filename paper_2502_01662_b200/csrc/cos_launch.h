@@ -8,7 +8,7 @@
 
 namespace cosv {
 
-// The streaming launch (mode: the Mode enum): a warp for each of the p.st_workers shares, blocks of `threads` threads; `report`:
+// The streaming launch (mode: the Mode enum): p.st_warps warps, blocks of `threads` threads; `report`:
 // the form that also decides and publishes.  mask: the launch before it that finds the plausibility threshold of every
 // position.  decide: a launch after it that decides the rows (greedy runs, and
 // ensembles of one or of more than four models).

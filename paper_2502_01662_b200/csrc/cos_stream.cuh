@@ -925,10 +925,10 @@ __device__ __forceinline__ int4 pack_arg(const ArgPart& a, float thr) {
   return make_int4(__double2loint(a.val), __double2hiint(a.val), a.idx, a.bad | (thr != thr ? 2 : 0));
 }
 
-// The part of one position, vectors [o0, o1) of every model, that lies in a warp's share: its records (lane 0 writes them).
+// The part of one position, vectors [o0, o1) of every model (ensembles: of models [i0, i1)), that lies in a warp's share: its records (lane 0 writes them).
 // `settled`: the inputs may be read before the kernel ahead in the stream is complete; this waits for it before it writes.
 template <int DT, int MODE, bool AL, bool PAIR, bool MASKED>
-__device__ __forceinline__ void sweep_part(const KParams& p, const char* base, int o0, int o1, int pis, float thr, int4* rec,
+__device__ __forceinline__ void sweep_part(const KParams& p, const char* base, int o0, int o1, int i0, int i1, int pis, float thr, int4* rec,
                                            bool& waited) {
   const int lane = threadIdx.x & 31;
   const VecRange whole = whole_vectors<DT, AL>(p.V);
@@ -943,9 +943,9 @@ __device__ __forceinline__ void sweep_part(const KParams& p, const char* base, i
     if (lane == 0) __stcg(rec + i, v);
   };
   if (MODE == kEnsembleSample) {
-    for (int i = 0; i < p.n; ++i) put(i, pack_soft(soft_segment<DT, AL>(base + i * row_step, v0, v1, ragged, p.V, p.cT), thr));
+    for (int i = i0; i < i1; ++i) put(i, pack_soft(soft_segment<DT, AL>(base + i * row_step, v0, v1, ragged, p.V, p.cT), thr));
   } else if (MODE == kEnsembleGreedy) {
-    for (int i = 0; i < p.n; ++i) put(i, pack_arg(arg_segment<DT, AL>(base + i * row_step, v0, v1, ragged, p.V), thr));
+    for (int i = i0; i < i1; ++i) put(i, pack_arg(arg_segment<DT, AL>(base + i * row_step, v0, v1, ragged, p.V), thr));
   } else if (MODE == kLogitSample) {
     const LaneSoft2 a = logit_segment<DT, AL, PAIR, MASKED>(p, base, row_step, logit_weights(p, pis, thr), p.cT, v0, v1, ragged);
     put(0, pack_soft(a.q, thr));
@@ -969,9 +969,16 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_stream_kernel(const __g
   bool waited = p.inputs_settled == 0;
   if (waited) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (w >= p.st_workers) return;
+  if (w >= p.st_warps) return;
   const int slots = record_slots<MODE>(p);
-  for (long long x = worker_lo(p, w), end = worker_lo(p, w + 1); x < end;) {
+  int share = w, i0 = 0, i1 = p.n;
+  if (kEns && p.st_split) {
+    const int row = w / p.st_split, unit = row / p.n;
+    share = unit * p.st_split + w - row * p.st_split;
+    i0 = row - unit * p.n;
+    i1 = i0 + 1;
+  }
+  for (long long x = worker_lo(p, share), end = worker_lo(p, share + 1); x < end;) {
     const int r = line_div(x, p.st_nv, p.st_inv_nv);
     const int o0 = static_cast<int>(x - static_cast<long long>(r) * p.st_nv);
     const int o1 = end - x < p.st_nv - o0 ? o0 + static_cast<int>(end - x) : p.st_nv;
@@ -986,8 +993,8 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_stream_kernel(const __g
       pis = (pi >= 0 && pi < p.n) ? pi : 0;
       if (MASKED) thr = mask_bound(p, __ldcg(&p.mask_key[r]));
     }
-    sweep_part<DT, MODE, AL, PAIR, MASKED>(p, base, o0, o1, pis, thr, p.st_rec + first_record(p, 0, p.num_units, r, slots) + static_cast<size_t>(w) * slots,
-                                           waited);
+    sweep_part<DT, MODE, AL, PAIR, MASKED>(p, base, o0, o1, i0, i1, pis, thr,
+                                           p.st_rec + first_record(p, 0, p.num_units, r, slots) + static_cast<size_t>(share) * slots, waited);
   }
 }
 
@@ -1036,11 +1043,11 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_report_kernel(const __g
       if (!skip) {
         int4* rec = p.st_rec + first_record(p, slab, units, r, slots) + static_cast<size_t>(w) * slots;
         if (kEns || (p.n == 2 && !masked))
-          sweep_part<DT, MODE, AL, true, false>(p, base, o0, o1, pis, thr, rec, waited);
+          sweep_part<DT, MODE, AL, true, false>(p, base, o0, o1, 0, p.n, pis, thr, rec, waited);
         else if (masked)
-          sweep_part<DT, MODE, AL, false, true>(p, base, o0, o1, pis, thr, rec, waited);
+          sweep_part<DT, MODE, AL, false, true>(p, base, o0, o1, 0, p.n, pis, thr, rec, waited);
         else
-          sweep_part<DT, MODE, AL, false, false>(p, base, o0, o1, pis, thr, rec, waited);
+          sweep_part<DT, MODE, AL, false, false>(p, base, o0, o1, 0, p.n, pis, thr, rec, waited);
       }
       int prev = 0;
       if (lane == 0) {

@@ -170,39 +170,48 @@ DrawPlan draw_plan(const cos_verify_config& c, long long units, int sm_count) {
 }
 
 constexpr int kStreamBlock = 512;   // threads of a block of a full streaming launch, two blocks per multiprocessor
-constexpr int kMinShare = 128;      // vectors a warp should have at least: four loads for each lane
 
 // Cut the line of `units` positions into shares for at most `workers` warps (see cos_stream.cuh).  Small runs take fewer warps, so
 // that each has a few loads in flight, in small blocks, so that they spread over the device.  Where nine tenths of the warps are
 // busy that way, every position is a whole number of shares (its end padded): a warp then has one part, not the end of one and
 // the beginning of the next, one after the other (16 rows of 50001 tokens and three models: the last warp ended after 17 us, the
-// average one after 10).  Returns the block size.
-int plan_line(KParams& p, const cos_verify_config& c, long long units, long long workers, int sm_count) {
+// average one after 10); and of an ensemble (`models` > 1) it has one model's, for the same reason.  Returns the block size.
+int plan_line(KParams& p, const cos_verify_config& c, long long units, int models, long long workers, int sm_count) {
   const int E = entries_per_vec(c.dtype), nvec = c.vocab / E;
   int nv = p.vec_ok ? nvec : nvec - 2;  // (unaligned rows: the first vector and the last one go entry by entry)
   if (nv < 1) nv = 1;                   // nothing but ragged entries
-  long long most = units * nv / kMinShare;
-  if (most < 8LL * sm_count) most /= 2;  // (where that leaves most of the device idle anyway: fewer records to merge)
+  // at least four loads for each lane; eight (all still on their way at once) where that leaves most of the device idle anyway,
+  // or for one model at a time: fewer records to merge
+  // (with 768 vectors or more the loads of one model after another leave no gap to speak of, and the split is coarser: 32 rows of
+  // 128256 tokens and four models 65 us in one, 68 apart)
+  if (units * models * nv >= 768 * workers) models = 1;
+  const long long rows = units * models;
+  long long most = rows * nv / 128;
+  if (most < 8LL * sm_count || models > 1) most /= 2;
   const bool small = workers > most;
-  if (small) workers = most;
-  if (workers < 1) workers = 1;
-  long long each = workers / units;  // shares of a position
-  if (small && each < 1 && units <= static_cast<long long>(sm_count) * 32) each = 1;
-  if (each >= 1 && (small || units * each * 10 >= workers * 9)) {
+  const long long busy = small ? (most < 1 ? 1 : most) : workers;
+  long long each = busy / rows;  // shares of a row
+  if (small && each < 1 && rows <= workers) each = 1;
+  if (each >= 1 && (small || rows * each * 10 >= busy * 9)) {
     p.st_share = static_cast<int>(((nv + each - 1) / each + 7) / 8 * 8);
     p.st_nv = (nv + p.st_share - 1) / p.st_share * p.st_share;
     p.st_line = units * p.st_nv;
+    p.st_split = models > 1 ? p.st_nv / p.st_share : 0;
   } else {
+    const long long line = units * nv;
+    const long long shares = busy < line / 128 ? busy : (line / 128 < 1 ? 1 : line / 128);
     p.st_nv = nv;
-    p.st_line = units * nv;
-    p.st_share = static_cast<int>(((p.st_line + workers - 1) / workers + 7) / 8 * 8);
+    p.st_line = line;
+    p.st_share = static_cast<int>(((line + shares - 1) / shares + 7) / 8 * 8);
+    p.st_split = 0;
   }
   p.st_workers = static_cast<int>((p.st_line + p.st_share - 1) / p.st_share);
+  p.st_warps = p.st_split ? p.st_workers * models : p.st_workers;
   p.st_inv_nv = 1.0 / p.st_nv;
   p.st_inv_share = 1.0 / p.st_share;
   const int slots = c.combine == COS_COMBINE_PROB_ENSEMBLE ? c.n : 2;
   p.slot_inv = (65536 + slots - 1) / slots;
-  return p.st_workers <= 16LL * sm_count ? 128 : kStreamBlock;
+  return p.st_warps <= 16LL * sm_count ? 128 : kStreamBlock;
 }
 
 // Warps of the streaming launch: what the device holds at once, or the cluster size's worth of blocks for every position.
@@ -227,12 +236,13 @@ cudaError_t launch_stream(const cos_verify_config& c, int mode, KParams& p, bool
     cudaError_t e = cudaSuccess;
     p.st_slabs = 1;
     if (p.mask_model >= 0) {
-      const int threads = plan_line(p, c, p.num_units, workers, sm_count);
+      const int threads = plan_line(p, c, p.num_units, 1, workers, sm_count);
       e = mask_launch<DT>(p, threads, stream);
     }
     // early exit: position by position, so that a row's rejection is known before its later positions are begun
     if (report && p.early_exit) p.st_slabs = p.P;
-    const int threads = plan_line(p, c, p.num_units / p.st_slabs, workers, sm_count);
+    const bool apart = c.combine == COS_COMBINE_PROB_ENSEMBLE && !report;
+    const int threads = plan_line(p, c, p.num_units / p.st_slabs, apart ? c.n : 1, workers, sm_count);
     if (e == cudaSuccess) e = stream_launch<DT>(p, mode, report, threads, stream);
     p.decide = report || decides_first(c) ? 0 : 1;
     const bool first = p.greedy || decides_first(c);
