@@ -23,10 +23,17 @@ KernelFn logit_kernel_of(bool pair, bool masked) {
   return masked ? cos_stream_kernel<DT, MODE, AL, false, true> : cos_stream_kernel<DT, MODE, AL, false, false>;
 }
 
+// Shares of an ensemble from this many vectors on are long (64 rows of 151936 tokens and two models, 2376 vectors: 84.6 us a call
+// with the short form, 82.8 with the long one; 32 rows of 128256 and four models, 768 vectors: 65.4 and 63.8; 32 rows of 32000
+// tokens, 288 vectors: 25.1 and 27.0).
+constexpr int kLongShare = 640;
+
 template <int DT, bool AL>
-KernelFn stream_kernel_of(int mode, bool report, bool pair, bool masked) {
+KernelFn stream_kernel_of(int mode, bool report, bool pair, bool masked, bool long_share) {
   switch (mode) {
-    case kEnsembleSample: return report ? cos_report_kernel<DT, kEnsembleSample, AL> : cos_stream_kernel<DT, kEnsembleSample, AL, true, false>;
+    case kEnsembleSample:
+      if (report) return cos_report_kernel<DT, kEnsembleSample, AL>;
+      return long_share ? cos_stream_kernel<DT, kEnsembleSample, AL, true, false> : cos_stream_kernel<DT, kEnsembleSample, AL, false, false>;
     case kEnsembleGreedy: return report ? cos_report_kernel<DT, kEnsembleGreedy, AL> : cos_stream_kernel<DT, kEnsembleGreedy, AL, true, false>;
     case kLogitSample: return report ? cos_report_kernel<DT, kLogitSample, AL> : logit_kernel_of<DT, kLogitSample, AL>(pair, masked);
     default: return report ? cos_report_kernel<DT, kLogitGreedy, AL> : logit_kernel_of<DT, kLogitGreedy, AL>(pair, masked);
@@ -55,9 +62,10 @@ inline cudaError_t launch(KernelFn fn, const KParams& p, int blocks, int threads
 template <int DT>
 cudaError_t stream_launch(const KParams& p, int mode, bool report, int threads, cudaStream_t stream) {
   const int blocks = (p.st_warps + threads / 32 - 1) / (threads / 32);
-  const bool pair = p.n == 2, masked = p.mask_model >= 0;
-  return launch(p.vec_ok ? stream_kernel_of<DT, true>(mode, report, pair, masked) : stream_kernel_of<DT, false>(mode, report, pair, masked), p,
-                blocks, threads, 0, stream);
+  const bool pair = p.n == 2, masked = p.mask_model >= 0, long_share = p.st_share >= kLongShare;
+  return launch(p.vec_ok ? stream_kernel_of<DT, true>(mode, report, pair, masked, long_share)
+                         : stream_kernel_of<DT, false>(mode, report, pair, masked, long_share),
+                p, blocks, threads, 0, stream);
 }
 
 template <int DT>

@@ -16,7 +16,7 @@ namespace cosv {
 // Measured on 1152 rows of 151936 bf16 entries (350 MB): 58 us (6.0 TB/s) for the sweep alone; whole positions per block of 16
 // warps, as before, 65 to 70 us; shares of blocks instead of warps 65 us; 4 vectors in flight per lane 60 us.  Reporting every part
 // (fence, counter) cost 20 us more, deciding in the same launch another 17, the sweep in a function of its own 8.
-constexpr int kStreamThreads = 512;  // (two blocks per multiprocessor: 64 registers)
+constexpr int kStreamThreads = 1024;  // most of a block: one per multiprocessor (64 registers)
 constexpr int kStreamDepth = 8;      // vectors in flight per lane
 constexpr int kSkipped = 1 << 16;    // a warp that left its part of a position unread (early exit)
 
@@ -149,7 +149,7 @@ __device__ __noinline__ LaneSoft soft_online(const char* row, int v, int v1, flo
 }
 
 // Softmax statistics of vectors [v0, v1) of one row and, with `ragged`, of its ragged entries; every lane's own part.
-template <int DT, bool AL>
+template <int DT, bool AL, bool LONG>
 __device__ __forceinline__ LaneSoft soft_segment(const char* row, int v0, int v1, bool ragged, int V, float c) {
   constexpr int U = kStreamDepth;
   const int lane = threadIdx.x & 31;
@@ -161,23 +161,40 @@ __device__ __forceinline__ LaneSoft soft_segment(const char* row, int v0, int v1
     uint4 raw[U];
     Comp2 total;
     total.init();
-    f32x2 nref2 = pack2(0.f, 0.f);
-    bool first = true;
-    for (; v < v1; v += U * 32) {
+    auto fetch = [&](int at, uint4& r) {
+      r = neg_inf_vector<DT>();
+      if (at < v1) r = load_whole<DT, AL>(row, at);
+    };
+    if (LONG) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        raw[u] = neg_inf_vector<DT>();
-        if (v + u * 32 < v1) raw[u] = load_whole<DT, AL>(row, v + u * 32);
-      }
-      if (first) {
-        acc.ref = seed_ref(vector_max<DT, false>(raw[0]), c);
-        nref2 = pack2(-acc.ref, -acc.ref);
-        first = false;
-      }
-      f32x2 s = vector_sum<DT>(raw[0], c2, nref2);
+      for (int u = 0; u < U; ++u) fetch(v + u * 32, raw[u]);
+      acc.ref = seed_ref(vector_max<DT, false>(raw[0]), c);
+      const f32x2 nref2 = pack2(-acc.ref, -acc.ref);
+      for (; v < v1; v += U * 32) {
+        f32x2 s = pack2(0.f, 0.f);
 #pragma unroll
-      for (int u = 1; u < U; ++u) s = add2(s, vector_sum<DT>(raw[u], c2, nref2));
-      total.add(s);
+        for (int u = 0; u < U; ++u) {
+          s = add2(s, vector_sum<DT>(raw[u], c2, nref2));
+          fetch(v + (U + u) * 32, raw[u]);
+        }
+        total.add(s);
+      }
+    } else {
+      f32x2 nref2 = pack2(0.f, 0.f);
+      bool first = true;
+      for (; v < v1; v += U * 32) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) fetch(v + u * 32, raw[u]);
+        if (first) {
+          acc.ref = seed_ref(vector_max<DT, false>(raw[0]), c);
+          nref2 = pack2(-acc.ref, -acc.ref);
+          first = false;
+        }
+        f32x2 s = vector_sum<DT>(raw[0], c2, nref2);
+#pragma unroll
+        for (int u = 1; u < U; ++u) s = add2(s, vector_sum<DT>(raw[u], c2, nref2));
+        total.add(s);
+      }
     }
     acc.s = total.total();
     if (!(acc.s < INFINITY)) acc = soft_online<DT, AL>(row, v0 + lane, v1, c);
@@ -872,7 +889,7 @@ __device__ __forceinline__ double draft_probability(const KParams& p, const Draf
 // Largest logit of the gating model at every position, for the plausibility mask: the same split, over that model's rows
 // alone.  (Positions need it before they can be swept, and the warps of the streaming launch do not wait for each other.)
 template <int DT, bool AL>
-__global__ void __launch_bounds__(kStreamThreads, 2) cos_mask_kernel(const __grid_constant__ KParams p) {
+__global__ void __launch_bounds__(kStreamThreads, 1) cos_mask_kernel(const __grid_constant__ KParams p) {
   constexpr int U = kStreamDepth;
   const int lane = threadIdx.x & 31;
   const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -943,7 +960,7 @@ __device__ __forceinline__ void sweep_part(const KParams& p, const char* base, i
     if (lane == 0) __stcg(rec + i, v);
   };
   if (MODE == kEnsembleSample) {
-    for (int i = i0; i < i1; ++i) put(i, pack_soft(soft_segment<DT, AL>(base + i * row_step, v0, v1, ragged, p.V, p.cT), thr));
+    for (int i = i0; i < i1; ++i) put(i, pack_soft(soft_segment<DT, AL, PAIR>(base + i * row_step, v0, v1, ragged, p.V, p.cT), thr));
   } else if (MODE == kEnsembleGreedy) {
     for (int i = i0; i < i1; ++i) put(i, pack_arg(arg_segment<DT, AL>(base + i * row_step, v0, v1, ragged, p.V), thr));
   } else if (MODE == kLogitSample) {
@@ -957,9 +974,10 @@ __device__ __forceinline__ void sweep_part(const KParams& p, const char* base, i
   }
 }
 
-// PAIR, MASKED: logit level with exactly two models, and with a mask (kernels of their own: straight code for each).
+// PAIR, MASKED: logit level with exactly two models, and with a mask (kernels of their own: straight code for each).  Ensembles: PAIR
+// is for long shares, which fetch a vector when the place of one before it is free; short ones fetch eight at a time.
 template <int DT, int MODE, bool AL, bool PAIR, bool MASKED>
-__global__ void __launch_bounds__(kStreamThreads, 2) cos_stream_kernel(const __grid_constant__ KParams p) {
+__global__ void __launch_bounds__(kStreamThreads, 1) cos_stream_kernel(const __grid_constant__ KParams p) {
   constexpr bool kEns = (MODE == kEnsembleSample || MODE == kEnsembleGreedy);
   const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   // Launched while the kernel before it in the stream drains (programmatic dependent launch): its blocks take their places
@@ -1003,7 +1021,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) cos_stream_kernel(const __g
 // reported, which needs the decisions while the sweep is under way (a line for each position of the rows, one after another),
 // and for those whose tokens the persistent kernel draws, which has no step that decides.
 template <int DT, int MODE, bool AL>
-__global__ void __launch_bounds__(kStreamThreads, 2) cos_report_kernel(const __grid_constant__ KParams p) {
+__global__ void __launch_bounds__(kStreamThreads, 1) cos_report_kernel(const __grid_constant__ KParams p) {
   constexpr bool kEns = (MODE == kEnsembleSample || MODE == kEnsembleGreedy);
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
   __shared__ Finish fins[kStreamThreads / 32];

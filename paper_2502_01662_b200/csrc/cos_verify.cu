@@ -169,7 +169,10 @@ DrawPlan draw_plan(const cos_verify_config& c, long long units, int sm_count) {
   return d;
 }
 
-constexpr int kStreamBlock = 512;   // threads of a block of a full streaming launch, two blocks per multiprocessor
+// Threads of a block of the streaming launch: 1024 where the launch fills the device (of two blocks of 512 on a multiprocessor the
+// older one's warps go first and leave it half empty in the end: 64 rows of 151936 tokens 86.0 us a call with two, 84.6 with one),
+// 512 and 128 where it does not, so that it spreads over all of it.
+constexpr int kStreamBlock = 512, kStreamFull = 1024, kStreamSmall = 128;
 
 // Cut the line of `units` positions into shares for at most `workers` warps (see cos_stream.cuh).  Small runs take fewer warps, so
 // that each has a few loads in flight, in small blocks, so that they spread over the device.  Where nine tenths of the warps are
@@ -211,7 +214,7 @@ int plan_line(KParams& p, const cos_verify_config& c, long long units, int model
   p.st_inv_share = 1.0 / p.st_share;
   const int slots = c.combine == COS_COMBINE_PROB_ENSEMBLE ? c.n : 2;
   p.slot_inv = (65536 + slots - 1) / slots;
-  return p.st_warps <= 16LL * sm_count ? 128 : kStreamBlock;
+  return p.st_warps <= 16LL * sm_count ? kStreamSmall : (p.st_warps <= 28LL * sm_count ? kStreamBlock : kStreamFull);
 }
 
 // Warps of the streaming launch: what the device holds at once, or the cluster size's worth of blocks for every position.
