@@ -90,6 +90,7 @@ struct KParams {
   int draw_all;            // it visits every position (test hook, residual masses)
   int decide;              // it also merges the records of the streaming launch and decides (else that is done)
   int keep_stats;          // ustats, unit_res and row_draw are wanted afterwards
+  float* lse;              // [B*P][records of a pair]: the log-sum-exps go here from the launch that decides
   int draw_parts;          // blocks of a position's cluster
   int draw_cs, draw_chunks;  // steps of a chunk, chunks of a warp
 };
@@ -237,6 +238,12 @@ struct SoftPart {  // sum over a set of tokens of 2^(arg - ref)
   float ref;
   int pad;
 };
+
+// ln sum_x exp(l(x) / T) of merged statistics, NaN where there is none.
+__device__ __forceinline__ float log_sum_exp(const SoftPart& f, bool there) {
+  if (!there) return __int_as_float(0x7fc00000);
+  return static_cast<float>((static_cast<double>(f.ref) + log2(f.s)) * 0.6931471805599453);
+}
 struct ArgPart {  // running maximum with the lowest index among equals
   double val;
   int idx;

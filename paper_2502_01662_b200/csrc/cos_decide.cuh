@@ -32,7 +32,7 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
   const int tid = threadIdx.x, lane = tid & 31, T = blockDim.x;
   const int slots = record_slots<MODE>(p);
-  const bool optional = p.diag != nullptr || p.keep_stats;
+  const bool optional = p.diag != nullptr || p.keep_stats || p.lse != nullptr;
   // lanes that share a pair: as many as the block has to spare (it has a thread for each at least)
   const int pairs = (p.P < kTile ? p.P : kTile) * slots;
   int lg = 5;
@@ -139,6 +139,11 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
           d[1] = static_cast<float>(f.dec.r_d);
           d[2] = static_cast<float>(f.dec.q_d);
           d[3] = static_cast<float>(f.dec.S);
+        }
+        if (p.lse) {  // ln sum_x exp(l(x) / T) = (ref + log2 s) ln 2
+#pragma unroll 1
+          for (int i = 0; i < slots; ++i)
+            p.lse[static_cast<long long>(uidx) * slots + i] = log_sum_exp(f.fsoft[i], kSample && !(f.dec.status & COS_ROW_NONFINITE));
         }
         if (p.keep_stats) {
           UnitStats& st = p.ustats[uidx];

@@ -65,8 +65,8 @@ struct cos_verify_ctx {
   unsigned wait_limit;  // idle polls after which a block of the one-launch kernel gives up
   int test_drop;        // test hook: one streaming warp never reports its first item
   void* d_logits;
-  int* d_small;   // host-pointer runs: drafts and proposers, then the outputs
-  int* h_small;   // the same, pinned: one copy each way
+  int* h_small;   // host-pointer runs, pinned: drafts and proposers, then the outputs
+  int* d_small;   // drafts and proposers on the device
   std::string err;
 };
 
@@ -426,8 +426,8 @@ extern "C" cos_status cos_verify_create(const cos_verify_config* config, cos_ver
   if (ok && config->host_staging) {
     const size_t V = static_cast<size_t>(config->vocab);
     ok = ok && cudaMalloc(&ctx->d_logits, static_cast<size_t>(config->n) * rows * P * V * elem_bytes(config->dtype)) == cudaSuccess;
-    const size_t small = rows * (2 * P + 3 + P + 4 * P) * sizeof(int);
-    ok = ok && cudaMalloc(&ctx->d_small, small) == cudaSuccess && cudaMallocHost(&ctx->h_small, small) == cudaSuccess;
+    const size_t small = rows * 2 * P * sizeof(int);
+    ok = ok && cudaMalloc(&ctx->d_small, small) == cudaSuccess && cudaMallocHost(&ctx->h_small, small + rows * (3 + 5 * P) * sizeof(int)) == cudaSuccess;
   }
   if (!ok) {
     (void)cudaGetLastError();
@@ -450,8 +450,8 @@ extern "C" cos_status cos_verify_create(const cos_verify_config* config, cos_ver
 }
 
 namespace {
-// the launches of one run (everything but the optional export of the log-sum-exps)
-cos_status run_launches(cos_verify_ctx* ctx, const cos_verify_args* a, void* cuda_stream) {
+// the launches of one run; `lse_done`: the optional log-sum-exps are written by them (not those that decide in the streaming launch)
+cos_status run_launches(cos_verify_ctx* ctx, const cos_verify_args* a, void* cuda_stream, bool* lse_done) {
   if (!ctx) return COS_ERR_INVALID_ARG;
   if (!a) {
     ctx->err = "null args";
@@ -545,8 +545,11 @@ cos_status run_launches(cos_verify_ctx* ctx, const cos_verify_args* a, void* cud
   // under way at once anyway and the hint is not taken.
   const long long workers = stream_workers(c, p.num_units, ctx->sm_count);
   if (static_cast<long long>(p.B) * c.n * (c.vocab / entries_per_vec(c.dtype)) / workers < 1024 || a->dump_r != nullptr) p.early_exit = 0;
-  p.keep_stats = (a->lse != nullptr || a->dump_r != nullptr || decides_first(c)) ? 1 : 0;
-  e = launch_stream(c, mode, p, p.early_exit || by_items, workers, ctx->sm_count, stream);
+  const bool report = p.early_exit || by_items;
+  p.lse = report ? nullptr : a->lse;
+  *lse_done = p.lse != nullptr;
+  p.keep_stats = (a->dump_r != nullptr || decides_first(c)) ? 1 : 0;
+  e = launch_stream(c, mode, p, report, workers, ctx->sm_count, stream);
   if (e != cudaSuccess) return cuda_fail(ctx, "kernel launch (streaming)", e);
   if (ctx->timing) cudaEventRecord(ctx->ev[1], stream);
   ctx->ev_used = 2;
@@ -570,18 +573,16 @@ cos_status run_launches(cos_verify_ctx* ctx, const cos_verify_args* a, void* cud
 }  // namespace
 
 namespace {
-// The log-sum-exp behind every softmax of a position, from the merged statistics a run leaves per position:
-// ln sum_x exp(l(x) / T) = (ref + log2 s) ln 2.  One thread per (position, slot).
+// The log-sum-exp behind every softmax of a position, from the merged statistics a run that decides in its first launch leaves
+// per position.  One thread per (position, slot).
 __global__ void export_lse_kernel(const UnitStats* ustats, const int4* unit_res, float* lse, int units, int slots, int sampling) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= units * slots) return;
   const int u = t / slots, k = t % slots;
-  float v = __int_as_float(0x7fc00000);
-  if (sampling && !(__ldcg(&unit_res[u]).y & COS_ROW_NONFINITE)) {
-    const double sum = ustats[u].s[k];
-    v = static_cast<float>((static_cast<double>(ustats[u].ref[k]) + log2(sum)) * 0.6931471805599453);
-  }
-  lse[t] = v;
+  SoftPart f;
+  f.s = ustats[u].s[k];
+  f.ref = ustats[u].ref[k];
+  lse[t] = log_sum_exp(f, sampling && !(__ldcg(&unit_res[u]).y & COS_ROW_NONFINITE));
 }
 
 }  // namespace
@@ -591,8 +592,9 @@ extern "C" cos_status cos_verify_run(cos_verify_ctx* ctx, const cos_verify_args*
     ctx->err = "lse is not 4-byte aligned";
     return COS_ERR_ALIGNMENT;
   }
-  const cos_status st = run_launches(ctx, a, cuda_stream);
-  if (st != COS_OK || a->lse == nullptr) return st;
+  bool lse_done = false;
+  const cos_status st = run_launches(ctx, a, cuda_stream, &lse_done);
+  if (st != COS_OK || a->lse == nullptr || lse_done) return st;
   const cos_verify_config& c = ctx->cfg;
   const int units = a->batch * (c.gamma + 1);
   const int slots = (c.combine == COS_COMBINE_PROB_ENSEMBLE) ? c.n : 2;
@@ -635,15 +637,19 @@ extern "C" cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   cudaError_t e = cudaSetDevice(c.device);
   if (e != cudaSuccess) return cuda_fail(ctx, "cudaSetDevice", e);
-  // The small arrays go over in one copy each way, by way of pinned memory of the context (the call waits for its copies, so that
-  // memory is free again when it returns): seven small copies of their own were half of the call for one row.
+  // The small arrays go by way of pinned memory of the context (the call waits for its launches, so that memory is free again when it
+  // returns), which the kernels write directly, and read directly where only the decisions need them: copies of their own, seven of
+  // them, were half of the call for one row, and one each way still 10 us of it.
   const size_t lbytes = static_cast<size_t>(c.n) * B * P * V * elem_bytes(c.dtype);
   const size_t ndraft = static_cast<size_t>(B * c.gamma), nprop = static_cast<size_t>((a->flags & COS_RUN_PROPOSER_PER_POSITION) ? B * P : B);
-  const size_t nout = static_cast<size_t>(B * (P + 3) + (a->diag ? B * P * 4 : 0));
-  int *out = ctx->d_small + ndraft + nprop, *h_out = ctx->h_small + ndraft + nprop;
+  int* out = ctx->h_small + ndraft + nprop;
+  int* in = ctx->h_small;
   if (ndraft) memcpy(ctx->h_small, a->draft_tokens, ndraft * sizeof(int));
   memcpy(ctx->h_small + ndraft, a->proposer, nprop * sizeof(int));
-  e = cudaMemcpyAsync(ctx->d_small, ctx->h_small, (ndraft + nprop) * sizeof(int), cudaMemcpyHostToDevice, stream);
+  if (c.combine != COS_COMBINE_PROB_ENSEMBLE || (ctx->fused && (ctx->use_fused || ctx->draw_fused))) {
+    in = ctx->d_small;  // (every warp of the streaming launch asks for the proposer)
+    e = cudaMemcpyAsync(ctx->d_small, ctx->h_small, (ndraft + nprop) * sizeof(int), cudaMemcpyHostToDevice, stream);
+  }
   if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_logits, a->logits, lbytes, cudaMemcpyHostToDevice, stream);
   if (e != cudaSuccess) {
     cudaStreamSynchronize(stream);
@@ -652,8 +658,8 @@ extern "C" cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_
   cos_verify_args d = *a;
   d.flags &= ~COS_RUN_INPUTS_SETTLED;  // the inputs are what the copies above have just written
   d.logits = ctx->d_logits;
-  d.draft_tokens = ctx->d_small;
-  d.proposer = ctx->d_small + ndraft;
+  d.draft_tokens = in;
+  d.proposer = in + ndraft;
   d.accept_count = out;
   d.row_status = reinterpret_cast<unsigned*>(out + B);
   d.bonus_prob = a->bonus_prob ? reinterpret_cast<float*>(out + 2 * B) : nullptr;
@@ -668,18 +674,16 @@ extern "C" cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_
     cudaStreamSynchronize(stream);
     return st;
   }
-  e = cudaMemcpyAsync(h_out, out, nout * sizeof(int), cudaMemcpyDeviceToHost, stream);
-  const cudaError_t done = cudaStreamSynchronize(stream);
-  if (e == cudaSuccess) e = done;
+  e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) {
     ctx->scratch_dirty = true;
-    return cuda_fail(ctx, "device to host copy", e);
+    return cuda_fail(ctx, "waiting for the launches", e);
   }
-  memcpy(a->accept_count, h_out, B * sizeof(int));
-  memcpy(a->row_status, h_out + B, B * sizeof(int));
-  if (a->bonus_prob) memcpy(a->bonus_prob, h_out + 2 * B, B * sizeof(int));
-  memcpy(a->out_tokens, h_out + 3 * B, B * P * sizeof(int));
-  if (a->diag) memcpy(a->diag, h_out + 3 * B + B * P, B * P * 4 * sizeof(int));
+  memcpy(a->accept_count, out, B * sizeof(int));
+  memcpy(a->row_status, out + B, B * sizeof(int));
+  if (a->bonus_prob) memcpy(a->bonus_prob, out + 2 * B, B * sizeof(int));
+  memcpy(a->out_tokens, out + 3 * B, B * P * sizeof(int));
+  if (a->diag) memcpy(a->diag, out + 3 * B + B * P, B * P * 4 * sizeof(int));
   return COS_OK;
 }
 
