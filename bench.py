@@ -31,7 +31,7 @@ from paper_2502_01662_b200.binding import COS_RUN_EARLY_EXIT, COS_RUN_INPUTS_SET
 HEADLINE = "cfg3"
 # dram read + write bytes of one launch of the dominant kernel, as RECORDED in the ncu capture summarised under
 # profiles/ (kernel name -> bytes); reported only while the kernel that runs carries the same name
-TRAFFIC_BYTES = {"cos_verify_kernel": 355468544}   # profiles/cos_verify_kernel_cfg3.md, stage 0 on workload 3
+TRAFFIC_BYTES = {"cos_stream_kernel": 0}
 FALLBACK_HBM_GBS = 6650.0
 NOMINAL_HBM_GBS = 8000.0
 REPORTED = ("cfg1", "cfg2", "cfg3", "cfg4", "cfg5", "cfg5_greedy")
@@ -250,16 +250,17 @@ def kernel_names(w, info):
     """What the launches of one call are (for the roofline's stage list)."""
     if info["one_launch"]:
         return ["cos_fused_kernel (every position: sweep, accept tests, row scan, token draw)"]
-    names = ["cos_verify_kernel stage 0 (every position: sweep, accept tests, row scan)"]
-    if info["launches_per_run"] == 2 and info.get("draw_items"):
-        names.append("cos_fused_kernel, drawing items only (token draw, one sweep)")
-    elif info["launches_per_run"] == 2 and w.combine == synth.COMBINE_PROB_ENSEMBLE and w.n > 2:
-        names.append("cos_verify_kernel stage 4 (token draw, one sweep, a channel per model)")
-    elif info["launches_per_run"] == 2:
-        names.append("cos_verify_kernel stage 3 (token draw, one sweep)")
-    elif info["launches_per_run"] == 3:
-        names += ["cos_verify_kernel stage 1 (normalisers of the drawing positions)",
-                  "cos_verify_kernel stage 2 (token masses and draw)"]
+    if w.temperature == 0.0:
+        return ["cos_stream_kernel (every position swept) with cos_decide_kernel (accept tests, row scan)"]
+    if info.get("draw_items"):
+        return ["cos_report_kernel (every position: sweep, accept tests, row scan)", "cos_fused_kernel, drawing items only (token draw)"]
+    names = ["cos_stream_kernel (every position swept)" if w.mask_model < 0 else
+             "cos_stream_kernel (every position swept) with cos_mask_kernel (largest logit of the gating model) before it"]
+    if w.combine == synth.COMBINE_PROB_ENSEMBLE and (w.n == 1 or w.n > 4):
+        names[0] += " and cos_decide_kernel (accept tests, row scan) after it"
+        names.append("cos_draw_kernel (token draw)")
+    else:
+        names.append("cos_draw_kernel (accept tests, row scan, token draw)")
     return names
 
 

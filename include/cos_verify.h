@@ -78,7 +78,9 @@ enum {
                                      /* accept_count, out_tokens, row_status and bonus_prob are those of */
                                      /* the full run; diag is NaN at a position that was left unread,    */
                                      /* and which positions those are depends on timing.  Taken by       */
-                                     /* cos_verify_run when no cluster size and no mask is configured.   */
+                                     /* cos_verify_run where a warp's share of the batch is long (16 KB  */
+                                     /* of every model or more); shorter runs have every position under  */
+                                     /* way at once, and read it.                                        */
   COS_RUN_INPUTS_SETTLED = 16        /* a promise by the caller: logits, draft_tokens and proposer were  */
                                      /* complete in device memory before the work that precedes this     */
                                      /* call in its stream was submitted (they are not written by the    */
@@ -89,10 +91,9 @@ enum {
                                      /* Outputs and results are those of an ordinary run.  Without the   */
                                      /* flag a run reads nothing before the work ahead of it in the      */
                                      /* stream is complete.  Taken by cos_verify_run at T > 0 for runs   */
-                                     /* of at least one position per multiprocessor whose drawing launch */
-                                     /* is a single wave of blocks, without cluster size, mask, test     */
-                                     /* hook or COS_RUN_EARLY_EXIT; ignored otherwise (cos_verify_get_   */
-                                     /* info does not tell).                                             */
+                                     /* of at least one position and at most one row per multiprocessor, */
+                                     /* without mask, test hook, COS_RUN_ALL_RESIDUALS or early exit;    */
+                                     /* ignored otherwise (cos_verify_get_info does not tell).           */
 };
 
 typedef struct {
@@ -109,8 +110,8 @@ typedef struct {
   int32_t max_batch;               /* largest batch a run may pass, >= 1                                */
   int32_t dtype;                   /* COS_DTYPE_* of the logits                                         */
   int32_t device;                  /* CUDA device ordinal                                               */
-  int32_t cluster_size;            /* thread blocks that share one (row, position) in the streaming     */
-                                   /* stage: 1, 2, 4, 8 or 16; 0 lets the library choose                */
+  int32_t cluster_size;            /* bound on the streaming launch: this many blocks' worth of warps   */
+                                   /* (16 each) per position, 1, 2, 4, 8 or 16; 0: the whole device     */
   int32_t host_staging;            /* non-zero: also allocate device staging for cos_verify_run_host    */
 } cos_verify_config;
 
@@ -148,13 +149,13 @@ typedef struct {
                                /* behind every softmax of a position (Sec. 3.1).  Ensemble: S = n, one  */
                                /* per model; logit level: S = 2, the proposer's logits and the combined */
                                /* (masked) logits.  NaN at T = 0 and where the position is not finite.  */
-                               /* One more small launch per run; may be NULL                            */
+                               /* may be NULL                                                           */
 } cos_verify_args;
 
 typedef struct {
-  int32_t cluster_size;      /* thread blocks per (row, position)                                     */
+  int32_t cluster_size;      /* blocks' worth of warps (16 each) per (row, position), rounded up       */
   int32_t threads_per_block;
-  int32_t max_clusters;      /* clusters that can be resident at once on the device                   */
+  int32_t max_clusters;      /* positions under way at once on the device                             */
   int32_t sm_count;
   int32_t launches_per_run;  /* kernels an ordinary cos_verify_run enqueues: 1 where the one-launch form was    */
                              /* chosen (reserved[2] bit 0); else 2, 3 for ensembles of one or of more than     */
@@ -189,10 +190,10 @@ cos_status cos_verify_create(const cos_verify_config* config, cos_verify_ctx** o
 cos_status cos_verify_run(cos_verify_ctx* ctx, const cos_verify_args* args, void* cuda_stream);
 
 /*
- * Same operation with every pointer in `args` a HOST pointer (pinned memory makes the
- * copies asynchronous): copies logits, drafts and proposers to staging owned by the
- * context, runs, copies accept_count / out_tokens / row_status (and diag if given)
- * back and waits for the stream.  Requires config.host_staging != 0 and contiguous
+ * Same operation with every pointer in `args` a HOST pointer (pinned memory makes the copy of the logits asynchronous):
+ * copies the logits to staging owned by the context, runs, waits for the stream and hands out accept_count / out_tokens /
+ * row_status (and bonus_prob and diag if given); the small arrays pass through pinned memory of the context.
+ * Requires config.host_staging != 0 and contiguous
  * logits (stride_pos = V, stride_row = (gamma+1) V, stride_model = B (gamma+1) V).
  * dump_r and lse are not supported here.
  */
@@ -206,9 +207,8 @@ cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_args* args,
  * do that at the point where they need a verification: an inference engine that has handed
  * the whole device to its own memory pool, or a serving loop in which the device-wide
  * synchronisation that cudaMalloc / cudaFree imply would stall every other stream.  This call
- * needs no context: the kernels' scratch (work and job counters, per-row arrival counters,
- * per-position results, statistics and partial sums, the list of positions that draw a token)
- * lives in an array that is part of the
+ * needs no context: the kernels' scratch (records of the streaming launch, per-position results and statistics, mask
+ * keys) lives in an array that is part of the
  * library image, COS_STATIC_SCRATCH_BYTES long, resident on every device that loads the
  * library until the process exits.  The call performs no cudaMalloc, cudaFree or other
  * device allocation; `config` is read on every call (max_batch and host_staging are ignored).
@@ -217,10 +217,10 @@ cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_args* args,
  * COS_STATIC_MAX_POSITIONS; anything larger returns COS_ERR_INVALID_ARG with the reason in
  * cos_verify_last_error(NULL) and enqueues nothing.
  *
- * The first call on a device looks up the array's device address (cudaGetSymbolAddress) and
- * sets kernel attributes; make that first call outside any stream capture.  Every call
- * re-initialises the part of the array that must start clean (memset on `cuda_stream`)
- * before the kernel, so a call does not depend on what the previous one left behind.
+ * The first call on a device looks up the array's device address (cudaGetSymbolAddress);
+ * make that first call outside any stream capture.  Nothing in the array is read before the call's own launches have
+ * written it (mask keys, which must start at zero, are cleared on `cuda_stream` first), so a call does not depend on what
+ * the previous one left behind.
  * All calls on a device share the one array: two calls that overlap on the GPU (different
  * streams without an ordering between them) race and give undefined results.  Calls ordered
  * on one stream, or otherwise serialised, are safe.  Inputs, outputs and semantics are those
@@ -236,8 +236,8 @@ cos_status cos_verify_run_static(const cos_verify_config* config, const cos_veri
 
 /*
  * Measurement aid: with `enable` non-zero, every later cos_verify_run records CUDA events on its
- * stream around each of its launches (stage 0: every position, Eq. 3-6 and the row scan; then the
- * launches that draw the tokens).  cos_verify_get_stage_ms waits for the last timed run and
+ * stream around its launches (first those that read every position, Eq. 3-5, with those that decide in a launch of their own; then
+ * the one that decides, Eq. 6, scans the rows and draws the tokens).  cos_verify_get_stage_ms waits for the last timed run and
  * returns the duration of each of its launches in milliseconds (at most 3 values) and their
  * number.  Timing adds a few event records per run and changes no result.
  */

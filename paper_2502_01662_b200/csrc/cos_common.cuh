@@ -47,7 +47,7 @@ struct KParams {
   int num_units;
   int per_pos;      // proposer is [B][gamma+1] (the model that proposed each draft) instead of [B]
   int early_exit;   // positions after a row's known first rejection may be left unread
-  int greedy;       // T = 0: no drawing stages; the fourth word of a unit's result carries the bonus probability
+  int greedy;       // T = 0: nothing is drawn; the fourth word of a unit's result carries the bonus probability
   int bonus_model;  // >= 0: the token after gamma acceptances follows this model's own distribution; -1: the combined one
   int inputs_settled;  // the inputs may be read before the kernel ahead in the stream is complete
   int max_jobs;  // capacity of the job list
@@ -72,7 +72,7 @@ struct KParams {
   int4* unit_res;          // [B*P]: x = accept flag, y = status bits, z = candidate token, w = a token can be drawn
   int* job_count;          // length of the job list (persistent kernel, which also clears it)
   int2* jobs;              // x = b * P + j of a unit that draws a token (y unused)
-  UnitStats* ustats;       // [B*P]: merged statistics of sweep 1, read back by the later stages
+  UnitStats* ustats;       // [B*P]: merged statistics, where a later launch reads them
   int use_jobs;            // the list of drawing positions is kept too (tokens drawn by the persistent kernel)
   // the streaming launch: a line of st_line vectors (st_nv for each position) in st_workers shares of st_share vectors (the last may
   // be shorter); st_slabs lines one after another (one, or one for each position of a row)

@@ -7,11 +7,16 @@
 
 namespace cosv {
 
-// A block decides a whole row: a few lanes merge the records of one (position, slot) pair each, then one warp goes on, a lane taking the accept
-// test of a position, a ballot finding the first rejection.  Every block of a row does it for itself (the records of a row are a
-// few KB, read from L2), which costs the device nothing that it would use otherwise and no word has to travel between blocks;
-// one of them writes the outputs.  It is a chain of latencies: what it needs of the inputs (drafts, proposers, the logits at the
-// drafts) is fetched before the launch waits for the streaming launch to end.
+// A block decides a whole row: a few lanes merge the records of one (position, slot) pair each, then one warp goes on, a lane taking
+// the accept test of a position, a ballot finding the first rejection.  Every block of a row does it for itself (the records of a
+// row are a few KB, read from L2), which costs the device nothing that it would use otherwise, and no word has to travel between
+// blocks; one of them writes the outputs.
+// What bounds it: a chain of latencies, and fetching instructions that no other block has run before (5 us from the end of the
+// streaming launch to the first load of the drawing sweep).  So what it needs of the inputs (drafts, proposers, the logits at the
+// drafts) is asked for before it waits for the streaming launch to end, there is one copy of everything and little is
+// unrolled: with fetches in two copies, 64-bit divisions and unrolled cold loops (35 KB instead of 20) it took 11 us.  Going
+// through it once on stale records before the wait, to have the instructions at hand, cost 4 to 8 us: the first time is the slow
+// one wherever it is.
 constexpr int kTile = 16;  // positions decided at a time
 
 struct RowShared {
@@ -24,9 +29,9 @@ struct RowShared {
 };
 
 // Decide row b.  `want` >= 0: a position whose statistics the block needs, whatever the first rejection; otherwise the first
-// rejected position is what it needs.  `keep(fin, j, word, accepted, drawable)` is called by the first warp with that
-// position's merged statistics and the random word its token is drawn with.  `writes_row(a)` / `writes_unit(j)`: whether this block writes the row's outputs and a
-// position's optional ones.
+// rejected position is what it needs.  `keep(fin, j, word, accepted, drawable)` is called by the first warp with that position's
+// merged statistics and the random word its token is drawn with.  `writes_row(a)` / `writes_unit(j)`: whether this block writes
+// the row's outputs and a position's optional ones.
 template <int DT, int MODE, typename K, typename WR, typename WU>
 __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int b, int want, K keep, WR writes_row, WU writes_unit) {
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);

@@ -20,7 +20,9 @@ namespace cosv {
 // that the launch fills the device in one wave (see draw_plan).
 // The part behind the sweep is a chain of latencies, issue slots and instruction fetches (counted on one row of 151936 tokens: most
 // stalls are for instructions), so what can be done by one warp is, and nothing is unrolled that need not be.
-// Records in global memory and the last block to report (fence and counter) took 5 us longer.
+// Measured (64 rows of 2 x 151936 tokens): 9 us of sweep, 3 until the cluster's last warp is done, 6 to find the token.  Records in
+// global memory and the last block to report (fence and counter) took 5 us longer; two more barriers of the cluster, for all
+// blocks to look for the token, 1.
 constexpr int kMaxDrawThreads = 512;
 constexpr int kMaxDrawWarps = kMaxDrawThreads / 32;
 constexpr int kMaxParts = 8;       // blocks of a cluster
@@ -310,9 +312,11 @@ __device__ __noinline__ void slow_vectors(const DrawConst& p, const DrawUnit<NCH
 
 // The steps [s_lo, s_hi) of a position by one warp, in chunks of cs steps: per channel the sum over the tokens with a positive mass,
 // for every chunk NCH sums to rec, and to part the normaliser's share, of all chunks together (both in the cluster's first block).
-// The fast loop adds vectors up in fp32; vectors that need the
-// slow path it only remembers until the end of the strip (their sums, in fp64, in the thread's slots of `acc`).
-// What bounds it: loads in flight (two steps of every model at a time) and issue (about 17 instructions per pair of terms).
+// The fast loop adds vectors up in fp32; vectors that need the slow path it only remembers until the end of the strip (their
+// sums, in fp64, in the thread's slots of `acc`).
+// What bounds it: instruction issue (counted at logit level, 128 rows of 256000 tokens: 211 instructions a step, 0.53 of the issue
+// slots of the average multiprocessor, 0.67 of the busiest).  Loads in flight do not: fetching a step as soon as a place is free,
+// so that two are always on their way, gained nothing with two channels and lost 2 to 7 % with four.
 // PAIR, MASKED: logit level with exactly two models, and with a mask.
 template <int DT, bool ENS, int NCH, bool AL, bool PAIR, bool MASKED>
 __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst& kc, const DrawUnit<NCH>& u, int cs, int s_lo, int s_hi, double* acc,

@@ -1,5 +1,4 @@
-// The streaming launch of a run: every logit is read once (Eq. 3-5), every position decided (Eq. 6), every row scanned for
-// its first rejection (Sec. 3.1).
+// The streaming launch of a run: every logit is read once (Eq. 3-5).
 #ifndef COS_STREAM_CUH
 #define COS_STREAM_CUH
 
@@ -8,14 +7,18 @@
 namespace cosv {
 
 // Split: the positions' 16-byte vectors (the same vectors of all models of a position go together) form one line in the order of
-// memory, cut into p.st_workers equal contiguous shares, one for each warp of a single wave of blocks, whatever the positions'
-// boundaries.  So every warp streams the same number of bytes for any batch and vocabulary, with 4 KB in flight, and does
-// nothing else: it leaves one record per model (partial softmax statistics or argmaxes) for every position it had a part of, and the
-// next launch merges the records of a row's positions and decides (see cos_decide.cuh).  Models that agree at a position are cut
-// at the same places, so that their statistics are the same bit for bit.
-// Measured on 1152 rows of 151936 bf16 entries (350 MB): 58 us (6.0 TB/s) for the sweep alone; whole positions per block of 16
-// warps, as before, 65 to 70 us; shares of blocks instead of warps 65 us; 4 vectors in flight per lane 60 us.  Reporting every part
-// (fence, counter) cost 20 us more, deciding in the same launch another 17, the sweep in a function of its own 8.
+// memory, cut into p.st_workers equal contiguous shares, one for each warp of a single wave of blocks.  So every warp streams the
+// same number of bytes for any batch and vocabulary, with 4 KB in flight, and does nothing else: it leaves one record per model
+// (partial softmax statistics or argmaxes) for every position it had a part of, and the next launch merges the records of a row's
+// positions and decides (see cos_decide.cuh).  Where there are enough shares to a position they end where it ends, and short
+// shares of an ensemble are one model's (see plan_line).  Models that agree at a position are cut at the same places, so that
+// their statistics are the same bit for bit.
+// What bounds it: HBM in large runs (256 rows of 256000 tokens, 2.36 GB: 355 us, 6.6 TB/s), in small ones the latency of one batch
+// of loads and the launch (one row of 6 x 2 x 151936 entries: 4 us).
+// Measured on 1152 rows of 151936 bf16 entries (350 MB): 60 us (5.8 TB/s); whole positions per block of 16 warps, as before, 65 to
+// 70 us; shares of blocks instead of warps 65; 4 vectors in flight per lane 2 us more.  Reporting every part (fence, counter) cost
+// 20 us more, deciding in the same launch another 17, the sweep in a function of its own 8; handing the last quarter out in
+// items of 8 KB as warps become free 10 (each item pays a memory round trip and a record).
 constexpr int kStreamThreads = 1024;  // most of a block: one per multiprocessor (64 registers)
 constexpr int kStreamDepth = 8;      // vectors in flight per lane
 constexpr int kSkipped = 1 << 16;    // a warp that left its part of a position unread (early exit)
