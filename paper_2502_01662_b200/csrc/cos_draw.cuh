@@ -47,11 +47,6 @@ __device__ __forceinline__ void store_cluster(unsigned a, double v) {
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
 }
 
-__device__ __forceinline__ double warp_sum(double t) {
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
-  return t;
-}
 // Sums of N values over the warp at once: lane L ends up with the sum of value (L * N / 32).
 template <int N>
 __device__ __forceinline__ double warp_sums(double (&v)[N], int lane) {
@@ -648,36 +643,40 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
     const int s0 = static_cast<int>(static_cast<long long>(p.nsteps) * ww / W) + win % p.draw_chunks * cs;
     const int end = static_cast<int>(static_cast<long long>(p.nsteps) * (ww + 1) / W);
     const int s1 = s0 + cs < end ? s0 + cs : end, gsz = (cs + 31) / 32;
-    double own = 0.0;
-    int held = -1;  // the step whose mass the lanes of this warp hold
+    // running total over the first `lanes` lanes
+    auto scan = [&](double m, int lanes) -> double {
+#pragma unroll 1
+      for (int d = 1; d < lanes; d <<= 1) {
+        const double o = __shfl_up_sync(0xffffffffu, m, d);
+        if (lane >= d) m += o;
+      }
+      return m;
+    };
+    // the first lane whose total `in` (its own mass: m) reaches the target, or the last with mass where rounding leaves none
+    auto first_reach = [&](double m, double in, double from, double& upto) -> int {
+      const unsigned some = __ballot_sync(0xffffffffu, m > 0.0), ok = __ballot_sync(0xffffffffu, m > 0.0 && from + in >= target);
+      const int k = ok ? __ffs(ok) - 1 : 31 - __clz(some);
+      upto = from + __shfl_sync(0xffffffffu, in - m, k & 31);
+      return ok ? k : k - 32;  // (negative: not reached; -33: no mass at all)
+    };
+    double own = 0.0, in = 0.0;
+    int held = -1;  // the step whose masses, and their running total, the lanes of this warp hold
 #pragma unroll 1
     for (int t = warp; s0 + t * gsz < s1; t += nw) {
       double rm = 0.0;
 #pragma unroll 1
       for (int s = s0 + t * gsz; s < s0 + (t + 1) * gsz && s < s1; ++s) {
         own = step_mass<DT, ENS, NCH, AL>(p, sh.kc, u, cf, inv, s);
-        rm += warp_sum(own);
+        in = scan(own, 32);
+        rm += __shfl_sync(0xffffffffu, in, 31);
         held = s;
       }
       if (lane == 0) sh.step_mass[t] = rm;
     }
     __syncthreads();
     if (held < 0) return;  // (no step of the chunk is this warp's)
-    // running total over the first `lanes` lanes; the first that reaches the target, or the last with mass where rounding leaves none
-    auto first_reach = [&](double m, int lanes, double from, double& upto) -> int {
-      double in = m;
-#pragma unroll 1
-      for (int d = 1; d < lanes; d <<= 1) {
-        const double o = __shfl_up_sync(0xffffffffu, in, d);
-        if (lane >= d) in += o;
-      }
-      const unsigned some = __ballot_sync(0xffffffffu, m > 0.0), ok = __ballot_sync(0xffffffffu, m > 0.0 && from + in >= target);
-      const int k = ok ? __ffs(ok) - 1 : 31 - __clz(some);
-      upto = from + __shfl_sync(0xffffffffu, in - m, k & 31);
-      return ok ? k : k - 32;  // (negative: not reached; -33: no mass at all)
-    };
-    double at;
-    int k = first_reach((s0 + lane * gsz < s1) ? sh.step_mass[lane] : 0.0, (s1 - s0 + gsz - 1) / gsz, sh.base, at);
+    double at, m = (s0 + lane * gsz < s1) ? sh.step_mass[lane] : 0.0;
+    int k = first_reach(m, scan(m, (s1 - s0 + gsz - 1) / gsz), sh.base, at);
     if (k == -33) return;
     if ((k & 31) % nw != warp) return;
     // one warp goes on: the record's steps in order, the lanes of a step, the tokens of a lane's vector
@@ -686,23 +685,26 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
     double before = 0.0;
 #pragma unroll 1
     for (int s = g0; s < g1; ++s) {
-      if (s != held) own = step_mass<DT, ENS, NCH, AL>(p, sh.kc, u, cf, inv, s);
+      if (s != held) {
+        own = step_mass<DT, ENS, NCH, AL>(p, sh.kc, u, cf, inv, s);
+        in = scan(own, 32);
+        held = s;
+      }
       double upto;
-      const int l = first_reach(own, 32, at, upto);
+      const int l = first_reach(own, in, at, upto);
       if (l != -33) {
         step = s;
         who = l & 31;
         before = upto;
       }
       if (l >= 0) break;
-      held = s;
-      if (s + 1 < g1) at += warp_sum(own);
+      at += __shfl_sync(0xffffffffu, in, 31);
     }
     if (step < 0) return;
     const int e = (step * 32 + who) * E + lane;
-    double m = 0.0;
+    m = 0.0;
     if (lane < E && e < p.V) m = token_mass<DT, ENS, NCH>(sh.kc, u, cf, inv, e);
-    k = first_reach(m, E, before, at);
+    k = first_reach(m, scan(m, E), before, at);
     const int token = (step * 32 + who) * E + (k & 31);
     if (lane == 0 && k != -33) {
       p.out_tokens[u.uidx] = token;
