@@ -136,8 +136,9 @@ bool decides_first(const cos_verify_config& c) { return c.combine == COS_COMBINE
 // How the drawing launch shares a position out.  The device holds 32 warps per multiprocessor (two channels) or 16; a
 // position gets a cluster of blocks of 16, 8 or 4 warps, whichever leaves least of the device idle.  Clusters of more than four
 // blocks are taken only where they need no more than two thirds of the device: they do not pack (32 clusters of 8 blocks
-// of 16 warps, on paper a fit, ran in two waves: 51 us instead of 37 for 32 rows of 32000 tokens; 64 of 8 blocks of 8 warps
-// 109 instead of 92 for 64 rows of 151936).
+// of 16 warps, on paper a fit, run in two waves: 31.8 us a call instead of 25.2 for 32 rows of 32000 tokens; 64 of 8 blocks of 8
+// warps 91 instead of 83 for 64 rows of 151936).  Fewer and smaller clusters: one row of 151936 tokens 18.5 us with 8 blocks of 16
+// warps, 20.7 with 4, 25.2 with 2.
 // A warp has a few chunks (one record of sums each), of eight steps where there is room for the records, so that the token is
 // searched in few steps.
 struct DrawPlan {
