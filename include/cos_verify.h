@@ -87,7 +87,8 @@ enum {
                                      /* kernel queued just before the call).  The streaming launch may   */
                                      /* then read them while that work drains - the drawing launch of    */
                                      /* the previous call, for one - and waits for it only before it     */
-                                     /* touches anything else; calls queued back to back overlap.        */
+                                     /* touches anything else (an offset in device memory included);     */
+                                     /* calls queued back to back overlap.                               */
                                      /* Outputs and results are those of an ordinary run.  Without the   */
                                      /* flag a run reads nothing before the work ahead of it in the      */
                                      /* stream is complete.  Taken by cos_verify_run at T > 0 for runs   */

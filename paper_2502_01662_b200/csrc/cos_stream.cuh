@@ -989,7 +989,9 @@ __global__ void __launch_bounds__(kStreamThreads, 1) cos_stream_kernel(const __g
   // promises that the inputs were complete earlier, a warp sweeps its first part first and waits only before it writes.
   bool waited = p.inputs_settled == 0;
   if (waited) asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // The drawing launch reads the counter offset before it waits for this launch.  The promise does not cover an offset in device
+  // memory, so there it may start only when every block of this launch is gone, and so has waited (each has a part to write).
+  if (waited || p.off_dev == nullptr) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (w >= p.st_warps) return;
   const int slots = record_slots<MODE>(p);
   int share = w, i0 = 0, i1 = p.n;

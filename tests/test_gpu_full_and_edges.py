@@ -378,3 +378,30 @@ def test_calls_queued_back_to_back_give_what_isolated_calls_give(name, kw, settl
         helpers.check_parity(w, got, ref)
     finally:
         v.close()
+
+
+@pytest.mark.parametrize("n", [2, 5])       # decisions in the drawing launch, and in a launch of their own
+def test_offset_written_just_before_a_call_on_settled_inputs_is_seen(n):
+    """COS_RUN_INPUTS_SETTLED promises logits, drafts and proposer, not the offset in device memory: a kernel that
+    advances the offset, queued directly before each call, is complete before the call reads it."""
+    weights = (0.6, 0.4) if n == 2 else (0.3, 0.25, 0.2, 0.15, 0.1)
+    w = synth.Workload("settled_offset", n, synth.COMBINE_PROB_ENSEMBLE, weights, 1.0, 40, 4, 20008, "bf16", "gauss", sigma=2.5, rho=0.8,
+                       proposer_rule="cycle")
+    inputs = synth.make_inputs(w, "cuda")
+    args = (inputs["logits"], inputs["drafts"], inputs["proposer"], inputs["seed"])
+    off = torch.zeros(1, dtype=torch.int64, device="cuda")
+    step = torch.ones(1 << 22, dtype=torch.int64, device="cuda")
+    v = helpers.make_verifier(w)
+    try:
+        torch.cuda.synchronize()
+        queued = []
+        for _ in range(24):
+            off += step.max()            # two kernels, the first of them longer than the tail of the call before
+            queued.append(v.run(*args, 0, offset_device=off, flags=COS_RUN_INPUTS_SETTLED))
+        torch.cuda.synchronize()
+        for k, outs in enumerate(queued):
+            want = v.run(*args, k + 1)
+            for key in ("accept_count", "out_tokens", "row_status"):
+                assert torch.equal(outs[key], want[key]), (k, key)
+    finally:
+        v.close()
