@@ -391,8 +391,16 @@ __device__ __forceinline__ uint4 load_vector(const char* row, int v, int V, cons
   return ragged_vector<DT>(row, v * Elem<DT>::E, V);
 }
 
+// A lane's sum is measured against a fixed reference exponent, seeded from its first vector, so it is 1 at least.  Where that vector
+// held nothing but -inf the reference is 0 until further notice, and a sum below this may have lost what it should hold
+// to underflow (or is of nothing): such a lane goes through its vectors again with a running maximum, and one with nothing
+// ends with the reference of an empty sum.
+constexpr float kTinySum = 8.67361738e-19f;  // 2^-60
+
 struct LaneSoft {
   float ref, s;
+  // whether the fixed reference held (a lane without any vector is as `init` left it)
+  __device__ __forceinline__ bool holds() const { return s < INFINITY && (s >= kTinySum || ref == -INFINITY); }
   __device__ __forceinline__ void init() {
     ref = -INFINITY;
     s = 0.f;
@@ -423,7 +431,7 @@ struct LaneSoft {
     float nref = (ref == -INFINITY) ? 0.f : -ref;
     s += ex2_approx(fmaf(x, c, nref));
   }
-  // reference exponent fixed (set from the first chunk); the caller checks s for overflow
+  // reference exponent fixed (set from the first chunk); the caller asks whether it held
   template <int E>
   __device__ __forceinline__ void seed(const float (&v)[E], float c) {
     float vmax = v[0];
@@ -612,7 +620,7 @@ __device__ __forceinline__ float pair_at(f32x2 v, int k) { return (k & 1) ? hi2(
 // Softmax statistics of a logit-level combine over the slice `sl` of one (row, position): accq = the proposer's
 // softmax, accc = the softmax of the combined logits sum_i w_i l_i (entries outside the plausibility mask count
 // as -inf).  Fast form: fixed reference exponents seeded from the thread's first vector, one vector of every model
-// per trip, the first two models fetched one trip ahead; overflow or a non-finite input falls back to the
+// per trip, the first two models fetched one trip ahead; overflow, underflow or a non-finite input falls back to the
 // running-maximum form.  `tid` in [0, NT): the threads that share the slice.
 template <int DT, int NT>
 __device__ __forceinline__ void logit_soft_slice(const KParams& p, const char* base, const Slice& sl, int tid, int pis,
@@ -691,14 +699,12 @@ __device__ __forceinline__ void logit_soft_slice(const KParams& p, const char* b
         accq.add_online1(xq, p.cT);
         accc.add_online1(cmb, p.cT);
       }
-      settled = (accq.s < INFINITY) && (accc.s < INFINITY);
+      settled = accq.holds() && accc.holds();
     }
-    // overflow or a non-finite input: the running-maximum form (two vectors of two models per trip)
-    for (int pass = 1; pass < 2 && !settled; ++pass) {
-      const bool fixed = (pass == 0);
+    // overflow, underflow or a non-finite input: the running-maximum form (two vectors of two models per trip)
+    if (!settled) {
       accq.init();
       accc.init();
-      bool seeded_q = false, seeded_c = false;
       // one model's vector: add to the combined logits; the proposer's row also feeds its own softmax,
       // the expert's row yields the mask bits
       auto take = [&](int i, const uint4& raw, float (&cmb)[E], unsigned& inbits) {
@@ -708,15 +714,7 @@ __device__ __forceinline__ void logit_soft_slice(const KParams& p, const char* b
 #pragma unroll
         for (int k = 0; k < E; ++k) cmb[k] = fmaf(wi, x[k], cmb[k]);
         if (i == pis) {
-          if (fixed) {
-            if (!seeded_q) {
-              accq.seed(x, p.cT);
-              seeded_q = true;
-            }
-            accq.add_fixed(x, p.cT);
-          } else {
-            accq.add_online(x, p.cT);
-          }
+          accq.add_online(x, p.cT);
         }
         if (masked && i == p.mask_model) {
           inbits = 0u;
@@ -729,15 +727,7 @@ __device__ __forceinline__ void logit_soft_slice(const KParams& p, const char* b
 #pragma unroll
           for (int k = 0; k < E; ++k) cmb[k] = (inbits & (1u << k)) ? cmb[k] : -INFINITY;
         }
-        if (fixed) {
-          if (!seeded_c) {
-            accc.seed(cmb, p.cT);
-            seeded_c = true;
-          }
-          accc.add_fixed(cmb, p.cT);
-        } else {
-          accc.add_online(cmb, p.cT);
-        }
+        accc.add_online(cmb, p.cT);
       };
       for (int v = sl.v_lo + tid; v < sl.v_hi; v += 2 * NT) {
         const bool have_b = (v + NT < sl.v_hi);
@@ -781,7 +771,6 @@ __device__ __forceinline__ void logit_soft_slice(const KParams& p, const char* b
         accq.add_online1(xq, p.cT);
         accc.add_online1(cmb, p.cT);
       }
-      if ((accq.s < INFINITY) && (accc.s < INFINITY)) break;
     }
 }
 

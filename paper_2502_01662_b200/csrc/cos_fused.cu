@@ -172,7 +172,7 @@ __device__ __forceinline__ uint4 ldg_ahead16(const void* p) {
   return v;
 }
 
-// One row's share of one thread again in the running-maximum form (after an overflow or a non-finite input).
+// One row's share of one thread again in the running-maximum form (after an overflow, an underflow or a non-finite input).
 template <int DT>
 __device__ __noinline__ LaneSoft online_redo(const char* row, int v_first, int v_hi, float c) {
   constexpr int E = Elem<DT>::E;
@@ -193,7 +193,7 @@ __device__ __noinline__ LaneSoft online_redo(const char* row, int v_first, int v
 // Ensemble: the softmax statistics of the chunk [lo, hi) of every model's row.  A thread's vectors are those at
 // lo + stid + 480 m, four per stage, read from shared memory once the stage's bulk copy has landed.  Fixed reference
 // exponent per row and thread, seeded from the thread's first vector (a whole number, so that sums rescale exactly);
-// overflow or a non-finite input redoes the thread's share of that row from global memory in the running-maximum
+// overflow, underflow or a non-finite input redoes the thread's share of that row from global memory in the running-maximum
 // form.  False when a wait gave up.
 template <int DT>
 __device__ __forceinline__ bool stream_ensemble(const FParams& fp, const ItemCtx& it, SoftPart* part, int stid, FShared& sh,
@@ -231,14 +231,14 @@ __device__ __forceinline__ bool stream_ensemble(const FParams& fp, const ItemCtx
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh.empty[slot]);
     }
-    if (!(acc.s < INFINITY)) acc = online_redo<DT>(base + i * row_step, it.lo + stid, it.hi, p.cT);
+    if (!acc.holds()) acc = online_redo<DT>(base + i * row_step, it.lo + stid, it.hi, p.cT);
     warp_merge_soft(acc, &part[i], lane);
   }
   return true;
 }
 
 // Logit level with two models: proposer's softmax and the softmax of the combined logits.  `settled` comes back
-// false when some lane of the warp met an overflow or a non-finite input (the caller then takes the general form
+// false when some lane of the warp met an overflow, an underflow or a non-finite input (the caller then takes the general form
 // from global memory).  False when a wait gave up.
 template <int DT>
 __device__ __forceinline__ bool stream_logit2(const FParams& fp, const ItemCtx& it, SoftPart* part, int stid, FShared& sh,
@@ -286,7 +286,7 @@ __device__ __forceinline__ bool stream_logit2(const FParams& fp, const ItemCtx& 
     __syncwarp();
     if (lane == 0) mbar_arrive(&sh.empty[slot]);
   }
-  const bool settled = (accq.s < INFINITY) && (accc.s < INFINITY);
+  const bool settled = accq.holds() && accc.holds();
   settled_all = __all_sync(0xffffffffu, settled);
   if (settled_all) {
     warp_merge_soft(accq, &part[0], lane);
@@ -348,7 +348,7 @@ __device__ __forceinline__ bool stream_item(const FParams& fp, const ItemCtx& it
     if (!stream_logit2<DT>(fp, it, part, stid, sh, ring, k, settled)) return false;
     if (settled) return true;
   }
-  // any other number of models, and the warps that met an overflow or a non-finite input: from global memory
+  // any other number of models, and the warps that met an overflow, an underflow or a non-finite input: from global memory
   const char* base = unit_base(p, it.b, it.j, Elem<DT>::bytes);
   Slice sl;
   sl.v_lo = it.lo;

@@ -90,6 +90,11 @@ __device__ __forceinline__ unsigned max2_nan(unsigned a, unsigned b) {
     asm("max.NaN.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
   return d;
 }
+__device__ __forceinline__ float max3(float a, float b, float c) {  // (a NaN counts for nothing)
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
 // The largest entry of a vector, NaN if there is one; MAG: the largest magnitude.
 template <int DT, bool MAG>
 __device__ __forceinline__ float vector_max(const uint4& r) {
@@ -117,7 +122,8 @@ struct Comp2 {
   __device__ __forceinline__ float total() const { return (lo2(sum) + hi2(sum)) + (lo2(nc) + hi2(nc)); }
 };
 
-// Reference exponent of a lane's sum: fixed, from its first vector, a whole number (sums with such references rescale exactly).
+// Reference exponent of a lane's sum: fixed, from its first vector, a whole number (sums with such references rescale exactly); 0 where
+// that is not finite (see kTinySum).
 __device__ __forceinline__ float seed_ref(float vmax, float c) {
   const float cand = vmax * c;
   return (fabsf(cand) < INFINITY) ? floorf(cand) : 0.f;
@@ -138,15 +144,26 @@ __device__ __forceinline__ f32x2 vector_sum(const uint4& r, f32x2 c2, f32x2 nref
   return s;
 }
 
-// The same segment with a running maximum, for the lane whose fixed reference overflowed or met a non-finite input.  Rare.
+// The same segment with a running maximum, for the lane whose fixed reference did not hold.  Rare, but for logits of which most are
+// -inf: four vectors at a time.
 template <int DT, bool AL>
 __device__ __noinline__ LaneSoft soft_online(const char* row, int v, int v1, float c) {
   LaneSoft acc;
   acc.init();
-  for (; v < v1; v += 32) {
-    float x[Elem<DT>::E];
-    Elem<DT>::unpack(load_whole<DT, AL>(row, v), x);
-    acc.add_online(x, c);
+#pragma unroll 1
+  for (; v < v1; v += 128) {
+    uint4 raw[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      raw[u] = neg_inf_vector<DT>();
+      if (v + u * 32 < v1) raw[u] = load_whole<DT, AL>(row, v + u * 32);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      float x[Elem<DT>::E];
+      Elem<DT>::unpack(raw[u], x);
+      acc.add_online(x, c);
+    }
   }
   return acc;
 }
@@ -171,9 +188,19 @@ __device__ __forceinline__ LaneSoft soft_segment(const char* row, int v0, int v1
     if (LONG) {
 #pragma unroll
       for (int u = 0; u < U; ++u) fetch(v + u * 32, raw[u]);
-      acc.ref = seed_ref(vector_max<DT, false>(raw[0]), c);
-      const f32x2 nref2 = pack2(-acc.ref, -acc.ref);
+      bool empty = true;
       for (; v < v1; v += U * 32) {
+        if (empty) {  // (nothing but -inf so far, if anything: nothing was added)
+          float m = vector_max<DT, false>(raw[0]);
+          if (m == -INFINITY) {
+#pragma unroll
+            for (int u = 1; u < U; ++u) m = max_nan(m, vector_max<DT, false>(raw[u]));
+          }
+          empty = m == -INFINITY;
+          acc.ref = empty ? -INFINITY : seed_ref(m, c);
+        }
+        const float n = empty ? 0.f : -acc.ref;
+        const f32x2 nref2 = pack2(n, n);
         f32x2 s = pack2(0.f, 0.f);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -200,7 +227,7 @@ __device__ __forceinline__ LaneSoft soft_segment(const char* row, int v0, int v1
       }
     }
     acc.s = total.total();
-    if (!(acc.s < INFINITY)) acc = soft_online<DT, AL>(row, v0 + lane, v1, c);
+    if (!acc.holds()) acc = soft_online<DT, AL>(row, v0 + lane, v1, c);
   }
   if (ragged) {
     const int e = ragged_entry(ragged_of<DT, AL>(V), V, lane);
@@ -254,7 +281,7 @@ __device__ __forceinline__ ArgPart arg_segment(const char* row, int v0, int v1, 
 struct LaneSoft2 {
   LaneSoft q, c;
 };
-// Tokens [e, end) one by one, running maximum: the ragged ends, and everything where a sum overflowed or met a non-finite input.
+// Tokens [e, end) one by one, running maximum: the ragged ends, and the lane whose fixed references did not hold.
 template <int DT>
 __device__ __noinline__ LaneSoft2 logit_online(const KParams& p, const char* base, int pis, float thr, int e, int end, LaneSoft2 a) {
   for (; e < end; ++e) {
@@ -293,6 +320,7 @@ __device__ __forceinline__ LaneSoft2 logit_segment(const KParams& p, const char*
     tc.init();
     f32x2 nq = pack2(0.f, 0.f), nc = nq;
     bool first = true;
+    float top = -INFINITY;  // with a mask: whether the lane has a token that counts
     for (; v < v1; v += U * 32) {
       uint4 r0[U], r1[U];
 #pragma unroll
@@ -328,6 +356,10 @@ __device__ __forceinline__ LaneSoft2 logit_segment(const KParams& p, const char*
           nc = pack2(-accc.ref, -accc.ref);
           first = false;
         }
+        if (MASKED) {
+#pragma unroll
+          for (int k = 0; k < H; ++k) top = max3(top, lo2(cmb[k]), hi2(cmb[k]));
+        }
         f32x2 vq = pack2(0.f, 0.f), vc = vq;
 #pragma unroll
         for (int k = 0; k < H; ++k) {
@@ -345,8 +377,9 @@ __device__ __forceinline__ LaneSoft2 logit_segment(const KParams& p, const char*
     }
     accq.s = tq.total();
     accc.s = tc.total();
+    if (MASKED && top == -INFINITY) accc.ref = -INFINITY;  // (the sum is 0, or NaN: a token inside the mask that is no number)
   }
-  if (!(accq.s < INFINITY) || !(accc.s < INFINITY)) {  // overflow or a non-finite input: rare
+  if (!accq.holds() || !accc.holds()) {  // rare
     accq.init();
     accc.init();
     for (v = v0 + lane; v < v1; v += 32) acc = logit_online<DT>(p, base, lw.pis, lw.thr, v * Elem<DT>::E, (v + 1) * Elem<DT>::E, acc);
