@@ -76,11 +76,11 @@ enum {
   COS_RUN_EARLY_EXIT = 8,            /* a hint: positions behind a rejection that their row has already  */
                                      /* reported may be left unread (Sec. 3.1 discards them anyway).     */
                                      /* accept_count, out_tokens, row_status and bonus_prob are those of */
-                                     /* the full run; diag is NaN at a position that was left unread,    */
-                                     /* and which positions those are depends on timing.  Taken by       */
-                                     /* cos_verify_run where a warp's share of the batch is long (16 KB  */
-                                     /* of every model or more); shorter runs have every position under  */
-                                     /* way at once, and read it.                                        */
+                                     /* the full run; diag and lse are NaN at a position that was left   */
+                                     /* unread, and which positions those are depends on timing.         */
+                                     /* Taken by cos_verify_run where a warp's share of the batch is     */
+                                     /* long (16 KB of every model or more); shorter runs have every     */
+                                     /* position under way at once, and read it.                         */
   COS_RUN_INPUTS_SETTLED = 16        /* a promise by the caller: logits, draft_tokens and proposer were  */
                                      /* complete in device memory before the work that precedes this     */
                                      /* call in its stream was submitted (they are not written by the    */
@@ -149,8 +149,8 @@ typedef struct {
   float* lse;                  /* optional out [B][gamma+1][S]: the log-sum-exp ln sum_x exp(l(x) / T)  */
                                /* behind every softmax of a position (Sec. 3.1).  Ensemble: S = n, one  */
                                /* per model; logit level: S = 2, the proposer's logits and the combined */
-                               /* (masked) logits.  NaN at T = 0 and where the position is not finite.  */
-                               /* may be NULL                                                           */
+                               /* (masked) logits.  NaN at T = 0, where the position is not finite and  */
+                               /* where it was left unread (COS_RUN_EARLY_EXIT); may be NULL            */
 } cos_verify_args;
 
 typedef struct {

@@ -1120,7 +1120,9 @@ __global__ void __launch_bounds__(kStreamThreads, 1) cos_report_kernel(const __g
         if (masked) p.mask_key[uidx] = 0u;
       }
       if (skip) {
-        // some warp left it unread: the unit reports "not accepted, no candidate", which the row's scan never reaches
+        // some warp left it unread: the unit reports "not accepted, no candidate", which the row's scan never reaches, and has no
+        // statistics (the log-sum-exps are exported from them)
+        if (lane < slots) p.ustats[uidx].s[lane] = __longlong_as_double(0x7ff8000000000000LL);
         if (lane == 0) {
           const double nan = __longlong_as_double(0x7ff8000000000000LL);
           publish_unit(p, b, j, 0, 0, -1, kSample ? 0 : 0x7fc00000, nan, nan, nan, nan);

@@ -405,3 +405,30 @@ def test_offset_written_just_before_a_call_on_settled_inputs_is_seen(n):
                 assert torch.equal(outs[key], want[key]), (k, key)
     finally:
         v.close()
+
+
+@pytest.mark.parametrize("combine,weights,mask_model", [(synth.COMBINE_PROB_ENSEMBLE, (0.6, 0.4), -1), (synth.COMBINE_LOGIT_LINEAR, (1.5, -0.5), -1),
+                                                        (synth.COMBINE_LOGIT_LINEAR, (1.0, -0.5), 0)])
+def test_positions_left_unread_report_no_log_sum_exp(combine, weights, mask_model):
+    """COS_RUN_EARLY_EXIT with `lse`: NaN at a position that was left unread, never what an earlier call left behind."""
+    from paper_2502_01662_b200 import COS_RUN_EARLY_EXIT
+    w = synth.Workload("unread", 2, combine, weights, 1.0, 16, 6, 458752, "bf16", "gauss", sigma=2.5, rho=0.3, proposer_rule="cycle",
+                       mask_model=mask_model, mask_alpha=0.1 if mask_model >= 0 else 1.0)
+    inputs = synth.make_inputs(w, "cuda")
+    v = helpers.make_verifier(w, cluster_size=1)      # long shares: the hint is taken
+    try:
+        full = helpers.run_gpu(w, inputs, verifier=v, diag=True, lse=True)
+        other = dict(inputs, logits=inputs["logits"] * 0.5)
+        helpers.run_gpu(w, other, verifier=v, diag=True, lse=True)          # leaves other statistics behind
+        hint = helpers.run_gpu(w, inputs, verifier=v, diag=True, lse=True, flags=COS_RUN_EARLY_EXIT)
+    finally:
+        v.close()
+    for k in ("accept_count", "out_tokens", "row_status"):
+        assert np.array_equal(hint[k], full[k]), k
+    drafts = w.gamma
+    unread = np.isnan(hint["diag"][:, :drafts, 1]) & ~np.isnan(full["diag"][:, :drafts, 1])
+    assert unread.any()
+    assert np.all(np.isnan(hint["lse"][:, :drafts][unread]))
+    assert np.allclose(hint["lse"][:, :drafts][~unread], full["lse"][:, :drafts][~unread], rtol=1e-6, atol=0)
+    del inputs, other
+    torch.cuda.empty_cache()
