@@ -624,7 +624,8 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
       if (u.law != kDrawResidual) return;
       __syncthreads();
       if (tid == 0) {
-        if (!u.accepted) atomicOr(&p.row_status[u.b], static_cast<unsigned>(COS_ROW_RESIDUAL_EMPTY));
+        // (this thread alone, after it or an earlier launch wrote the row's status, which may lie in host memory: no atomic)
+        if (!u.accepted) p.row_status[u.b] |= static_cast<unsigned>(COS_ROW_RESIDUAL_EMPTY);
         u.law = kDrawR;
 #pragma unroll
         for (int i = 0; i < NCH; ++i)

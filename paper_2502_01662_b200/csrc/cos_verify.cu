@@ -66,7 +66,7 @@ struct cos_verify_ctx {
   int test_drop;        // test hook: one streaming warp never reports its first item
   void* d_logits;
   int* h_small;   // host-pointer runs, pinned: drafts and proposers, then the outputs
-  int* d_small;   // drafts and proposers on the device
+  int* d_small;   // the same on the device, for the launches that read them often or write the outputs with atomics
   std::string err;
 };
 
@@ -427,8 +427,8 @@ extern "C" cos_status cos_verify_create(const cos_verify_config* config, cos_ver
   if (ok && config->host_staging) {
     const size_t V = static_cast<size_t>(config->vocab);
     ok = ok && cudaMalloc(&ctx->d_logits, static_cast<size_t>(config->n) * rows * P * V * elem_bytes(config->dtype)) == cudaSuccess;
-    const size_t small = rows * 2 * P * sizeof(int);
-    ok = ok && cudaMalloc(&ctx->d_small, small) == cudaSuccess && cudaMallocHost(&ctx->h_small, small + rows * (3 + 5 * P) * sizeof(int)) == cudaSuccess;
+    const size_t small = rows * (2 * P + 3 + 5 * P) * sizeof(int);
+    ok = ok && cudaMalloc(&ctx->d_small, small) == cudaSuccess && cudaMallocHost(&ctx->h_small, small) == cudaSuccess;
   }
   if (!ok) {
     (void)cudaGetLastError();
@@ -645,9 +645,12 @@ extern "C" cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_
   const size_t ndraft = static_cast<size_t>(B * c.gamma), nprop = static_cast<size_t>((a->flags & COS_RUN_PROPOSER_PER_POSITION) ? B * P : B);
   int* out = ctx->h_small + ndraft + nprop;
   int* in = ctx->h_small;
+  // the persistent kernel adds status bits with atomics, which are for device memory: its outputs are copied
+  const bool items = ctx->fused && (ctx->use_fused || ctx->draw_fused);
+  int* written = items ? ctx->d_small + ndraft + nprop : out;
   if (ndraft) memcpy(ctx->h_small, a->draft_tokens, ndraft * sizeof(int));
   memcpy(ctx->h_small + ndraft, a->proposer, nprop * sizeof(int));
-  if (c.combine != COS_COMBINE_PROB_ENSEMBLE || (ctx->fused && (ctx->use_fused || ctx->draw_fused))) {
+  if (c.combine != COS_COMBINE_PROB_ENSEMBLE || items) {
     in = ctx->d_small;  // (every warp of the streaming launch asks for the proposer)
     e = cudaMemcpyAsync(ctx->d_small, ctx->h_small, (ndraft + nprop) * sizeof(int), cudaMemcpyHostToDevice, stream);
   }
@@ -661,11 +664,11 @@ extern "C" cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_
   d.logits = ctx->d_logits;
   d.draft_tokens = in;
   d.proposer = in + ndraft;
-  d.accept_count = out;
-  d.row_status = reinterpret_cast<unsigned*>(out + B);
-  d.bonus_prob = a->bonus_prob ? reinterpret_cast<float*>(out + 2 * B) : nullptr;
-  d.out_tokens = out + 3 * B;
-  d.diag = a->diag ? reinterpret_cast<float*>(out + 3 * B + B * P) : nullptr;
+  d.accept_count = written;
+  d.row_status = reinterpret_cast<unsigned*>(written + B);
+  d.bonus_prob = a->bonus_prob ? reinterpret_cast<float*>(written + 2 * B) : nullptr;
+  d.out_tokens = written + 3 * B;
+  d.diag = a->diag ? reinterpret_cast<float*>(written + 3 * B + B * P) : nullptr;
   if (a->offset_device) {  // a host address here, like every other pointer of this call
     d.offset = *a->offset_device;
     d.offset_device = nullptr;
@@ -675,7 +678,9 @@ extern "C" cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_
     cudaStreamSynchronize(stream);
     return st;
   }
-  e = cudaStreamSynchronize(stream);
+  if (items) e = cudaMemcpyAsync(out, written, (3 * B + B * P * (a->diag ? 5 : 1)) * sizeof(int), cudaMemcpyDeviceToHost, stream);
+  const cudaError_t waited = cudaStreamSynchronize(stream);
+  if (e == cudaSuccess) e = waited;
   if (e != cudaSuccess) {
     ctx->scratch_dirty = true;
     return cuda_fail(ctx, "waiting for the launches", e);

@@ -127,6 +127,34 @@ def test_host_pointer_entry_matches_device_entry():
         v.close()
 
 
+@pytest.mark.parametrize("n,form", [(1, 0), (2, 0), (3, 0), (5, 0), (1, 1), (2, 1), (3, 1), (1, 2), (2, 2), (3, 2)])
+def test_host_pointer_entry_with_problems_in_the_rows(n, form):
+    """Status bits that are added after a row's outputs were written (a residual without mass: identical models and a
+    bad draft) reach host memory in every form of a run."""
+    weights = {1: (1.0,), 2: (0.5, 0.5), 3: (0.5, 0.25, 0.25), 5: (0.5, 0.5, 0.0, 0.0, 0.0)}[n]   # (r cancels against q exactly)
+    w = synth.Workload("host_rows", n, synth.COMBINE_PROB_ENSEMBLE, weights, 1.0, 6, 3, 8192, "bf16", "gauss", sigma=2.0, proposer_rule="zero")
+    inputs = synth.make_inputs(w, "cuda")
+    logits, drafts = inputs["logits"].clone(), inputs["drafts"].clone()
+    logits[:, :4] = logits[0, :4].clone()
+    drafts[0, 0] = w.vocab
+    drafts[2, 1] = -1
+    logits[n - 1, 3, 2, 7] = float("nan")
+    v = helpers.make_verifier(w, host_staging=True)
+    try:
+        v.set_one_launch(form)
+        want = {k: t.cpu() for k, t in v.run(logits, drafts, inputs["proposer"], inputs["seed"], 3, diag=True).items()}
+        got = v.run_host(logits.cpu(), drafts.cpu(), inputs["proposer"].cpu(), inputs["seed"], 3, diag=True)
+    finally:
+        v.close()
+    assert got["row_status"][0] == COS_ROW_BAD_DRAFT | COS_ROW_RESIDUAL_EMPTY
+    assert got["row_status"][2] == COS_ROW_BAD_DRAFT | COS_ROW_RESIDUAL_EMPTY and got["accept_count"][2] == 1
+    assert got["row_status"][3] == COS_ROW_NONFINITE and got["accept_count"][3] == 2
+    for k in ("accept_count", "out_tokens", "row_status"):
+        assert torch.equal(got[k], want[k]), k
+    for k in ("diag", "bonus_prob"):
+        assert torch.equal(torch.nan_to_num(got[k], nan=-7.0), torch.nan_to_num(want[k], nan=-7.0)), k
+
+
 def test_data_dependent_problems_are_flagged_not_trapped():
     w = _small("cfg3", batch=6, vocab=2048, gamma=3, name="flags")
     inputs = synth.make_inputs(w, "cuda")
