@@ -36,6 +36,9 @@ EXPORTS = ("cos_verify_create", "cos_verify_run", "cos_verify_run_host", "cos_ve
            "cos_verify_run_static", "cos_verify_set_wait_limit", "cos_verify_measure_ceiling", "cos_verify_set_one_launch")
 
 
+_OUTPUTS = ("accept_count", "out_tokens", "row_status", "bonus_prob", "diag", "r", "lse")   # (a caller's dict may hold more)
+
+
 class CosVerifyError(RuntimeError):
     def __init__(self, status: int, message: str):
         super().__init__(f"{_STATUS_NAMES.get(status, status)}: {message}")
@@ -194,7 +197,7 @@ class CosVerifier:
         if _dtype_code(logits.dtype) != self._dtype:
             raise ValueError("logits dtype does not match the context")
         if ptr is None:
-            ptr = {k: t.data_ptr() for k, t in outs.items()}
+            ptr = {k: outs[k].data_ptr() for k in _OUTPUTS if k in outs}
         get = ptr.get
         return cos_verify_args(
             logits.data_ptr(), sm, sr, sp, drafts.data_ptr() if (drafts is not None and drafts.numel() > 0) else None,
