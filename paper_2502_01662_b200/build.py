@@ -28,7 +28,7 @@ def sources():
 
 
 def dependencies():
-    return sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + [os.path.join(INCLUDE, "cos_verify.h")]
+    return sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))) + [os.path.join(INCLUDE, "cos_verify.h")]
 
 
 def needs_build() -> bool:

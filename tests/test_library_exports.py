@@ -56,3 +56,10 @@ def test_binding_constants_are_the_headers():
                  "COS_RUN_INPUTS_SETTLED", "COS_ROW_FAULT", "COS_ROW_NONFINITE"):
         assert name in found and hasattr(binding, name), name
     assert checked >= 12, checked
+
+
+def test_every_header_makes_the_library_stale():
+    import os
+    from paper_2502_01662_b200 import build
+    headers = {os.path.join(build.CSRC, f) for f in os.listdir(build.CSRC) if f.endswith((".h", ".cuh"))}
+    assert headers <= set(build.dependencies())
