@@ -393,60 +393,52 @@ __device__ __forceinline__ LaneSoft2 logit_segment(const KParams& p, const char*
 
 // The argmax of the combined logits must be the fp64 one (the same chain of fused multiply-adds on every token, lowest index
 // among equals).  A vector gets its largest fp32 value and a bound on the distance of any of its fp32 values from the
-// fp64 ones, n 2^-23 sum_i |w_i| max |l_i|; only the tokens of a vector that could reach the best fp64 value seen so far are
-// evaluated in fp64.  (A bound for every token cost 5 instructions more for each logit: 564 us instead of 418 for 2304
-// positions of two 256000-token models.)
-struct BestCombined {
-  double best;
-  int idx, bad;
-  float lo;  // best rounded down
-};
-template <int DT>
-__device__ __noinline__ void consider_tokens(const KParams& p, const char* base, int e0, int count, float thr, BestCombined* b) {
-  const long long row_step = p.s_model * Elem<DT>::bytes;
-  const bool masked = p.mask_model >= 0;
-  for (int e = e0; e < e0 + count; ++e) {
-    double cm = 0.0;
-    float xe = 0.f;
-    int bad = 0;
-    for (int i = 0; i < p.n; ++i) {
-      const float x = Elem<DT>::load1(base + i * row_step, e);
-      bad |= !(x < INFINITY);
-      cm = fma(p.w64[i], static_cast<double>(x), cm);
-      if (i == p.mask_model) xe = x;
-    }
-    const bool in = !masked || xe >= thr;
-    b->bad |= bad | (in && cm != cm);
-    if (in && cm > b->best) {  // tokens come in increasing order within a lane: ties keep the earlier one
-      b->best = cm;
-      b->idx = e;
-      const float lo = __double2float_rd(cm);
-      if (lo > b->lo) b->lo = lo;
-    }
-  }
-}
-
+// fp64 ones, n 2^-23 sum_i |w_i| max |l_i|; the warp's largest value less its bound is below the maximum for certain, and
+// only vectors that could reach it are evaluated in fp64, one or two of a batch, a token a lane.  (A bound for every token
+// cost 5 instructions more for each logit: 564 us instead of 418 for 2304 positions of two 256000-token models.  Without a bound to
+// start from every first vector was evaluated, each by its lane: one row of 32000 tokens took 21.4 us on the device, with it 7.6;
+// 64 rows of 256000 with a mask 309 and 93.)
 struct ArgPart2 {
   ArgPart q, c;
 };
+__device__ __forceinline__ float warp_max(float x) {  // (floats ordered as unsigned integers; no NaN)
+  const unsigned bits = __float_as_uint(x);
+  const unsigned top = __reduce_max_sync(0xffffffffu, bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u));
+  return __uint_as_float(top ^ ((top >> 31) ? 0x80000000u : 0xffffffffu));
+}
 template <int DT, bool AL, bool PAIR, bool MASKED>
 __device__ __forceinline__ ArgPart2 logit_arg_segment(const KParams& p, const char* base, long long row_step, LogitWeights lw, int v0,
                                                    int v1, bool ragged) {
-  constexpr int U = kStreamDepth / 2, E = Elem<DT>::E, H = E / 2;
+  constexpr int U = kStreamDepth / 2, E = Elem<DT>::E, H = E / 2, G = 32 / E;
   const int lane = threadIdx.x & 31;
   const bool pair = PAIR || p.n >= 2;
   const int pis = lw.pis;
-  const float thr = lw.thr;
   const float slack = static_cast<float>(PAIR ? 2 : p.n) * 1.1920929e-07f;  // n * 2^-23
   const float wa0 = fabsf(lw.w0), wa1 = pair ? fabsf(lw.w1) : 0.f;
-  BestCombined b;
-  b.best = -INFINITY;
-  b.idx = kNoReject;
-  b.bad = 0;
-  b.lo = -INFINITY;
-  float lo = -INFINITY, qbest = -INFINITY;
+  double best = -INFINITY;
+  int idx = kNoReject, bad = 0;
+  float lo = -INFINITY, qbest = -INFINITY;  // lo: below the maximum, the same for the whole warp
   int qv = -1;
-  for (int v = v0 + lane; __any_sync(0xffffffffu, v < v1); v += U * 32) {
+  auto consider = [&](int e) {
+    double cm = 0.0;
+    float gate = 0.f;
+    const int n = PAIR ? 2 : p.n;
+#pragma unroll 2
+    for (int i = 0; i < n; ++i) {
+      const float x = Elem<DT>::load1(base + i * row_step, e);
+      bad |= !(x < INFINITY);
+      cm = fma(p.w64[i], static_cast<double>(x), cm);
+      if (MASKED && i == lw.mask_model) gate = x;
+    }
+    const bool in = !MASKED || gate >= lw.thr;
+    bad |= (in && cm != cm);
+    if (in && arg_better(cm, e, best, idx)) {
+      best = cm;
+      idx = e;
+    }
+  };
+  for (int vb = v0; vb < v1; vb += U * 32) {  // (a warp goes through the loop as one)
+    const int v = vb + lane;
     uint4 r0[U], r1[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -456,43 +448,58 @@ __device__ __forceinline__ ArgPart2 logit_arg_segment(const KParams& p, const ch
         if (pair) r1[u] = load_whole<DT, AL>(base + row_step, v + u * 32);
       }
     }
+    float hi[U], low = -INFINITY;  // no value of the vector is above hi; some value of the lane's is not below low
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int vu = v + u * 32;
-      if (vu < v1) {
-        float bound = wa0 * vector_max<DT, true>(r0[u]);
-        if (pair) bound = fmaf(wa1, vector_max<DT, true>(r1[u]), bound);
-        uint4 rq = pick_vector(pis == 0, r0[u], r1[u]);
-        f32x2 xq[H], cmb[H];
-        logit_args<DT, PAIR, MASKED>(p, lw, r0[u], r1[u],
-                                     [&](int i) {
-                                       const uint4 r = load_whole<DT, AL>(base + i * row_step, vu);
-                                       if (i == pis) rq = r;
-                                       bound = fmaf(fabsf(p.w[i]), vector_max<DT, true>(r), bound);
-                                       return r;
-                                     },
-                                     xq, cmb);
-        const float mq = vector_max<DT, false>(rq);
-        if (mq > qbest) {
-          qbest = mq;
-          qv = vu;
-        }
-        float mc = -INFINITY;
+      const bool there = vu < v1;
+      float bound = wa0 * vector_max<DT, true>(r0[u]);
+      if (pair) bound = fmaf(wa1, vector_max<DT, true>(r1[u]), bound);
+      uint4 rq = pick_vector(pis == 0, r0[u], r1[u]);
+      f32x2 xq[H], cmb[H];
+      logit_args<DT, PAIR, MASKED>(p, lw, r0[u], r1[u],
+                                   [&](int i) {
+                                     uint4 r = neg_inf_vector<DT>();
+                                     if (there) r = load_whole<DT, AL>(base + i * row_step, vu);
+                                     if (i == pis) rq = r;
+                                     bound = fmaf(fabsf(p.w[i]), vector_max<DT, true>(r), bound);
+                                     return r;
+                                   },
+                                   xq, cmb);
+      const float mq = vector_max<DT, false>(rq);
+      if (mq > qbest) {
+        qbest = mq;
+        qv = vu;
+      }
+      float mc = -INFINITY;
 #pragma unroll
-        for (int k = 0; k < H; ++k) mc = fmaxf(mc, fmaxf(lo2(cmb[k]), hi2(cmb[k])));
-        if (!(__fmaf_ru(bound, slack, mc) < lo)) {  // (a NaN or an infinity among the logits comes here too: the bound is not finite)
-          b.lo = lo;
-          consider_tokens<DT>(p, base, vu * E, E, thr, &b);
-          lo = b.lo;
+      for (int k = 0; k < H; ++k) mc = max3(mc, lo2(cmb[k]), hi2(cmb[k]));
+      const bool sound = bound < INFINITY;  // (a NaN or an infinity among the logits has to be looked at)
+      hi[u] = !there ? -INFINITY : (sound ? __fmaf_ru(bound, slack, mc) : INFINITY);
+      if (there && sound) low = fmaxf(low, __fmaf_rd(-bound, slack, mc));
+    }
+    lo = fmaxf(lo, warp_max(low));
+    unsigned reach = 0u;  // (-inf: no token of the vector counts)
+#pragma unroll
+    for (int u = 0; u < U; ++u) reach |= (hi[u] >= lo && hi[u] > -INFINITY) ? 1u << u : 0u;
+    unsigned any = __reduce_or_sync(0xffffffffu, reach);
+    if (any) {
+#pragma unroll 1
+      for (; any; any &= any - 1) {
+        const int u = __ffs(any) - 1;
+        unsigned m = __ballot_sync(0xffffffffu, (reach >> u) & 1u);
+#pragma unroll 1
+        while (m) {
+          unsigned t = m;
+#pragma unroll
+          for (int q = 0; q < G; ++q) {
+            if (q < lane / E) t &= t - 1;
+            m &= m - 1;
+          }
+          if (t) consider((vb + u * 32 + __ffs(t) - 1) * E + lane % E);
         }
       }
-      if (u == 0 || u == U - 1) {
-        // any exact value found by a lane of the warp is a lower bound of the maximum for all of them: share the
-        // largest (floats ordered as unsigned integers, one warp-wide max)
-        const unsigned bits = __float_as_uint(lo);
-        const unsigned top = __reduce_max_sync(0xffffffffu, bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u));
-        lo = fmaxf(lo, __uint_as_float(top ^ ((top >> 31) ? 0x80000000u : 0xffffffffu)));
-      }
+      lo = fmaxf(lo, warp_max(__double2float_rd(best)));
     }
   }
   int qidx = kNoReject;
@@ -505,17 +512,7 @@ __device__ __forceinline__ ArgPart2 logit_arg_segment(const KParams& p, const ch
   if (ragged) {
     const int e = ragged_entry(ragged_of<DT, AL>(p.V), p.V, lane);
     if (e >= 0) {
-      BestCombined one;
-      one.best = -INFINITY;
-      one.idx = kNoReject;
-      one.bad = 0;
-      one.lo = -INFINITY;
-      consider_tokens<DT>(p, base, e, 1, thr, &one);
-      b.bad |= one.bad;
-      if (arg_better(one.best, one.idx, b.best, b.idx)) {
-        b.best = one.best;
-        b.idx = one.idx;
-      }
+      consider(e);
       const float x = Elem<DT>::load1(base + pis * row_step, e);
       if (arg_better(x, e, qbest, qidx)) {
         qbest = x;
@@ -524,8 +521,8 @@ __device__ __forceinline__ ArgPart2 logit_arg_segment(const KParams& p, const ch
     }
   }
   ArgPart2 out;
-  out.q = warp_reduce_arg(static_cast<double>(qbest), qidx, b.bad, lane);
-  out.c = warp_reduce_arg(b.best, b.idx, b.bad, lane);
+  out.q = warp_reduce_arg(static_cast<double>(qbest), qidx, bad, lane);
+  out.c = warp_reduce_arg(best, idx, bad, lane);
   return out;
 }
 
