@@ -78,9 +78,10 @@ enum {
                                      /* accept_count, out_tokens, row_status and bonus_prob are those of */
                                      /* the full run; diag and lse are NaN at a position that was left   */
                                      /* unread, and which positions those are depends on timing.         */
-                                     /* Taken by cos_verify_run where a warp's share of the batch is     */
-                                     /* long (16 KB of every model or more); shorter runs have every     */
-                                     /* position under way at once, and read it.                         */
+                                     /* Taken by cos_verify_run where it pays: six positions and 5 MB of */
+                                     /* logits for every multiprocessor, or more (0.76 GB on a B200);    */
+                                     /* smaller runs have most positions under way at once, and read     */
+                                     /* them all.                                                        */
   COS_RUN_INPUTS_SETTLED = 16        /* a promise by the caller: logits, draft_tokens and proposer were  */
                                      /* complete in device memory before the work that precedes this     */
                                      /* call in its stream was submitted (they are not written by the    */
@@ -230,7 +231,7 @@ cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_args* args,
 #define COS_STATIC_MAX_BATCH 1024
 #define COS_STATIC_MAX_POSITIONS 8192
 #define COS_STATIC_SCRATCH_BYTES                                                                          \
-  (256 + 4 * (COS_STATIC_MAX_BATCH + 3 * COS_STATIC_MAX_POSITIONS) + 16 * COS_STATIC_MAX_POSITIONS +     \
+  (256 + 4 * COS_STATIC_MAX_POSITIONS + 16 * COS_STATIC_MAX_POSITIONS +                                  \
    16 * COS_MAX_MODELS * (COS_STATIC_MAX_POSITIONS + 5120) + 112 * COS_STATIC_MAX_POSITIONS +            \
    4 * COS_STATIC_MAX_BATCH)
 cos_status cos_verify_run_static(const cos_verify_config* config, const cos_verify_args* args, void* cuda_stream);

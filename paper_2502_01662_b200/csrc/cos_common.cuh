@@ -23,6 +23,8 @@ namespace cosv {
 constexpr int kNoReject = 0x7fffffff;
 constexpr int kPackedP = 13;  // rows of up to this many positions keep their accept flags in the arrival word
 constexpr int kDrawResidual = 0, kDrawR = 1, kDrawQ = 2;  // what a token is drawn from: max(0, r - q), r, or q
+// The streaming launch with early exit: a block's threads, the warps of it that sweep, blocks on a multiprocessor.
+constexpr int kEarlyThreads = 512, kEarlySweepers = kEarlyThreads / 32 - 1, kEarlyBlocks = 2;
 constexpr double kBigShare = 1.0 / 256.0;  // probabilities above 2^-8 get fp64 treatment when tokens are drawn
 
 enum Mode { kEnsembleSample = 0, kLogitSample = 1, kEnsembleGreedy = 2, kLogitGreedy = 3 };
@@ -66,7 +68,7 @@ struct KParams {
   float* dump_r;
   float* bonus_prob;
   // scratch owned by the context
-  unsigned* work_counter;  // (persistent kernel: cleared by a launch that only draws tokens)
+  unsigned* work_counter;  // next position to be taken, blocks that have left (early exit); zero between runs
   int* row_arrivals;       // [B], zero between runs
   int* row_reject;         // [B]: earliest rejected position published so far; kNoReject between runs
   int4* unit_res;          // [B*P]: x = accept flag, y = status bits, z = candidate token, w = a token can be drawn
@@ -75,8 +77,8 @@ struct KParams {
   UnitStats* ustats;       // [B*P]: merged statistics, where a later launch reads them
   int use_jobs;            // the list of drawing positions is kept too (tokens drawn by the persistent kernel)
   // the streaming launch: a line of st_line vectors (st_nv for each position) in st_workers shares of st_share vectors (the last may
-  // be shorter); st_slabs lines one after another (one, or one for each position of a row)
-  int st_workers, st_slabs, st_nv, st_share;
+  // be shorter)
+  int st_workers, st_nv, st_share;
   int st_split;            // ensembles: shares of a position, each model's a warp of its own; 0: a warp sweeps all models of its share
   int st_warps;            // warps of the launch
   long long st_line;

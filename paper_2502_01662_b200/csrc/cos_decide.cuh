@@ -61,7 +61,7 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
     const char* base = row + static_cast<long long>(j0 + pos) * p.s_pos * Elem<DT>::bytes;
     if (live) {
       const int j = j0 + pos;
-      range = records_of<MODE>(p, 0, p.num_units, b * p.P + j);
+      range = records_of<MODE>(p, b * p.P + j);
       if (kSample && sub == 0 && j < p.gamma) {
         at = __ldg(p.drafts + b * p.gamma + j);
         if (at >= p.V) at = -1;

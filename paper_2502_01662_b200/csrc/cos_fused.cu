@@ -1487,7 +1487,6 @@ __device__ __forceinline__ void service_role(const FParams& fp, FShared& sh) {
       fp.s.ctr[kCtrFault] = faulted ? 2u : 0u;  // 2: the scratch may be dirty; the host clears it before the next run
       if (fp.draw_only) {  // what the staged launches leave clean for the next run
         *fp.k.job_count = 0;
-        *fp.k.work_counter = 0u;
       }
       __threadfence();
     }

@@ -29,14 +29,22 @@ KernelFn logit_kernel_of(bool pair, bool masked) {
 constexpr int kLongShare = 640;
 
 template <int DT, bool AL>
-KernelFn stream_kernel_of(int mode, bool report, bool pair, bool masked, bool long_share) {
+KernelFn stream_kernel_of(int mode, bool pair, bool masked, bool long_share) {
   switch (mode) {
     case kEnsembleSample:
-      if (report) return cos_report_kernel<DT, kEnsembleSample, AL>;
       return long_share ? cos_stream_kernel<DT, kEnsembleSample, AL, true, false> : cos_stream_kernel<DT, kEnsembleSample, AL, false, false>;
-    case kEnsembleGreedy: return report ? cos_report_kernel<DT, kEnsembleGreedy, AL> : cos_stream_kernel<DT, kEnsembleGreedy, AL, true, false>;
-    case kLogitSample: return report ? cos_report_kernel<DT, kLogitSample, AL> : logit_kernel_of<DT, kLogitSample, AL>(pair, masked);
-    default: return report ? cos_report_kernel<DT, kLogitGreedy, AL> : logit_kernel_of<DT, kLogitGreedy, AL>(pair, masked);
+    case kEnsembleGreedy: return cos_stream_kernel<DT, kEnsembleGreedy, AL, true, false>;
+    case kLogitSample: return logit_kernel_of<DT, kLogitSample, AL>(pair, masked);
+    default: return logit_kernel_of<DT, kLogitGreedy, AL>(pair, masked);
+  }
+}
+template <int DT, bool AL>
+KernelFn early_kernel_of(int mode) {
+  switch (mode) {
+    case kEnsembleSample: return cos_early_kernel<DT, kEnsembleSample, AL>;
+    case kEnsembleGreedy: return cos_early_kernel<DT, kEnsembleGreedy, AL>;
+    case kLogitSample: return cos_early_kernel<DT, kLogitSample, AL>;
+    default: return cos_early_kernel<DT, kLogitGreedy, AL>;
   }
 }
 
@@ -60,12 +68,14 @@ inline cudaError_t launch(KernelFn fn, const KParams& p, int blocks, int threads
 }
 
 template <int DT>
-cudaError_t stream_launch(const KParams& p, int mode, bool report, int threads, cudaStream_t stream) {
+cudaError_t stream_launch(const KParams& p, int mode, int threads, cudaStream_t stream) {
+  if (p.early_exit) return launch(p.vec_ok ? early_kernel_of<DT, true>(mode) : early_kernel_of<DT, false>(mode), p, p.st_workers, threads, 0, stream);
   const int blocks = (p.st_warps + threads / 32 - 1) / (threads / 32);
+  if (p.use_jobs)  // (aligned rows, no mask)
+    return launch(mode == kEnsembleSample ? cos_report_kernel<DT, kEnsembleSample> : cos_report_kernel<DT, kLogitSample>, p, blocks, threads, 0, stream);
   const bool pair = p.n == 2, masked = p.mask_model >= 0, long_share = p.st_share >= kLongShare;
-  return launch(p.vec_ok ? stream_kernel_of<DT, true>(mode, report, pair, masked, long_share)
-                         : stream_kernel_of<DT, false>(mode, report, pair, masked, long_share),
-                p, blocks, threads, 0, stream);
+  return launch(p.vec_ok ? stream_kernel_of<DT, true>(mode, pair, masked, long_share) : stream_kernel_of<DT, false>(mode, pair, masked, long_share), p,
+                blocks, threads, 0, stream);
 }
 
 template <int DT>

@@ -8,12 +8,12 @@
 
 namespace cosv {
 
-// The streaming launch (mode: the Mode enum): p.st_warps warps, blocks of `threads` threads; `report`:
-// the form that also decides and publishes.  mask: the launch before it that finds the plausibility threshold of every
+// The streaming launch (mode: the Mode enum): p.st_warps warps, blocks of `threads` threads; with p.early_exit (p.st_workers blocks) or
+// p.use_jobs a form that also decides and publishes.  mask: the launch before it that finds the plausibility threshold of every
 // position.  decide: a launch after it that decides the rows (greedy runs, and
 // ensembles of one or of more than four models).
 template <int DT>
-cudaError_t stream_launch(const KParams& p, int mode, bool report, int threads, cudaStream_t stream);
+cudaError_t stream_launch(const KParams& p, int mode, int threads, cudaStream_t stream);
 template <int DT>
 cudaError_t decide_launch(const KParams& p, int mode, cudaStream_t stream);
 template <int DT>

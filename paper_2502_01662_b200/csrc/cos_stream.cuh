@@ -21,7 +21,6 @@ namespace cosv {
 // items of 8 KB as warps become free 10 (each item pays a memory round trip and a record).
 constexpr int kStreamThreads = 1024;  // most of a block: one per multiprocessor (64 registers)
 constexpr int kStreamDepth = 8;      // vectors in flight per lane
-constexpr int kSkipped = 1 << 16;    // a warp that left its part of a position unread (early exit)
 
 struct Decision {  // one position's outcome
   int accept, status, cand;
@@ -775,28 +774,24 @@ __device__ __forceinline__ double rescale(double s, float ref, float R) {
   return s * __hiloint2double((1023 + static_cast<int>(d)) << 20, 0);
 }
 
-// The records of a line: `slots` (a model each, or the proposer's and the combined logits) for every position r that share w
-// has a part of; the pairs (r, w) of a line follow one another with r + w rising.
+// The records of the line: `slots` (a model each, or the proposer's and the combined logits) for every position r that share w
+// has a part of; the pairs (r, w) follow one another with r + w rising.
 template <int MODE>
 __device__ __forceinline__ int record_slots(const KParams& p) {
   return (MODE == kEnsembleSample || MODE == kEnsembleGreedy) ? p.n : 2;
 }
-__device__ __forceinline__ size_t first_record(const KParams& p, int slab, int units, int r, int slots) {
-  return (static_cast<size_t>(slab) * (static_cast<size_t>(units) + p.st_workers) + static_cast<size_t>(r)) * slots;
-}
-
 // Where the records of position r are: `count` times `slots` of them.
 struct RecordRange {
   const int4* first;
   int count;
 };
 template <int MODE>
-__device__ __forceinline__ RecordRange records_of(const KParams& p, int slab, int units, int r) {
+__device__ __forceinline__ RecordRange records_of(const KParams& p, int r) {
   const int slots = record_slots<MODE>(p);
   const long long at = static_cast<long long>(r) * p.st_nv;
   const int w0 = worker_of(p, at), w1 = worker_of(p, at + p.st_nv - 1);
   RecordRange q;
-  q.first = p.st_rec + first_record(p, slab, units, r, slots) + static_cast<size_t>(w0) * slots;
+  q.first = p.st_rec + (static_cast<size_t>(r) + w0) * slots;
   q.count = w1 - w0 + 1;
   return q;
 }
@@ -1047,120 +1042,209 @@ __global__ void __launch_bounds__(kStreamThreads, 1) cos_stream_kernel(const __g
       if (MASKED) thr = mask_bound(p, __ldcg(&p.mask_key[r]));
     }
     sweep_part<DT, MODE, AL, PAIR, MASKED>(p, base, o0, o1, i0, i1, pis, thr,
-                                           p.st_rec + first_record(p, 0, p.num_units, r, slots) + static_cast<size_t>(share) * slots, waited);
+                                           p.st_rec + (static_cast<size_t>(r) + share) * slots, waited);
   }
 }
 
-// The same with every part reported (fence and counter): the warp that completes a position merges its records, decides and
-// publishes it at once.  Slower (see above); for runs that leave positions unread behind a rejection their row has already
-// reported, which needs the decisions while the sweep is under way (a line for each position of the rows, one after another),
-// and for those whose tokens the persistent kernel draws, which has no step that decides.
-template <int DT, int MODE, bool AL>
-__global__ void __launch_bounds__(kStreamThreads, 1) cos_report_kernel(const __grid_constant__ KParams p) {
+// Forms of the streaming launch that decide while the sweep is under way.  One warp: the position (b, j) from its records `q`.
+template <int DT, int MODE>
+__device__ __forceinline__ void decide_and_publish(const KParams& p, Finish& fin, int b, int j, RecordRange q) {
   constexpr bool kEns = (MODE == kEnsembleSample || MODE == kEnsembleGreedy);
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
+  const int lane = threadIdx.x & 31, uidx = b * p.P + j, slots = record_slots<MODE>(p);
+  const int g = slots <= 1 ? 32 : (slots <= 2 ? 16 : (slots <= 4 ? 8 : 4)), i = lane / g;
+  const bool masked = !kEns && p.mask_model >= 0;
+  const char* base = reinterpret_cast<const char*>(p.logits) +
+                     (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
+  const int pi = proposer_of(p, b, j);
+  const bool pi_ok = (pi >= 0 && pi < p.n);
+  const int pis = pi_ok ? pi : 0;
+  const bool is_bonus = (j == p.gamma);
+  const int draft = is_bonus ? 0 : __ldg(p.drafts + b * p.gamma + j);
+  const bool draft_ok = is_bonus || (draft >= 0 && draft < p.V);
+  const int at = is_bonus || !draft_ok ? -1 : draft;
+  DraftLogits d = {0.f, 0.f};
+  if (kSample && i < slots && lane % g == 0) d = draft_logits<DT, MODE>(p, base, i, pis, at);  // (asked for before the records are)
+  const float thr = masked ? mask_bound(p, __ldcg(&p.mask_key[uidx])) : -INFINITY;
+  if (i >= slots) q.count = 0;
+  const Merged m = merge_slot<MODE>(p, q, i, g, lane % g);
+  if (i < slots && lane % g == 0) {
+    if (kSample) {
+      fin.fsoft[i] = m.soft;
+      fin.pdraft[i] = draft_probability<DT, MODE>(p, d, base, i, at, thr, m.soft, 1.0 / m.soft.s);
+    } else {
+      fin.farg[i] = m.arg;
+    }
+  }
+  if (lane == 0) fin.thr = thr;
+  __syncwarp();
+  if (kSample && lane < slots) {  // kept for the drawing launch
+    p.ustats[uidx].s[lane] = fin.fsoft[lane].s;
+    p.ustats[uidx].ref[lane] = fin.fsoft[lane].ref;
+  }
+  if (kSample && lane == 31) p.ustats[uidx].thr32 = thr;
+  if (lane == 0) {
+    if (masked) p.mask_key[uidx] = 0u;  // ready for the next run
+    unsigned rnd[4];
+    philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
+    decide_unit<DT, MODE>(p, fin, fin.dec, word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), is_bonus, draft, draft_ok, pi, pi_ok, pis);
+    const Decision& e = fin.dec;
+    publish_unit(p, b, j, e.accept, e.status, e.cand, kSample ? e.drawable : __float_as_int(static_cast<float>(e.prob)), e.ratio, e.r_d,
+                 e.q_d, e.S);
+  }
+  __syncwarp();
+}
+
+// For runs whose tokens the persistent kernel draws, which has no step that decides: the shares of the ordinary form, every part of a
+// position reported (fence and counter); the warp that completes the position decides and publishes it.  Slower than deciding in
+// the next launch (see above).
+template <int DT, int MODE>
+__global__ void __launch_bounds__(kStreamThreads, 1) cos_report_kernel(const __grid_constant__ KParams p) {
+  constexpr bool kEns = (MODE == kEnsembleSample);
   __shared__ Finish fins[kStreamThreads / 32];
   const int lane = threadIdx.x & 31;
   const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  Finish& fin = fins[threadIdx.x >> 5];
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (w >= p.st_workers) return;
-  const bool masked = !kEns && p.mask_model >= 0;
-  const int units = p.st_slabs > 1 ? p.B : p.num_units;  // positions of a line
   const int slots = record_slots<MODE>(p);
-  const long long row_step = p.s_model * Elem<DT>::bytes;
   bool waited = true;
-  for (int slab = 0; slab < p.st_slabs; ++slab) {
-    for (long long x = worker_lo(p, w), end = worker_lo(p, w + 1); x < end;) {
-      const int r = line_div(x, p.st_nv, p.st_inv_nv);
-      const int o0 = static_cast<int>(x - static_cast<long long>(r) * p.st_nv);
-      const int o1 = end - x < p.st_nv - o0 ? o0 + static_cast<int>(end - x) : p.st_nv;
-      x += o1 - o0;
-      const int b = p.st_slabs > 1 ? r : r / p.P, j = p.st_slabs > 1 ? slab : r % p.P;
-      const int uidx = b * p.P + j;
-      const char* base = reinterpret_cast<const char*>(p.logits) +
-                         (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
-      const int pi = proposer_of(p, b, j);
-      const bool pi_ok = (pi >= 0 && pi < p.n);
-      const int pis = pi_ok ? pi : 0;
-      const float thr = masked ? mask_bound(p, __ldcg(&p.mask_key[uidx])) : -INFINITY;
-      // A position behind a rejection that its row has already published decides nothing (Sec. 3.1: the tokens after the
-      // first rejection are discarded).  Every warp looks for itself; one that skips marks the position.
-      bool skip = false;
-      if (p.early_exit) {
-        int rej = 0;
-        if (lane == 0) rej = *reinterpret_cast<volatile int*>(&p.row_reject[b]);
-        skip = __shfl_sync(0xffffffffu, rej, 0) < j;
-      }
-      if (!skip) {
-        int4* rec = p.st_rec + first_record(p, slab, units, r, slots) + static_cast<size_t>(w) * slots;
-        if (kEns || (p.n == 2 && !masked))
-          sweep_part<DT, MODE, AL, true, false>(p, base, o0, o1, 0, p.n, pis, thr, rec, waited);
-        else if (masked)
-          sweep_part<DT, MODE, AL, false, true>(p, base, o0, o1, 0, p.n, pis, thr, rec, waited);
-        else
-          sweep_part<DT, MODE, AL, false, false>(p, base, o0, o1, 0, p.n, pis, thr, rec, waited);
-      }
-      int prev = 0;
-      if (lane == 0) {
-        __threadfence();
-        prev = atomicAdd(&p.st_arrivals[uidx], skip ? 1 + kSkipped : 1);
-        __threadfence();
-      }
-      prev = __shfl_sync(0xffffffffu, prev, 0);
-      const long long at = static_cast<long long>(r) * p.st_nv;
-      if ((prev & (kSkipped - 1)) != worker_of(p, at + p.st_nv - 1) - worker_of(p, at)) continue;
-      skip = skip || prev >= kSkipped;
-      if (lane == 0) {
-        p.st_arrivals[uidx] = 0;  // ready for the next run
-        if (masked) p.mask_key[uidx] = 0u;
-      }
-      if (skip) {
-        // some warp left it unread: the unit reports "not accepted, no candidate", which the row's scan never reaches, and has no
-        // statistics (the log-sum-exps are exported from them)
-        if (lane < slots) p.ustats[uidx].s[lane] = __longlong_as_double(0x7ff8000000000000LL);
-        if (lane == 0) {
-          const double nan = __longlong_as_double(0x7ff8000000000000LL);
-          publish_unit(p, b, j, 0, 0, -1, kSample ? 0 : 0x7fc00000, nan, nan, nan, nan);
-        }
-        __syncwarp();
-        continue;
-      }
-      const bool is_bonus = (j == p.gamma);
-      const int draft = is_bonus ? 0 : __ldg(p.drafts + b * p.gamma + j);
-      const bool draft_ok = is_bonus || (draft >= 0 && draft < p.V);
-      const int g = slots <= 1 ? 32 : (slots <= 2 ? 16 : (slots <= 4 ? 8 : 4)), i = lane / g;
-      RecordRange q = records_of<MODE>(p, slab, units, r);
-      if (i >= slots) q.count = 0;
-      const Merged m = merge_slot<MODE>(p, q, i, g, lane % g);
-      if (i < slots && lane % g == 0) {
-        if (kSample) {
-          fin.fsoft[i] = m.soft;
-          const int at = is_bonus || !draft_ok ? -1 : draft;
-          fin.pdraft[i] = draft_probability<DT, MODE>(p, draft_logits<DT, MODE>(p, base, i, pis, at), base, i, at, thr, m.soft, 1.0 / m.soft.s);
+  for (long long x = worker_lo(p, w), end = worker_lo(p, w + 1); x < end;) {
+    const int r = line_div(x, p.st_nv, p.st_inv_nv);
+    const int o0 = static_cast<int>(x - static_cast<long long>(r) * p.st_nv);
+    const int o1 = end - x < p.st_nv - o0 ? o0 + static_cast<int>(end - x) : p.st_nv;
+    x += o1 - o0;
+    const int b = r / p.P, j = r - b * p.P;
+    const char* base = reinterpret_cast<const char*>(p.logits) +
+                       (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
+    const int pi = kEns ? 0 : proposer_of(p, b, j);
+    const int pis = (pi >= 0 && pi < p.n) ? pi : 0;
+    int4* rec = p.st_rec + (static_cast<size_t>(r) + w) * slots;
+    if (kEns || p.n == 2)
+      sweep_part<DT, MODE, true, true, false>(p, base, o0, o1, 0, p.n, pis, -INFINITY, rec, waited);
+    else
+      sweep_part<DT, MODE, true, false, false>(p, base, o0, o1, 0, p.n, pis, -INFINITY, rec, waited);
+    const RecordRange q = records_of<MODE>(p, r);
+    int prev = 0;
+    if (lane == 0) {
+      __threadfence();
+      prev = atomicAdd(&p.st_arrivals[r], 1);
+      __threadfence();
+    }
+    prev = __shfl_sync(0xffffffffu, prev, 0);
+    if (prev != q.count - 1) continue;
+    if (lane == 0) p.st_arrivals[r] = 0;  // ready for the next run
+    decide_and_publish<DT, MODE>(p, fins[threadIdx.x >> 5], b, j, q);
+  }
+}
+
+// For runs that leave positions unread behind a rejection their row has already reported.  A block takes a whole position at a time,
+// the first positions of every row before the second ones, from a counter: 15 warps sweep it in equal contiguous parts, one
+// decides and publishes the position before it and takes the next one while they do.  One barrier a position; two blocks on a
+// multiprocessor, so that one streams while the other meets.
+// What bounds it: HBM at what is read, and how much is read before a row's rejection is known (592 positions are under way at
+// once, in order).  Shares of all warps over the first positions of every row, then over the second ones, and so on, read less (0.30
+// of the positions instead of 0.48 for 256 rows of 256000 tokens), but the warps whose rows are rejected have nothing to do: whole calls
+// 437 us sampled and 281 greedy, now 293 and 166.
+__device__ __forceinline__ void early_barrier() {
+  __syncwarp();
+  asm volatile("barrier.sync 1, %0;" ::"n"(kEarlyThreads) : "memory");
+}
+
+template <int DT, int MODE, bool AL>
+__global__ void __launch_bounds__(kEarlyThreads, kEarlyBlocks) cos_early_kernel(const __grid_constant__ KParams p) {
+  constexpr bool kEns = (MODE == kEnsembleSample || MODE == kEnsembleGreedy);
+  constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
+  __shared__ Finish fin;
+  __shared__ int next[2];     // the position after the present one (by parity); num_units: none
+  __shared__ int skipped[2];  // some warp left it unread
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool masked = !kEns && p.mask_model >= 0;
+  const int slots = record_slots<MODE>(p);
+  const int parts = (p.st_nv + p.st_share - 1) / p.st_share;
+  int4* const recs = p.st_rec + static_cast<size_t>(blockIdx.x) * 2 * kEarlySweepers * slots;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (threadIdx.x == 0) {
+    next[0] = blockIdx.x;
+    skipped[0] = skipped[1] = 0;
+  }
+  __syncthreads();
+  // a position behind a rejection that its row has already published decides nothing (Sec. 3.1: the tokens after the first
+  // rejection are discarded); it reports "not accepted, no candidate", which the row's scan never reaches, and has no
+  // statistics (the log-sum-exps are exported from them)
+  auto rejected = [&](int b, int j) {
+    int rej = 0;
+    if (lane == 0) rej = *reinterpret_cast<volatile int*>(&p.row_reject[b]);
+    return __shfl_sync(0xffffffffu, rej, 0) < j;
+  };
+  auto leave = [&](int b, int j) {
+    const double nan = __longlong_as_double(0x7ff8000000000000LL);
+    if (lane < slots) p.ustats[b * p.P + j].s[lane] = nan;
+    if (lane == 0) {
+      if (masked) p.mask_key[b * p.P + j] = 0u;  // ready for the next run
+      publish_unit(p, b, j, 0, 0, -1, kSample ? 0 : 0x7fc00000, nan, nan, nan, nan);
+    }
+    __syncwarp();
+  };
+  if (warp < kEarlySweepers) {
+    bool waited = true;
+#pragma unroll 1
+    for (int k = 0;; k ^= 1) {
+      const int unit = next[k];
+      if (unit >= p.num_units) return;
+      const int j = unit / p.B, b = unit - j * p.B;
+      if (warp < parts) {
+        if (rejected(b, j)) {  // (every warp looks for itself)
+          if (lane == 0) skipped[k] = 1;
         } else {
-          fin.farg[i] = m.arg;
+          const int o0 = warp * p.st_share, o1 = o0 + p.st_share < p.st_nv ? o0 + p.st_share : p.st_nv;
+          const char* base = reinterpret_cast<const char*>(p.logits) +
+                             (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
+          const int pi = kEns ? 0 : proposer_of(p, b, j);
+          const int pis = (pi >= 0 && pi < p.n) ? pi : 0;
+          const float thr = masked ? mask_bound(p, __ldcg(&p.mask_key[b * p.P + j])) : -INFINITY;
+          int4* rec = recs + (k * kEarlySweepers + warp) * slots;
+          if (kEns || (p.n == 2 && !masked))
+            sweep_part<DT, MODE, AL, true, false>(p, base, o0, o1, 0, p.n, pis, thr, rec, waited);
+          else if (masked)
+            sweep_part<DT, MODE, AL, false, true>(p, base, o0, o1, 0, p.n, pis, thr, rec, waited);
+          else
+            sweep_part<DT, MODE, AL, false, false>(p, base, o0, o1, 0, p.n, pis, thr, rec, waited);
         }
       }
-      if (lane == 0) fin.thr = thr;
-      __syncwarp();
-      if (kSample && lane < slots) {  // kept for the drawing launch
-        p.ustats[uidx].s[lane] = fin.fsoft[lane].s;
-        p.ustats[uidx].ref[lane] = fin.fsoft[lane].ref;
-      }
-      if (kSample && lane == 31) p.ustats[uidx].thr32 = thr;
-      if (lane == 0) {
-        unsigned rnd[4];
-        philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
-        decide_unit<DT, MODE>(p, fin, fin.dec, word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), is_bonus, draft, draft_ok, pi, pi_ok, pis);
-        const Decision& d = fin.dec;
-        publish_unit(p, b, j, d.accept, d.status, d.cand, kSample ? d.drawable : __float_as_int(static_cast<float>(d.prob)), d.ratio,
-                     d.r_d, d.q_d, d.S);
-      }
-      __syncwarp();
+      early_barrier();
     }
   }
+#pragma unroll 1
+  for (int k = 0;; k ^= 1) {
+    const int unit = next[k];
+    if (unit >= p.num_units) break;
+    // the next position, while this one is swept
+    int then = p.num_units;
+#pragma unroll 1
+    for (;;) {
+      if (lane == 0) then = static_cast<int>(gridDim.x + atomicAdd(p.work_counter, 1u));
+      then = __shfl_sync(0xffffffffu, then, 0);
+      if (then >= p.num_units) break;
+      const int tj = then / p.B, tb = then - tj * p.B;
+      if (!rejected(tb, tj)) break;
+      leave(tb, tj);
+    }
+    if (lane == 0) next[k ^ 1] = then;
+    early_barrier();  // this position's records are written (and the warps go on with the next one)
+    const int j = unit / p.B, b = unit - j * p.B;
+    const bool skip = skipped[k] != 0;
+    __syncwarp();
+    if (skip) {
+      if (lane == 0) skipped[k] = 0;
+      leave(b, j);
+    } else {
+      decide_and_publish<DT, MODE>(p, fin, b, j, RecordRange{recs + k * kEarlySweepers * slots, parts});
+    }
+  }
+  // the last block to leave puts the counters back, for the next run
+  if (lane == 0 && atomicAdd(&p.work_counter[1], 1u) == gridDim.x - 1) p.work_counter[0] = p.work_counter[1] = 0u;
 }
 
 // Test hook, greedy runs: r is a handful of atoms.

@@ -218,6 +218,26 @@ int plan_line(KParams& p, const cos_verify_config& c, long long units, int model
   return p.st_warps <= 16LL * sm_count ? kStreamSmall : (p.st_warps <= 28LL * sm_count ? kStreamBlock : kStreamFull);
 }
 
+// The streaming launch with early exit (cos_early_kernel): a block a position, st_workers blocks.
+int plan_positions(KParams& p, const cos_verify_config& c, int sm_count) {
+  const int nvec = c.vocab / entries_per_vec(c.dtype), nv = p.vec_ok ? nvec : nvec - 2;
+  p.st_nv = nv < 1 ? 1 : nv;
+  p.st_share = ((p.st_nv + kEarlySweepers - 1) / kEarlySweepers + 7) / 8 * 8;
+  p.st_workers = p.num_units < kEarlyBlocks * sm_count ? p.num_units : kEarlyBlocks * sm_count;
+  return kEarlyThreads;
+}
+
+// Whether the hint to leave positions unread is taken.  It needs the decisions while the sweep is under way (cos_early_kernel, a block a
+// position), which costs 20 to 40 us more than the streaming launch and what follows it, and where a block has few
+// positions all are under way before a rejection is known.  Whole calls without and with it, in us: 256 rows of 9 positions of 2 x 128256 bf16
+// (1.2 GB) 221 and 195, 512 rows of 2 x 50001 (0.9 GB) 335 and 246, 128 rows of 3 x 128256 with a mask (0.9 GB) 284 and 251, but
+// 128 rows of 2 x 128256 (0.6 GB) 122 and 136, 512 rows of 2 x 32000 (0.6 GB) 137 and 149, and 64 rows of 7 positions of 8 x 128256 (0.9 GB,
+// one and a half positions a block) 233 and 303.
+bool early_exit_pays(const cos_verify_config& c, long long units, int sm_count) {
+  const long long blocks = static_cast<long long>(kEarlyBlocks) * sm_count;
+  return units >= 3 * blocks && units * c.n * (c.vocab / entries_per_vec(c.dtype)) >= blocks * 160000;
+}
+
 // Warps of the streaming launch: what the device holds at once, or the cluster size's worth of blocks for every position.
 long long stream_workers(const cos_verify_config& c, long long units, int sm_count) {
   const long long most = static_cast<long long>(sm_count) * 2 * (kStreamBlock / 32);
@@ -233,21 +253,19 @@ cudaError_t by_dtype(int dtype, F f) {
 }
 
 // The streaming launch, before it the one that finds the plausibility thresholds, and after it, at T = 0, the one that
-// decides.  `report`: the streaming launch decides itself (see cos_report_kernel).
-cudaError_t launch_stream(const cos_verify_config& c, int mode, KParams& p, bool report, long long workers, int sm_count, cudaStream_t stream) {
+// decides (with early exit or a job list the streaming launch decides itself).
+cudaError_t launch_stream(const cos_verify_config& c, int mode, KParams& p, long long workers, int sm_count, cudaStream_t stream) {
   return by_dtype(c.dtype, [&](auto dt) {
     constexpr int DT = decltype(dt)::value;
     cudaError_t e = cudaSuccess;
-    p.st_slabs = 1;
     if (p.mask_model >= 0) {
       const int threads = plan_line(p, c, p.num_units, 1, workers, sm_count);
       e = mask_launch<DT>(p, threads, stream);
     }
-    // early exit: position by position, so that a row's rejection is known before its later positions are begun
-    if (report && p.early_exit) p.st_slabs = p.P;
-    const bool apart = c.combine == COS_COMBINE_PROB_ENSEMBLE && !report;
-    const int threads = plan_line(p, c, p.num_units / p.st_slabs, apart ? c.n : 1, workers, sm_count);
-    if (e == cudaSuccess) e = stream_launch<DT>(p, mode, report, threads, stream);
+    const bool report = p.early_exit || p.use_jobs;
+    const int apart = c.combine == COS_COMBINE_PROB_ENSEMBLE && !report ? c.n : 1;
+    const int threads = p.early_exit ? plan_positions(p, c, sm_count) : plan_line(p, c, p.num_units, apart, workers, sm_count);
+    if (e == cudaSuccess) e = stream_launch<DT>(p, mode, threads, stream);
     p.decide = report || decides_first(c) ? 0 : 1;
     const bool first = p.greedy || decides_first(c);
     if (e == cudaSuccess && !report && first) e = decide_launch<DT>(p, mode, stream);
@@ -385,9 +403,11 @@ extern "C" cos_status cos_verify_create(const cos_verify_config* config, cos_ver
   ok = ok && cudaMalloc(&ctx->d_jobs, (rows * P + rows) * sizeof(int2)) == cudaSuccess;
   ok = ok && cudaMalloc(&ctx->d_ustats, rows * P * sizeof(UnitStats)) == cudaSuccess;
   {
-    // records of a slot for each model (logit level: two) for every position of the line and for every warp and slab
-    const size_t warps = static_cast<size_t>(ctx->sm_count) * 2 * (kStreamBlock / 32) * P;
-    const size_t recs = (rows * P + warps) * (config->combine == COS_COMBINE_PROB_ENSEMBLE ? config->n : 2);
+    // records of a slot for each model (logit level: two) for every position of the line and for every warp; with early exit two
+    // positions' worth for every block
+    const size_t line = rows * P + static_cast<size_t>(ctx->sm_count) * 2 * (kStreamBlock / 32);
+    const size_t apiece = static_cast<size_t>(ctx->sm_count) * kEarlyBlocks * 2 * kEarlySweepers;
+    const size_t recs = (line > apiece ? line : apiece) * (config->combine == COS_COMBINE_PROB_ENSEMBLE ? config->n : 2);
     ok = ok && cudaMalloc(&ctx->d_st_rec, recs * sizeof(int4)) == cudaSuccess;
   }
   ok = ok && cudaMalloc(&ctx->d_st_arrivals, rows * P * sizeof(int)) == cudaSuccess;
@@ -542,15 +562,13 @@ cos_status run_launches(cos_verify_ctx* ctx, const cos_verify_args* a, void* cud
                          : 0;
   const bool by_items = draws && !all && ctx->fused && ctx->draw_fused && p.vec_ok && a->lse == nullptr;
   p.use_jobs = by_items ? 1 : 0;
-  // Early exit needs the decisions while the sweep is under way; where a warp's part of a position is short, every position is
-  // under way at once anyway and the hint is not taken.
   const long long workers = stream_workers(c, p.num_units, ctx->sm_count);
-  if (static_cast<long long>(p.B) * c.n * (c.vocab / entries_per_vec(c.dtype)) / workers < 1024 || a->dump_r != nullptr) p.early_exit = 0;
+  if (a->dump_r != nullptr || !early_exit_pays(c, p.num_units, ctx->sm_count)) p.early_exit = 0;
   const bool report = p.early_exit || by_items;
   p.lse = report ? nullptr : a->lse;
   *lse_done = p.lse != nullptr;
   p.keep_stats = (a->dump_r != nullptr || decides_first(c)) ? 1 : 0;
-  e = launch_stream(c, mode, p, report, workers, ctx->sm_count, stream);
+  e = launch_stream(c, mode, p, workers, ctx->sm_count, stream);
   if (e != cudaSuccess) return cuda_fail(ctx, "kernel launch (streaming)", e);
   if (ctx->timing) cudaEventRecord(ctx->ev[1], stream);
   ctx->ev_used = 2;
@@ -650,8 +668,8 @@ extern "C" cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_
   int* written = items ? ctx->d_small + ndraft + nprop : out;
   if (ndraft) memcpy(ctx->h_small, a->draft_tokens, ndraft * sizeof(int));
   memcpy(ctx->h_small + ndraft, a->proposer, nprop * sizeof(int));
-  if (c.combine != COS_COMBINE_PROB_ENSEMBLE || items) {
-    in = ctx->d_small;  // (every warp of the streaming launch asks for the proposer)
+  if (c.combine != COS_COMBINE_PROB_ENSEMBLE || items || (a->flags & COS_RUN_EARLY_EXIT)) {
+    in = ctx->d_small;  // (every warp of the streaming launch asks for the proposer, or every position of the reporting one)
     e = cudaMemcpyAsync(ctx->d_small, ctx->h_small, (ndraft + nprop) * sizeof(int), cudaMemcpyHostToDevice, stream);
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_logits, a->logits, lbytes, cudaMemcpyHostToDevice, stream);
@@ -805,7 +823,7 @@ namespace {
 
 // Scratch of the context-free entry point.  It is part of the library image: every device
 // that loads the library holds these COS_STATIC_SCRATCH_BYTES until the process exits.
-// Layout: [0, 256) unused | arrival counters and mask keys | unit results | records of the streaming launch | unit
+// Layout: [0, 256) unused | mask keys | unit results | records of the streaming launch | unit
 // statistics | drawing positions.
 static __device__ __align__(256) unsigned char g_static_scratch[COS_STATIC_SCRATCH_BYTES];
 
@@ -880,15 +898,13 @@ extern "C" cos_status cos_verify_run_static(const cos_verify_config* config, con
   const bool draws = c.temperature > 0.0f;
   const bool all = draws && ((a->dump_r != nullptr) || (a->flags & COS_RUN_ALL_RESIDUALS));
   const bool masked = c.combine == COS_COMBINE_LOGIT_LINEAR && c.mask_model >= 0;
-  const size_t n_units = static_cast<size_t>(units), n_rows = static_cast<size_t>(a->batch);
+  const size_t n_units = static_cast<size_t>(units);
   unsigned char* basep = g_static_addr[c.device];
-  int* d_arrivals = reinterpret_cast<int*>(basep + 256);
-  int* d_st_arrivals = d_arrivals + n_rows;
-  unsigned* d_mask_key = reinterpret_cast<unsigned*>(d_st_arrivals + n_units);
+  unsigned* d_mask_key = reinterpret_cast<unsigned*>(basep + 256);
   // (only the mask keys have to start clean: without a mask nothing in the array is read before the launches write it)
   if (masked) e = cudaMemsetAsync(d_mask_key, 0, n_units * sizeof(unsigned), stream);
   if (e != cudaSuccess) return cuda_fail(nullptr, "clearing the built-in scratch", e);
-  int4* d_unit_res = reinterpret_cast<int4*>(basep + 256 + 4 * (COS_STATIC_MAX_BATCH + 3 * COS_STATIC_MAX_POSITIONS));
+  int4* d_unit_res = reinterpret_cast<int4*>(basep + 256 + 4 * COS_STATIC_MAX_POSITIONS);
   int4* d_st_rec = d_unit_res + COS_STATIC_MAX_POSITIONS;
   UnitStats* d_ustats = reinterpret_cast<UnitStats*>(d_st_rec + COS_MAX_MODELS * (COS_STATIC_MAX_POSITIONS + kStaticWorkers));
   static_assert(sizeof(UnitStats) == 112, "COS_STATIC_SCRATCH_BYTES assumes 112 bytes of statistics per position");
@@ -897,20 +913,18 @@ extern "C" cos_status cos_verify_run_static(const cos_verify_config* config, con
   KParams p;
   fill_params(c, a, p);
   p.num_units = static_cast<int>(units);
-  p.row_arrivals = d_arrivals;
-  p.row_reject = nullptr;  // the hint to leave positions unread is not taken here
+  // (the hint to leave positions unread is not taken here)
   p.early_exit = 0;
   p.unit_res = d_unit_res;
   p.ustats = d_ustats;
   p.st_rec = d_st_rec;
-  p.st_arrivals = d_st_arrivals;
   p.mask_key = d_mask_key;
   p.row_draw = d_row_draw;
 
   long long workers = stream_workers(c, units, sm_count);
   if (workers > kStaticWorkers) workers = kStaticWorkers;
   p.keep_stats = (a->dump_r != nullptr || decides_first(c)) ? 1 : 0;
-  e = launch_stream(c, mode_of(c), p, false, workers, sm_count, stream);
+  e = launch_stream(c, mode_of(c), p, workers, sm_count, stream);
   if (e != cudaSuccess) return cuda_fail(nullptr, "kernel launch (streaming)", e);
   if (draws) {
     e = launch_draw(c, p, all, sm_count, stream);

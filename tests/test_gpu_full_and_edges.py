@@ -284,13 +284,23 @@ def test_invalid_arguments_return_errors():
         v.close()
 
 
-@pytest.mark.parametrize("name", ["cfg3", "cfg5_greedy"])
-def test_early_exit_hint_gives_the_rows_of_the_full_run(name):
+_E, _L = synth.COMBINE_PROB_ENSEMBLE, synth.COMBINE_LOGIT_LINEAR
+_early = dict(proposer_rule="cycle", sigma=2.5, rho=0.8)
+EARLY = [C["cfg3"],                                                # not taken: every position is read
+         C["cfg3"].scaled(batch=256), C["cfg5"], C["cfg5_greedy"],
+         synth.Workload("mask", 3, _L, (1.0, -0.25, -0.25), 1.0, 128, 8, 128256, "bf16", "gauss", mask_model=2, mask_alpha=0.1, **_early),
+         synth.Workload("mask_greedy", 2, _L, (1.0, -0.5), 0.0, 256, 8, 90001, "f16", "gauss", mask_model=0, mask_alpha=0.1, **_early),
+         synth.Workload("one", 1, _E, (1.0,), 1.0, 512, 8, 90001, "bf16", "gauss", **_early),
+         synth.Workload("five", 5, _E, (0.3, 0.25, 0.2, 0.15, 0.1), 0.7, 180, 6, 40000, "f32", "gauss", **_early),
+         synth.Workload("greedy", 4, _E, (0.4, 0.3, 0.2, 0.1), 0.0, 160, 15, 50001, "bf16", "gauss", **_early)]   # long rows
+
+
+@pytest.mark.parametrize("w", EARLY, ids=lambda w: f"{w.name}-{w.batch}")
+def test_early_exit_hint_gives_the_rows_of_the_full_run(w):
     """COS_RUN_EARLY_EXIT: positions behind a rejection their row has already reported may be left unread
     (Sec. 3.1 discards them).  The rows must be those of the full run; what is reported for positions up to
     and including the first rejection must be there; some later positions are in fact left unread."""
     from paper_2502_01662_b200 import COS_RUN_EARLY_EXIT
-    w = C[name]
     inputs = synth.make_inputs(w, "cuda")
     v = helpers.make_verifier(w)
     try:
@@ -313,12 +323,15 @@ def test_early_exit_hint_gives_the_rows_of_the_full_run(name):
     for b in range(w.batch):
         for j in range(g):
             if j <= a[b]:
-                assert np.array_equal(hint["diag"][b, j, :3], full["diag"][b, j, :3], equal_nan=True), (b, j)
+                # the same sums in another order: an argument up to 64 rounds by 2^-19, which is 1.4e-6 of its exponential with
+                # the exponential's own 2^-22; r and q are quotients of two such terms (3e-6), the ratio one of theirs
+                tol = 0.0 if w.temperature == 0.0 else 6e-6
+                np.testing.assert_allclose(hint["diag"][b, j, :3], full["diag"][b, j, :3], rtol=tol, atol=0, err_msg=f"{b}, {j}")
             elif np.isnan(hint["diag"][b, j, 1]) and not np.isnan(full["diag"][b, j, 1]):
                 unread += 1
-    # workload 3 keeps every position resident at once, so nothing can be known in time there; workload 5
-    # runs in many waves and leaves positions unread
-    assert unread > 0 or name == "cfg3"
+    # large runs go through their positions in many waves and leave some unread; in smaller ones nothing can be known in time, and
+    # one model rejects nothing
+    assert (unread > 0) == (w.batch > 64 and w.n > 1), unread
     del inputs
     torch.cuda.empty_cache()
 
@@ -440,10 +453,10 @@ def test_offset_written_just_before_a_call_on_settled_inputs_is_seen(n):
 def test_positions_left_unread_report_no_log_sum_exp(combine, weights, mask_model):
     """COS_RUN_EARLY_EXIT with `lse`: NaN at a position that was left unread, never what an earlier call left behind."""
     from paper_2502_01662_b200 import COS_RUN_EARLY_EXIT
-    w = synth.Workload("unread", 2, combine, weights, 1.0, 16, 6, 458752, "bf16", "gauss", sigma=2.5, rho=0.3, proposer_rule="cycle",
-                       mask_model=mask_model, mask_alpha=0.1 if mask_model >= 0 else 1.0)
+    w = synth.Workload("unread", 2, combine, weights, 1.0, 192, 6, 143360, "bf16", "gauss", sigma=2.5, rho=0.3, proposer_rule="cycle",
+                       mask_model=mask_model, mask_alpha=0.1 if mask_model >= 0 else 1.0)     # large: the hint is taken
     inputs = synth.make_inputs(w, "cuda")
-    v = helpers.make_verifier(w, cluster_size=1)      # long shares: the hint is taken
+    v = helpers.make_verifier(w)
     try:
         full = helpers.run_gpu(w, inputs, verifier=v, diag=True, lse=True)
         other = dict(inputs, logits=inputs["logits"] * 0.5)
