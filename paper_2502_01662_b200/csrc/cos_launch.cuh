@@ -38,6 +38,11 @@ KernelFn stream_kernel_of(int mode, bool pair, bool masked, bool long_share) {
     default: return logit_kernel_of<DT, kLogitGreedy, AL>(pair, masked);
   }
 }
+template <int DT>
+KernelFn report_kernel_of(int mode, bool pair, bool long_share) {
+  if (mode == kEnsembleSample) return long_share ? cos_report_kernel<DT, kEnsembleSample, true> : cos_report_kernel<DT, kEnsembleSample, false>;
+  return pair ? cos_report_kernel<DT, kLogitSample, true> : cos_report_kernel<DT, kLogitSample, false>;
+}
 template <int DT, bool AL>
 KernelFn early_kernel_of(int mode) {
   switch (mode) {
@@ -71,9 +76,9 @@ template <int DT>
 cudaError_t stream_launch(const KParams& p, int mode, int threads, cudaStream_t stream) {
   if (p.early_exit) return launch(p.vec_ok ? early_kernel_of<DT, true>(mode) : early_kernel_of<DT, false>(mode), p, p.st_workers, threads, 0, stream);
   const int blocks = (p.st_warps + threads / 32 - 1) / (threads / 32);
-  if (p.use_jobs)  // (aligned rows, no mask)
-    return launch(mode == kEnsembleSample ? cos_report_kernel<DT, kEnsembleSample> : cos_report_kernel<DT, kLogitSample>, p, blocks, threads, 0, stream);
   const bool pair = p.n == 2, masked = p.mask_model >= 0, long_share = p.st_share >= kLongShare;
+  if (p.use_jobs)  // (aligned rows, no mask)
+    return launch(report_kernel_of<DT>(mode, pair, long_share), p, blocks, threads, 0, stream);
   return launch(p.vec_ok ? stream_kernel_of<DT, true>(mode, pair, masked, long_share) : stream_kernel_of<DT, false>(mode, pair, masked, long_share), p,
                 blocks, threads, 0, stream);
 }

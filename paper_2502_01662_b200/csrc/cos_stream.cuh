@@ -1098,7 +1098,8 @@ __device__ __forceinline__ void decide_and_publish(const KParams& p, Finish& fin
 // For runs whose tokens the persistent kernel draws, which has no step that decides: the shares of the ordinary form, every part of a
 // position reported (fence and counter); the warp that completes the position decides and publishes it.  Slower than deciding in
 // the next launch (see above).
-template <int DT, int MODE>
+// PAIR: as in cos_stream_kernel.
+template <int DT, int MODE, bool PAIR>
 __global__ void __launch_bounds__(kStreamThreads, 1) cos_report_kernel(const __grid_constant__ KParams p) {
   constexpr bool kEns = (MODE == kEnsembleSample);
   __shared__ Finish fins[kStreamThreads / 32];
@@ -1119,11 +1120,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) cos_report_kernel(const __g
                        (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
     const int pi = kEns ? 0 : proposer_of(p, b, j);
     const int pis = (pi >= 0 && pi < p.n) ? pi : 0;
-    int4* rec = p.st_rec + (static_cast<size_t>(r) + w) * slots;
-    if (kEns || p.n == 2)
-      sweep_part<DT, MODE, true, true, false>(p, base, o0, o1, 0, p.n, pis, -INFINITY, rec, waited);
-    else
-      sweep_part<DT, MODE, true, false, false>(p, base, o0, o1, 0, p.n, pis, -INFINITY, rec, waited);
+    sweep_part<DT, MODE, true, PAIR, false>(p, base, o0, o1, 0, p.n, pis, -INFINITY, p.st_rec + (static_cast<size_t>(r) + w) * slots, waited);
     const RecordRange q = records_of<MODE>(p, r);
     int prev = 0;
     if (lane == 0) {
