@@ -129,9 +129,6 @@ struct Elem<COS_DTYPE_F32> {
   static __device__ __forceinline__ float load1(const void* row, long long x) {
     return __ldg(reinterpret_cast<const float*>(row) + x);
   }
-  static __device__ __forceinline__ float pick(const uint4* vec, int k) {  // entry k of a vector in shared memory
-    return reinterpret_cast<const float*>(vec)[k];
-  }
 };
 template <>
 struct Elem<COS_DTYPE_F16> {  // IEEE half: 8 entries per 16-byte vector, widened exactly
@@ -148,9 +145,6 @@ struct Elem<COS_DTYPE_F16> {  // IEEE half: 8 entries per 16-byte vector, widene
   }
   static __device__ __forceinline__ float load1(const void* row, long long x) {
     return __half2float(__ldg(reinterpret_cast<const __half*>(row) + x));
-  }
-  static __device__ __forceinline__ float pick(const uint4* vec, int k) {  // entry k of a vector in shared memory
-    return __half2float(reinterpret_cast<const __half*>(vec)[k]);
   }
 };
 template <>
@@ -170,9 +164,6 @@ struct Elem<COS_DTYPE_BF16> {
   static __device__ __forceinline__ float load1(const void* row, long long x) {
     unsigned short h = __ldg(reinterpret_cast<const unsigned short*>(row) + x);
     return __uint_as_float(static_cast<unsigned>(h) << 16);
-  }
-  static __device__ __forceinline__ float pick(const uint4* vec, int k) {  // entry k of a vector in shared memory
-    return __uint_as_float(static_cast<unsigned>(reinterpret_cast<const unsigned short*>(vec)[k]) << 16);
   }
 };
 

@@ -23,9 +23,10 @@ KernelFn logit_kernel_of(bool pair, bool masked) {
   return masked ? cos_stream_kernel<DT, MODE, AL, false, true> : cos_stream_kernel<DT, MODE, AL, false, false>;
 }
 
-// Shares of an ensemble from this many vectors on are long (64 rows of 151936 tokens and two models, 2376 vectors: 84.6 us a call
-// with the short form, 82.8 with the long one; 32 rows of 128256 and four models, 768 vectors: 65.4 and 63.8; 32 rows of 32000
-// tokens, 288 vectors: 25.1 and 27.0).
+// Shares of an ensemble from this many vectors on are long.  Device time of a call with the short and with the long form, in us: 2376
+// vectors (64 rows of 9 positions of 2 x 151936 bf16) 84.5 and 81.8, 1625 (96 rows of 5 of 2 x 128256) 83.1 and 81.1, 1083 (64 of
+// them) 53.6 and 53.4, 758 (32 rows of 7 of 4 x 128256) 64.6 and 64.0, 507 (48 rows of 5 of 2 x 80000) 39.6 and 40.4, 288 (32 rows
+// of 6 of 2 x 32000) 25.1 and 27.0.
 constexpr int kLongShare = 640;
 
 template <int DT, bool AL>

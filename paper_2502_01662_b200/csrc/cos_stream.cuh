@@ -878,9 +878,8 @@ __device__ __forceinline__ float mask_bound(const KParams& p, unsigned key) {
   return __double2float_ru(static_cast<double>(top) + p.ln_alpha);
 }
 
-// What the probability of the draft token under slot i needs of the logits there (draft < 0: nothing), and that probability once
-// the statistics are merged, with the constant the sweep used.
-// Probability of the draft token under softmax i: what it needs of the logits (fetched early), and the rest (whose first use of them it is).
+// Probability of the draft token under softmax i, with the constant the sweep used: what it needs of the logits (fetched early; nothing
+// where draft < 0), and the rest once the statistics are merged.
 struct DraftLogits {
   float a, b;  // the slot's logit; combined logits: those of models 0 and 1
 };
@@ -1139,8 +1138,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1) cos_report_kernel(const __g
 // the first positions of every row before the second ones, from a counter: 15 warps sweep it in equal contiguous parts, one
 // decides and publishes the position before it and takes the next one while they do.  One barrier a position; two blocks on a
 // multiprocessor, so that one streams while the other meets.
-// What bounds it: HBM at what is read, and how much is read before a row's rejection is known (592 positions are under way at
-// once, in order).  Shares of all warps over the first positions of every row, then over the second ones, and so on, read less (0.30
+// What bounds it: how much is read before a row's rejection is known (592 positions are under way or next, in order), and memory latency
+// and the barrier at what is read (1344 positions of 2 x 143360: half of the nominal DRAM rate, 4.2 and 2.4 warps waiting for them).  Shares of all warps over the first positions of every row, then over the second ones, and so on, read less (0.30
 // of the positions instead of 0.48 for 256 rows of 256000 tokens), but the warps whose rows are rejected have nothing to do: whole calls
 // 437 us sampled and 281 greedy, now 293 and 166.
 __device__ __forceinline__ void early_barrier() {

@@ -9,7 +9,7 @@
 //   drawing    merge them, take the accept tests in fp64, find every row's first rejection, write the row's outputs
 //              (cos_decide.cuh; at T = 0 that is all), and draw the row's token: one more sweep of the one position that
 //              needs it (cos_draw.cuh).
-// Between blocks there are only fences and arrival counters: nothing waits for another block.
+// Blocks wait for one another only at the hardware barrier of their cluster.
 //
 // This file is the host side of the library (contexts, launches, the C entry points).  The kernels are compiled in
 // cos_bf16.cu, cos_f16.cu and cos_f32.cu; cos_common.cuh holds constants, launch parameters, loads, Philox and softmax
@@ -186,8 +186,9 @@ int plan_line(KParams& p, const cos_verify_config& c, long long units, int model
   if (nv < 1) nv = 1;                   // nothing but ragged entries
   // at least four loads for each lane; eight (all still on their way at once) where that leaves most of the device idle anyway,
   // or for one model at a time: fewer records to merge
-  // (with 768 vectors or more the loads of one model after another leave no gap to speak of, and the split is coarser: 32 rows of
-  // 128256 tokens and four models 65 us in one, 68 apart)
+  // (with many vectors a warp the loads of one model after another leave no gap to speak of, and the split is coarser: 32 rows of 7
+  // positions of 4 x 128256, 3030 vectors, 65 us in one, 68 apart; 24 rows of 5 of 4 x 48000, 608 vectors, 34.6 in one, 32.8 apart.
+  // From 768 to 1200 or so apart was the faster one too: 4 x 80000, 1013 vectors, 48.1 in one, 41.8 apart, 2 x 80000 39.7 and 37.8)
   if (units * models * nv >= 768 * workers) models = 1;
   const long long rows = units * models;
   long long most = rows * nv / 128;
