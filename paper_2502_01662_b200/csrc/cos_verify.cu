@@ -66,7 +66,7 @@ struct cos_verify_ctx {
   int test_drop;        // test hook: one streaming warp never reports its first item
   void* d_logits;
   int* h_small;   // host-pointer runs, pinned: drafts and proposers, then the outputs
-  int* d_small;   // the same on the device, for the launches that read them often or write the outputs with atomics
+  int* d_small;   // the same on the device
   std::string err;
 };
 
@@ -658,8 +658,9 @@ extern "C" cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_
   cudaError_t e = cudaSetDevice(c.device);
   if (e != cudaSuccess) return cuda_fail(ctx, "cudaSetDevice", e);
   // The small arrays go by way of pinned memory of the context (the call waits for its launches, so that memory is free again when it
-  // returns), which the kernels write directly, and read directly where only the decisions need them: copies of their own, seven of
-  // them, were half of the call for one row, and one each way still 10 us of it.
+  // returns), which the kernels write directly: copies of their own, seven of them, were half of the call for one row.  The inputs
+  // are copied together, but for one row of an ensemble, of which only the decisions read them (2 x 9 x 2000 bf16, in us, read where they are
+  // and copied: one row 49.2 and 52.7, two 54.9 and 55.5, four 58.5 and 57.3, 64 rows 140.5 and 139.3).
   const size_t lbytes = static_cast<size_t>(c.n) * B * P * V * elem_bytes(c.dtype);
   const size_t ndraft = static_cast<size_t>(B * c.gamma), nprop = static_cast<size_t>((a->flags & COS_RUN_PROPOSER_PER_POSITION) ? B * P : B);
   int* out = ctx->h_small + ndraft + nprop;
@@ -669,8 +670,8 @@ extern "C" cos_status cos_verify_run_host(cos_verify_ctx* ctx, const cos_verify_
   int* written = items ? ctx->d_small + ndraft + nprop : out;
   if (ndraft) memcpy(ctx->h_small, a->draft_tokens, ndraft * sizeof(int));
   memcpy(ctx->h_small + ndraft, a->proposer, nprop * sizeof(int));
-  if (c.combine != COS_COMBINE_PROB_ENSEMBLE || items || (a->flags & COS_RUN_EARLY_EXIT)) {
-    in = ctx->d_small;  // (every warp of the streaming launch asks for the proposer, or every position of the reporting one)
+  if (B > 1 || c.combine != COS_COMBINE_PROB_ENSEMBLE || items) {
+    in = ctx->d_small;
     e = cudaMemcpyAsync(ctx->d_small, ctx->h_small, (ndraft + nprop) * sizeof(int), cudaMemcpyHostToDevice, stream);
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_logits, a->logits, lbytes, cudaMemcpyHostToDevice, stream);

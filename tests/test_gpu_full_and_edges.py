@@ -306,12 +306,14 @@ def test_early_exit_hint_gives_the_rows_of_the_full_run(w):
     try:
         full = helpers.run_gpu(w, inputs, verifier=v, diag=True)
         hint = helpers.run_gpu(w, inputs, verifier=v, diag=True, flags=COS_RUN_EARLY_EXIT)
+        once_more = helpers.run_gpu(w, inputs, verifier=v, flags=COS_RUN_EARLY_EXIT)
         again = helpers.run_gpu(w, inputs, verifier=v, diag=True)        # the scratch was left clean
     finally:
         v.close()
     for k in ("accept_count", "out_tokens", "row_status"):
         assert np.array_equal(hint[k], full[k]), k
         assert np.array_equal(again[k], full[k]), k
+        assert np.array_equal(once_more[k], full[k]), k
     assert np.array_equal(np.isnan(hint["bonus_prob"]), np.isnan(full["bonus_prob"]))
     # and a sample of the hinted run's rows against the oracle itself
     rows = sorted(np.random.default_rng(13).choice(w.batch, size=24, replace=False).tolist())
