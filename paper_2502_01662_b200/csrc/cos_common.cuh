@@ -487,14 +487,24 @@ __device__ __forceinline__ SoftPart warp_reduce_soft(float ref, double s) {
   return o;
 }
 
-__device__ __forceinline__ void warp_merge_soft(LaneSoft a, SoftPart* dst, int lane) {
+// The sum of a warp's lanes and its reference exponent: the largest of theirs and 8, since the lanes together may hold more than 32
+// bits do.  A lane's sum may reach 127 powers of two above its own reference, so the distance between references is taken in two steps
+// (in one, a lane whose reference lay 127 below the largest was lost, whatever it held).
+__device__ __forceinline__ float warp_sum_soft(const LaneSoft& a, float& R) {
   // lanes of one warp: fp32 is enough here, the errors of the 32 scale factors average out
-  float R = a.ref;
+  R = a.ref;
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) R = fmaxf(R, __shfl_xor_sync(0xffffffffu, R, d));
-  float t = (a.ref == R) ? a.s : a.s * ex2_approx(a.ref - R);
+  const float far = fmaxf(a.ref - R, -300.f), half = floorf(0.5f * far);  // (an empty sum's reference is minus infinity)
+  float t = a.s * ex2_approx(half - 4.f) * ex2_approx(far - half - 4.f);
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+  R += 8.f;
+  return t;
+}
+__device__ __forceinline__ void warp_merge_soft(LaneSoft a, SoftPart* dst, int lane) {
+  float R;
+  const float t = warp_sum_soft(a, R);
   if (lane == 0) {
     dst->s = static_cast<double>(t);
     dst->ref = R;

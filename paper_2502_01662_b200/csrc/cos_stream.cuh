@@ -955,14 +955,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1) cos_mask_kernel(const __gri
 }
 
 __device__ __forceinline__ int4 pack_soft(const LaneSoft& a, float thr) {
-  // lanes of one warp: fp32 is enough here, the errors of the 32 scale factors average out
-  float R = a.ref;
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) R = fmaxf(R, __shfl_xor_sync(0xffffffffu, R, d));
-  float t = (a.ref == R) ? a.s : a.s * ex2_approx(a.ref - R);
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
-  const double s = static_cast<double>(t);
+  float R;
+  const double s = static_cast<double>(warp_sum_soft(a, R));
   return make_int4(__double2loint(s), __double2hiint(s), __float_as_int(R), __float_as_int(thr));
 }
 __device__ __forceinline__ int4 pack_arg(const ArgPart& a, float thr) {

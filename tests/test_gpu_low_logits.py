@@ -67,3 +67,39 @@ def test_low_logits_in_the_one_launch_forms(case, form):
         v.close()
     assert not np.any(gpu["row_status"] & COS_ROW_NONFINITE)
     helpers.check_parity(w, gpu, helpers.run_oracle(w, inputs))
+
+
+# Logits of two heights, 126 to 128 powers of two apart: as far as a 32-bit sum reaches from the reference of its first vector.
+FAR = [(combine, n, dtype, where) for combine, n in ((ENS, 1), (ENS, 2), (ENS, 3), (LOGIT, 1), (LOGIT, 2), (LOGIT, 3)) for dtype in ("f32", "bf16")
+       for where in ("scattered", "behind", "long")]
+
+
+@pytest.mark.parametrize("form", [0, 1, 2])
+@pytest.mark.parametrize("case", FAR, ids=lambda c: "-".join(str(x) for x in c))
+def test_sums_far_above_their_reference(case, form):
+    """A warp adds up lanes whose references differ by more than a 32-bit power of two can hold ("scattered": the high tokens lie in
+    the first vectors of some lanes only), and lanes whose sums together are more than 32 bits hold ("behind": one high token a
+    lane, none in a first vector)."""
+    combine, n, dtype, where = case
+    weights = {1: (1.0,), 2: (0.5, 0.5), 3: (0.5, 0.25, 0.25)}[n]
+    E, V = (4, 8192) if dtype == "f32" else (8, 16384)
+    if where == "long":
+        V = 800000
+    w = synth.Workload("far", n, combine, weights, 1.0, 2, 2, V, dtype, "gauss", proposer_rule="zero")
+    g = torch.Generator(device="cuda").manual_seed(7)
+    high = torch.zeros(V, dtype=torch.bool, device="cuda")
+    if where == "behind":
+        high[32 * E:64 * E:E] = True
+    else:
+        high = torch.rand(V, generator=g, device="cuda") < 0.02
+    logits = torch.where(high, 44.25, -44.0).to(w.torch_dtype).expand(n, 2, 3, V).clone()
+    drafts = torch.nonzero(high)[:2].flatten().to(torch.int32).repeat(2, 1)
+    inputs = {"logits": logits, "drafts": drafts, "proposer": torch.zeros(2, dtype=torch.int32, device="cuda"), "seed": 11, "offset": 3}
+    v = helpers.make_verifier(w)
+    try:
+        v.set_one_launch(form)
+        gpu = helpers.run_gpu(w, inputs, verifier=v, diag=True)
+    finally:
+        v.close()
+    assert not np.any(gpu["row_status"] & COS_ROW_NONFINITE)
+    helpers.check_parity(w, gpu, helpers.run_oracle(w, inputs, native=True))
