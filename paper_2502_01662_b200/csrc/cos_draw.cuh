@@ -90,6 +90,7 @@ struct DrawUnit {
   int accepted, drawable;
   float thr;             // plausibility threshold
   float nref[NCH], bt[NCH], ct[NCH];  // minus the reference exponents, "big" bounds, k / Z in fp32
+  double ck[NCH];                     // k / Z
 };
 
 template <bool ENS>
@@ -137,7 +138,8 @@ __device__ __forceinline__ bool load_unit(const KParams& p, int u, DrawUnit<NCH>
     const double z = live ? __ldcg(&st->s[i]) : 1.0;
     d.nref[i] = live ? -__ldcg(&st->ref[i]) : 0.f;
     d.bt[i] = live ? static_cast<float>(z * kBigShare) : INFINITY;
-    d.ct[i] = static_cast<float>(coefficient<ENS>(p, i, d.pis, d.law) / z);
+    d.ck[i] = coefficient<ENS>(p, i, d.pis, d.law) / z;
+    d.ct[i] = static_cast<float>(d.ck[i]);
   }
   return true;
 }
@@ -292,7 +294,7 @@ __device__ __noinline__ void slow_vectors(const DrawConst& p, const DrawUnit<NCH
           exact_terms<DT, ENS, NCH>(p, u, e, x, d);
           double t64 = 0.0;
 #pragma unroll
-          for (int i = 0; i < NCH; ++i) t64 += static_cast<double>(u.ct[i]) * d[i];
+          for (int i = 0; i < NCH; ++i) t64 = __dadd_rn(t64, __dmul_rn(u.ck[i], d[i]));
           counts = t64 > 0.0;
         }
 #pragma unroll
@@ -471,7 +473,7 @@ struct DrawShared {
   double inv[NCH];      // one over the normalisers
   double base, target;  // mass before the winning chunk; the running total to be reached
   float cf[NCH];        // k / Z
-  int win;              // the winning chunk; -1: nothing to draw, -2: no mass
+  int win;              // the winning chunk; -1: nothing to draw, -2: no mass, -3: the set of tokens is to be decided again
 };
 
 // The share of warp w of W; chunks without steps get sums of zero.
@@ -531,15 +533,19 @@ __device__ __forceinline__ double token_mass(const DrawConst& p, const DrawUnit<
   return big ? big_mass<DT, ENS, NCH>(p, u, inv, e) : static_cast<double>(fmaxf(0.f, tot));
 }
 
-// The whole position again by the cluster's first block, for another law.  Rare; out of line.
+// The whole position again by the cluster's first block, for another law or other coefficients.  Rare; out of line.
 template <int DT, bool ENS, int NCH, bool AL>
 __device__ __noinline__ void draw_sweep_again(const KParams& p, DrawShared<NCH>& sh, int W, double* acc) {
   for (int w = threadIdx.x >> 5; w < W; w += blockDim.x >> 5) draw_sweep<DT, ENS, NCH, AL>(p, sh, w, W, acc);
 }
 
-// The normalisers from the shares of all W warps, and the chunk that holds the token.  One warp.
+// The normalisers from the shares of all W warps, and the chunk that holds the token.  One warp.  `first_pass`: the set of tokens with a
+// positive mass was decided with the streaming launch's normalisers.  A token whose sign that got wrong counts for no more than their
+// error (1e-7, a few 1e-6 at low temperature), which matters only where the whole residual mass is below a thousand times that: there
+// the set is decided again with the refined ones (sh.win = -3).  (Where the normalisers of all channels are the same number, r is q and
+// nothing is left.)
 template <bool ENS, int NCH>
-__device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh, int W) {
+__device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh, int W, bool first_pass) {
   constexpr int G = 32 / NCH;  // lanes of a channel
   const int lane = threadIdx.x & 31, i = lane / G, live = ENS ? p.n : 2;
   const DrawUnit<NCH>& u = sh.unit;
@@ -594,6 +600,13 @@ __device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh
       }
       before += m;
     }
+  bool again = false;
+  if (first_pass && u.law == kDrawResidual) {  // (the whole warp)
+    const bool off = i < live && fabs(z * kBigShare - static_cast<double>(u.bt[i])) * 1000.0 > S * static_cast<double>(u.bt[i]);
+    const double z0 = __shfl_sync(0xffffffffu, z, 0);
+    const unsigned offs = __ballot_sync(0xffffffffu, off), unlike = __ballot_sync(0xffffffffu, i < live && z != z0);
+    again = offs != 0u && unlike != 0u;
+  }
   const unsigned hit = __ballot_sync(0xffffffffu, first >= 0), some = __ballot_sync(0xffffffffu, last >= 0);
   const int winner = hit ? __ffs(hit) - 1 : 31 - __clz(some);
   if (some != 0u ? lane == winner : lane == 0) {
@@ -601,6 +614,7 @@ __device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh
     sh.base = base;
     sh.target = target;
     if (!u.emit) sh.win = -1;
+    if (again) sh.win = -3;
     if (p.diag && u.j != p.gamma && u.law == kDrawResidual) p.diag[static_cast<long long>(u.uidx) * 4 + 3] = static_cast<float>(S);
   }
 }
@@ -614,8 +628,8 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
   DrawUnit<NCH>& u = sh.unit;
   const int cs = p.draw_cs;
 #pragma unroll 1
-  for (int pass = 0; pass < 2; ++pass) {
-    if (warp == 0) find_chunk<ENS, NCH>(p, sh, W);
+  for (int pass = 0; pass < 3; ++pass) {
+    if (warp == 0) find_chunk<ENS, NCH>(p, sh, W, pass == 0);
     __syncthreads();
     const int win = sh.win;
     if (win == -1) return;
@@ -623,13 +637,21 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
       // no residual mass although a token is needed: this block draws from r instead, over the whole position
       if (u.law != kDrawResidual) return;
       __syncthreads();
-      if (tid == 0) {
+      if (tid == 0 && win == -3) {
+#pragma unroll
+        for (int i = 0; i < NCH; ++i) {
+          u.ct[i] = sh.cf[i];
+          u.ck[i] = coefficient<ENS>(p, i, u.pis, kDrawResidual) * sh.inv[i];
+        }
+      } else if (tid == 0) {
         // (this thread alone, after it or an earlier launch wrote the row's status, which may lie in host memory: no atomic)
         if (!u.accepted) p.row_status[u.b] |= static_cast<unsigned>(COS_ROW_RESIDUAL_EMPTY);
         u.law = kDrawR;
 #pragma unroll
-        for (int i = 0; i < NCH; ++i)
-          u.ct[i] = static_cast<float>(coefficient<ENS>(p, i, u.pis, kDrawR) / (i < live ? static_cast<double>(u.bt[i]) / kBigShare : 1.0));
+        for (int i = 0; i < NCH; ++i) {
+          u.ck[i] = coefficient<ENS>(p, i, u.pis, kDrawR) * sh.inv[i];
+          u.ct[i] = static_cast<float>(u.ck[i]);
+        }
       }
       __syncthreads();
       draw_sweep_again<DT, ENS, NCH, AL>(p, sh, W, acc);
@@ -738,7 +760,8 @@ __device__ __forceinline__ bool decide_unit_to_draw(const KParams& p, DrawShared
           const bool live = tid < (ENS ? p.n : 2);
           u.nref[tid] = live ? -f.fsoft[tid].ref : 0.f;
           u.bt[tid] = live ? static_cast<float>(f.fsoft[tid].s * kBigShare) : INFINITY;
-          u.ct[tid] = live ? static_cast<float>(coefficient<ENS>(p, tid, pis, law) * f.inv[tid]) : 0.f;
+          u.ck[tid] = live ? coefficient<ENS>(p, tid, pis, law) * f.inv[tid] : 0.0;
+          u.ct[tid] = static_cast<float>(u.ck[tid]);
         }
         if (tid == 0) {
           u.b = b;

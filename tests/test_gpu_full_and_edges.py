@@ -87,6 +87,25 @@ def test_statistics_of_acceptance_match_eq7():
     assert np.all(alpha >= np.asarray(w.weights)[inputs["proposer"].cpu().numpy()][:, None] - 1e-6)   # Thm 3.2
 
 
+@pytest.mark.parametrize("combine,weights,temperature,vocab,dtype", [
+    (synth.COMBINE_PROB_ENSEMBLE, (0.16, 0.84), 0.3, 9559, "f32"), (synth.COMBINE_PROB_ENSEMBLE, (0.5, 0.3, 0.2), 0.3, 3920, "bf16"),
+    (synth.COMBINE_PROB_ENSEMBLE, (0.3, 0.25, 0.2, 0.15, 0.1), 0.3, 4096, "bf16"), (synth.COMBINE_PROB_ENSEMBLE, (0.54, 0.46), 1.0, 9, "f16"),
+    (synth.COMBINE_LOGIT_LINEAR, (1.5,), 0.3, 32, "f32"), (synth.COMBINE_LOGIT_LINEAR, (0.75, 0.75), 0.3, 18664, "f32"),
+    (synth.COMBINE_LOGIT_LINEAR, (-0.5, 1.5), 0.3, 28128, "f16")])
+def test_residual_masses_next_to_nothing(combine, weights, temperature, vocab, dtype):
+    """Distributions of one token or two: r and q agree there to 1e-6 or so, and the residual mass is what is left of
+    their difference, a few 1e-7.  To the tolerance of the parity check (1e-7 and 1e-5 of the mass)."""
+    w = synth.Workload("nothing", len(weights), combine, weights, temperature, 24, 20, vocab, dtype, "gauss", sigma=6.0, rho=0.9,
+                       proposer_rule="cycle")
+    inputs = synth.make_inputs(w, "cuda")
+    ref = helpers.run_oracle(w, inputs, native=True)
+    S = ref["S"][:, : w.gamma]
+    assert np.any((S > 2e-7) & (S < 1e-4))
+    gpu = helpers.run_gpu(w, inputs, diag=True, flags=COS_RUN_ALL_RESIDUALS)
+    got = gpu["diag"][:, : w.gamma, 3]
+    assert np.all(np.abs(got - S) <= 1e-5 * np.maximum(S, 1e-3) + 1e-7), np.max(np.abs(got - S))
+
+
 def test_row_base_and_partial_batches_and_strides():
     w = _small("cfg3", batch=6, vocab=4096, gamma=3, name="layout")
     inputs = synth.make_inputs(w, "cuda")
@@ -475,3 +494,18 @@ def test_positions_left_unread_report_no_log_sum_exp(combine, weights, mask_mode
     assert np.allclose(hint["lse"][:, :drafts][~unread], full["lse"][:, :drafts][~unread], rtol=1e-6, atol=0)
     del inputs, other
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("n,combine,weights", [(4, synth.COMBINE_PROB_ENSEMBLE, (0.41, 0.435, 0.042, 0.113)), (2, synth.COMBINE_LOGIT_LINEAR, (1.5, -0.25)),
+                                               (2, synth.COMBINE_PROB_ENSEMBLE, (0.6, 0.4))])
+def test_tokens_from_residuals_next_to_nothing(n, combine, weights):
+    """A token that has to be drawn (bad drafts) from a residual of a few 1e-7, with and without the masses of all positions."""
+    w = synth.Workload("scraps", n, combine, weights, 0.3, 64, 3, 3000, "f16", "gauss", sigma=6.0, rho=0.9, proposer_rule="cycle")
+    inputs = synth.make_inputs(w, "cuda")
+    drafts = inputs["drafts"].clone()
+    drafts[:, 0] = w.vocab
+    inputs = dict(inputs, drafts=drafts)
+    ref = helpers.run_oracle(w, inputs, native=True)
+    assert np.any((ref["S"][:, 0] > 1e-7) & (ref["S"][:, 0] < 1e-3))
+    for flags in (0, COS_RUN_ALL_RESIDUALS):
+        helpers.check_parity(w, helpers.run_gpu(w, inputs, diag=True, flags=flags), ref)
