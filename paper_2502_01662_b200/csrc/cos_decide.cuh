@@ -11,41 +11,201 @@ namespace cosv {
 // the accept test of a position, a ballot finding the first rejection.  Every block of a row does it for itself (the records of a
 // row are a few KB, read from L2), which costs the device nothing that it would use otherwise, and no word has to travel between
 // blocks; one of them writes the outputs.
-// What bounds it: a chain of latencies, and fetching instructions that no other block has run before (5 us from the end of the
-// streaming launch to the first load of the drawing sweep).  So what it needs of the inputs (drafts, proposers, the logits at the
-// drafts) is asked for before it waits for the streaming launch to end, there is one copy of everything and little is
-// unrolled: with fetches in two copies, 64-bit divisions and unrolled cold loops (35 KB instead of 20) it took 11 us.  Going
-// through it once on stale records before the wait, to have the instructions at hand, cost 4 to 8 us: the first time is the slow
-// one wherever it is.
+// What bounds it: a chain of latencies, the same the second time that a block goes through it (so not of instructions fetched for the first
+// time).  So what it needs of the inputs (drafts, proposers, the logits at the drafts, random words) is there before it waits for the
+// streaming launch to end, nothing is read from global memory after the records, the tests multiply where they could divide, and the
+// lane of the position to be drawn has all that is needed to draw it.  (With what follows in the drawing launch, device time of a call:
+// one row of 5 x 2 x 32000 fp32 14.8 us before and 12.7 now, 32 rows of 6 x 2 x 32000 bf16 25.0 and 22.6.)
 constexpr int kTile = 16;  // positions decided at a time
 
+struct PairStats {  // one softmax of a position
+  double p;    // probability of the draft token; NaN where the statistics are of no use
+  double inv;  // one over the normaliser
+  double s;
+  float ref, thr;
+};
 struct RowShared {
-  Finish fin[kTile];
-  int a;            // the row's first rejected position, or gamma; -1 until it is known
-  int drawable;     // whether a token can be drawn there
-  int cand;         // greedy: the token there
-  float prob;       // greedy: the bonus token's probability
-  unsigned status;  // status bits up to there
+  union {
+    PairStats pair[kTile][COS_MAX_MODELS];  // sampling
+    Finish fin[kTile];                      // greedy
+  };
+  int a;             // the row's first rejected position, or gamma; -1 until it is known
+  int cand;          // greedy: the token there
+  float prob;        // greedy: the bonus token's probability
+  unsigned status;   // greedy: status bits up to there
+  int draft[kTile];  // the draft tokens of the tile
 };
 
-// Decide row b.  `want` >= 0: a position whose statistics the block needs, whatever the first rejection; otherwise the first
-// rejected position is what it needs.  `keep(fin, j, word, accepted, drawable)` is called by the first warp with that position's
-// merged statistics and the random word its token is drawn with.  `writes_row(a)` / `writes_unit(j)`: whether this block writes
-// the row's outputs and a position's optional ones.
-template <int DT, int MODE, typename K, typename WR, typename WU>
-__device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int b, int want, K keep, WR writes_row, WU writes_unit) {
+// What the merge and the accept tests of a tile need of the inputs, fetched before the records are there.
+struct TileInputs {
+  RecordRange range;  // the thread's pair
+  DraftLogit d;
+  int at;             // its draft token
+  int draft, pi;      // the lane's position
+  unsigned word0, word1;
+};
+struct TilePlan {  // pairs of (position, slot) and the lanes that share one: as many as the block has to spare (a thread for each at least)
+  int lg, pos, slot, sub;
+};
+template <int MODE>
+__device__ __forceinline__ TilePlan tile_plan(const KParams& p) {
+  const int slots = record_slots<MODE>(p), pairs = (p.P < kTile ? p.P : kTile) * slots;
+  TilePlan t;
+  t.lg = 5;
+#pragma unroll 1
+  while (pairs << t.lg > blockDim.x) --t.lg;
+  const int mine = threadIdx.x >> t.lg;
+  t.sub = threadIdx.x & ((1 << t.lg) - 1);
+  t.pos = (mine * p.slot_inv) >> 16;
+  t.slot = mine - t.pos * slots;
+  return t;
+}
+template <int DT, int MODE>
+__device__ __forceinline__ TileInputs tile_inputs(const KParams& p, const TilePlan& t, int b, int j0) {
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
+  const int count = p.P - j0 < kTile ? p.P - j0 : kTile;
+  TileInputs in;
+  in.d = {0.0, 0.f};
+  in.range = {nullptr, 0};
+  in.at = -1;
+  if (t.pos < count) {
+    const int j = j0 + t.pos;
+    in.range = records_of<MODE>(p, b, j);
+    if (kSample && t.sub == 0 && j < p.gamma) {
+      in.at = __ldg(p.drafts + b * p.gamma + j);
+      if (in.at >= p.V) in.at = -1;
+      const int pi = (MODE == kLogitSample) ? proposer_of(p, b, j) : 0;
+      const char* base = reinterpret_cast<const char*>(p.logits) +
+                         (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
+      in.d = draft_logit<DT, MODE>(p, base, t.slot, (pi >= 0 && pi < p.n) ? pi : 0, in.at);
+    }
+  }
+  in.draft = in.pi = 0;
+  unsigned rnd[4] = {0u, 0u, 0u, 0u};
+  if (threadIdx.x < count) {
+    const int j = j0 + threadIdx.x;
+    if (j < p.gamma) in.draft = __ldg(p.drafts + b * p.gamma + j);
+    in.pi = proposer_of(p, b, j);
+    philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
+  }
+  in.word0 = rnd[0];
+  in.word1 = rnd[1];
+  // (all of it now, not where it is used)
+  asm volatile("" : "+r"(in.word0), "+r"(in.word1), "+l"(in.range.first), "+r"(in.range.count), "+d"(in.d.x), "+f"(in.d.gate), "+r"(in.pi), "+r"(in.draft));
+  return in;
+}
+
+// Decide row b, sampling.  `want` >= 0: a position whose statistics the block needs, whatever the first rejection; otherwise the first
+// rejected position is what it needs.  `in`: the inputs of the first tile; `ready()` waits for the records.  `keep(stats, j, proposer,
+// word, accepted, drawable)` is called by one thread of the first warp with that position's merged statistics, its proposer and the
+// random word its token is drawn with.  `writes_row(a)` / `writes_unit(j)`: whether this block writes the row's outputs and a
+// position's optional ones.
+template <int DT, int MODE, typename R, typename K, typename WR, typename WU>
+__device__ __forceinline__ void decide_sampled(const KParams& p, RowShared& sh, const TilePlan& t, TileInputs in, int b, int want, R ready, K keep,
+                                               WR writes_row, WU writes_unit) {
+  constexpr bool kEns = (MODE == kEnsembleSample);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int slots = record_slots<MODE>(p);
+  const bool optional = p.diag != nullptr || p.keep_stats || p.lse != nullptr;
+  int a = -1, drawable = 0;  // (of the first warp)
+  unsigned status = 0u;
+#pragma unroll 1
+  for (int j0 = 0; j0 < p.P; j0 += kTile) {
+    const int count = p.P - j0 < kTile ? p.P - j0 : kTile;
+    if (j0 > 0) in = tile_inputs<DT, MODE>(p, t, b, j0);
+    if (tid < count) sh.draft[tid] = in.draft;
+    if (j0 == 0) ready();
+    {
+      const Merged m = merge_slot<MODE>(p, in.range, t.slot, 1 << t.lg, t.sub);
+      if (t.pos < count && t.sub == 0) {
+        PairStats o;
+        o.s = m.soft.s;
+        o.ref = m.soft.ref;
+        o.thr = m.thr;
+        o.inv = 1.0 / m.soft.s;
+        o.p = draft_probability<MODE>(p, in.d, t.slot, in.at, m.thr, m.soft, o.inv);
+        sh.pair[t.pos][t.slot] = o;
+      }
+    }
+    __syncthreads();
+    if (tid < 32) {
+      const int j = j0 + lane;
+      const bool is_bonus = j == p.gamma, pi_ok = in.pi >= 0 && in.pi < p.n, draft_ok = is_bonus || (in.draft >= 0 && in.draft < p.V);
+      const PairStats* f = sh.pair[lane < count ? lane : 0];
+      double r_d = 0.0;
+      const double q_d = f[kEns ? (pi_ok ? in.pi : 0) : 0].p;
+      if (kEns) {
+#pragma unroll 1
+        for (int k = 0; k < p.n; ++k) r_d += p.w64[k] * f[k].p;
+      } else {
+        r_d = f[1].p;
+      }
+      const bool finite = pi_ok && r_d == r_d && q_d == q_d, tested = finite && !is_bonus && draft_ok;
+      // u <= min(1, r / q), u < 1
+      const bool accept = tested && (q_d > 0.0 ? word_to_uniform(in.word0) * q_d <= r_d : r_d > 0.0);
+      const unsigned stops = __ballot_sync(0xffffffffu, lane < count && !accept);  // (the bonus position accepts nothing)
+      const bool known = a >= 0;
+      if (!known && stops) a = j0 + __ffs(stops) - 1;
+      const int asked = want >= 0 ? want : a;
+      if (j == asked && lane < count) keep(f, j, in.pi, in.word1, accept ? 1 : 0, finite ? 1 : 0);
+      const unsigned own = !finite ? static_cast<unsigned>(COS_ROW_NONFINITE)
+                                   : (!draft_ok ? static_cast<unsigned>(COS_ROW_BAD_DRAFT)
+                                                : (tested && !(q_d > 0.0) ? static_cast<unsigned>(COS_ROW_Q_ZERO) : 0u));
+      if (!known) status |= __reduce_or_sync(0xffffffffu, lane < count && (a < 0 || j <= a) ? own : 0u);
+      if (!known && a >= 0) drawable = __shfl_sync(0xffffffffu, finite ? 1 : 0, a - j0);
+      if (lane == 0) sh.a = a;
+      if (optional && lane < count && writes_unit(j)) {
+        const int uidx = b * p.P + j;
+        if (p.diag) {
+          const float nan = __int_as_float(0x7fc00000);
+          float* o = p.diag + static_cast<long long>(uidx) * 4;
+          o[0] = !tested ? nan : (q_d > 0.0 ? static_cast<float>(r_d / q_d) : (r_d > 0.0 ? INFINITY : 0.f));
+          o[1] = tested ? static_cast<float>(r_d) : nan;
+          o[2] = tested ? static_cast<float>(q_d) : nan;
+          o[3] = nan;
+        }
+#pragma unroll 1
+        for (int k = 0; k < slots; ++k) {
+          if (p.lse) {  // ln sum_x exp(l(x) / T) = (ref + log2 s) ln 2
+            SoftPart part;
+            part.s = f[k].s;
+            part.ref = f[k].ref;
+            p.lse[static_cast<long long>(uidx) * slots + k] = log_sum_exp(part, finite);
+          }
+          if (p.keep_stats) {
+            p.ustats[uidx].s[k] = f[k].s;
+            p.ustats[uidx].ref[k] = f[k].ref;
+            p.ustats[uidx].thr32 = f[k].thr;
+          }
+        }
+        if (p.keep_stats) p.unit_res[uidx] = make_int4(accept ? 1 : 0, static_cast<int>(own), -1, finite ? 1 : 0);
+      }
+      if (!kEns && p.mask_model >= 0 && lane < count && writes_unit(j)) p.mask_key[b * p.P + j] = 0u;  // ready for the next run
+    }
+    __syncthreads();
+    const int first = sh.a;
+    if (first >= 0 && (want < 0 || want < j0 + count) && !optional && p.mask_model < 0) break;
+    if (j0 + kTile < p.P) __syncthreads();  // the tile is about to be overwritten
+  }
+  if (tid < 32 && writes_row(a)) {
+#pragma unroll 1
+    for (int k = lane; k < p.P; k += 32)
+      p.out_tokens[static_cast<long long>(b) * p.P + k] = k < a ? (p.P <= kTile ? sh.draft[k] : p.drafts[b * p.gamma + k]) : -1;
+    if (lane == 0) {
+      p.accept_count[b] = a;
+      p.row_status[b] = status;
+      if (p.bonus_prob != nullptr) p.bonus_prob[b] = __int_as_float(0x7fc00000);
+      if (p.keep_stats) p.row_draw[b] = drawable ? a : -1;
+    }
+  }
+}
+
+// The same for greedy runs, whose tokens come out of the decisions.
+template <int DT, int MODE, typename R>
+__device__ __forceinline__ void decide_greedy(const KParams& p, RowShared& sh, const TilePlan& t, TileInputs in, int b, R ready) {
   const int tid = threadIdx.x, lane = tid & 31, T = blockDim.x;
   const int slots = record_slots<MODE>(p);
   const bool optional = p.diag != nullptr || p.keep_stats || p.lse != nullptr;
-  // lanes that share a pair: as many as the block has to spare (it has a thread for each at least)
-  const int pairs = (p.P < kTile ? p.P : kTile) * slots;
-  int lg = 5;
-#pragma unroll 1
-  while (pairs << lg > T) --lg;
-  const int mine = tid >> lg, sub = tid & ((1 << lg) - 1);
-  const int pos = (mine * p.slot_inv) >> 16, i = mine - pos * slots;
-  const char* row = reinterpret_cast<const char*>(p.logits) + static_cast<long long>(b) * p.s_row * Elem<DT>::bytes;
   if (tid == 0) {
     sh.a = -1;
     sh.status = 0u;
@@ -53,90 +213,51 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
 #pragma unroll 1
   for (int j0 = 0; j0 < p.P; j0 += kTile) {
     const int count = p.P - j0 < kTile ? p.P - j0 : kTile;
-    const bool live = pos < count;
-    // what the merge and the accept test need of the inputs
-    DraftLogits d = {0.f, 0.f};
-    RecordRange range = {nullptr, 0};
-    int at = -1;  // the pair's draft token
-    const char* base = row + static_cast<long long>(j0 + pos) * p.s_pos * Elem<DT>::bytes;
-    if (live) {
-      const int j = j0 + pos;
-      range = records_of<MODE>(p, b * p.P + j);
-      if (kSample && sub == 0 && j < p.gamma) {
-        at = __ldg(p.drafts + b * p.gamma + j);
-        if (at >= p.V) at = -1;
-        const int pi = (MODE == kLogitSample) ? proposer_of(p, b, j) : 0;
-        d = draft_logits<DT, MODE>(p, base, i, (pi >= 0 && pi < p.n) ? pi : 0, at);
-      }
-    }
-    int draft = 0, pi = 0;
-    unsigned rnd[4] = {0u, 0u, 0u, 0u};
-    if (tid < count) {
-      const int j = j0 + tid;
-      if (j < p.gamma) draft = __ldg(p.drafts + b * p.gamma + j);
-      pi = proposer_of(p, b, j);
-      philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
-    }
-    if (j0 == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (j0 > 0) in = tile_inputs<DT, MODE>(p, t, b, j0);
+    if (tid < count) sh.draft[tid] = in.draft;
+    if (j0 == 0) ready();
     {
-      const Merged m = merge_slot<MODE>(p, range, i, 1 << lg, sub);
-      if (live && sub == 0) {
-        Finish& f = sh.fin[pos];
-        if (kSample) {
-          f.fsoft[i] = m.soft;
-          f.inv[i] = 1.0 / m.soft.s;
-          f.pdraft[i] = draft_probability<DT, MODE>(p, d, base, i, at, m.thr, m.soft, f.inv[i]);
-        } else {
-          f.farg[i] = m.arg;
-        }
-        if (i == slots - 1) f.thr = m.thr;
+      const Merged m = merge_slot<MODE>(p, in.range, t.slot, 1 << t.lg, t.sub);
+      if (t.pos < count && t.sub == 0) {
+        Finish& f = sh.fin[t.pos];
+        f.farg[t.slot] = m.arg;
+        if (t.slot == slots - 1) f.thr = m.thr;
       }
     }
     __syncthreads();
     if (tid < 32) {
-      // (sampling: the decision stays in registers but where somebody asked to see it)
-      Decision own;
-      own.accept = own.status = own.drawable = 0;
-      Decision& dec = kSample || lane >= count ? own : sh.fin[lane].dec;
+      Decision& dec = sh.fin[lane < count ? lane : 0].dec;
+      int accept = 0;
+      unsigned own = 0u;
       if (lane < count) {
         const bool is_bonus = (j0 + lane == p.gamma);
-        const bool draft_ok = is_bonus || (draft >= 0 && draft < p.V);
-        const bool pi_ok = (pi >= 0 && pi < p.n);
-        decide_unit<DT, MODE>(p, sh.fin[lane], dec, word_to_uniform(rnd[0]), word_to_uniform(rnd[1]), is_bonus, draft, draft_ok, pi, pi_ok,
-                              pi_ok ? pi : 0);
-        if (kSample && optional) sh.fin[lane].dec = dec;
+        const bool draft_ok = is_bonus || (in.draft >= 0 && in.draft < p.V);
+        const bool pi_ok = (in.pi >= 0 && in.pi < p.n);
+        decide_unit<DT, MODE>(p, sh.fin[lane], dec, word_to_uniform(in.word0), word_to_uniform(in.word1), is_bonus, in.draft, draft_ok, in.pi, pi_ok,
+                              pi_ok ? in.pi : 0);
+        accept = dec.accept;
+        own = static_cast<unsigned>(dec.status);
       }
-      int a = sh.a;
+      const int a = sh.a;
       __syncwarp();
       if (a < 0) {
-        const unsigned stops = __ballot_sync(0xffffffffu, lane < count && (!dec.accept || j0 + lane == p.gamma));
+        const unsigned stops = __ballot_sync(0xffffffffu, lane < count && (!accept || j0 + lane == p.gamma));
         const int k = stops ? __ffs(stops) - 1 : count - 1;
-        const unsigned st = __reduce_or_sync(0xffffffffu, lane <= k && lane < count ? static_cast<unsigned>(dec.status) : 0u);
-        if (stops) a = j0 + k;
+        const unsigned st = __reduce_or_sync(0xffffffffu, lane <= k && lane < count ? own : 0u);
         if (lane == k) {
           sh.status |= st;
-          sh.a = a;
-          sh.drawable = dec.drawable;
-          if (!kSample) {
-            sh.cand = dec.cand;
-            sh.prob = static_cast<float>(dec.prob);
-          }
+          sh.a = stops ? j0 + k : -1;
+          sh.cand = dec.cand;
+          sh.prob = static_cast<float>(dec.prob);
         }
       }
-      const int asked = want >= 0 ? want : a;
-      const int k = asked >= j0 && asked < j0 + count ? asked - j0 : 0;
-      const int accepted = __shfl_sync(0xffffffffu, dec.accept, k), drawable = __shfl_sync(0xffffffffu, dec.drawable, k);
-      const unsigned word = __shfl_sync(0xffffffffu, rnd[1], k);
-      if (asked >= j0 && asked < j0 + count) keep(sh.fin[k], asked, word, accepted, drawable);
     }
     __syncthreads();
     const int a = sh.a;
-    const int asked = want >= 0 ? want : a;
     if (optional) {
 #pragma unroll 1
       for (int k = tid; k < count; k += T) {
-        const int j = j0 + k, uidx = b * p.P + j;
-        if (!writes_unit(j)) continue;
+        const int uidx = b * p.P + j0 + k;
         const Finish& f = sh.fin[k];
         if (p.diag) {
           float* d = p.diag + static_cast<long long>(uidx) * 4;
@@ -145,51 +266,37 @@ __device__ __forceinline__ void decide_row(const KParams& p, RowShared& sh, int 
           d[2] = static_cast<float>(f.dec.q_d);
           d[3] = static_cast<float>(f.dec.S);
         }
-        if (p.lse) {  // ln sum_x exp(l(x) / T) = (ref + log2 s) ln 2
+        if (p.lse) {
 #pragma unroll 1
-          for (int i = 0; i < slots; ++i)
-            p.lse[static_cast<long long>(uidx) * slots + i] = log_sum_exp(f.fsoft[i], kSample && !(f.dec.status & COS_ROW_NONFINITE));
+          for (int i = 0; i < slots; ++i) p.lse[static_cast<long long>(uidx) * slots + i] = __int_as_float(0x7fc00000);
         }
-        if (p.keep_stats) {
+        if (p.keep_stats) {  // the atoms of r, for the test hook
           UnitStats& st = p.ustats[uidx];
-          if (kSample) {
+          st.pad[0] = (f.dec.status & COS_ROW_NONFINITE) ? -1 : f.dec.natoms;
 #pragma unroll 1
-            for (int i = 0; i < slots; ++i) {
-              st.s[i] = f.fsoft[i].s;
-              st.ref[i] = f.fsoft[i].ref;
-            }
-            st.thr32 = f.thr;
-          } else {  // the atoms of r, for the test hook
-            st.pad[0] = (f.dec.status & COS_ROW_NONFINITE) ? -1 : f.dec.natoms;
-#pragma unroll 1
-            for (int i = 0; i < f.dec.natoms; ++i) {
-              st.s[i] = f.dec.atom_mass[i];
-              st.ref[i] = __int_as_float(f.dec.atom_tok[i]);
-            }
+          for (int i = 0; i < f.dec.natoms; ++i) {
+            st.s[i] = f.dec.atom_mass[i];
+            st.ref[i] = __int_as_float(f.dec.atom_tok[i]);
           }
           p.unit_res[uidx] = make_int4(f.dec.accept, f.dec.status, f.dec.cand, f.dec.drawable);
         }
       }
     }
-    if (MODE == kLogitSample || MODE == kLogitGreedy) {
+    if (MODE == kLogitGreedy) {
 #pragma unroll 1
-      for (int k = p.mask_model >= 0 ? tid : count; k < count; k += T)
-        if (writes_unit(j0 + k)) p.mask_key[b * p.P + j0 + k] = 0u;  // ready for the next run
+      for (int k = p.mask_model >= 0 ? tid : count; k < count; k += T) p.mask_key[b * p.P + j0 + k] = 0u;  // ready for the next run
     }
-    if (a >= 0 && asked < j0 + count && !optional && p.mask_model < 0) break;
+    if (a >= 0 && !optional && p.mask_model < 0) break;
     __syncthreads();  // the tile is about to be overwritten
   }
   const int a = sh.a;
-  if (writes_row(a)) {
 #pragma unroll 1
-    for (int k = tid; k < p.P; k += T)
-      p.out_tokens[static_cast<long long>(b) * p.P + k] = k < a ? p.drafts[b * p.gamma + k] : (k == a && !kSample ? sh.cand : -1);
-    if (tid == 0) {
-      p.accept_count[b] = a;
-      p.row_status[b] = sh.status;
-      if (p.bonus_prob != nullptr) p.bonus_prob[b] = (!kSample && a == p.gamma && sh.cand >= 0) ? sh.prob : __int_as_float(0x7fc00000);
-      if (kSample && p.keep_stats) p.row_draw[b] = sh.drawable ? a : -1;
-    }
+  for (int k = tid; k < p.P; k += T)
+    p.out_tokens[static_cast<long long>(b) * p.P + k] = k < a ? (p.P <= kTile ? sh.draft[k] : p.drafts[b * p.gamma + k]) : (k == a ? sh.cand : -1);
+  if (tid == 0) {
+    p.accept_count[b] = a;
+    p.row_status[b] = sh.status;
+    if (p.bonus_prob != nullptr) p.bonus_prob[b] = (a == p.gamma && sh.cand >= 0) ? sh.prob : __int_as_float(0x7fc00000);
   }
 }
 
@@ -199,7 +306,14 @@ template <int DT, int MODE>
 __global__ void __launch_bounds__(128) cos_decide_kernel(const __grid_constant__ KParams p) {
   __shared__ RowShared sh;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  decide_row<DT, MODE>(p, sh, blockIdx.x, -1, [](const Finish&, int, unsigned, int, int) {}, [](int) { return true; }, [](int) { return true; });
+  const TilePlan t = tile_plan<MODE>(p);
+  const TileInputs in = tile_inputs<DT, MODE>(p, t, blockIdx.x, 0);
+  auto ready = [] { asm volatile("griddepcontrol.wait;" ::: "memory"); };
+  if (MODE == kEnsembleSample)
+    decide_sampled<DT, MODE>(p, sh, t, in, blockIdx.x, -1, ready, [](const PairStats*, int, int, unsigned, int, int) {}, [](int) { return true; },
+                             [](int) { return true; });
+  else
+    decide_greedy<DT, MODE>(p, sh, t, in, blockIdx.x, ready);
 }
 
 }  // namespace cosv

@@ -18,10 +18,10 @@ namespace cosv {
 // the shared memory of the cluster's first block, nothing per step.  After one barrier of the cluster that block alone
 // adds the records up, finds the chunk that holds the token, then the step, then the token.  The host picks block size and parts so
 // that the launch fills the device in one wave (see draw_plan).
-// The part behind the sweep is a chain of latencies, issue slots and instruction fetches (counted on one row of 151936 tokens: most
-// stalls are for instructions), so what can be done by one warp is, and nothing is unrolled that need not be.
-// Measured (64 rows of 2 x 151936 tokens): 9 us of sweep, 3 until the cluster's last warp is done, 6 to find the token.  Records in
-// global memory and the last block to report (fence and counter) took 5 us longer; two more barriers of the cluster, for all
+// The part behind the sweep is a chain of latencies: bank conflicts, loops that need not be loops and second trips to memory for what is in
+// registers are what it can do without (cycles in one row of 5 x 2 x 32000 fp32: chunk 3900 with conflicts and serial searches, 2500
+// without; the steps' masses 4000, entries and exponentials of big tokens fetched again; token 1000 to 2000 with a load of its entries).
+// Records in global memory and the last block to report (fence and counter) took 5 us longer; two more barriers of the cluster, for all
 // blocks to look for the token, 1.
 constexpr int kMaxDrawThreads = 512;
 constexpr int kMaxDrawWarps = kMaxDrawThreads / 32;
@@ -69,6 +69,21 @@ __device__ __forceinline__ double warp_sums(double (&v)[N], int lane) {
   return v[0];
 }
 
+// Where the sums of chunk c are among the records: a record is left out after every eight, so that lanes that each go through a few
+// consecutive chunks read from different banks (without, all 32 from the same two: 2.4 of the 6.1 thousand cycles of the search in 512).
+__device__ __forceinline__ int record_at(int c) { return c + (c >> 3); }
+
+// Running total over the lanes of a warp (the first N of them are asked for).  Unrolled: 220 cycles for 32 lanes, in a loop 480.
+template <int N>
+__device__ __forceinline__ double running_total(double m, int lane) {
+#pragma unroll
+  for (int d = 1; d < N; d <<= 1) {
+    const double o = __shfl_up_sync(0xffffffffu, m, d);
+    if (lane >= d) m += o;
+  }
+  return m;
+}
+
 // What the functions that are not inlined need of the parameters, in shared memory: behind a call the parameters are no longer
 // operands from the constant bank but loads through a generic address, a trip to L2 for each line of them the first time.
 struct DrawConst {
@@ -77,6 +92,22 @@ struct DrawConst {
   float cT, w[COS_MAX_MODELS];
   int n, V, mask_model;
 };
+
+template <int DT>
+__device__ __forceinline__ void fill_const(const KParams& p, DrawConst& kc) {
+  if (threadIdx.x < COS_MAX_MODELS) {
+    kc.w[threadIdx.x] = p.w[threadIdx.x];
+    kc.w64[threadIdx.x] = p.w64[threadIdx.x];
+    if (threadIdx.x == 0) {
+      kc.row_step = p.s_model * Elem<DT>::bytes;
+      kc.cT64 = p.cT64;
+      kc.cT = p.cT;
+      kc.n = p.n;
+      kc.V = p.V;
+      kc.mask_model = p.mask_model;
+    }
+  }
+}
 
 // What a block knows about its position.
 template <int NCH>
@@ -144,54 +175,55 @@ __device__ __forceinline__ bool load_unit(const KParams& p, int u, DrawUnit<NCH>
   return true;
 }
 
-// The arguments of the channels for one token.
-template <int DT, bool ENS, int NCH>
-__device__ __forceinline__ void entry_args(const DrawConst& p, const DrawUnit<NCH>& u, int e, float (&x)[NCH]) {
-  if (ENS) {
-#pragma unroll
-    for (int i = 0; i < NCH; ++i) {
-      x[i] = -INFINITY;
-      if (i < p.n) x[i] = Elem<DT>::load1(u.base + i * p.row_step, e);
-    }
-  } else {
-    const float l0 = Elem<DT>::load1(u.base, e);
-    float l1 = 0.f, gate = l0;
-    if (p.n >= 2) l1 = Elem<DT>::load1(u.base + p.row_step, e);
-    x[0] = u.pis == 0 ? l0 : l1;
-    if (p.mask_model == 1) gate = l1;
-    x[1] = __fmul_rn(p.w[0], l0);
-    if (p.n >= 2) x[1] = fmaf(p.w[1], l1, x[1]);
-    for (int i = 2; i < p.n; ++i) {
-      const float l = Elem<DT>::load1(u.base + i * p.row_step, e);
-      if (i == u.pis) x[0] = l;
-      if (i == p.mask_model) gate = l;
-      x[1] = fmaf(p.w[i], l, x[1]);
-    }
-    if (p.mask_model >= 0 && !(gate >= u.thr)) x[1] = -INFINITY;
-  }
+// A vector of every model (logit level: of the first two).
+template <int N>
+struct Vectors {
+  uint4 r[N];
+};
+// One entry of a vector, any of them.
+template <int DT>
+__device__ __forceinline__ float entry_at(const uint4& r, int k) {
+  const int w = DT == COS_DTYPE_F32 ? k : k >> 1;
+  const unsigned a = (w & 1) ? r.y : r.x, b = (w & 1) ? r.w : r.z, h = (w & 2) ? b : a;
+  if (DT == COS_DTYPE_F32) return __uint_as_float(h);
+  return entry<DT>(make_uint4((k & 1) ? h >> 16 : h, 0u, 0u, 0u), 0);
 }
 
-// fp64 terms of one token (its arguments: x): e_i of every channel.  For "big" tokens (more than 2^-8 of a normaliser) and the
-// bonus token's probability.
-template <int DT, bool ENS, int NCH>
-__device__ __forceinline__ void exact_terms(const DrawConst& p, const DrawUnit<NCH>& u, int e, const float (&x)[NCH], double (&out)[NCH]) {
+// fp64 terms of token e, the k-th of the vectors: e_i of every channel (in: whether the token is inside the mask).  For "big" tokens (more
+// than 2^-8 of a normaliser) and the bonus token's probability.
+template <int DT, bool ENS, int NCH, int FORM>
+__device__ __forceinline__ void exact_terms(const DrawConst& p, const DrawUnit<NCH>& u, const Vectors<ENS ? NCH : 2>& v, int e, int k, bool in,
+                                            double (&out)[NCH]) {
   double t[NCH];
+  if (ENS) {
 #pragma unroll
-  for (int i = 0; i < NCH; ++i) t[i] = static_cast<double>(x[i]);
-  if (!ENS && !(x[1] == -INFINITY)) {  // (the combination again, in fp64)
-    t[1] = 0.0;
-    for (int i = 0; i < p.n; ++i) t[1] = fma(p.w64[i], static_cast<double>(Elem<DT>::load1(u.base + i * p.row_step, e)), t[1]);
-  }
+    for (int i = 0; i < NCH; ++i) t[i] = static_cast<double>(entry_at<DT>(v.r[i], k));
+  } else {
+    const float l0 = entry_at<DT>(v.r[0], k), l1 = entry_at<DT>(v.r[1], k);
+    float q = u.pis == 0 ? l0 : l1;
+    t[1] = p.w64[0] * static_cast<double>(l0);
+    if ((FORM & 1) || p.n >= 2) t[1] = fma(p.w64[1], static_cast<double>(l1), t[1]);
+    if (!(FORM & 1)) {
 #pragma unroll 1
-  for (int k = 0; k < NCH; ++k) {  // (one copy of the exponential)
-    double v = 0.0;
+      for (int i = 2; i < p.n; ++i) {
+        const float l = Elem<DT>::load1(u.base + i * p.row_step, e);
+        if (i == u.pis) q = l;
+        t[1] = fma(p.w64[i], static_cast<double>(l), t[1]);
+      }
+    }
+    t[0] = static_cast<double>(q);
+    if (!in) t[1] = -INFINITY;
+  }
+#pragma unroll(NCH == 2 ? 2 : 1)
+  for (int k2 = 0; k2 < NCH; ++k2) {  // (more than two channels: one copy of the exponential)
+    double x = 0.0;
 #pragma unroll
     for (int i = 0; i < NCH; ++i)
-      if (i == k) v = t[i] * p.cT64 + static_cast<double>(u.nref[i]);
-    v = exp2(v);
+      if (i == k2) x = t[i] * p.cT64 + static_cast<double>(u.nref[i]);
+    x = exp2(x);
 #pragma unroll
     for (int i = 0; i < NCH; ++i)
-      if (i == k) out[i] = v;
+      if (i == k2) out[i] = x;
   }
 }
 
@@ -215,109 +247,112 @@ __device__ __forceinline__ double exact_mass(const DrawConst& p, const double* e
   return law == kDrawR ? r : (law == kDrawQ ? q : fmax(0.0, r - q));
 }
 
-// The arguments of the NCH channels for the E tokens of vector v (any vector of the row; -inf beyond V), one lane.
-template <int DT, bool ENS, int NCH, bool AL>
-__device__ __forceinline__ void vector_args(const KParams& p, const DrawUnit<NCH>& u, int v, float (&x)[NCH][Elem<DT>::E]) {
+// The arguments of the NCH channels for the E tokens of vector v of the row from the vectors of the models; beyond V they are -inf.
+template <int DT, bool ENS, int NCH, bool AL, int FORM>
+__device__ __forceinline__ void vector_args(const KParams& p, const DrawConst& kc, const DrawUnit<NCH>& u, const Vectors<ENS ? NCH : 2>& rv, int v,
+                                            float (&x)[NCH][Elem<DT>::E]) {
   constexpr int E = Elem<DT>::E;
-  const VecRange whole = whole_vectors<DT, AL>(p.V);
-  const long long row_step = p.s_model * Elem<DT>::bytes;
   if (ENS) {
 #pragma unroll
-    for (int i = 0; i < NCH; ++i) {
-      uint4 r = neg_inf_vector<DT>();
-      if (i < p.n) r = load_vector<DT, AL>(u.base + i * row_step, v, p.V, whole);
+    for (int i = 0; i < NCH; ++i)
 #pragma unroll
-      for (int k = 0; k < E; ++k) x[i][k] = entry<DT>(r, k);
-    }
+      for (int k = 0; k < E; ++k) x[i][k] = entry<DT>(rv.r[i], k);
   } else {
-    auto row = [&](int i) { return load_vector<DT, AL>(u.base + i * row_step, v, p.V, whole); };
-    const uint4 r0 = row(0);
-    const uint4 r1 = p.n >= 2 ? row(1) : r0;
+    const VecRange whole = whole_vectors<DT, AL>(kc.V);
     f32x2 xq[E / 2], cmb[E / 2];
-    const LogitWeights lw = logit_weights(p, u.pis, u.thr);
-    if (p.mask_model >= 0)
-      logit_args<DT, false, true>(p, lw, r0, r1, row, xq, cmb);
-    else
-      logit_args<DT, false, false>(p, lw, r0, r1, row, xq, cmb);
+    const LogitWeights lw = {kc.w[0], kc.w[1], u.pis, kc.mask_model, u.thr};
+    logit_args<DT, (FORM & 1) != 0, (FORM & 2) != 0>(
+        p, lw, rv.r[0], rv.r[1], [&](int i) { return load_vector<DT, AL>(u.base + i * kc.row_step, v, kc.V, whole); }, xq, cmb);
 #pragma unroll
     for (int k = 0; k < E; ++k) {  // (beyond V the combination of -inf could be anything)
       x[0][k] = pair_at(xq[k / 2], k);
-      x[1][k] = (v * E + k < p.V) ? pair_at(cmb[k / 2], k) : -INFINITY;
+      x[1][k] = (v * E + k < kc.V) ? pair_at(cmb[k / 2], k) : -INFINITY;
     }
   }
 }
 
-// The mass of one big token.  Out of line.
-template <int DT, bool ENS, int NCH>
-__device__ __noinline__ double big_mass(const DrawConst& p, const DrawUnit<NCH>& u, const double* inv, int e) {
-  float x[NCH];
+// The mass of one big token, the k-th of the vectors.  Out of line.
+template <int DT, bool ENS, int NCH, int FORM>
+__device__ __noinline__ double big_mass(const DrawConst& p, const DrawUnit<NCH>& u, const double* inv, Vectors<ENS ? NCH : 2> rv, int e, int k, bool in) {
   double d[NCH];
-  entry_args<DT, ENS, NCH>(p, u, e, x);
-  exact_terms<DT, ENS, NCH>(p, u, e, x, d);
+  exact_terms<DT, ENS, NCH, FORM>(p, u, rv, e, k, in, d);
   return exact_mass<ENS, NCH>(p, d, inv, u.pis, u.law);
 }
 
-// The vectors the fast loop left out (bit k of a lane's `slow`: its vector of step c + k): those with a big entry, which is summed in
-// fp64 then, and the ragged ends of the row.  The warp takes 32 entries at a time, one a lane; the sums go to the lanes'
-// slots of `acc`.  Out of line.  (One lane going through its vector while the others waited took 2 us a vector, and the warp that
-// happened on most big tokens was the last of its cluster by 5 to 8 us.)
-template <int DT, bool ENS, int NCH>
-__device__ __noinline__ void slow_vectors(const DrawConst& p, const DrawUnit<NCH>& u, int c, unsigned slow, double* acc) {
-  constexpr int E = Elem<DT>::E, G = 32 / E;
-  const int T = blockDim.x, lane = threadIdx.x & 31;
-  for (unsigned any = __reduce_or_sync(0xffffffffu, slow); any; any &= any - 1) {
-    const int k = __ffs(any) - 1;
-    unsigned m = __ballot_sync(0xffffffffu, (slow >> k) & 1u);
-    while (m) {
-      unsigned t = m;
+// A lane's vector v that the fast loop left out: one with a big entry, which is summed in fp64 then, or one at a ragged end of the
+// row (fetched here).  The sums go to the lane's slots of `acc`, which are cleared where `first`.  Out of line.  (What the fast loop had
+// left out, put off until the end of 32 steps, fetched again and dealt out over the warp entry by entry, took a warp 1400 cycles for every
+// step that had any.)
+template <int DT, bool ENS, int NCH, bool AL, int FORM>
+__device__ __noinline__ void slow_vector(const KParams& p, const DrawConst& kc, const DrawUnit<NCH>& u, Vectors<ENS ? NCH : 2> rv, int v, bool ragged,
+                                         bool first, double* acc) {
+  constexpr int E = Elem<DT>::E, NR = ENS ? NCH : 2;
+  const int T = blockDim.x;
+  if (ragged) {
+    const VecRange whole = whole_vectors<DT, AL>(kc.V);
 #pragma unroll
-      for (int q = 0; q < G; ++q) {
-        if (q < lane / E) t &= t - 1;
-        m &= m - 1;
-      }
-      const int e = t ? ((c + k) * 32 + __ffs(t) - 1) * E + lane % E : p.V;
-      if (e < p.V) {
-        float x[NCH], f[NCH], tot = 0.f;
-        bool big = false;
-        entry_args<DT, ENS, NCH>(p, u, e, x);
+    for (int i = 0; i < NR; ++i)
+      if (i < kc.n) rv.r[i] = load_vector<DT, AL>(u.base + i * kc.row_step, v, kc.V, whole);
+  }
+  float x[NCH][E], z[NCH], a[NCH];
+  vector_args<DT, ENS, NCH, AL, FORM>(p, kc, u, rv, v, x);
 #pragma unroll
-        for (int i = 0; i < NCH; ++i) {
-          f[i] = ex2_approx(fmaf(x[i], p.cT, u.nref[i]));
-          big = big || f[i] > u.bt[i];
-          tot = __fadd_rn(tot, __fmul_rn(u.ct[i], f[i]));
-        }
-        double d[NCH];
+  for (int i = 0; i < NCH; ++i) z[i] = a[i] = 0.f;
+  unsigned bigbits = 0u, inbits = 0u;
 #pragma unroll
-        for (int i = 0; i < NCH; ++i) d[i] = static_cast<double>(f[i]);
-        bool counts = tot > 0.f;
-        if (big) {
-          exact_terms<DT, ENS, NCH>(p, u, e, x, d);
-          double t64 = 0.0;
+  for (int k = 0; k < E; ++k) {
+    float f[NCH], tot = 0.f;
+    bool big = false;
 #pragma unroll
-          for (int i = 0; i < NCH; ++i) t64 = __dadd_rn(t64, __dmul_rn(u.ck[i], d[i]));
-          counts = t64 > 0.0;
-        }
-#pragma unroll
-        for (int i = 0; i < NCH; ++i) {
-          acc[i * T] += d[i];
-          if (counts) acc[(NCH + i) * T] += d[i];
-        }
-      }
+    for (int i = 0; i < NCH; ++i) {
+      f[i] = ex2_approx(fmaf(x[i][k], kc.cT, u.nref[i]));
+      big = big || f[i] > u.bt[i];
+      tot = __fadd_rn(tot, __fmul_rn(u.ct[i], f[i]));
     }
+    if (big) bigbits |= 1u << k;
+    if (ENS || x[1][k] != -INFINITY) inbits |= 1u << k;
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      z[i] += big ? 0.f : f[i];
+      a[i] += !big && tot > 0.f ? f[i] : 0.f;
+    }
+  }
+  double sz[NCH], sa[NCH];
+#pragma unroll
+  for (int i = 0; i < NCH; ++i) {
+    sz[i] = static_cast<double>(z[i]) + (first ? 0.0 : acc[i * T]);
+    sa[i] = static_cast<double>(a[i]) + (first ? 0.0 : acc[(NCH + i) * T]);
+  }
+#pragma unroll 1
+  for (; bigbits; bigbits &= bigbits - 1) {
+    const int k = __ffs(bigbits) - 1;
+    double d[NCH], t = 0.0;
+    exact_terms<DT, ENS, NCH, FORM>(kc, u, rv, v * E + k, k, (inbits >> k) & 1u, d);
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) t = __dadd_rn(t, __dmul_rn(u.ck[i], d[i]));
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      sz[i] += d[i];
+      sa[i] += t > 0.0 ? d[i] : 0.0;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NCH; ++i) {
+    acc[i * T] = sz[i];
+    acc[(NCH + i) * T] = sa[i];
   }
 }
 
 // The steps [s_lo, s_hi) of a position by one warp, in chunks of cs steps: per channel the sum over the tokens with a positive mass,
-// for every chunk NCH sums to rec, and to part the normaliser's share, of all chunks together (both in the cluster's first block).
-// The fast loop adds vectors up in fp32; vectors that need the slow path it only remembers until the end of the strip (their
-// sums, in fp64, in the thread's slots of `acc`).
+// for every chunk NCH sums to the records from the rec-th on, and to part the normaliser's share, of all chunks together (both in the cluster's first block).
+// The fast loop adds vectors up in fp32 and leaves those with a big entry, and the ragged ends, to slow_vector.
 // What bounds it: instruction issue (counted at logit level, 128 rows of 256000 tokens: 211 instructions a step, 0.53 of the issue
 // slots of the average multiprocessor, 0.67 of the busiest).  Loads in flight do not: fetching a step as soon as a place is free,
 // so that two are always on their way, gained nothing with two channels and lost 2 to 7 % with four.
-// PAIR, MASKED: logit level with exactly two models, and with a mask.
-template <int DT, bool ENS, int NCH, bool AL, bool PAIR, bool MASKED>
+template <int DT, bool ENS, int NCH, bool AL, int FORM>
 __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst& kc, const DrawUnit<NCH>& u, int cs, int s_lo, int s_hi, double* acc,
-                                              unsigned rec, unsigned part) {
+                                              int rec, unsigned recs, unsigned part) {
+  constexpr bool PAIR = (FORM & 1) != 0, MASKED = (FORM & 2) != 0;
   constexpr int E = Elem<DT>::E;
   constexpr int NP = NCH / 2;
   constexpr int NR = ENS ? NCH : 2;         // vectors of a step kept in registers
@@ -339,28 +374,25 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
   const LogitWeights lw = logit_weights(p, u.pis, u.thr);
   double all = 0.0;
 #pragma unroll 1
-  for (int begin = s_lo; begin < s_hi; begin += cs, rec += NCH * 8) {
+  for (int begin = s_lo; begin < s_hi; begin += cs, ++rec) {
     const int end = begin + cs < s_hi ? begin + cs : s_hi;
-    double sums[2 * NCH];
-    // in strips of 32 steps: a bit each in the slow-path mask
-    for (int c = begin; c < end; c += 32) {
-      const int ce = c + 32 < end ? c + 32 : end;
-      unsigned slow = 0u;
-      f32x2 zc[NP], ac[NP];
+    bool slow = false;  // (whether the lane's slots hold anything)
+    f32x2 zc[NP], ac[NP];
 #pragma unroll
-      for (int q = 0; q < NP; ++q) zc[q] = ac[q] = pack2(0.f, 0.f);
-      for (int s = c; s < ce; s += US) {
-        uint4 r[US][NR];
+    for (int q = 0; q < NP; ++q) zc[q] = ac[q] = pack2(0.f, 0.f);
+    {
+#pragma unroll 1
+      for (int s = begin; s < end; s += US) {
+        Vectors<NR> r[US];
 #pragma unroll
         for (int t = 0; t < US; ++t) {
           const int v = (s + t) * 32 + lane;
           const bool in = v >= whole.lo && v < whole.hi;
 #pragma unroll
           for (int i = 0; i < NR; ++i) {
-            r[t][i] = neg_inf_vector<DT>();
-            if (in && s + t < ce && i < p.n) r[t][i] = load_whole<DT, AL>(base + i * row_step, v);
+            r[t].r[i] = neg_inf_vector<DT>();
+            if (in && s + t < end && i < p.n) r[t].r[i] = load_whole<DT, AL>(base + i * row_step, v);
           }
-          if (!in && s + t < ce) slow |= 1u << (s + t - c);
         }
 #pragma unroll
         for (int t = 0; t < US; ++t) {
@@ -374,7 +406,7 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
               f32x2 e[NP], m[NP];
 #pragma unroll
               for (int q = 0; q < NP; ++q) {
-                const f32x2 arg = fma2(pack2(entry<DT>(r[t][2 * q], k), entry<DT>(r[t][2 * q + 1], k)), c2, nref[q]);
+                const f32x2 arg = fma2(pack2(entry<DT>(r[t].r[2 * q], k), entry<DT>(r[t].r[2 * q + 1], k)), c2, nref[q]);
                 e[q] = pack2(ex2_approx(lo2(arg)), ex2_approx(hi2(arg)));
                 vz[q] = add2(vz[q], e[q]);
                 m[q] = mul2(ct[q], e[q]);
@@ -389,8 +421,8 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
             // two neighbouring tokens side by side
             f32x2 xq[E / 2], cmb[E / 2];
             const int v = (s + t) * 32 + lane;
-            const bool in = v >= whole.lo && v < whole.hi && s + t < ce;
-            logit_args<DT, PAIR, MASKED>(p, lw, r[t][0], r[t][1],
+            const bool in = v >= whole.lo && v < whole.hi && s + t < end;
+            logit_args<DT, PAIR, MASKED>(p, lw, r[t].r[0], r[t].r[1],
                                          [&](int i) {
                                            uint4 m = neg_inf_vector<DT>();
                                            if (in) m = load_whole<DT, AL>(base + i * row_step, v);
@@ -425,8 +457,11 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
           bool big = false;
 #pragma unroll
           for (int q = 0; q < NP; ++q) big = big || lo2(vz[q]) > bt[2 * q] || hi2(vz[q]) > bt[2 * q + 1];
-          if (big) {
-            slow |= 1u << (s + t - c);
+          const int v = (s + t) * 32 + lane;
+          const bool ragged = s + t < end && (v < whole.lo || v >= whole.hi) && v * E < p.V;
+          if (big || ragged) {
+            slow_vector<DT, ENS, NCH, AL, FORM>(p, kc, u, r[t], v, ragged, !slow, acc);
+            slow = true;
           } else {
 #pragma unroll
             for (int q = 0; q < NP; ++q) {
@@ -436,39 +471,38 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
           }
         }
       }
+    }
+    double sums[2 * NCH];
+    {
       const int T = blockDim.x;
-      const bool more = c > begin;
 #pragma unroll
       for (int q = 0; q < NP; ++q) {
-        sums[2 * q] = static_cast<double>(lo2(zc[q])) + (more ? acc[(2 * q) * T] : 0.0);
-        sums[2 * q + 1] = static_cast<double>(hi2(zc[q])) + (more ? acc[(2 * q + 1) * T] : 0.0);
-        sums[NCH + 2 * q] = static_cast<double>(lo2(ac[q])) + (more ? acc[(NCH + 2 * q) * T] : 0.0);
-        sums[NCH + 2 * q + 1] = static_cast<double>(hi2(ac[q])) + (more ? acc[(NCH + 2 * q + 1) * T] : 0.0);
+        sums[2 * q] = static_cast<double>(lo2(zc[q]));
+        sums[2 * q + 1] = static_cast<double>(hi2(zc[q]));
+        sums[NCH + 2 * q] = static_cast<double>(lo2(ac[q]));
+        sums[NCH + 2 * q + 1] = static_cast<double>(hi2(ac[q]));
       }
-      if (ce < end || __any_sync(0xffffffffu, slow != 0u)) {
+      if (slow) {
 #pragma unroll
-        for (int q = 0; q < 2 * NCH; ++q) acc[q * T] = sums[q];
-        slow_vectors<DT, ENS, NCH>(kc, u, c, slow, acc);
-#pragma unroll
-        for (int q = 0; q < 2 * NCH; ++q) sums[q] = acc[q * T];
+        for (int q = 0; q < 2 * NCH; ++q) sums[q] += acc[q * T];
       }
     }
     __syncwarp();
     const double mine = warp_sums<2 * NCH>(sums, lane);
-    if (lane >= 16 && lane % (16 / NCH) == 0) store_cluster(rec + (lane - 16) / (16 / NCH) * 8, mine);
+    if (lane >= 16 && lane % (16 / NCH) == 0) store_cluster(recs + (record_at(rec) * NCH + (lane - 16) / (16 / NCH)) * 8, mine);
     all += mine;
   }
   if (lane < 16 && lane % (16 / NCH) == 0) store_cluster(part + lane / (16 / NCH) * 8, all);
 }
 
 // Shared memory of a block, in front of every thread's 2 NCH slots of the slow path.
-template <int NCH>
+template <int NCH, int PARTS = kMaxParts, int SUMS = kMaxSums>
 struct DrawShared {
   DrawConst kc;
   DrawUnit<NCH> unit;
   // (of the cluster's first block)
-  double recs[kMaxSums];                         // sums of the chunks
-  double part[kMaxParts * kMaxDrawWarps][NCH];   // shares of the normalisers, of every warp
+  double recs[SUMS / 8 * 9];                 // sums of the chunks (see record_at)
+  double part[PARTS * kMaxDrawWarps][NCH];   // shares of the normalisers, of every warp
   double step_mass[32];
   double inv[NCH];      // one over the normalisers
   double base, target;  // mass before the winning chunk; the running total to be reached
@@ -476,67 +510,59 @@ struct DrawShared {
   int win;              // the winning chunk; -1: nothing to draw, -2: no mass, -3: the set of tokens is to be decided again
 };
 
-// The share of warp w of W; chunks without steps get sums of zero.
-template <int DT, bool ENS, int NCH, bool AL>
-__device__ __forceinline__ void draw_sweep(const KParams& p, DrawShared<NCH>& sh, int w, int W, double* acc) {
+// The share of warp w of W; chunks without steps get sums of zero.  FORM: logit level: bit 0: two models, bit 1: with a mask.
+template <int DT, bool ENS, int NCH, bool AL, int FORM, typename SH>
+__device__ __forceinline__ void draw_sweep(const KParams& p, SH& sh, int w, int W, double* acc) {
   const int s_lo = static_cast<int>(static_cast<long long>(p.nsteps) * w / W);
   const int s_hi = static_cast<int>(static_cast<long long>(p.nsteps) * (w + 1) / W);
-  const unsigned rec = at_first(&sh.recs[w * p.draw_chunks * NCH]), part = at_first(sh.part[w]);
-  const int cs = p.draw_cs, used = (s_hi - s_lo + cs - 1) / cs;
-  for (int k = used * NCH + (threadIdx.x & 31); k < p.draw_chunks * NCH; k += 32) store_cluster(rec + k * 8, 0.0);
-  const DrawUnit<NCH>& u = sh.unit;
-  if (ENS) return draw_sweep_as<DT, ENS, NCH, AL, true, false>(p, sh.kc, u, cs, s_lo, s_hi, acc, rec, part);
-  if (p.n == 2 && p.mask_model < 0) return draw_sweep_as<DT, ENS, NCH, AL, true, false>(p, sh.kc, u, cs, s_lo, s_hi, acc, rec, part);
-  if (p.n == 2) return draw_sweep_as<DT, ENS, NCH, AL, true, true>(p, sh.kc, u, cs, s_lo, s_hi, acc, rec, part);
-  if (p.mask_model < 0) return draw_sweep_as<DT, ENS, NCH, AL, false, false>(p, sh.kc, u, cs, s_lo, s_hi, acc, rec, part);
-  draw_sweep_as<DT, ENS, NCH, AL, false, true>(p, sh.kc, u, cs, s_lo, s_hi, acc, rec, part);
+  const unsigned recs = at_first(sh.recs), part = at_first(sh.part[w]);
+  const int cs = p.draw_cs, rec = w * p.draw_chunks, used = (s_hi - s_lo + cs - 1) / cs;
+  for (int k = used * NCH + (threadIdx.x & 31); k < p.draw_chunks * NCH; k += 32) store_cluster(recs + (record_at(rec + k / NCH) * NCH + k % NCH) * 8, 0.0);
+  draw_sweep_as<DT, ENS, NCH, AL, FORM>(p, sh.kc, sh.unit, cs, s_lo, s_hi, acc, rec, recs, part);
 }
 
-// The mass of one lane's tokens of step s under the refined normalisers (coefficients cf = k / Z): small ones in fp32, big
-// ones in fp64.
-template <int DT, bool ENS, int NCH, bool AL>
-__device__ __forceinline__ double step_mass(const KParams& p, const DrawConst& kc, const DrawUnit<NCH>& u, const float* cf, const double* inv, int s) {
-  constexpr int E = Elem<DT>::E;
+// The masses of one lane's tokens of step s under the refined normalisers (coefficients cf = k / Z): small ones in fp32; the bits of big
+// ones, which are for fp64 (big_mass), with 0 in their place; and the bits of those inside the mask.
+template <int DT, bool ENS, int NCH, bool AL, int FORM>
+__device__ __forceinline__ void step_masses(const KParams& p, const DrawConst& kc, const DrawUnit<NCH>& u, const float* cf, int s,
+                                            Vectors<ENS ? NCH : 2>& rv, float (&m)[Elem<DT>::E], unsigned& bigbits, unsigned& inbits) {
+  constexpr int E = Elem<DT>::E, NR = ENS ? NCH : 2;
   const int v = s * 32 + (threadIdx.x & 31);
+  const VecRange whole = whole_vectors<DT, AL>(kc.V);
+  const bool in = v >= whole.lo && v < whole.hi;
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    rv.r[i] = neg_inf_vector<DT>();
+    if (in && i < kc.n) rv.r[i] = load_whole<DT, AL>(u.base + i * kc.row_step, v);
+  }
+  if (!in && v * E < kc.V) {
+#pragma unroll
+    for (int i = 0; i < NR; ++i)
+      if (i < kc.n) rv.r[i] = load_vector<DT, AL>(u.base + i * kc.row_step, v, kc.V, whole);
+  }
   float x[NCH][E];
-  vector_args<DT, ENS, NCH, AL>(p, u, v, x);
-  unsigned bigbits = 0u;
-  float ls = 0.f;
+  vector_args<DT, ENS, NCH, AL, FORM>(p, kc, u, rv, v, x);
+  bigbits = inbits = 0u;
 #pragma unroll
   for (int k = 0; k < E; ++k) {
     float tot = 0.f;
     bool big = false;
 #pragma unroll
     for (int i = 0; i < NCH; ++i) {
-      const float e = ex2_approx(fmaf(x[i][k], p.cT, u.nref[i]));
+      const float e = ex2_approx(fmaf(x[i][k], kc.cT, u.nref[i]));
       big = big || e > u.bt[i];
       tot = __fadd_rn(tot, __fmul_rn(cf[i], e));
     }
-    ls += big ? 0.f : fmaxf(0.f, tot);
-    bigbits |= big ? (1u << k) : 0u;
+    m[k] = big ? 0.f : fmaxf(0.f, tot);
+    if (big) bigbits |= 1u << k;
+    if (ENS || x[1][k] != -INFINITY) inbits |= 1u << k;
   }
-  double own = static_cast<double>(ls);
-  for (; bigbits; bigbits &= bigbits - 1) own += big_mass<DT, ENS, NCH>(kc, u, inv, v * E + __ffs(bigbits) - 1);
-  return own;
-}
-template <int DT, bool ENS, int NCH>
-__device__ __forceinline__ double token_mass(const DrawConst& p, const DrawUnit<NCH>& u, const float* cf, const double* inv, int e) {
-  float x[NCH], tot = 0.f;
-  bool big = false;
-  entry_args<DT, ENS, NCH>(p, u, e, x);
-#pragma unroll
-  for (int i = 0; i < NCH; ++i) {
-    const float f = ex2_approx(fmaf(x[i], p.cT, u.nref[i]));
-    big = big || f > u.bt[i];
-    tot = __fadd_rn(tot, __fmul_rn(cf[i], f));
-  }
-  return big ? big_mass<DT, ENS, NCH>(p, u, inv, e) : static_cast<double>(fmaxf(0.f, tot));
 }
 
 // The whole position again by the cluster's first block, for another law or other coefficients.  Rare; out of line.
-template <int DT, bool ENS, int NCH, bool AL>
-__device__ __noinline__ void draw_sweep_again(const KParams& p, DrawShared<NCH>& sh, int W, double* acc) {
-  for (int w = threadIdx.x >> 5; w < W; w += blockDim.x >> 5) draw_sweep<DT, ENS, NCH, AL>(p, sh, w, W, acc);
+template <int DT, bool ENS, int NCH, bool AL, int FORM, typename SH>
+__device__ __noinline__ void draw_sweep_again(const KParams& p, SH& sh, int W, double* acc) {
+  for (int w = threadIdx.x >> 5; w < W; w += blockDim.x >> 5) draw_sweep<DT, ENS, NCH, AL, FORM>(p, sh, w, W, acc);
 }
 
 // The normalisers from the shares of all W warps, and the chunk that holds the token.  One warp.  `first_pass`: the set of tokens with a
@@ -544,8 +570,8 @@ __device__ __noinline__ void draw_sweep_again(const KParams& p, DrawShared<NCH>&
 // error (1e-7, a few 1e-6 at low temperature), which matters only where the whole residual mass is below a thousand times that: there
 // the set is decided again with the refined ones (sh.win = -3).  (Where the normalisers of all channels are the same number, r is q and
 // nothing is left.)
-template <bool ENS, int NCH>
-__device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh, int W, bool first_pass) {
+template <bool ENS, int NCH, typename SH>
+__device__ __forceinline__ void find_chunk(const KParams& p, SH& sh, int W, bool first_pass) {
   constexpr int G = 32 / NCH;  // lanes of a channel
   const int lane = threadIdx.x & 31, i = lane / G, live = ENS ? p.n : 2;
   const DrawUnit<NCH>& u = sh.unit;
@@ -563,43 +589,38 @@ __device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh
 #pragma unroll
   for (int q = 0; q < NCH; ++q) c64[q] = __shfl_sync(0xffffffffu, k, q * G);
   auto mass_of = [&](int c) -> double {  // (products rounded one by one: equal sums under opposite coefficients cancel)
-    const double* a = &sh.recs[c * NCH];
+    const double* a = &sh.recs[record_at(c) * NCH];
     double m = __dmul_rn(c64[0], a[0]);
 #pragma unroll
     for (int q = 1; q < NCH; ++q) m = __dadd_rn(m, __dmul_rn(c64[q], a[q]));
-    return fmax(0.0, m);
+    return m > 0.0 ? m : 0.0;
   };
-  // consecutive chunks to a lane, their masses in the place of their first sums
+  // consecutive chunks to a lane; then the chunks of the lane that holds the target, one to a lane (32 and more of them: in a few goes)
   const int chunks = W * p.draw_chunks, per = (chunks + 31) / 32;
   const int c_lo = lane * per, c_hi = c_lo + per < chunks ? c_lo + per : chunks;
   double mine = 0.0;
 #pragma unroll 4
-  for (int c = c_lo; c < c_hi; ++c) {
-    const double m = mass_of(c);
-    sh.recs[c * NCH] = m;
-    mine += m;
-  }
-  double incl = mine;
-#pragma unroll 1
-  for (int d = 1; d < 32; d <<= 1) {
-    const double o = __shfl_up_sync(0xffffffffu, incl, d);
-    if (lane >= d) incl += o;
-  }
+  for (int c = c_lo; c < c_hi; ++c) mine += mass_of(c);
+  const double incl = running_total<32>(mine, lane);
   const double S = __shfl_sync(0xffffffffu, incl, 31), target = word_to_uniform(u.word) * S;
-  // the first chunk whose running total reaches the target; where rounding leaves none, the last chunk with mass
-  double before = incl - mine, base = 0.0;
-  int first = -1, last = -1;
-  if (mine > 0.0)
+  // the first that reaches the target; where rounding leaves none, the last with mass
+  const unsigned some = __ballot_sync(0xffffffffu, mine > 0.0), hit = __ballot_sync(0xffffffffu, mine > 0.0 && incl >= target);
+  const int who = hit ? __ffs(hit) - 1 : 31 - __clz(some);
+  double base = __shfl_sync(0xffffffffu, incl - mine, who & 31), win_base = 0.0;
+  int win = -1;
+  const int w_lo = (who & 31) * per, w_hi = w_lo + per < chunks ? w_lo + per : chunks;
 #pragma unroll 1
-    for (int c = c_lo; c < c_hi; ++c) {
-      const double m = sh.recs[c * NCH];
-      if (m > 0.0 && first < 0) {
-        last = c;
-        base = before;
-        if (before + m >= target) first = c;
-      }
-      before += m;
+  for (int c0 = w_lo; c0 < w_hi && some != 0u; c0 += 32) {
+    const double m = c0 + lane < w_hi ? mass_of(c0 + lane) : 0.0, in = running_total<32>(m, lane);
+    const unsigned with = __ballot_sync(0xffffffffu, m > 0.0), ok = __ballot_sync(0xffffffffu, m > 0.0 && base + in >= target);
+    if (with) {
+      const int k = ok ? __ffs(ok) - 1 : 31 - __clz(with);
+      win = c0 + k;
+      win_base = base + __shfl_sync(0xffffffffu, in - m, k);
     }
+    if (ok) break;
+    base += __shfl_sync(0xffffffffu, in, 31);
+  }
   bool again = false;
   if (first_pass && u.law == kDrawResidual) {  // (the whole warp)
     const bool off = i < live && fabs(z * kBigShare - static_cast<double>(u.bt[i])) * 1000.0 > S * static_cast<double>(u.bt[i]);
@@ -607,11 +628,9 @@ __device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh
     const unsigned offs = __ballot_sync(0xffffffffu, off), unlike = __ballot_sync(0xffffffffu, i < live && z != z0);
     again = offs != 0u && unlike != 0u;
   }
-  const unsigned hit = __ballot_sync(0xffffffffu, first >= 0), some = __ballot_sync(0xffffffffu, last >= 0);
-  const int winner = hit ? __ffs(hit) - 1 : 31 - __clz(some);
-  if (some != 0u ? lane == winner : lane == 0) {
-    sh.win = some != 0u && S > 0.0 ? last : -2;
-    sh.base = base;
+  if (lane == 0) {
+    sh.win = some != 0u && S > 0.0 ? win : -2;
+    sh.base = win_base;
     sh.target = target;
     if (!u.emit) sh.win = -1;
     if (again) sh.win = -3;
@@ -620,11 +639,11 @@ __device__ __forceinline__ void find_chunk(const KParams& p, DrawShared<NCH>& sh
 }
 
 // The rest of a position, after the sweep: the block that has the sums finds the chunk, the step and the token.
-template <int DT, bool ENS, int NCH, bool AL>
-__device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, double* acc) {
+template <int DT, bool ENS, int NCH, bool AL, int FORM, typename SH>
+__device__ __forceinline__ void locate(const KParams& p, SH& sh, double* acc) {
   constexpr int E = Elem<DT>::E;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const int live = ENS ? p.n : 2, W = p.draw_parts * nw;
+  const int W = p.draw_parts * nw;
   DrawUnit<NCH>& u = sh.unit;
   const int cs = p.draw_cs;
 #pragma unroll 1
@@ -654,7 +673,7 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
         }
       }
       __syncthreads();
-      draw_sweep_again<DT, ENS, NCH, AL>(p, sh, W, acc);
+      draw_sweep_again<DT, ENS, NCH, AL, FORM>(p, sh, W, acc);
       __syncthreads();
       continue;
     }
@@ -666,15 +685,6 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
     const int s0 = static_cast<int>(static_cast<long long>(p.nsteps) * ww / W) + win % p.draw_chunks * cs;
     const int end = static_cast<int>(static_cast<long long>(p.nsteps) * (ww + 1) / W);
     const int s1 = s0 + cs < end ? s0 + cs : end, gsz = (cs + 31) / 32;
-    // running total over the first `lanes` lanes
-    auto scan = [&](double m, int lanes) -> double {
-#pragma unroll 1
-      for (int d = 1; d < lanes; d <<= 1) {
-        const double o = __shfl_up_sync(0xffffffffu, m, d);
-        if (lane >= d) m += o;
-      }
-      return m;
-    };
     // the first lane whose total `in` (its own mass: m) reaches the target, or the last with mass where rounding leaves none
     auto first_reach = [&](double m, double in, double from, double& upto) -> int {
       const unsigned some = __ballot_sync(0xffffffffu, m > 0.0), ok = __ballot_sync(0xffffffffu, m > 0.0 && from + in >= target);
@@ -682,100 +692,132 @@ __device__ __forceinline__ void locate(const KParams& p, DrawShared<NCH>& sh, do
       upto = from + __shfl_sync(0xffffffffu, in - m, k & 31);
       return ok ? k : k - 32;  // (negative: not reached; -33: no mass at all)
     };
+    // (what the lanes of this warp hold of step `held`: their masses, the running total, the masses of their tokens)
     double own = 0.0, in = 0.0;
-    int held = -1;  // the step whose masses, and their running total, the lanes of this warp hold
+    int held = -1;
+    Vectors<ENS ? NCH : 2> rv;
+    float m[E];
+    unsigned bigbits = 0u, inbits = 0u;
+    auto hold = [&](int s) {
+      step_masses<DT, ENS, NCH, AL, FORM>(p, sh.kc, u, cf, s, rv, m, bigbits, inbits);
+      own = 0.0;
+#pragma unroll
+      for (int k = 0; k < E; ++k) own += static_cast<double>(m[k]);
+#pragma unroll 1
+      for (unsigned bits = bigbits; bits; bits &= bits - 1) {
+        const int k = __ffs(bits) - 1;
+        own += big_mass<DT, ENS, NCH, FORM>(sh.kc, u, inv, rv, (s * 32 + lane) * E + k, k, (inbits >> k) & 1u);
+      }
+      in = running_total<32>(own, lane);
+      held = s;
+    };
 #pragma unroll 1
     for (int t = warp; s0 + t * gsz < s1; t += nw) {
       double rm = 0.0;
 #pragma unroll 1
       for (int s = s0 + t * gsz; s < s0 + (t + 1) * gsz && s < s1; ++s) {
-        own = step_mass<DT, ENS, NCH, AL>(p, sh.kc, u, cf, inv, s);
-        in = scan(own, 32);
+        hold(s);
         rm += __shfl_sync(0xffffffffu, in, 31);
-        held = s;
       }
       if (lane == 0) sh.step_mass[t] = rm;
     }
     __syncthreads();
     if (held < 0) return;  // (no step of the chunk is this warp's)
-    double at, m = (s0 + lane * gsz < s1) ? sh.step_mass[lane] : 0.0;
-    int k = first_reach(m, scan(m, (s1 - s0 + gsz - 1) / gsz), sh.base, at);
+    double at;
+    const double sm = (s0 + lane * gsz < s1) ? sh.step_mass[lane] : 0.0;
+    const int k = first_reach(sm, running_total<32>(sm, lane), sh.base, at);
     if (k == -33) return;
     if ((k & 31) % nw != warp) return;
     // one warp goes on: the record's steps in order, the lanes of a step, the tokens of a lane's vector
     const int g0 = s0 + (k & 31) * gsz, g1 = g0 + gsz < s1 ? g0 + gsz : s1;
-    int step = -1, who = 0;
-    double before = 0.0;
+    int some = -1;  // the last step with mass, and the total before it
+    double some_at = 0.0;
 #pragma unroll 1
-    for (int s = g0; s < g1; ++s) {
-      if (s != held) {
-        own = step_mass<DT, ENS, NCH, AL>(p, sh.kc, u, cf, inv, s);
-        in = scan(own, 32);
-        held = s;
-      }
-      double upto;
-      const int l = first_reach(own, in, at, upto);
+    for (int s = g0;;) {
+      if (s != held) hold(s);
+      double before;
+      const int l = first_reach(own, in, at, before);
       if (l != -33) {
-        step = s;
-        who = l & 31;
-        before = upto;
+        some = s;
+        some_at = at;
       }
-      if (l >= 0) break;
-      at += __shfl_sync(0xffffffffu, in, 31);
+      if (l < 0) {  // (not reached in this step)
+        at += __shfl_sync(0xffffffffu, in, 31);
+        if (++s < g1) continue;
+        if (some < 0) return;
+        if (some != held) hold(some);  // (rounding left none that reaches the target: the last token with mass)
+        first_reach(own, in, some_at, before);
+      }
+      const unsigned with = __ballot_sync(0xffffffffu, own > 0.0);
+      const int who = l >= 0 ? l : 31 - __clz(with);
+      if (lane == who) {
+        double run = before;
+        int last = -1;
+        bool reached = false;
+        auto take = [&](int q, double mass) {
+          run += mass;
+          if (mass > 0.0 && !reached) {
+            last = q;
+            reached = run >= target;
+          }
+        };
+        const int e0 = (held * 32 + lane) * E;
+        if (bigbits == 0u) {
+#pragma unroll
+          for (int q = 0; q < E; ++q) take(q, static_cast<double>(m[q]));
+        } else {
+#pragma unroll 1
+          for (int q = 0; q < E; ++q) {
+            float small = m[0];
+#pragma unroll
+            for (int r = 1; r < E; ++r) small = r == q ? m[r] : small;
+            take(q, (bigbits >> q) & 1u ? big_mass<DT, ENS, NCH, FORM>(sh.kc, u, inv, rv, e0 + q, q, (inbits >> q) & 1u) : static_cast<double>(small));
+          }
+        }
+        if (last >= 0) {
+          p.out_tokens[u.uidx] = e0 + last;
+          // Algorithm 2's Score returns the bonus token with its probability under the law it came from
+          if (u.j == p.gamma && p.bonus_prob != nullptr)
+            p.bonus_prob[u.b] = static_cast<float>(big_mass<DT, ENS, NCH, FORM>(sh.kc, u, inv, rv, e0 + last, last, (inbits >> last) & 1u));
+        }
+      }
+      return;
     }
-    if (step < 0) return;
-    const int e = (step * 32 + who) * E + lane;
-    m = 0.0;
-    if (lane < E && e < p.V) m = token_mass<DT, ENS, NCH>(sh.kc, u, cf, inv, e);
-    k = first_reach(m, scan(m, E), before, at);
-    const int token = (step * 32 + who) * E + (k & 31);
-    if (lane == 0 && k != -33) {
-      p.out_tokens[u.uidx] = token;
-      // Algorithm 2's Score returns the bonus token with its probability under the law it came from
-      if (u.j == p.gamma && p.bonus_prob != nullptr) p.bonus_prob[u.b] = static_cast<float>(big_mass<DT, ENS, NCH>(sh.kc, u, inv, token));
-    }
-    return;
   }
 }
 
 // The block's position from the records of the streaming launch (and the row's outputs, see decide_row): every block decides
 // its row for itself.  False when there is nothing to draw.
-template <int DT, bool ENS, int NCH>
-__device__ __forceinline__ bool decide_unit_to_draw(const KParams& p, DrawShared<NCH>& sh, RowShared& rs, int slot, int part) {
+template <int DT, bool ENS, int NCH, typename SH, typename R>
+__device__ __forceinline__ bool decide_unit_to_draw(const KParams& p, SH& sh, RowShared& rs, const TilePlan& t, const TileInputs& in, int b, int want,
+                                                    int part, R ready) {
   const int tid = threadIdx.x;
-  int b = slot, want = -1;
-  if (p.draw_all) {
-    const int drafts = p.B * p.gamma;  // every draft position, then the bonus positions
-    b = slot < drafts ? slot / p.gamma : slot - drafts;
-    want = slot < drafts ? slot % p.gamma : p.gamma;
-  }
   DrawUnit<NCH>& u = sh.unit;
-  decide_row<DT, ENS ? kEnsembleSample : kLogitSample>(
-      p, rs, b, want,
-      [&](const Finish& f, int j, unsigned word, int accepted, int drawable) {
-        const int pi = proposer_of(p, b, j);
+  decide_sampled<DT, ENS ? kEnsembleSample : kLogitSample>(
+      p, rs, t, in, b, want, ready,
+      [&](const PairStats* f, int j, int pi, unsigned word, int accepted, int drawable) {
         const int pis = (pi >= 0 && pi < p.n) ? pi : 0;
         const int law = (j == p.gamma) ? (p.bonus_model >= 0 ? kDrawQ : kDrawR) : kDrawResidual;
-        if (tid < NCH) {
-          const bool live = tid < (ENS ? p.n : 2);
-          u.nref[tid] = live ? -f.fsoft[tid].ref : 0.f;
-          u.bt[tid] = live ? static_cast<float>(f.fsoft[tid].s * kBigShare) : INFINITY;
-          u.ck[tid] = live ? coefficient<ENS>(p, tid, pis, law) * f.inv[tid] : 0.0;
-          u.ct[tid] = static_cast<float>(u.ck[tid]);
+#pragma unroll
+        for (int i = 0; i < NCH; ++i) {
+          const bool live = i < (ENS ? p.n : 2);
+          const double ck = live ? coefficient<ENS>(p, i, pis, law) * f[i].inv : 0.0;
+          u.nref[i] = live ? -f[i].ref : 0.f;
+          u.bt[i] = live ? static_cast<float>(f[i].s * kBigShare) : INFINITY;
+          u.ck[i] = ck;
+          u.ct[i] = static_cast<float>(ck);
         }
-        if (tid == 0) {
-          u.b = b;
-          u.j = j;
-          u.uidx = b * p.P + j;
-          u.pis = pis;
-          u.law = law;
-          u.word = word;
-          u.accepted = accepted;
-          u.drawable = drawable;
-          u.thr = (!ENS && p.mask_model >= 0) ? f.thr : -INFINITY;
-          u.base = reinterpret_cast<const char*>(p.logits) +
-                   (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
-        }
+        u.b = b;
+        u.j = j;
+        u.uidx = b * p.P + j;
+        u.pis = pis;
+        u.law = law;
+        u.word = word;
+        u.accepted = accepted;
+        u.drawable = drawable;
+        u.thr = (!ENS && p.mask_model >= 0) ? f[1].thr : -INFINITY;
+        u.base = reinterpret_cast<const char*>(p.logits) +
+                 (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
       },
       [&](int a) { return part == 0 && (want < 0 || want == a); }, [&](int j) { return part == 0 && (want < 0 || want == j); });
   const bool emit = (rs.a == u.j);
@@ -784,32 +826,29 @@ __device__ __forceinline__ bool decide_unit_to_draw(const KParams& p, DrawShared
 }
 
 // One cluster of p.draw_parts blocks for each position.  All blocks of a cluster take the same way, and so meet at its barriers.
-template <int DT, bool ENS, int NCH, bool AL>
+template <int DT, bool ENS, int NCH, bool AL, int FORM>
 __global__ void __launch_bounds__(NCH == 8 ? 256 : kMaxDrawThreads, NCH == 2 ? 2 : (NCH == 4 ? 1 : 2)) cos_draw_kernel(const __grid_constant__ KParams p) {
   extern __shared__ __align__(16) unsigned char draw_smem_raw[];
   DrawShared<NCH>& sh = *reinterpret_cast<DrawShared<NCH>*>(draw_smem_raw);
   double* slots = reinterpret_cast<double*>(draw_smem_raw + sizeof(DrawShared<NCH>));
   double* acc = slots + threadIdx.x;
   const int slot = blockIdx.x / p.draw_parts, rank = blockIdx.x % p.draw_parts, nw = blockDim.x >> 5;
-  if (threadIdx.x < COS_MAX_MODELS) {
-    DrawConst& kc = sh.kc;
-    kc.w[threadIdx.x] = p.w[threadIdx.x];
-    kc.w64[threadIdx.x] = p.w64[threadIdx.x];
-    if (threadIdx.x == 0) {
-      kc.row_step = p.s_model * Elem<DT>::bytes;
-      kc.cT64 = p.cT64;
-      kc.cT = p.cT;
-      kc.n = p.n;
-      kc.V = p.V;
-      kc.mask_model = p.mask_model;
-    }
-  }
+  fill_const<DT>(p, sh.kc);
   cluster_arrive();  // (the first block has begun: its shared memory may be written to)
   // launched while the kernel before it drains; nothing but inputs is read before that one is complete
   bool draws;
   if (NCH != 8 && p.decide) {
     RowShared& rs = *reinterpret_cast<RowShared*>(slots);
-    draws = decide_unit_to_draw<DT, ENS, NCH>(p, sh, rs, slot, rank);
+    int b = slot, want = -1;
+    if (p.draw_all) {
+      const int drafts = p.B * p.gamma;  // every draft position, then the bonus positions
+      b = slot < drafts ? slot / p.gamma : slot - drafts;
+      want = slot < drafts ? slot % p.gamma : p.gamma;
+    }
+    constexpr int kMode = ENS ? kEnsembleSample : kLogitSample;
+    const TilePlan t = tile_plan<kMode>(p);
+    draws = decide_unit_to_draw<DT, ENS, NCH>(p, sh, rs, t, tile_inputs<DT, kMode>(p, t, b, 0), b, want, rank,
+                                              [] { asm volatile("griddepcontrol.wait;" ::: "memory"); });
   } else {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     DrawUnit<NCH> d;
@@ -819,13 +858,13 @@ __global__ void __launch_bounds__(NCH == 8 ? 256 : kMaxDrawThreads, NCH == 2 ? 2
   cluster_wait();
   if (!draws) return;
   __syncthreads();
-  draw_sweep<DT, ENS, NCH, AL>(p, sh, rank * nw + (threadIdx.x >> 5), p.draw_parts * nw, acc);
+  draw_sweep<DT, ENS, NCH, AL, FORM>(p, sh, rank * nw + (threadIdx.x >> 5), p.draw_parts * nw, acc);
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   cluster_arrive();
   cluster_wait();
   if (rank == 0) {
     __syncthreads();
-    locate<DT, ENS, NCH, AL>(p, sh, acc);
+    locate<DT, ENS, NCH, AL, FORM>(p, sh, acc);
   }
 }
 

@@ -11,10 +11,11 @@ namespace cosv {
 using KernelFn = void (*)(const KParams);
 
 template <int DT, bool AL>
-KernelFn draw_kernel_of(bool ens, int channels) {
-  if (!ens) return cos_draw_kernel<DT, false, 2, AL>;
-  if (channels == 2) return cos_draw_kernel<DT, true, 2, AL>;
-  return channels == 4 ? cos_draw_kernel<DT, true, 4, AL> : cos_draw_kernel<DT, true, 8, AL>;
+KernelFn draw_kernel_of(bool ens, int channels, bool pair, bool masked) {
+  if (!ens && pair) return masked ? cos_draw_kernel<DT, false, 2, AL, 3> : cos_draw_kernel<DT, false, 2, AL, 1>;
+  if (!ens) return masked ? cos_draw_kernel<DT, false, 2, AL, 2> : cos_draw_kernel<DT, false, 2, AL, 0>;
+  if (channels == 2) return cos_draw_kernel<DT, true, 2, AL, 0>;
+  return channels == 4 ? cos_draw_kernel<DT, true, 4, AL, 0> : cos_draw_kernel<DT, true, 8, AL, 0>;
 }
 
 template <int DT, int MODE, bool AL>
@@ -99,7 +100,8 @@ cudaError_t mask_launch(const KParams& p, int threads, cudaStream_t stream) {
 
 template <int DT>
 cudaError_t draw_launch(const KParams& p, bool ens, int channels, int units, int threads, cudaStream_t stream) {
-  KernelFn fn = p.vec_ok ? draw_kernel_of<DT, true>(ens, channels) : draw_kernel_of<DT, false>(ens, channels);
+  const bool pair = p.n == 2, masked = p.mask_model >= 0;
+  KernelFn fn = p.vec_ok ? draw_kernel_of<DT, true>(ens, channels, pair, masked) : draw_kernel_of<DT, false>(ens, channels, pair, masked);
   const size_t fixed = channels == 2 ? sizeof(DrawShared<2>) : (channels == 4 ? sizeof(DrawShared<4>) : sizeof(DrawShared<8>));
   static_assert(sizeof(DrawShared<4>) + 8 * 8 * kMaxDrawThreads <= 48 * 1024 && sizeof(DrawShared<8>) + 8 * 16 * 256 <= 48 * 1024,
                 "no opt-in for large shared memory is made");

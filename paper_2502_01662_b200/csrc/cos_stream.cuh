@@ -36,7 +36,7 @@ struct Finish {  // what a position is decided from, and the decision
     SoftPart fsoft[COS_MAX_MODELS];  // merged statistics (sampling)
     ArgPart farg[COS_MAX_MODELS];    // merged argmaxes (greedy)
   };
-  double pdraft[COS_MAX_MODELS];     // sampling: probability of the draft token under each softmax
+  double pdraft[COS_MAX_MODELS];     // sampling: probability of the draft token under each softmax, NaN where its statistics are of no use
   double inv[COS_MAX_MODELS];        // sampling: one over each normaliser
   float thr;                         // plausibility threshold (NaN: the gating model's logits hold one)
   Decision dec;
@@ -614,7 +614,7 @@ __device__ __forceinline__ void publish_unit(const KParams& p, int b, int j, int
 template <int DT, int MODE>
 __device__ __forceinline__ void decide_unit(const KParams& p, const Finish& sh, Decision& d, double u_acc, double u_smp, bool is_bonus, int draft, bool draft_ok,
                                             int pi, bool pi_ok, int pis) {
-  const bool mask_bad = (MODE == kLogitSample || MODE == kLogitGreedy) && p.mask_model >= 0 && sh.thr != sh.thr;
+  const bool mask_bad = MODE == kLogitGreedy && p.mask_model >= 0 && sh.thr != sh.thr;
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
   const double kNaN = __longlong_as_double(0x7ff8000000000000LL);
   const double kInf = __longlong_as_double(0x7ff0000000000000LL);
@@ -625,41 +625,31 @@ __device__ __forceinline__ void decide_unit(const KParams& p, const Finish& sh, 
   d.ratio = d.r_d = d.q_d = d.S = d.prob = kNaN;
   bool finite = pi_ok;
   if (kSample) {
-    const int nsoft = (MODE == kEnsembleSample) ? p.n : 2;
+    double r_d = 0.0, q_d;
+    if (MODE == kEnsembleSample) {
 #pragma unroll 1
-    for (int k = 0; k < nsoft; ++k) {
-      const SoftPart& f = sh.fsoft[k];
-      finite = finite && isfinite(f.ref) && isfinite(f.s) && (f.s > 0.0);
+      for (int i = 0; i < p.n; ++i) r_d += p.w64[i] * sh.pdraft[i];
+      q_d = sh.pdraft[pis];
+    } else {
+      q_d = sh.pdraft[0];
+      r_d = sh.pdraft[1];
     }
-    if (mask_bad) finite = false;
+    finite = finite && r_d == r_d && q_d == q_d;
     if (!finite) {
       d.status |= COS_ROW_NONFINITE;
-    } else {
-      if (!is_bonus) {
-        if (draft_ok) {
-          double r_d = 0.0, q_d = 0.0;
-          if (MODE == kEnsembleSample) {
-#pragma unroll 1
-            for (int i = 0; i < p.n; ++i) {
-              r_d += p.w64[i] * sh.pdraft[i];
-              if (i == pi) q_d = sh.pdraft[i];
-            }
-          } else {
-            q_d = sh.pdraft[0];
-            r_d = sh.pdraft[1];
-          }
-          d.r_d = r_d;
-          d.q_d = q_d;
-          if (q_d > 0.0) {
-            d.ratio = r_d / q_d;
-          } else {
-            d.status |= COS_ROW_Q_ZERO;
-            d.ratio = (r_d > 0.0) ? kInf : 0.0;
-          }
-          d.accept = (u_acc <= fmin(1.0, d.ratio)) ? 1 : 0;
+    } else if (!is_bonus) {
+      if (draft_ok) {
+        d.r_d = r_d;
+        d.q_d = q_d;
+        if (q_d > 0.0) {
+          d.ratio = r_d / q_d;
         } else {
-          d.status |= COS_ROW_BAD_DRAFT;
+          d.status |= COS_ROW_Q_ZERO;
+          d.ratio = (r_d > 0.0) ? kInf : 0.0;
         }
+        d.accept = (u_acc <= fmin(1.0, d.ratio)) ? 1 : 0;
+      } else {
+        d.status |= COS_ROW_BAD_DRAFT;
       }
     }
   } else {
@@ -780,14 +770,15 @@ template <int MODE>
 __device__ __forceinline__ int record_slots(const KParams& p) {
   return (MODE == kEnsembleSample || MODE == kEnsembleGreedy) ? p.n : 2;
 }
-// Where the records of position r are: `count` times `slots` of them.
+// Where the records of position j of row b are: `count` times `slots` of them.
 struct RecordRange {
   const int4* first;
   int count;
 };
 template <int MODE>
-__device__ __forceinline__ RecordRange records_of(const KParams& p, int r) {
+__device__ __forceinline__ RecordRange records_of(const KParams& p, int b, int j) {
   const int slots = record_slots<MODE>(p);
+  const int r = b * p.P + j;
   const long long at = static_cast<long long>(r) * p.st_nv;
   const int w0 = worker_of(p, at), w1 = worker_of(p, at + p.st_nv - 1);
   RecordRange q;
@@ -797,9 +788,9 @@ __device__ __forceinline__ RecordRange records_of(const KParams& p, int r) {
 }
 
 // Merge slot i of a position over its records; `g` lanes (a power of two, aligned) share the work, `sub` is the lane's place
-// among them.  Every lane of the warp calls this (one with an empty range only takes part in the exchanges).  The first lane
-// of a group gets the result.  Eight records at a time are on their way, and every sum is rescaled once: one record after
-// another took 10 us for the 148 of each position of a 6-position row.
+// among them.  Every lane of the warp calls this (one with an empty range only takes part in the exchanges).  All lanes of a
+// group get the sums, the first one of them argmaxes.  Four records at a time are on their way, and every sum is rescaled once, to the
+// reference of the whole group: one record after another took 10 us for the 148 of each position of a 6-position row.
 struct Merged {
   SoftPart soft;
   ArgPart arg;
@@ -808,7 +799,7 @@ struct Merged {
 template <int MODE>
 __device__ __forceinline__ Merged merge_slot(const KParams& p, const RecordRange& q, int i, int g, int sub) {
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
-  constexpr int kAtOnce = 8;
+  constexpr int kAtOnce = 4;
   const int slots = record_slots<MODE>(p);
   Merged m;
   m.soft.ref = -INFINITY;
@@ -817,25 +808,44 @@ __device__ __forceinline__ Merged merge_slot(const KParams& p, const RecordRange
   m.arg.idx = kNoReject;
   m.arg.bad = 0;
   m.thr = -INFINITY;
-  for (int c0 = sub; c0 < q.count; c0 += kAtOnce * g) {
-    int4 v4[kAtOnce];
+  int4 v4[kAtOnce];
+  auto fetch = [&](int c0) {
 #pragma unroll
     for (int k = 0; k < kAtOnce; ++k) {
       const int c = c0 + k * g;
       v4[k] = make_int4(0, kSample ? 0 : static_cast<int>(0xfff00000u), kSample ? static_cast<int>(0xff800000u) : kNoReject, 0);
       if (c < q.count) v4[k] = __ldcg(q.first + static_cast<size_t>(c) * slots + i);
     }
-    if (kSample) {
+  };
+  if (kSample) {
+    fetch(sub);
+    if (sub < q.count) m.thr = __int_as_float(v4[0].w);
+#pragma unroll 1
+    for (int c0 = sub;;) {
       float top = m.soft.ref;
 #pragma unroll
       for (int k = 0; k < kAtOnce; ++k) top = fmaxf(top, __int_as_float(v4[k].z));
-      double s = rescale(m.soft.s, m.soft.ref, top);
+      const bool more = __any_sync(0xffffffffu, c0 + kAtOnce * g < q.count);
+      if (!more) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1)
+          if (d < g) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, d));
+      }
+      double s = c0 == sub ? 0.0 : rescale(m.soft.s, m.soft.ref, top);
 #pragma unroll
       for (int k = 0; k < kAtOnce; ++k) s += rescale(__hiloint2double(v4[k].y, v4[k].x), __int_as_float(v4[k].z), top);
       m.soft.s = s;
       m.soft.ref = top;
-      if (c0 == sub) m.thr = __int_as_float(v4[0].w);
-    } else {
+      if (!more) break;
+      c0 += kAtOnce * g;
+      fetch(c0);
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1)
+      if (d < g) m.soft.s += __shfl_xor_sync(0xffffffffu, m.soft.s, d);
+  } else {
+    for (int c0 = sub; c0 < q.count; c0 += kAtOnce * g) {
+      fetch(c0);
 #pragma unroll
       for (int k = 0; k < kAtOnce; ++k) {
         const double v = __hiloint2double(v4[k].y, v4[k].x);
@@ -847,15 +857,6 @@ __device__ __forceinline__ Merged merge_slot(const KParams& p, const RecordRange
         }
       }
     }
-  }
-  if (kSample) {
-    float top = m.soft.ref;
-    for (int d = g / 2; d > 0; d >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, d));
-    double s = rescale(m.soft.s, m.soft.ref, top);
-    for (int d = g / 2; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-    m.soft.s = s;
-    m.soft.ref = top;
-  } else {
     for (int d = g / 2; d > 0; d >>= 1) {
       const double ov = __shfl_xor_sync(0xffffffffu, m.arg.val, d);
       const int oi = __shfl_xor_sync(0xffffffffu, m.arg.idx, d);
@@ -878,39 +879,39 @@ __device__ __forceinline__ float mask_bound(const KParams& p, unsigned key) {
   return __double2float_ru(static_cast<double>(top) + p.ln_alpha);
 }
 
-// Probability of the draft token under softmax i, with the constant the sweep used: what it needs of the logits (fetched early; nothing
-// where draft < 0), and the rest once the statistics are merged.
-struct DraftLogits {
-  float a, b;  // the slot's logit; combined logits: those of models 0 and 1
+// Probability of the draft token under softmax i, with the constant the sweep used: what it needs of the logits (fetched, and combined,
+// before the statistics are there; nothing where draft < 0), and the rest once they are merged.
+struct DraftLogit {
+  double x;    // the softmax's logit
+  float gate;  // what the plausibility threshold is compared with
 };
 template <int DT, int MODE>
-__device__ __forceinline__ DraftLogits draft_logits(const KParams& p, const char* base, int i, int pis, int draft) {
-  DraftLogits d;
-  d.a = d.b = -INFINITY;
+__device__ __forceinline__ DraftLogit draft_logit(const KParams& p, const char* base, int i, int pis, int draft) {
+  DraftLogit d = {0.0, 0.f};
   if (draft < 0) return d;
   const long long row_step = p.s_model * Elem<DT>::bytes;
-  const int first = MODE == kEnsembleSample ? i : (i == 0 ? pis : 0);
-  d.a = Elem<DT>::load1(base + first * row_step, draft);
-  if (MODE == kLogitSample && i == 1 && p.n >= 2) d.b = Elem<DT>::load1(base + row_step, draft);
+  if (MODE == kEnsembleSample || i == 0) {
+    d.x = static_cast<double>(Elem<DT>::load1(base + (MODE == kEnsembleSample ? i : pis) * row_step, draft));
+  } else {
+#pragma unroll 2
+    for (int k = 0; k < p.n; ++k) {
+      const float l = Elem<DT>::load1(base + k * row_step, draft);
+      d.x = k == 0 ? p.w64[0] * static_cast<double>(l) : fma(p.w64[k], static_cast<double>(l), d.x);
+      if (k == p.mask_model) d.gate = l;
+    }
+  }
   return d;
 }
-template <int DT, int MODE>
-__device__ __forceinline__ double draft_probability(const KParams& p, const DraftLogits& d, const char* base, int i, int draft, float thr,
-                                                    const SoftPart& f, double inv) {
-  if (draft < 0) return 0.0;
-  double x = static_cast<double>(d.a);
-  if (MODE == kLogitSample && i == 1) {
-    float gate = p.mask_model == 1 ? d.b : d.a;
-    x = p.w64[0] * x;
-    if (p.n >= 2) x = fma(p.w64[1], static_cast<double>(d.b), x);
-    for (int k = 2; k < p.n; ++k) {
-      const float l = Elem<DT>::load1(base + k * p.s_model * Elem<DT>::bytes, draft);
-      x = fma(p.w64[k], static_cast<double>(l), x);
-      if (k == p.mask_model) gate = l;
-    }
-    if (p.mask_model >= 0 && !(gate >= thr)) return 0.0;
+// NaN where the statistics, or the threshold, are of no use.
+template <int MODE>
+__device__ __forceinline__ double draft_probability(const KParams& p, const DraftLogit& d, int i, int draft, float thr, const SoftPart& f, double inv) {
+  const double nan = __longlong_as_double(0x7ff8000000000000LL);
+  if (!(isfinite(f.ref) && isfinite(f.s) && f.s > 0.0)) return nan;
+  if (MODE == kLogitSample && p.mask_model >= 0) {
+    if (thr != thr) return nan;
+    if (i == 1 && !(d.gate >= thr)) return 0.0;
   }
-  return exp2(x * p.cT64 - static_cast<double>(f.ref)) * inv;
+  return draft < 0 ? 0.0 : exp2(d.x * p.cT64 - static_cast<double>(f.ref)) * inv;
 }
 
 // Largest logit of the gating model at every position, for the plausibility mask: the same split, over that model's rows
@@ -1056,15 +1057,15 @@ __device__ __forceinline__ void decide_and_publish(const KParams& p, Finish& fin
   const int draft = is_bonus ? 0 : __ldg(p.drafts + b * p.gamma + j);
   const bool draft_ok = is_bonus || (draft >= 0 && draft < p.V);
   const int at = is_bonus || !draft_ok ? -1 : draft;
-  DraftLogits d = {0.f, 0.f};
-  if (kSample && i < slots && lane % g == 0) d = draft_logits<DT, MODE>(p, base, i, pis, at);  // (asked for before the records are)
+  DraftLogit d = {0.0, 0.f};
+  if (kSample && i < slots && lane % g == 0) d = draft_logit<DT, MODE>(p, base, i, pis, at);  // (asked for before the records are)
   const float thr = masked ? mask_bound(p, __ldcg(&p.mask_key[uidx])) : -INFINITY;
   if (i >= slots) q.count = 0;
   const Merged m = merge_slot<MODE>(p, q, i, g, lane % g);
   if (i < slots && lane % g == 0) {
     if (kSample) {
       fin.fsoft[i] = m.soft;
-      fin.pdraft[i] = draft_probability<DT, MODE>(p, d, base, i, at, thr, m.soft, 1.0 / m.soft.s);
+      fin.pdraft[i] = draft_probability<MODE>(p, d, i, at, thr, m.soft, 1.0 / m.soft.s);
     } else {
       fin.farg[i] = m.arg;
     }
@@ -1114,7 +1115,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) cos_report_kernel(const __g
     const int pi = kEns ? 0 : proposer_of(p, b, j);
     const int pis = (pi >= 0 && pi < p.n) ? pi : 0;
     sweep_part<DT, MODE, true, PAIR, false>(p, base, o0, o1, 0, p.n, pis, -INFINITY, p.st_rec + (static_cast<size_t>(r) + w) * slots, waited);
-    const RecordRange q = records_of<MODE>(p, r);
+    const RecordRange q = records_of<MODE>(p, b, j);
     int prev = 0;
     if (lane == 0) {
       __threadfence();
