@@ -246,10 +246,17 @@ def run_reference(args, w):
     print(json.dumps(line))
 
 
+def launches_of(info):
+    """Kernels of one ordinary call of a full batch."""
+    return 1 if info["rows_at_once"] else info["launches_per_run"]
+
+
 def kernel_names(w, info):
     """What the launches of one call are (for the roofline's stage list)."""
     if info["one_launch"]:
         return ["cos_fused_kernel (every position: sweep, accept tests, row scan, token draw)"]
+    if info["rows_at_once"]:
+        return ["cos_row_kernel (every position swept, accept tests, row scan, token draw)"]
     if w.temperature == 0.0:
         return ["cos_stream_kernel (every position swept) with cos_decide_kernel (accept tests, row scan)"]
     if info.get("draw_items"):
@@ -323,7 +330,7 @@ def measure_workload(w, dev, local, steps, warmup, row_base=0, sampler=None, clu
             v2.close()
     res = {"us_per_call": 1e6 * per_call, "positions_per_s": w.positions / per_call, "GBps": nbytes / per_call / 1e9,
            "frac": nbytes / per_call / 1e9 / peak, "frac_of_nominal_8TBps": nbytes / per_call / 1e9 / NOMINAL_HBM_GBS,
-           "bytes_per_call": nbytes, "launches_per_call": info["launches_per_run"], "stages": stages,
+           "bytes_per_call": nbytes, "launches_per_call": launches_of(info), "stages": stages,
            "buffers": len(sets), "one_launch": info["one_launch"],
            "inputs_settled": {"us_per_call": 1e6 * t_settled / settled_steps,
                               "frac": nbytes / (t_settled / settled_steps) / 1e9 / peak,
@@ -484,7 +491,7 @@ def main():
             k2 = 400 if ww.positions * ww.bytes_per_position < (1 << 30) else 100
             res, _, _, inf2, s2 = measure_workload(ww, dev, local, k2, 5, stage_runs=20, try_one_launch=True)
             del s2
-            extra_launches += (k2 + 5 + 25) * inf2["launches_per_run"]
+            extra_launches += (k2 + 5 + 25) * launches_of(inf2)
             if name == "cfg2":
                 res.update(sustained_small_calls(ww, dev, local))
             res["three_streams"] = three_streams(ww, dev, local)
@@ -524,7 +531,7 @@ def main():
                      # not the headline either: independent calls on three contexts and streams overlap one call's
                      # drawing launch with another's streaming launch
                      "three_streams": (table or {}).get(w.name, {}).get("three_streams")},
-        "gpu_launches": args.steps * info["launches_per_run"],
+        "gpu_launches": args.steps * launches_of(info),
         "clocks": sampler.summary() if sampler else None,
     }
     if e2e:

@@ -159,7 +159,8 @@ typedef struct {
   int32_t threads_per_block;
   int32_t max_clusters;      /* positions under way at once on the device                             */
   int32_t sm_count;
-  int32_t launches_per_run;  /* kernels an ordinary cos_verify_run enqueues: 1 where the one-launch form was    */
+  int32_t launches_per_run;  /* kernels an ordinary cos_verify_run enqueues where its rows are not all at work at */
+                             /* once (reserved[2] bit 2: there it is one): 1 where the one-launch form was        */
                              /* chosen (reserved[2] bit 0); else 2, 3 for ensembles of one or of more than     */
                              /* four models at T > 0, and one more with a plausibility mask.  Every            */
                              /* launch takes its places on the device while the kernel before it in    */
@@ -167,7 +168,8 @@ typedef struct {
                              /* until it is complete (unless COS_RUN_INPUTS_SETTLED says the inputs may be read) */
   int32_t reserved[3];       /* [0], [1]: work items per position when streaming / drawing; [2]: bit  */
                              /* 0: an ordinary run is one launch; bit 1: the tokens of a staged run   */
-                             /* are drawn by the persistent kernel's drawing items                    */
+                             /* are drawn by the persistent kernel's drawing items; bit 2: an ordinary */
+                             /* run of max_batch aligned rows has them all at work at once, in one launch */
 } cos_verify_info;
 
 /*

@@ -174,6 +174,7 @@ class CosVerifier:
         out["items_per_position"], out["draw_items_per_position"] = inf.reserved[0], inf.reserved[1]
         out["one_launch"] = bool(inf.reserved[2] & 1)
         out["draw_items"] = bool(inf.reserved[2] & 2)   # tokens are drawn by the persistent kernel's drawing items
+        out["rows_at_once"] = bool(inf.reserved[2] & 4)  # a run of max_batch aligned rows is one launch, a cluster of blocks a row
         return out
 
     def _fill_args(self, logits, drafts, proposer, seed, offset, row_base, flags, outs,

@@ -81,6 +81,7 @@ struct KParams {
   int st_workers, st_nv, st_share;
   int st_split;            // ensembles: shares of a position, each model's a warp of its own; 0: a warp sweeps all models of its share
   int st_warps;            // warps of the launch
+  int st_row;              // > 0: every row is a line of its own, in this many shares (st_workers, st_warps and st_line are a row's, too)
   long long st_line;
   double st_inv_nv, st_inv_share;  // one over them, for divisions
   int slot_inv;            // 65536 over the records of a (share, position) pair, rounded up: likewise

@@ -36,14 +36,23 @@ struct RowShared {
   int draft[kTile];  // the draft tokens of the tile
 };
 
-// What the merge and the accept tests of a tile need of the inputs, fetched before the records are there.
+// What the merge and the accept tests of a tile need of the inputs, asked for before the records are there.
 struct TileInputs {
   RecordRange range;  // the thread's pair
-  DraftLogit d;
-  int at;             // its draft token
+  int at, pair_pi;    // its draft token and proposer
+  DraftLogit d;       // (tile_logits)
   int draft, pi;      // the lane's position
   unsigned word0, word1;
 };
+// A load that stays where it is, before what takes long.
+__device__ __forceinline__ int load_now(const int* at) {
+  int v;
+  asm volatile("ld.global.nc.s32 %0, [%1];" : "=r"(v) : "l"(at));
+  return v;
+}
+__device__ __forceinline__ int proposer_now(const KParams& p, int b, int j) {  // (see proposer_of)
+  return j == p.gamma && p.bonus_model >= 0 ? p.bonus_model : load_now(p.proposer + (p.per_pos ? b * p.P + j : b));
+}
 struct TilePlan {  // pairs of (position, slot) and the lanes that share one: as many as the block has to spare (a thread for each at least)
   int lg, pos, slot, sub;
 };
@@ -68,31 +77,35 @@ __device__ __forceinline__ TileInputs tile_inputs(const KParams& p, const TilePl
   in.d = {0.0, 0.f};
   in.range = {nullptr, 0};
   in.at = -1;
-  if (t.pos < count) {
-    const int j = j0 + t.pos;
-    in.range = records_of<MODE>(p, b, j);
-    if (kSample && t.sub == 0 && j < p.gamma) {
-      in.at = __ldg(p.drafts + b * p.gamma + j);
-      if (in.at >= p.V) in.at = -1;
-      const int pi = (MODE == kLogitSample) ? proposer_of(p, b, j) : 0;
-      const char* base = reinterpret_cast<const char*>(p.logits) +
-                         (static_cast<long long>(b) * p.s_row + static_cast<long long>(j) * p.s_pos) * Elem<DT>::bytes;
-      in.d = draft_logit<DT, MODE>(p, base, t.slot, (pi >= 0 && pi < p.n) ? pi : 0, in.at);
-    }
+  in.pair_pi = in.draft = in.pi = 0;
+  const bool mine = kSample && t.pos < count && t.sub == 0 && j0 + t.pos < p.gamma;
+  if (mine) {
+    in.at = load_now(p.drafts + b * p.gamma + j0 + t.pos);
+    if (MODE == kLogitSample) in.pair_pi = proposer_now(p, b, j0 + t.pos);
   }
-  in.draft = in.pi = 0;
-  unsigned rnd[4] = {0u, 0u, 0u, 0u};
+  const int j = j0 + threadIdx.x;
   if (threadIdx.x < count) {
-    const int j = j0 + threadIdx.x;
-    if (j < p.gamma) in.draft = __ldg(p.drafts + b * p.gamma + j);
-    in.pi = proposer_of(p, b, j);
-    philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
+    if (j < p.gamma) in.draft = load_now(p.drafts + b * p.gamma + j);
+    in.pi = proposer_now(p, b, j);
   }
+  if (t.pos < count) in.range = records_of<MODE>(p, b, j0 + t.pos);
+  unsigned rnd[4] = {0u, 0u, 0u, 0u};
+  if (threadIdx.x < count)
+    philox4x32_10(static_cast<unsigned>(p.row_base + b), static_cast<unsigned>(j), offset_lo(p), offset_hi(p), p.seed_lo, p.seed_hi, rnd);
   in.word0 = rnd[0];
   in.word1 = rnd[1];
-  // (all of it now, not where it is used)
-  asm volatile("" : "+r"(in.word0), "+r"(in.word1), "+l"(in.range.first), "+r"(in.range.count), "+d"(in.d.x), "+f"(in.d.gate), "+r"(in.pi), "+r"(in.draft));
+  asm volatile("" : "+r"(in.word0), "+r"(in.word1), "+l"(in.range.first), "+r"(in.range.count));  // (now, not where it is used)
   return in;
+}
+// The logits at the draft tokens, of tile_inputs.
+template <int DT, int MODE>
+__device__ __forceinline__ void tile_logits(const KParams& p, const TilePlan& t, int b, int j0, TileInputs& in) {
+  if (MODE != kEnsembleSample && MODE != kLogitSample) return;
+  const char* base = reinterpret_cast<const char*>(p.logits) +
+                     (static_cast<long long>(b) * p.s_row + static_cast<long long>(j0 + t.pos) * p.s_pos) * Elem<DT>::bytes;
+  if (in.at >= p.V) in.at = -1;
+  in.d = draft_logit<DT, MODE>(p, base, t.slot, (in.pair_pi >= 0 && in.pair_pi < p.n) ? in.pair_pi : 0, in.at);
+  asm volatile("" : "+d"(in.d.x), "+f"(in.d.gate));
 }
 
 // Decide row b, sampling.  `want` >= 0: a position whose statistics the block needs, whatever the first rejection; otherwise the first
@@ -114,6 +127,7 @@ __device__ __forceinline__ void decide_sampled(const KParams& p, RowShared& sh, 
     const int count = p.P - j0 < kTile ? p.P - j0 : kTile;
     if (j0 > 0) in = tile_inputs<DT, MODE>(p, t, b, j0);
     if (tid < count) sh.draft[tid] = in.draft;
+    tile_logits<DT, MODE>(p, t, b, j0, in);
     if (j0 == 0) ready();
     {
       const Merged m = merge_slot<MODE>(p, in.range, t.slot, 1 << t.lg, t.sub);

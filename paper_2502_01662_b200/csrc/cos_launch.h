@@ -22,6 +22,12 @@ cudaError_t mask_launch(const KParams& p, int threads, cudaStream_t stream);
 // threads for each.
 template <int DT>
 cudaError_t draw_launch(const KParams& p, bool ensemble, int channels, int units, int threads, cudaStream_t stream);
+// A run in one launch (cos_row.cuh): a cluster of p.draw_parts blocks for each of the p.B rows.
+constexpr int kRowThreads = 512, kRowParts = 16, kRowSums = 2048;  // threads of a block, most blocks of a cluster, chunks times channels
+template <int DT>
+cudaError_t row_launch(const KParams& p, int mode, int channels, cudaStream_t stream);
+// Clusters of `parts` such blocks that the current device holds at once; 0: it takes none.
+int row_clusters(int parts);
 // Test hook: the combined distribution of every position.
 template <int DT>
 cudaError_t dump_launch(const KParams& p, int mode, cudaStream_t stream);

@@ -778,18 +778,18 @@ struct RecordRange {
 template <int MODE>
 __device__ __forceinline__ RecordRange records_of(const KParams& p, int b, int j) {
   const int slots = record_slots<MODE>(p);
-  const int r = b * p.P + j;
-  const long long at = static_cast<long long>(r) * p.st_nv;
+  // (where every row has a line of its own, the records of a row follow those of the row before)
+  const long long at = static_cast<long long>(p.st_row ? j : b * p.P + j) * p.st_nv;
   const int w0 = worker_of(p, at), w1 = worker_of(p, at + p.st_nv - 1);
   RecordRange q;
-  q.first = p.st_rec + (static_cast<size_t>(r) + w0) * slots;
+  q.first = p.st_rec + (static_cast<size_t>(b) * (p.P + p.st_row) + j + w0) * slots;
   q.count = w1 - w0 + 1;
   return q;
 }
 
 // Merge slot i of a position over its records; `g` lanes (a power of two, aligned) share the work, `sub` is the lane's place
 // among them.  Every lane of the warp calls this (one with an empty range only takes part in the exchanges).  All lanes of a
-// group get the sums, the first one of them argmaxes.  Four records at a time are on their way, and every sum is rescaled once, to the
+// group get the sums, the first one of them argmaxes.  Four records or eight at a time are on their way, and every sum is rescaled once, to the
 // reference of the whole group: one record after another took 10 us for the 148 of each position of a 6-position row.
 struct Merged {
   SoftPart soft;
@@ -799,7 +799,7 @@ struct Merged {
 template <int MODE>
 __device__ __forceinline__ Merged merge_slot(const KParams& p, const RecordRange& q, int i, int g, int sub) {
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
-  constexpr int kAtOnce = 4;
+  constexpr int kAtOnce = kSample ? 4 : 8;  // (argmaxes are compared one after the other, so that fewer trips count for more)
   const int slots = record_slots<MODE>(p);
   Merged m;
   m.soft.ref = -INFINITY;

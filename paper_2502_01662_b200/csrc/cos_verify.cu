@@ -9,10 +9,12 @@
 //   drawing    merge them, take the accept tests in fp64, find every row's first rejection, write the row's outputs
 //              (cos_decide.cuh; at T = 0 that is all), and draw the row's token: one more sweep of the one position that
 //              needs it (cos_draw.cuh).
+// Runs whose rows have their places on the device side by side, each on a cluster of blocks, are one launch that does all of it
+// (cos_row.cuh, plan_row).
 // Blocks wait for one another only at the hardware barrier of their cluster.
 //
 // This file is the host side of the library (contexts, launches, the C entry points).  The kernels are compiled in
-// cos_bf16.cu, cos_f16.cu and cos_f32.cu; cos_common.cuh holds constants, launch parameters, loads, Philox and softmax
+// cos_bf16.cu, cos_f16.cu and cos_f32.cu (those of cos_row.cuh in cos_row_*.cu); cos_common.cuh holds constants, launch parameters, loads, Philox and softmax
 // partials, cos_fused.cu the persistent one-launch kernel, cos_probe.cu the two streaming ceilings.
 
 #include <mutex>
@@ -36,6 +38,7 @@ thread_local std::string g_create_error;
 struct cos_verify_ctx {
   cos_verify_config cfg;
   int sm_count;
+  int clusters[kRowParts + 1];  // clusters of so many blocks that the device holds at once
   unsigned* d_work_counter;
   bool scratch_dirty;
   int4* d_st_rec;
@@ -275,6 +278,75 @@ cudaError_t launch_stream(const cos_verify_config& c, int mode, KParams& p, long
   });
 }
 
+// Runs of one launch: a cluster of blocks a row, all rows at once (cos_row.cuh).  Whether this one is, and its plan.  `clusters[k]`:
+// clusters of k blocks that the device holds at once.
+// A row has the largest clusters of which the device holds one for each row (16 blocks up to 7 rows, 6 for 16, 4 for 33, 2 for 48 on a B200).
+// That leaves multiprocessors idle which the launches of whole batches use, so it pays where a block's part is small (`mine`: its vectors)
+// or little is left idle (`spread`: vectors for each multiprocessor if all of them shared the work).  Device time in us of the launches
+// apart and of this one (5 positions; models x vocabulary, bf16):
+//   two models sampled: 1 row of 2 x 128256 15.1 and 14.9, of 6 x 2 x 151936 16.2 and 17.6, 7 of 2 x 32000 17.0 and 14.9, of 2 x 128256 23.3 and
+//     16.7, 33 of 2 x 128256 38.6 and 34.8, 48 of 2 x 64000 32.0 and 34.6;
+//   four: 1 row of 4 x 32000 15.9 and 17.6, 7 of 4 x 64000 24.9 and 20.7, 12 of them 26.4 and 30.9;
+//   logit level: 7 rows of 2 x 128256 27.4 and 17.3, with a mask 33.8 and 21.1, 48 of them 49.5 and 55.1, with a mask 67.2 and 71.6, 48 of
+//     2 x 64000 36.8 and 35.0; 16 of 3 x 64000 with a mask 40.0 and 37.1, 24 of 3 x 128256 59.4 and 64.9;
+//   greedy (little to save but launches): 4 rows of 2 x 32000 6.3 and 7.4, of 2 x 128256 9.7 and 8.1, 24 of 2 x 64000 12.0 and 13.1; logit
+//     level: 1 row of 2 x 32000 7.6 and 7.9, 4 of 2 x 128256 13.3 and 9.8, with a mask 18.9 and 13.0.
+bool plan_row(const cos_verify_config& c, const int* clusters, int sm_count, KParams& p) {
+  const int mode = mode_of(c), ch = draw_channels(c);
+  if (c.cluster_size > 0 || (mode == kEnsembleSample && (c.n < 2 || c.n > 4))) return false;
+  int parts = 0;
+  for (int k = 1; k <= kRowParts; ++k)
+    if (clusters[k] >= p.B) parts = k;
+  if (parts == 0 || p.B * parts > sm_count) return false;
+  // (vectors of unaligned rows cost half as much again)
+  const long long row = static_cast<long long>(c.n) * p.P * (c.vocab / entries_per_vec(c.dtype)) * (p.vec_ok ? 2 : 3) / 2;
+  const long long mine = row / parts, spread = row * p.B / sm_count, beyond = mine - spread * 17 / 20;
+  switch (mode) {
+    case kEnsembleSample:
+      if (ch == 2 ? beyond > 10000 : mine > 10000 || spread < 2500) return false;
+      break;
+    case kLogitSample:
+      if (beyond > (c.n == 2 ? 18000 : 12000)) return false;
+      break;
+    case kEnsembleGreedy:
+      if (spread < 3000 || beyond > 4500) return false;
+      break;
+    default:
+      if (spread < 2000 || beyond > 8000) return false;
+  }
+  const int warps = parts * (kRowThreads / 32);
+  plan_line(p, c, p.P, c.combine == COS_COMBINE_PROB_ENSEMBLE ? c.n : 1, warps, parts);
+  p.st_row = p.st_workers;
+  p.draw_parts = parts;
+  const int steps = (p.nsteps + warps - 1) / warps, room = kRowSums / ch / warps;  // steps and records of a warp
+  p.draw_chunks = (steps + 7) / 8 < room ? (steps + 7) / 8 : room;
+  p.draw_cs = (steps + p.draw_chunks - 1) / p.draw_chunks;
+  return true;
+}
+
+// What plan_row asks of a device, once for each (for runs without a context; a context keeps its own).
+constexpr int kMaxDevices = 64;
+struct DeviceShape {
+  int sm_count, clusters[kRowParts + 1];
+};
+cudaError_t device_shape(int device, DeviceShape* out) {
+  static DeviceShape shapes[kMaxDevices];
+  static std::mutex guard;
+  std::lock_guard<std::mutex> lock(guard);
+  DeviceShape fresh = {};
+  DeviceShape& d = device >= 0 && device < kMaxDevices ? shapes[device] : fresh;
+  if (d.sm_count == 0) {
+    for (int k = 1; k <= kRowParts; ++k) d.clusters[k] = row_clusters(k);
+    const cudaError_t e = cudaDeviceGetAttribute(&d.sm_count, cudaDevAttrMultiProcessorCount, device);
+    if (e != cudaSuccess) {
+      d.sm_count = 0;
+      return e;
+    }
+  }
+  *out = d;
+  return cudaSuccess;
+}
+
 // The launches that draw the tokens: of every position (`all`: test hook, residual masses) or of one per row.
 cudaError_t launch_draw(const cos_verify_config& c, KParams& p, bool all, int sm_count, cudaStream_t stream) {
   const bool ens = c.combine == COS_COMBINE_PROB_ENSEMBLE;
@@ -394,6 +466,13 @@ extern "C" cos_status cos_verify_create(const cos_verify_config* config, cos_ver
     return cuda_fail(nullptr, "cudaGetDeviceProperties", e);
   }
   ctx->sm_count = prop.multiProcessorCount;
+  DeviceShape shape;
+  e = device_shape(config->device, &shape);
+  if (e != cudaSuccess) {
+    delete ctx;
+    return cuda_fail(nullptr, "cudaDeviceGetAttribute", e);
+  }
+  memcpy(ctx->clusters, shape.clusters, sizeof(shape.clusters));
   const size_t rows = static_cast<size_t>(config->max_batch), P = static_cast<size_t>(config->gamma) + 1;
   bool ok = true;
   ok = ok && cudaMalloc(&ctx->d_work_counter, 256) == cudaSuccess;
@@ -565,6 +644,16 @@ cos_status run_launches(cos_verify_ctx* ctx, const cos_verify_args* a, void* cud
   p.use_jobs = by_items ? 1 : 0;
   const long long workers = stream_workers(c, p.num_units, ctx->sm_count);
   if (a->dump_r != nullptr || !early_exit_pays(c, p.num_units, ctx->sm_count)) p.early_exit = 0;
+  if (!p.early_exit && !by_items && !all && a->dump_r == nullptr && plan_row(c, ctx->clusters, ctx->sm_count, p)) {
+    p.lse = a->lse;
+    *lse_done = p.lse != nullptr;
+    e = by_dtype(c.dtype, [&](auto dt) { return row_launch<decltype(dt)::value>(p, mode, draw_channels(c), stream); });
+    if (e != cudaSuccess) return cuda_fail(ctx, "kernel launch (rows at once)", e);
+    if (ctx->timing) cudaEventRecord(ctx->ev[1], stream);
+    ctx->ev_used = 2;
+    ctx->scratch_dirty = false;
+    return COS_OK;
+  }
   const bool report = p.early_exit || by_items;
   p.lse = report ? nullptr : a->lse;
   *lse_done = p.lse != nullptr;
@@ -784,7 +873,14 @@ extern "C" cos_status cos_verify_get_info(const cos_verify_ctx* ctx, cos_verify_
   }
   info->reserved[0] = ctx->fused ? ctx->fplan.chunks : 1;
   info->reserved[1] = ctx->fused ? ctx->fplan.dchunks : 1;
-  info->reserved[2] = ((ctx->fused && ctx->use_fused) ? 1 : 0) | ((ctx->fused && ctx->draw_fused) ? 2 : 0);
+  KParams p = {};
+  p.B = ctx->cfg.max_batch;
+  p.P = ctx->cfg.gamma + 1;
+  p.vec_ok = 1;
+  p.nsteps = (ctx->cfg.vocab + 32 * entries_per_vec(ctx->cfg.dtype) - 1) / (32 * entries_per_vec(ctx->cfg.dtype));
+  const bool staged = !ctx->fused || !(ctx->use_fused || ctx->draw_fused);
+  info->reserved[2] = ((ctx->fused && ctx->use_fused) ? 1 : 0) | ((ctx->fused && ctx->draw_fused) ? 2 : 0) |
+                      (staged && plan_row(ctx->cfg, ctx->clusters, ctx->sm_count, p) ? 4 : 0);
   return COS_OK;
 }
 
@@ -892,9 +988,10 @@ extern "C" cos_status cos_verify_run_static(const cos_verify_config* config, con
       g_static_ready[c.device] = true;
     }
   }
-  int sm_count = 0;
-  e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, c.device);
+  DeviceShape shape;
+  e = device_shape(c.device, &shape);
   if (e != cudaSuccess) return cuda_fail(nullptr, "cudaDeviceGetAttribute", e);
+  const int sm_count = shape.sm_count;
 
   // carve the array; what must start clean comes first and is cleared on the caller's stream before the kernels
   const bool draws = c.temperature > 0.0f;
@@ -923,6 +1020,11 @@ extern "C" cos_status cos_verify_run_static(const cos_verify_config* config, con
   p.mask_key = d_mask_key;
   p.row_draw = d_row_draw;
 
+  if (!all && a->dump_r == nullptr && sm_count * (kRowThreads / 32) <= kStaticWorkers && plan_row(c, shape.clusters, sm_count, p)) {
+    e = by_dtype(c.dtype, [&](auto dt) { return row_launch<decltype(dt)::value>(p, mode_of(c), draw_channels(c), stream); });
+    if (e != cudaSuccess) return cuda_fail(nullptr, "kernel launch (rows at once)", e);
+    return COS_OK;
+  }
   long long workers = stream_workers(c, units, sm_count);
   if (workers > kStaticWorkers) workers = kStaticWorkers;
   p.keep_stats = (a->dump_r != nullptr || decides_first(c)) ? 1 : 0;
