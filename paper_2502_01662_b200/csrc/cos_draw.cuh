@@ -345,7 +345,7 @@ __device__ __noinline__ void slow_vector(const KParams& p, const DrawConst& kc, 
 
 // The steps [s_lo, s_hi) of a position by one warp, in chunks of cs steps: per channel the sum over the tokens with a positive mass,
 // for every chunk NCH sums to the records from the rec-th on, and to part the normaliser's share, of all chunks together (both in the cluster's first block).
-// The fast loop adds vectors up in fp32 and leaves those with a big entry, and the ragged ends, to slow_vector.
+// The fast loop adds vectors up in fp32, up to 32 of a lane, and leaves those with a big entry, and the ragged ends, to slow_vector.
 // What bounds it: instruction issue (counted at logit level, 128 rows of 256000 tokens: 211 instructions a step, 0.53 of the issue
 // slots of the average multiprocessor, 0.67 of the busiest).  Loads in flight do not: fetching a step as soon as a place is free,
 // so that two are always on their way, gained nothing with two channels and lost 2 to 7 % with four.
@@ -357,6 +357,11 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
   constexpr int NP = NCH / 2;
   constexpr int NR = ENS ? NCH : 2;         // vectors of a step kept in registers
   constexpr int US = (NR == 2) ? 2 : 1;     // steps fetched at a time
+  // Slow vectors are finished where they are, which is the shorter chain, or behind the (up to 32) steps that have them, fetched again, where
+  // the call in the loop costs registers.  Where they are and behind, device time in us: two models, 64 rows of 9 x 151936 80.7 and 81.6, one
+  // row 16.1 and 16.8; three, 16 rows of 6 x 50001 unaligned 32.2 and 33.0; four, 32 rows of 7 x 128256 65.2 and 62.5; logit level, 200 rows of
+  // 5 x 2 x 128256 138.5 and 136.8, 48 of 3 x 128256 with a mask 94.7 and 88.0.
+  constexpr bool kLater = !ENS || NCH == 8 || (NCH == 4 && AL);
   const int lane = threadIdx.x & 31;
   const f32x2 c2 = pack2(p.cT, p.cT);
   const VecRange whole = whole_vectors<DT, AL>(p.V);
@@ -380,9 +385,12 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
     f32x2 zc[NP], ac[NP];
 #pragma unroll
     for (int q = 0; q < NP; ++q) zc[q] = ac[q] = pack2(0.f, 0.f);
-    {
 #pragma unroll 1
-      for (int s = begin; s < end; s += US) {
+    for (int c = begin; c < end; c += 32) {  // (not more in fp32)
+      const int ce = c + 32 < end ? c + 32 : end;
+      unsigned later = 0u;
+#pragma unroll 1
+      for (int s = c; s < ce; s += US) {
         Vectors<NR> r[US];
 #pragma unroll
         for (int t = 0; t < US; ++t) {
@@ -391,7 +399,7 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
 #pragma unroll
           for (int i = 0; i < NR; ++i) {
             r[t].r[i] = neg_inf_vector<DT>();
-            if (in && s + t < end && i < p.n) r[t].r[i] = load_whole<DT, AL>(base + i * row_step, v);
+            if (in && s + t < ce && i < p.n) r[t].r[i] = load_whole<DT, AL>(base + i * row_step, v);
           }
         }
 #pragma unroll
@@ -421,7 +429,7 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
             // two neighbouring tokens side by side
             f32x2 xq[E / 2], cmb[E / 2];
             const int v = (s + t) * 32 + lane;
-            const bool in = v >= whole.lo && v < whole.hi && s + t < end;
+            const bool in = v >= whole.lo && v < whole.hi && s + t < ce;
             logit_args<DT, PAIR, MASKED>(p, lw, r[t].r[0], r[t].r[1],
                                          [&](int i) {
                                            uint4 m = neg_inf_vector<DT>();
@@ -458,8 +466,12 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
 #pragma unroll
           for (int q = 0; q < NP; ++q) big = big || lo2(vz[q]) > bt[2 * q] || hi2(vz[q]) > bt[2 * q + 1];
           const int v = (s + t) * 32 + lane;
-          const bool ragged = s + t < end && (v < whole.lo || v >= whole.hi) && v * E < p.V;
+          const bool ragged = s + t < ce && (v < whole.lo || v >= whole.hi) && v * E < p.V;
           if (big || ragged) {
+            if (kLater) {
+              later |= 1u << (s + t - c);
+              continue;
+            }
             slow_vector<DT, ENS, NCH, AL, FORM>(p, kc, u, r[t], v, ragged, !slow, acc);
             slow = true;
           } else {
@@ -470,6 +482,28 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
             }
           }
         }
+      }
+      if (kLater) {
+#pragma unroll 1
+        for (; later; later &= later - 1) {
+          Vectors<NR> none;
+#pragma unroll
+          for (int i = 0; i < NR; ++i) none.r[i] = neg_inf_vector<DT>();
+          slow_vector<DT, ENS, NCH, AL, FORM>(p, kc, u, none, (c + __ffs(later) - 1) * 32 + lane, true, !slow, acc);
+          slow = true;
+        }
+      }
+      if (ce < end) {  // (the lane's slots take over)
+        const int T = blockDim.x;
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+          acc[(2 * q) * T] = static_cast<double>(lo2(zc[q])) + (slow ? acc[(2 * q) * T] : 0.0);
+          acc[(2 * q + 1) * T] = static_cast<double>(hi2(zc[q])) + (slow ? acc[(2 * q + 1) * T] : 0.0);
+          acc[(NCH + 2 * q) * T] = static_cast<double>(lo2(ac[q])) + (slow ? acc[(NCH + 2 * q) * T] : 0.0);
+          acc[(NCH + 2 * q + 1) * T] = static_cast<double>(hi2(ac[q])) + (slow ? acc[(NCH + 2 * q + 1) * T] : 0.0);
+          zc[q] = ac[q] = pack2(0.f, 0.f);
+        }
+        slow = true;
       }
     }
     double sums[2 * NCH];

@@ -986,7 +986,16 @@ __device__ __forceinline__ void sweep_part(const KParams& p, const char* base, i
   } else if (MODE == kEnsembleGreedy) {
     for (int i = i0; i < i1; ++i) put(i, pack_arg(arg_segment<DT, AL>(base + i * row_step, v0, v1, ragged, p.V), thr));
   } else if (MODE == kLogitSample) {
-    const LaneSoft2 a = logit_segment<DT, AL, PAIR, MASKED>(p, base, row_step, logit_weights(p, pis, thr), p.cT, v0, v1, ragged);
+    LaneSoft2 a;
+    // (with a mask, which of two vectors is the proposer's is known to the code, not chosen entry by entry: 100 rows of 5 x 2 x 128256
+    // 108.4 and 105.3 us a call; without one it is as fast one way, 256 rows of 9 x 2 x 256000 448.9 and 446.2, and slower the other,
+    // 200 of 5 x 2 x 128256 136.2 and 139.5)
+    if (PAIR && MASKED && pis == 0)
+      a = logit_segment<DT, AL, PAIR, MASKED>(p, base, row_step, logit_weights(p, 0, thr), p.cT, v0, v1, ragged);
+    else if (PAIR && MASKED)
+      a = logit_segment<DT, AL, PAIR, MASKED>(p, base, row_step, logit_weights(p, 1, thr), p.cT, v0, v1, ragged);
+    else
+      a = logit_segment<DT, AL, PAIR, MASKED>(p, base, row_step, logit_weights(p, pis, thr), p.cT, v0, v1, ragged);
     put(0, pack_soft(a.q, thr));
     put(1, pack_soft(a.c, thr));
   } else {
