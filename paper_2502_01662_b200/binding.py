@@ -114,6 +114,24 @@ def load_library(rebuild: bool = False) -> ctypes.CDLL:
     return lib
 
 
+_call = None
+
+
+def load_call():
+    """The call of cos_verify_run on device tensors in native code (csrc/call.cpp); raises if it cannot be opened."""
+    global _call
+    if _call is None:
+        import importlib.util
+
+        import torch  # noqa: F401  (its libraries are what the module links to)
+        load_library()
+        spec = importlib.util.spec_from_file_location("_call", _build.CALL)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _call = module
+    return _call
+
+
 def _dtype_code(torch_dtype) -> int:
     import torch
     if torch_dtype == torch.float32:
@@ -145,6 +163,7 @@ class CosVerifier:
                  device: int = 0, cluster_size: int = 0, host_staging: bool = False):
         self._lib = load_library()
         self._ctx = ctypes.c_void_p()
+        self._callee = None
         cfg = cos_verify_config()
         cfg.n, cfg.combine = n, combine
         for i, w in enumerate(list(weights)[:COS_MAX_MODELS]):
@@ -160,6 +179,9 @@ class CosVerifier:
             msg = self._lib.cos_verify_last_error(None).decode()
             self._ctx = ctypes.c_void_p()
             raise CosVerifyError(st, msg)
+        call = load_call()
+        self._run = call.run
+        self._callee = call.callee(ctypes.cast(self._lib.cos_verify_run, ctypes.c_void_p).value, self._ctx.value, n, gamma + 1, vocab, cfg.dtype)
 
     # -- helpers ---------------------------------------------------------------------
     def _check(self, st: int):
@@ -178,7 +200,7 @@ class CosVerifier:
         return out
 
     def _fill_args(self, logits, drafts, proposer, seed, offset, row_base, flags, outs,
-                   bonus_model=None, offset_device=None, ptr=None) -> cos_verify_args:
+                   bonus_model=None, offset_device=None) -> cos_verify_args:
         n, B, P, V = logits.shape
         # a [B, gamma+1] proposer table selects the per-position form; a bonus model selects its flag
         if proposer.dim() == 2:
@@ -197,8 +219,7 @@ class CosVerifier:
             raise ValueError("the vocabulary axis of logits must be contiguous")
         if _dtype_code(logits.dtype) != self._dtype:
             raise ValueError("logits dtype does not match the context")
-        if ptr is None:
-            ptr = {k: outs[k].data_ptr() for k in _OUTPUTS if k in outs}
+        ptr = {k: outs[k].data_ptr() for k in _OUTPUTS if k in outs}
         get = ptr.get
         return cos_verify_args(
             logits.data_ptr(), sm, sr, sp, drafts.data_ptr() if (drafts is not None and drafts.numel() > 0) else None,
@@ -257,6 +278,13 @@ class CosVerifier:
         include "bonus_prob" [B]: the bonus token's probability under the law it was drawn from.
         `offset_device` (a one-element int64 device tensor) replaces `offset`: the kernels read it, so a
         run captured in a CUDA graph can be replayed with a new offset each time."""
+        if outs is None and stream is None and not (diag or dump_r or lse) and self._callee is not None:
+            got = self._run(self._callee, logits, drafts, proposer, seed, offset, row_base, flags, bonus_model, offset_device)
+            if type(got) is dict:
+                return got
+            if got is not None:
+                self._check(got)
+        # (what does not fit there, and whatever there is to complain about)
         import torch
         if not logits.is_cuda:
             raise ValueError("run() needs device tensors; use run_host() for host tensors")
@@ -267,22 +295,15 @@ class CosVerifier:
         if (proposer is not None and proposer.numel() > 0 and
                 (proposer.dtype is not i32 or not proposer.is_contiguous() or not proposer.is_cuda)):
             raise ValueError("proposer must be a contiguous int32 device tensor")
-        ptr = None
         if outs is None:
             n, B, P, V = logits.shape
-            if diag or dump_r or lse:
-                outs = self._alloc_outs(B, P, V, logits.device, diag, dump_r)
-                if lse:     # log-sum-exp behind every softmax of a position: [B, gamma+1, n] (ensemble) or [B, gamma+1, 2]
-                    slots = self.cfg.n if self.cfg.combine == COS_COMBINE_PROB_ENSEMBLE else 2
-                    outs["lse"] = torch.empty((B, P, slots), dtype=torch.float32, device=logits.device)
-            else:
-                buf = logits.new_empty(B * (P + 3), dtype=i32)
-                outs = self._small_outs(buf, B, P)
-                at, b4 = buf.data_ptr(), 4 * B
-                ptr = {"accept_count": at, "row_status": at + b4, "bonus_prob": at + 2 * b4, "out_tokens": at + 3 * b4}
+            outs = self._alloc_outs(B, P, V, logits.device, diag, dump_r)
+            if lse:     # log-sum-exp behind every softmax of a position: [B, gamma+1, n] (ensemble) or [B, gamma+1, 2]
+                slots = self.cfg.n if self.cfg.combine == COS_COMBINE_PROB_ENSEMBLE else 2
+                outs["lse"] = torch.empty((B, P, slots), dtype=torch.float32, device=logits.device)
         if offset_device is not None and (offset_device.dtype != torch.int64 or not offset_device.is_cuda):
             raise ValueError("offset_device must be an int64 device tensor")
-        a = self._fill_args(logits, drafts, proposer, seed, offset, row_base, flags, outs, bonus_model, offset_device, ptr)
+        a = self._fill_args(logits, drafts, proposer, seed, offset, row_base, flags, outs, bonus_model, offset_device)
         s = _current_stream(torch, logits.get_device()) if stream is None else stream.cuda_stream
         st = self._lib.cos_verify_run(self._ctx, ctypes.byref(a), s)
         if st != COS_OK:
@@ -308,6 +329,7 @@ class CosVerifier:
         return outs
 
     def close(self):
+        self._callee = None
         if getattr(self, "_ctx", None) is not None and self._ctx.value:
             self._lib.cos_verify_destroy(self._ctx)
             self._ctx = ctypes.c_void_p()

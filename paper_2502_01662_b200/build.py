@@ -1,4 +1,4 @@
-"""Builds libcos_verify.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds libcos_verify.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and _call.so, the call from Python, with g++."""
 from __future__ import annotations
 
 import glob
@@ -6,6 +6,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
@@ -13,6 +14,7 @@ ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(PKG_DIR, "libcos_verify.so")
+CALL = os.path.join(PKG_DIR, "_call.so")
 OBJ_DIR = os.path.join(PKG_DIR, "_build")
 
 
@@ -28,13 +30,13 @@ def sources():
 
 
 def dependencies():
-    return sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))) + [os.path.join(INCLUDE, "cos_verify.h")]
+    return sources() + [os.path.join(CSRC, "call.cpp")] + sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))) + [os.path.join(INCLUDE, "cos_verify.h")]
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALL):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALL))
     return any(os.path.getmtime(d) > t for d in dependencies())
 
 
@@ -50,6 +52,19 @@ def _compile(src: str, verbose: bool):
     return obj, res.stdout + res.stderr
 
 
+def _compile_call():
+    import torch
+    inc = os.path.join(os.path.dirname(torch.__file__), "include")
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(nvcc_path())), "include")
+    cmd = ["g++", "-O2", "-std=c++20", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI, "-I", INCLUDE, "-isystem", inc,
+           "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"), "-isystem", cuda, "-isystem", sysconfig.get_paths()["include"], "-o", CALL,
+           os.path.join(CSRC, "call.cpp"), "-L", lib, "-Wl,-rpath," + lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed:\n" + " ".join(cmd) + "\n" + res.stdout + res.stderr)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile the CUDA library if it is missing or older than its sources; return its path.
     Every csrc/*.cu is one translation unit; they are compiled side by side and linked into one library."""
@@ -57,8 +72,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
         return LIB
     os.makedirs(OBJ_DIR, exist_ok=True)
     srcs = sources()
-    with ThreadPoolExecutor(max_workers=len(srcs)) as pool:
+    with ThreadPoolExecutor(max_workers=len(srcs) + 1) as pool:
+        call = pool.submit(_compile_call)
         done = list(pool.map(lambda s: _compile(s, verbose), srcs))
+        call.result()
     cmd = [nvcc_path(), "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-Xcompiler", "-fPIC", "-o", LIB]
     cmd += [obj for obj, _ in done] + ["-lcudart"]
     res = subprocess.run(cmd, capture_output=True, text=True)
