@@ -37,7 +37,6 @@ struct Finish {  // what a position is decided from, and the decision
     ArgPart farg[COS_MAX_MODELS];    // merged argmaxes (greedy)
   };
   double pdraft[COS_MAX_MODELS];     // sampling: probability of the draft token under each softmax, NaN where its statistics are of no use
-  double inv[COS_MAX_MODELS];        // sampling: one over each normaliser
   float thr;                         // plausibility threshold (NaN: the gating model's logits hold one)
   Decision dec;
 };
