@@ -211,6 +211,14 @@ __device__ __forceinline__ double word_to_uniform(unsigned w) {
   return (2.0 * static_cast<double>(w >> 9) + 1.0) * 5.9604644775390625e-08;  // 2^-24
 }
 
+// Eq. 6: u <= min(1, r / q), 0 < u < 1, from the probabilities of the draft token (q = 0: the ratio is infinite, or 0 where r is 0 too).  Without the
+// quotient, which costs the decisions 0.3 us (contrastive decoding of 8 rows of 32000 tokens 18.1 and 18.4 us).  Both sides are taken far from
+// the subnormal numbers first: there the product rounds to 0, or up to r, and lets pass what the ratio rules out.
+__device__ __forceinline__ bool accepts(double u, double r_d, double q_d) {
+  const double up = 0x1p300;  // (probabilities: nothing overflows)
+  return q_d > 0.0 ? u * (q_d * up) <= r_d * up : r_d > 0.0;
+}
+
 __device__ __forceinline__ double shfl_double(double x, int src) {
   int lo = __double2loint(x), hi = __double2hiint(x);
   lo = __shfl_sync(0xffffffffu, lo, src);

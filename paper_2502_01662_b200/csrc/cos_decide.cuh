@@ -13,7 +13,7 @@ namespace cosv {
 // blocks; one of them writes the outputs.
 // What bounds it: a chain of latencies, the same the second time that a block goes through it (so not of instructions fetched for the first
 // time).  So what it needs of the inputs (drafts, proposers, the logits at the drafts, random words) is there before it waits for the
-// streaming launch to end, nothing is read from global memory after the records, the tests multiply where they could divide, and the
+// streaming launch to end, nothing is read from global memory after the records, and the
 // lane of the position to be drawn has all that is needed to draw it.  (With what follows in the drawing launch, device time of a call:
 // one row of 5 x 2 x 32000 fp32 14.8 us before and 12.7 now, 32 rows of 6 x 2 x 32000 bf16 25.0 and 22.6.)
 constexpr int kTile = 16;  // positions decided at a time
@@ -155,8 +155,7 @@ __device__ __forceinline__ void decide_sampled(const KParams& p, RowShared& sh, 
         r_d = f[1].p;
       }
       const bool finite = pi_ok && r_d == r_d && q_d == q_d, tested = finite && !is_bonus && draft_ok;
-      // u <= min(1, r / q), u < 1
-      const bool accept = tested && (q_d > 0.0 ? word_to_uniform(in.word0) * q_d <= r_d : r_d > 0.0);
+      const bool accept = tested && accepts(word_to_uniform(in.word0), r_d, q_d);
       const unsigned stops = __ballot_sync(0xffffffffu, lane < count && !accept);  // (the bonus position accepts nothing)
       const bool known = a >= 0;
       if (!known && stops) a = j0 + __ffs(stops) - 1;

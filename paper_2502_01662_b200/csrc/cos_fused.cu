@@ -846,7 +846,7 @@ __device__ __forceinline__ void finish_position(const FParams& fp, int b, int j,
         status |= COS_ROW_Q_ZERO;
         ratio = (rr > 0.0) ? kInf : 0.0;
       }
-      accept = (un.u_acc <= fmin(1.0, ratio)) ? 1 : 0;
+      accept = accepts(un.u_acc, rr, qq) ? 1 : 0;
     } else {
       status |= COS_ROW_BAD_DRAFT;
     }

@@ -646,7 +646,7 @@ __device__ __forceinline__ void decide_unit(const KParams& p, const Finish& sh, 
           d.status |= COS_ROW_Q_ZERO;
           d.ratio = (r_d > 0.0) ? kInf : 0.0;
         }
-        d.accept = (u_acc <= fmin(1.0, d.ratio)) ? 1 : 0;
+        d.accept = accepts(u_acc, r_d, q_d) ? 1 : 0;
       } else {
         d.status |= COS_ROW_BAD_DRAFT;
       }
