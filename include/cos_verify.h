@@ -82,20 +82,21 @@ enum {
                                      /* logits for every multiprocessor, or more (0.76 GB on a B200);    */
                                      /* smaller runs have most positions under way at once, and read     */
                                      /* them all.                                                        */
-  COS_RUN_INPUTS_SETTLED = 16        /* a promise by the caller: logits, draft_tokens and proposer were  */
-                                     /* complete in device memory before the work that precedes this     */
-                                     /* call in its stream was submitted (they are not written by the    */
-                                     /* kernel queued just before the call).  The streaming launch may   */
-                                     /* then read them while that work drains - the drawing launch of    */
-                                     /* the previous call, for one - and waits for it only before it     */
-                                     /* touches anything else (an offset in device memory included);     */
-                                     /* calls queued back to back overlap.                               */
-                                     /* Outputs and results are those of an ordinary run.  Without the   */
-                                     /* flag a run reads nothing before the work ahead of it in the      */
-                                     /* stream is complete.  Taken by cos_verify_run at T > 0 for runs   */
-                                     /* of at least one position and at most one row per multiprocessor, */
-                                     /* without mask, test hook, COS_RUN_ALL_RESIDUALS or early exit;    */
-                                     /* ignored otherwise (cos_verify_get_info does not tell).           */
+  COS_RUN_INPUTS_SETTLED = 16        /* a promise by the caller: the work queued just before this call   */
+                                     /* in its stream (a kernel, a copy, or a call of this library) does */
+                                     /* not write logits, draft_tokens or proposer; what lies before     */
+                                     /* that may.  The launch that reads the logits (of a run of one     */
+                                     /* launch: that one) may then read them while the work just ahead   */
+                                     /* drains - the drawing launch of the previous call, for one - and  */
+                                     /* waits for it only before it touches anything else (an offset in  */
+                                     /* device memory included); no later call starts before it has      */
+                                     /* waited.  Calls queued back to back overlap.  Outputs and results */
+                                     /* are those of an ordinary run.  Without the flag a run reads      */
+                                     /* nothing before the work ahead of it in the stream is complete.   */
+                                     /* Taken by cos_verify_run at T > 0 for runs of at least one        */
+                                     /* position and at most one row per multiprocessor, without mask,   */
+                                     /* test hook, COS_RUN_ALL_RESIDUALS or early exit; ignored          */
+                                     /* otherwise (cos_verify_get_info does not tell).                   */
 };
 
 typedef struct {

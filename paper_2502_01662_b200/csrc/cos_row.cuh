@@ -93,11 +93,15 @@ __global__ void __launch_bounds__(kRowThreads, 1) cos_row_kernel(const __grid_co
   double* acc = slots + threadIdx.x;
   const int b = blockIdx.x / p.draw_parts, rank = blockIdx.x % p.draw_parts, nw = blockDim.x >> 5, warp = threadIdx.x >> 5;
   if (kSample) fill_const<DT>(p, sh.kc);
-  // (where the caller promises that the inputs were complete earlier, a warp waits for the kernel ahead only before it writes; the
-  // promise does not cover an offset in device memory)
-  bool waited = p.inputs_settled == 0 || p.off_dev != nullptr;
-  if (waited) asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // Where the caller promises that the inputs are not what the kernel ahead writes, a warp waits for that one only before it writes itself;
+  // the promise does not cover an offset in device memory.  Nor does it cover what may run beside the kernel ahead, if that let this one
+  // start early: so the call behind may start only when every block of this one has waited.
+  const bool settled = p.inputs_settled != 0 && p.off_dev == nullptr;
+  bool waited = !settled;
+  if (!settled) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
   const TilePlan t = tile_plan<MODE>(p);
   const TileInputs in = tile_inputs<DT, MODE>(p, t, b, 0);
   if (kMasked) {
@@ -107,6 +111,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) cos_row_kernel(const __grid_co
   }
   for (int w = rank * nw + warp; w < p.st_warps; w += p.draw_parts * nw) row_share<DT, MODE, AL, kPair, kMasked>(p, b, w, waited);
   if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (settled) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   cluster_arrive();  // (the records of this block are there, and its shared memory may be written to)
   if (kSample) {
     if (!decide_unit_to_draw<DT, kEns, NCH>(p, sh, rs, t, in, b, -1, rank, [] { cluster_wait(); })) return;
