@@ -118,18 +118,21 @@ _call = None
 
 
 def load_call():
-    """The call of cos_verify_run on device tensors in native code (csrc/call.cpp); raises if it cannot be opened."""
+    """The call of cos_verify_run on device tensors in native code (csrc/call.cpp).  None, and a warning the first time, where it cannot be
+    built or opened: the same call goes the long way then."""
     global _call
     if _call is None:
         import importlib.util
-
-        import torch  # noqa: F401  (its libraries are what the module links to)
-        load_library()
-        spec = importlib.util.spec_from_file_location("_call", _build.CALL)
-        module = importlib.util.module_from_spec(spec)
-        spec.loader.exec_module(module)
-        _call = module
-    return _call
+        import warnings
+        try:
+            import torch  # noqa: F401  (its libraries are what the module links to)
+            spec = importlib.util.spec_from_file_location("_call", _build.build_call())
+            _call = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(_call)
+        except Exception as e:
+            _call = False
+            warnings.warn(f"calls from Python go the long way, without csrc/call.cpp: {e}", RuntimeWarning, stacklevel=2)
+    return _call or None
 
 
 def _dtype_code(torch_dtype) -> int:
@@ -180,8 +183,9 @@ class CosVerifier:
             self._ctx = ctypes.c_void_p()
             raise CosVerifyError(st, msg)
         call = load_call()
-        self._run = call.run
-        self._callee = call.callee(ctypes.cast(self._lib.cos_verify_run, ctypes.c_void_p).value, self._ctx.value, n, gamma + 1, vocab, cfg.dtype)
+        if call is not None:
+            self._run = call.run
+            self._callee = call.callee(ctypes.cast(self._lib.cos_verify_run, ctypes.c_void_p).value, self._ctx.value, n, gamma + 1, vocab, cfg.dtype)
 
     # -- helpers ---------------------------------------------------------------------
     def _check(self, st: int):

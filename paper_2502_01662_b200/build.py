@@ -1,7 +1,8 @@
-"""Builds libcos_verify.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and _call.so, the call from Python, with g++."""
+"""Builds libcos_verify.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the module _call, the call from Python, with g++."""
 from __future__ import annotations
 
 import glob
+import importlib.metadata
 import os
 import shutil
 import subprocess
@@ -14,7 +15,7 @@ ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(PKG_DIR, "libcos_verify.so")
-CALL = os.path.join(PKG_DIR, "_call.so")
+CALL_SOURCE = os.path.join(CSRC, "call.cpp")
 OBJ_DIR = os.path.join(PKG_DIR, "_build")
 
 
@@ -30,14 +31,25 @@ def sources():
 
 
 def dependencies():
-    return sources() + [os.path.join(CSRC, "call.cpp")] + sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))) + [os.path.join(INCLUDE, "cos_verify.h")]
+    return sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))) + [os.path.join(INCLUDE, "cos_verify.h")]
+
+
+def _stale(path: str, deps) -> bool:
+    return not os.path.exists(path) or any(os.path.getmtime(d) > os.path.getmtime(path) for d in deps)
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(CALL):
-        return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(CALL))
-    return any(os.path.getmtime(d) > t for d in dependencies())
+    return _stale(LIB, dependencies())
+
+
+def call_path() -> str:
+    """Where the module of csrc/call.cpp for this interpreter and this torch is: it holds inline code of both, so that one made for others is
+    not to be opened.  Raises PackageNotFoundError without torch."""
+    return os.path.join(PKG_DIR, "_call.%s.torch-%s.so" % (sysconfig.get_config_var("SOABI"), importlib.metadata.version("torch")))
+
+
+def call_needs_build() -> bool:
+    return _stale(call_path(), [CALL_SOURCE, os.path.join(INCLUDE, "cos_verify.h")])
 
 
 def _compile(src: str, verbose: bool):
@@ -52,17 +64,27 @@ def _compile(src: str, verbose: bool):
     return obj, res.stdout + res.stderr
 
 
-def _compile_call():
+def _compile_call(out: str):
     import torch
     inc = os.path.join(os.path.dirname(torch.__file__), "include")
     lib = os.path.join(os.path.dirname(torch.__file__), "lib")
     cuda = os.path.join(os.path.dirname(os.path.dirname(nvcc_path())), "include")
     cmd = ["g++", "-O2", "-std=c++20", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI, "-I", INCLUDE, "-isystem", inc,
-           "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"), "-isystem", cuda, "-isystem", sysconfig.get_paths()["include"], "-o", CALL,
-           os.path.join(CSRC, "call.cpp"), "-L", lib, "-Wl,-rpath," + lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+           "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"), "-isystem", cuda, "-isystem", sysconfig.get_paths()["include"], "-o", out,
+           CALL_SOURCE, "-L", lib, "-Wl,-rpath," + lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError("g++ failed:\n" + " ".join(cmd) + "\n" + res.stdout + res.stderr)
+
+
+def build_call(force: bool = False) -> str:
+    """Compile the module of csrc/call.cpp if there is none for this interpreter and this torch, or an older one; return its path."""
+    path = call_path()
+    if force or call_needs_build():
+        fresh = "%s.%d" % (path, os.getpid())
+        _compile_call(fresh)
+        os.replace(fresh, path)  # (another process may be at it too)
+    return path
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -72,10 +94,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         return LIB
     os.makedirs(OBJ_DIR, exist_ok=True)
     srcs = sources()
-    with ThreadPoolExecutor(max_workers=len(srcs) + 1) as pool:
-        call = pool.submit(_compile_call)
+    with ThreadPoolExecutor(max_workers=len(srcs)) as pool:
         done = list(pool.map(lambda s: _compile(s, verbose), srcs))
-        call.result()
     cmd = [nvcc_path(), "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-Xcompiler", "-fPIC", "-o", LIB]
     cmd += [obj for obj, _ in done] + ["-lcudart"]
     res = subprocess.run(cmd, capture_output=True, text=True)
@@ -89,3 +109,4 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 if __name__ == "__main__":
     print(build(force=True, verbose="-v" in sys.argv))
+    print(build_call(force=True))
