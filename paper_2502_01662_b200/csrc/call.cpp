@@ -7,6 +7,7 @@
 #include <ATen/ops/empty.h>
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <new>
@@ -62,7 +63,8 @@ PyObject* run(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   }
   const Callee* c = static_cast<Callee*>(PyCapsule_GetPointer(a[0], kCapsule));
   if (!c) return nullptr;
-  try {
+  HANDLE_TH_ERRORS  // (what the allocation of the outputs raises is what torch raises from Python)
+  {
     if (!THPVariable_CheckExact(a[1]) || !plain_int32(a[3])) Py_RETURN_NONE;
     const at::Tensor &logits = THPVariable_Unpack(a[1]), &proposer = THPVariable_Unpack(a[3]);
     if (!logits.is_cuda() || logits.layout() != at::kStrided || logits.dim() != 4 || logits.scalar_type() != c->dtype) Py_RETURN_NONE;
@@ -136,10 +138,8 @@ PyObject* run(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
       Py_XDECREF(t);
     }
     return d;
-  } catch (const std::exception& e) {
-    if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, e.what());
-    return nullptr;
   }
+  END_HANDLE_TH_ERRORS
 }
 
 PyMethodDef methods[] = {{"callee", callee, METH_VARARGS, "a context, for run"},
