@@ -96,7 +96,8 @@ __global__ void __launch_bounds__(kRowThreads, 1) cos_row_kernel(const __grid_co
   // Where the caller promises that the inputs are not what the kernel ahead writes, a warp waits for that one only before it writes itself;
   // the promise does not cover an offset in device memory.  Nor does it cover what may run beside the kernel ahead, if that let this one
   // start early: so the call behind may start only when every block of this one has waited.
-  const bool settled = p.inputs_settled != 0 && p.off_dev == nullptr;
+  // (With a mask the promise is not taken; left open to the compiler it costs the masked sweep 4 to 8 %: 60 rows of 5 x 2 x 64000 46.3 us and 43.1.)
+  const bool settled = !kMasked && p.inputs_settled != 0 && p.off_dev == nullptr;
   bool waited = !settled;
   if (!settled) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
