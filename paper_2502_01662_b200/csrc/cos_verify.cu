@@ -283,14 +283,22 @@ cudaError_t launch_stream(const cos_verify_config& c, int mode, KParams& p, long
 // A row has the largest clusters of which the device holds one for each row (16 blocks up to 7 rows, 6 for 16, 4 for 33, 2 for 48 on a B200).
 // That leaves multiprocessors idle which the launches of whole batches use, so it pays where a block's part is small (`mine`: its vectors)
 // or little is left idle (`spread`: vectors for each multiprocessor if all of them shared the work).  Device time in us of the launches
-// apart and of this one (5 positions; models x vocabulary, bf16):
-//   two models sampled: 1 row of 2 x 128256 15.1 and 14.9, of 6 x 2 x 151936 16.2 and 17.6, 7 of 2 x 32000 17.0 and 14.9, of 2 x 128256 23.3 and
-//     16.7, 33 of 2 x 128256 38.6 and 34.8, 48 of 2 x 64000 32.0 and 34.6;
-//   four: 1 row of 4 x 32000 15.9 and 17.6, 7 of 4 x 64000 24.9 and 20.7, 12 of them 26.4 and 30.9;
-//   logit level: 7 rows of 2 x 128256 27.4 and 17.3, with a mask 33.8 and 21.1, 48 of them 49.5 and 55.1, with a mask 67.2 and 71.6, 48 of
-//     2 x 64000 36.8 and 35.0; 16 of 3 x 64000 with a mask 40.0 and 37.1, 24 of 3 x 128256 59.4 and 64.9;
-//   greedy (little to save but launches): 4 rows of 2 x 32000 6.3 and 7.4, of 2 x 128256 9.7 and 8.1, 24 of 2 x 64000 12.0 and 13.1; logit
-//     level: 1 row of 2 x 32000 7.6 and 7.9, 4 of 2 x 128256 13.3 and 9.8, with a mask 18.9 and 13.0.
+// apart and of this one (5 positions; models x vocabulary, bf16 where nothing is said; some 1300 calls of 1 to 148 rows, every type, were compared):
+//   two models sampled: 1 row of 2 x 128256 15.6 and 15.8, of 6 x 2 x 151936 16.2 and 17.6, 7 of 2 x 32000 17.6 and 15.4, of 2 x 128256 24.1 and
+//     17.7, 33 of 2 x 128256 39.0 and 35.9, 48 of 2 x 64000 32.2 and 36.1;
+//   three and four: 1 row of 4 x 32000 16.3 and 18.2, 7 of 4 x 64000 24.1 and 21.3, 12 of them 26.1 and 31.2; with 50 positions shares of four models no
+//     longer end where positions do, 7 rows of 4 x 4000 22.3 and 29.8;
+//   logit level: 7 rows of 2 x 128256 26.8 and 18.6, with a mask 33.5 and 22.6, 48 of them 48.4 and 55.0, with a mask 62.2 and 71.2, 48 of
+//     2 x 64000 35.7 and 34.7; 124 of 3 x 2 x 71936 with a mask 64.9 and 68.0; 16 of 3 x 64000 with a mask 40.1 and 36.5; 24 of 3 x 64000 33.8 and
+//     35.1, 25 of 8 x 3 x 47488 fp16 39.3 and 44.0; 57 of 9 x 1 x 57664 fp16 41.5 and 44.1;
+//   greedy (little to save but launches): 12 rows of 2 x 32000 7.4 and 7.7, 16 of them 8.8 and 7.7, 24 of 2 x 64000 12.1 and 13.1; logit
+//     level: 4 rows of 2 x 64000 7.9 and 8.6, 7 of them 9.6 and 8.7, with a mask 14.9 and 11.6; 24 of 3 x 64000 20.0 and 25.8.
+// Unaligned rows, whose vectors are cut out of two, keep a block busy for as long again (fp32 twice as long): two models of 50001, 16 rows 25.2 and 22.8, 24
+// rows 27.2 and 28.7, fp32 12 rows 26.5 and 26.0, 16 rows 30.5 and 38.0; logit level 24 rows 29.5 and 27.7, 33 rows 34.5 and 36.2, with a mask in
+// fp32 12 rows 35.0 and 32.4, 16 rows 37.6 and 49.7; greedy 16 rows 14.2 and 13.1, 24 rows 15.5 and 18.1.  With nothing idle it pays further (74 rows, two
+// blocks each, 62.1 and 59.6; fp32 85.4 and 99.2).
+// A position takes a warp its round trips, however few vectors it has, and a vocabulary of next to nothing leaves a few warps with all of them: one row of
+// 500 positions of 2 x 7 at logit level 19 and 558, of 2 x 100 18.9 and 88.9; of two models of 1000 15.2 and 22.2.
 bool plan_row(const cos_verify_config& c, const int* clusters, int sm_count, KParams& p) {
   const int mode = mode_of(c), ch = draw_channels(c);
   if (c.cluster_size > 0 || (mode == kEnsembleSample && (c.n < 2 || c.n > 4))) return false;
@@ -298,24 +306,41 @@ bool plan_row(const cos_verify_config& c, const int* clusters, int sm_count, KPa
   for (int k = 1; k <= kRowParts; ++k)
     if (clusters[k] >= p.B) parts = k;
   if (parts == 0 || p.B * parts > sm_count) return false;
-  // (vectors of unaligned rows cost half as much again)
-  const long long row = static_cast<long long>(c.n) * p.P * (c.vocab / entries_per_vec(c.dtype)) * (p.vec_ok ? 2 : 3) / 2;
-  const long long mine = row / parts, spread = row * p.B / sm_count, beyond = mine - spread * 17 / 20;
+  const long long pairs = static_cast<long long>(c.n) * p.P, nv = c.vocab / entries_per_vec(c.dtype);
+  const long long mine = pairs * (nv < 192 ? 192 : nv) / parts, spread = pairs * nv * p.B / sm_count, beyond = mine - spread * 17 / 20;
+  const bool full = (mine - spread) * 16 <= spread;                // nothing idle
+  const long long further = c.dtype != COS_DTYPE_F32 ? 47000 : 0;  // (unaligned rows)
+  bool pays;
   switch (mode) {
     case kEnsembleSample:
-      if (ch == 2 ? beyond > 10000 : mine > 10000 || spread < 2500) return false;
+      if (ch == 2)
+        pays = p.vec_ok ? beyond <= 10000 : mine <= 12000 || (full && mine <= further);
+      else
+        pays = p.P <= 16 && spread >= 2500 && mine <= (p.vec_ok ? 10000 : 8000);
       break;
     case kLogitSample:
-      if (beyond > (c.n == 2 ? 18000 : 12000)) return false;
+      if (!p.vec_ok)
+        pays = mine <= (c.n > 2 ? 18000 : (spread <= 8000 ? 17000 : 14000)) || (full && mine <= further);
+      else if (c.n == 2)
+        pays = beyond <= (c.mask_model < 0 || parts >= 6 ? 18000 : 14000);
+      else
+        pays = beyond <= (c.n == 1 ? 9000 : (c.mask_model >= 0 || parts >= 6 || full ? 12000 : 7300));
       break;
     case kEnsembleGreedy:
-      if (spread < 3000 || beyond > 4500) return false;
+      pays = spread >= 3500 && (p.vec_ok ? beyond <= 4500 : mine <= 8000);
       break;
     default:
-      if (spread < 2000 || beyond > 8000) return false;
+      if (!p.vec_ok)
+        pays = spread >= 1600 && mine <= 12000 && mine - 2 * spread <= 2500;
+      else if (c.n <= 2)
+        pays = spread >= 2500 && beyond <= 8000;
+      else
+        pays = mine - 2 * spread <= 500 && mine - spread * 3 / 5 <= (c.dtype != COS_DTYPE_F32 && spread <= 10000 ? 7500 : 6200);
   }
+  if (!pays) return false;
   const int warps = parts * (kRowThreads / 32);
   plan_line(p, c, p.P, c.combine == COS_COMBINE_PROB_ENSEMBLE ? c.n : 1, warps, parts);
+  if (p.P > 4 * p.st_workers) return false;
   p.st_row = p.st_workers;
   p.draw_parts = parts;
   const int steps = (p.nsteps + warps - 1) / warps, room = kRowSums / ch / warps;  // steps and records of a warp
