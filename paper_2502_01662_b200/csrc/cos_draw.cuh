@@ -279,8 +279,8 @@ __device__ __noinline__ double big_mass(const DrawConst& p, const DrawUnit<NCH>&
   return exact_mass<ENS, NCH>(p, d, inv, u.pis, u.law);
 }
 
-// A lane's vector v that the fast loop left out: one with a big entry, which is summed in fp64 then, or one at a ragged end of the
-// row (fetched here).  The sums go to the lane's slots of `acc`, which are cleared where `first`.  Out of line.  (What the fast loop had
+// A lane's vector v that the fast loop left out: one with a big entry, or one at a ragged end of the row (fetched here).  Every entry is added in
+// fp64, and a big one's exponential is fp64 too.  The sums go to the lane's slots of `acc`, which are cleared where `first`.  Out of line.  (What the fast loop had
 // left out, put off until the end of 32 steps, fetched again and dealt out over the warp entry by entry, took a warp 1400 cycles for every
 // step that had any.)
 template <int DT, bool ENS, int NCH, bool AL, int FORM>
@@ -294,10 +294,14 @@ __device__ __noinline__ void slow_vector(const KParams& p, const DrawConst& kc, 
     for (int i = 0; i < NR; ++i)
       if (i < kc.n) rv.r[i] = load_vector<DT, AL>(u.base + i * kc.row_step, v, kc.V, whole);
   }
-  float x[NCH][E], z[NCH], a[NCH];
+  float x[NCH][E];
   vector_args<DT, ENS, NCH, AL, FORM>(p, kc, u, rv, v, x);
+  double sz[NCH], sa[NCH];
 #pragma unroll
-  for (int i = 0; i < NCH; ++i) z[i] = a[i] = 0.f;
+  for (int i = 0; i < NCH; ++i) {
+    sz[i] = first ? 0.0 : acc[i * T];
+    sa[i] = first ? 0.0 : acc[(NCH + i) * T];
+  }
   unsigned bigbits = 0u, inbits = 0u;
 #pragma unroll
   for (int k = 0; k < E; ++k) {
@@ -313,15 +317,9 @@ __device__ __noinline__ void slow_vector(const KParams& p, const DrawConst& kc, 
     if (ENS || x[1][k] != -INFINITY) inbits |= 1u << k;
 #pragma unroll
     for (int i = 0; i < NCH; ++i) {
-      z[i] += big ? 0.f : f[i];
-      a[i] += !big && tot > 0.f ? f[i] : 0.f;
+      sz[i] += big ? 0.0 : static_cast<double>(f[i]);
+      sa[i] += !big && tot > 0.f ? static_cast<double>(f[i]) : 0.0;
     }
-  }
-  double sz[NCH], sa[NCH];
-#pragma unroll
-  for (int i = 0; i < NCH; ++i) {
-    sz[i] = static_cast<double>(z[i]) + (first ? 0.0 : acc[i * T]);
-    sa[i] = static_cast<double>(a[i]) + (first ? 0.0 : acc[(NCH + i) * T]);
   }
 #pragma unroll 1
   for (; bigbits; bigbits &= bigbits - 1) {
