@@ -341,6 +341,68 @@ __device__ __noinline__ void slow_vector(const KParams& p, const DrawConst& kc, 
   }
 }
 
+// The vectors of steps c to c + 31 that the fast loop left out (bit k of a lane's `left`: its vector of step c + k), of an ensemble: the warp takes 32
+// of their entries at a time, one a lane, and adds them to the lanes' slots of `acc`.  Out of line.
+template <int DT, int NCH>
+__device__ __noinline__ void slow_entries(const DrawConst& p, const DrawUnit<NCH>& u, int c, unsigned left, double* acc) {
+  constexpr int E = Elem<DT>::E, G = 32 / E;
+  const int T = blockDim.x, lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (unsigned any = __reduce_or_sync(0xffffffffu, left); any; any &= any - 1) {
+    const int k = __ffs(any) - 1;
+    unsigned m = __ballot_sync(0xffffffffu, (left >> k) & 1u);
+#pragma unroll 1
+    while (m) {
+      unsigned t = m;
+#pragma unroll
+      for (int q = 0; q < G; ++q) {
+        if (q < lane / E) t &= t - 1;
+        m &= m - 1;
+      }
+      const int e = t ? ((c + k) * 32 + __ffs(t) - 1) * E + lane % E : p.V;
+      if (e >= p.V) continue;
+      float x[NCH], tot = 0.f;
+      double d[NCH];
+      bool big = false;
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) {
+        x[i] = -INFINITY;
+        if (i < p.n) x[i] = Elem<DT>::load1(u.base + i * p.row_step, e);
+      }
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) {
+        const float f = ex2_approx(fmaf(x[i], p.cT, u.nref[i]));
+        big = big || f > u.bt[i];
+        tot = __fadd_rn(tot, __fmul_rn(u.ct[i], f));
+        d[i] = static_cast<double>(f);
+      }
+      bool counts = tot > 0.f;
+      if (big) {
+#pragma unroll 1
+        for (int q = 0; q < NCH; ++q) {  // (one copy of the exponential)
+          double v = 0.0;
+#pragma unroll
+          for (int i = 0; i < NCH; ++i)
+            if (i == q) v = static_cast<double>(x[i]) * p.cT64 + static_cast<double>(u.nref[i]);
+          v = exp2(v);
+#pragma unroll
+          for (int i = 0; i < NCH; ++i)
+            if (i == q) d[i] = v;
+        }
+        double t64 = 0.0;
+#pragma unroll
+        for (int i = 0; i < NCH; ++i) t64 = __dadd_rn(t64, __dmul_rn(u.ck[i], d[i]));
+        counts = t64 > 0.0;
+      }
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) {
+        acc[i * T] += d[i];
+        if (counts) acc[(NCH + i) * T] += d[i];
+      }
+    }
+  }
+}
+
 // The steps [s_lo, s_hi) of a position by one warp, in chunks of cs steps: per channel the sum over the tokens with a positive mass,
 // for every chunk NCH sums to the records from the rec-th on, and to part the normaliser's share, of all chunks together (both in the cluster's first block).
 // The fast loop adds vectors up in fp32, up to 32 of a lane, and leaves those with a big entry, and the ragged ends, to slow_vector.
@@ -358,8 +420,10 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
   // Slow vectors are finished where they are, which is the shorter chain, or behind the (up to 32) steps that have them, fetched again, where
   // the call in the loop costs registers.  Where they are and behind, device time in us: two models, 64 rows of 9 x 151936 80.7 and 81.6, one
   // row 16.1 and 16.8; three, 16 rows of 6 x 50001 unaligned 32.2 and 33.0; four, 32 rows of 7 x 128256 65.2 and 62.5; logit level, 200 rows of
-  // 5 x 2 x 128256 138.5 and 136.8, 48 of 3 x 128256 with a mask 94.7 and 88.0.
-  constexpr bool kLater = !ENS || NCH == 8 || (NCH == 4 && AL);
+  // 5 x 2 x 128256 138.5 and 136.8, 48 of 3 x 128256 with a mask 94.7 and 88.0.  Eight channels entry by entry over the warp (`kShared`), with nothing live across
+  // the call: by the lane that left a vector out the kernel spilled 400 bytes a thread around it, and five models took, by the lane and over
+  // the warp, 7 rows of 5 x 32000 47.1 and 37.5, 40 of 50001 120.4 and 106.5, the same in fp32 165.9 and 145.5, 60 of 64000 99.8 and 102.1.
+  constexpr bool kShared = ENS && NCH == 8, kLater = kShared || !ENS || (NCH == 4 && AL);
   const int lane = threadIdx.x & 31;
   const f32x2 c2 = pack2(p.cT, p.cT);
   const VecRange whole = whole_vectors<DT, AL>(p.V);
@@ -481,7 +545,21 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
           }
         }
       }
-      if (kLater) {
+      if constexpr (kShared) {
+        if (__any_sync(0xffffffffu, later != 0u)) {
+          const int T = blockDim.x;
+#pragma unroll
+          for (int q = 0; q < NP; ++q) {
+            acc[(2 * q) * T] = static_cast<double>(lo2(zc[q])) + (slow ? acc[(2 * q) * T] : 0.0);
+            acc[(2 * q + 1) * T] = static_cast<double>(hi2(zc[q])) + (slow ? acc[(2 * q + 1) * T] : 0.0);
+            acc[(NCH + 2 * q) * T] = static_cast<double>(lo2(ac[q])) + (slow ? acc[(NCH + 2 * q) * T] : 0.0);
+            acc[(NCH + 2 * q + 1) * T] = static_cast<double>(hi2(ac[q])) + (slow ? acc[(NCH + 2 * q + 1) * T] : 0.0);
+            zc[q] = ac[q] = pack2(0.f, 0.f);
+          }
+          slow = true;
+          slow_entries<DT, NCH>(kc, u, c, later, acc);
+        }
+      } else if (kLater) {
 #pragma unroll 1
         for (; later; later &= later - 1) {
           Vectors<NR> none;

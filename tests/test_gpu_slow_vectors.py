@@ -36,3 +36,23 @@ def test_small_tokens_beside_a_big_one_keep_their_bits(combine, n, vocab, cluste
     # half a unit of the last place for the store, and a tenth of one for the few 64-bit operations and the tokens of 2^-200
     assert np.all(np.abs(S - want) <= 0.6 * np.spacing(np.float32(want))), (S - want) / want
     assert np.all(got["accept_count"].cpu().numpy() == 0) and np.all(got["out_tokens"][:, 0].cpu().numpy() < 8)
+
+
+@pytest.mark.parametrize("cluster_size", [0, 1])
+@pytest.mark.parametrize("n,vocab,dtype,sigma", [(3, 4099, "bf16", 6.0), (4, 23, "f32", 2.0), (5, 3, "bf16", 3.0), (5, 4097, "f32", 8.0), (6, 257, "f16", 1.0),
+                                                 (6, 20000, "bf16", 6.0), (7, 23, "f32", 2.0), (8, 9001, "bf16", 8.0), (8, 64, "f16", 0.1), (8, 32768, "f32", 5.0)])
+def test_many_channels_with_many_big_tokens(n, vocab, dtype, sigma, cluster_size):
+    """Nothing but big tokens, a few among many, ragged ends at both sides of a row, several in a warp's vectors at once."""
+    w = synth.Workload("many", n, ENS, tuple([1.0 - 0.125 * (n - 1)] + [0.125] * (n - 1)), 1.0, 6, 3, vocab, dtype, "gauss", sigma=sigma, rho=0.6,
+                       proposer_rule="cycle")
+    inputs = synth.make_inputs(w, "cuda")
+    drafts = inputs["drafts"].clone()
+    drafts[0, 0] = vocab
+    inputs = dict(inputs, drafts=drafts)
+    ref = helpers.run_oracle(w, inputs)
+    v = helpers.make_verifier(w, cluster_size=cluster_size)
+    try:
+        for opts in ({}, {"flags": 1}):     # the token's position alone, and every position's mass
+            helpers.check_parity(w, helpers.run_gpu(w, inputs, verifier=v, diag=True, **opts), ref)
+    finally:
+        v.close()
