@@ -112,8 +112,8 @@ __device__ __forceinline__ void tile_logits(const KParams& p, const TilePlan& t,
 // rejected position is what it needs.  `in`: the inputs of the first tile; `ready()` waits for the records.  `keep(stats, j, proposer,
 // word, accepted, drawable)` is called by one thread of the first warp with that position's merged statistics, its proposer and the
 // random word its token is drawn with.  `writes_row(a)` / `writes_unit(j)`: whether this block writes the row's outputs and a
-// position's optional ones.
-template <int DT, int MODE, typename R, typename K, typename WR, typename WU>
+// position's optional ones.  `AT`: see merge_slot.
+template <int DT, int MODE, int AT, typename R, typename K, typename WR, typename WU>
 __device__ __forceinline__ void decide_sampled(const KParams& p, RowShared& sh, const TilePlan& t, TileInputs in, int b, int want, R ready, K keep,
                                                WR writes_row, WU writes_unit) {
   constexpr bool kEns = (MODE == kEnsembleSample);
@@ -130,7 +130,7 @@ __device__ __forceinline__ void decide_sampled(const KParams& p, RowShared& sh, 
     tile_logits<DT, MODE>(p, t, b, j0, in);
     if (j0 == 0) ready();
     {
-      const Merged m = merge_slot<MODE>(p, in.range, t.slot, 1 << t.lg, t.sub);
+      const Merged m = merge_slot<MODE, AT>(p, in.range, t.slot, 1 << t.lg, t.sub);
       if (t.pos < count && t.sub == 0) {
         PairStats o;
         o.s = m.soft.s;
@@ -230,7 +230,7 @@ __device__ __forceinline__ void decide_greedy(const KParams& p, RowShared& sh, c
     if (tid < count) sh.draft[tid] = in.draft;
     if (j0 == 0) ready();
     {
-      const Merged m = merge_slot<MODE>(p, in.range, t.slot, 1 << t.lg, t.sub);
+      const Merged m = merge_slot<MODE, 8>(p, in.range, t.slot, 1 << t.lg, t.sub);
       if (t.pos < count && t.sub == 0) {
         Finish& f = sh.fin[t.pos];
         f.farg[t.slot] = m.arg;
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(128) cos_decide_kernel(const __grid_constant__
   const TileInputs in = tile_inputs<DT, MODE>(p, t, blockIdx.x, 0);
   auto ready = [] { asm volatile("griddepcontrol.wait;" ::: "memory"); };
   if (MODE == kEnsembleSample)
-    decide_sampled<DT, MODE>(p, sh, t, in, blockIdx.x, -1, ready, [](const PairStats*, int, int, unsigned, int, int) {}, [](int) { return true; },
+    decide_sampled<DT, MODE, 8>(p, sh, t, in, blockIdx.x, -1, ready, [](const PairStats*, int, int, unsigned, int, int) {}, [](int) { return true; },
                              [](int) { return true; });
   else
     decide_greedy<DT, MODE>(p, sh, t, in, blockIdx.x, ready);

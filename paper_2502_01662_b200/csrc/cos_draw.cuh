@@ -903,7 +903,7 @@ __device__ __forceinline__ bool decide_unit_to_draw(const KParams& p, SH& sh, Ro
                                                     int part, R ready) {
   const int tid = threadIdx.x;
   DrawUnit<NCH>& u = sh.unit;
-  decide_sampled<DT, ENS ? kEnsembleSample : kLogitSample>(
+  decide_sampled<DT, ENS ? kEnsembleSample : kLogitSample, 4>(
       p, rs, t, in, b, want, ready,
       [&](const PairStats* f, int j, int pi, unsigned word, int accepted, int drawable) {
         const int pis = (pi >= 0 && pi < p.n) ? pi : 0;

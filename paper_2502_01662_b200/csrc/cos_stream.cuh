@@ -788,17 +788,20 @@ __device__ __forceinline__ RecordRange records_of(const KParams& p, int b, int j
 
 // Merge slot i of a position over its records; `g` lanes (a power of two, aligned) share the work, `sub` is the lane's place
 // among them.  Every lane of the warp calls this (one with an empty range only takes part in the exchanges).  All lanes of a
-// group get the sums, the first one of them argmaxes.  Four records or eight at a time are on their way, and every sum is rescaled once, to the
-// reference of the whole group: one record after another took 10 us for the 148 of each position of a 6-position row.
+// group get the sums, the first one of them argmaxes.  `AT` records at a time are on their way, and every sum is rescaled once, to the
+// reference of the whole group: one record after another took 10 us for the 148 of each position of a 6-position row.  Sums four at a time
+// where a block of 512 threads leaves a pair more lanes than that many trips need, otherwise eight (in the deciding launch, whose groups are of a
+// few lanes, one row of 5 x 8 x 128256 fp32 takes 58.3 us with four and 53.8 with eight, of 5 x 5 x 128256 50.4 and 49.0); argmaxes are
+// compared one after the other, so that fewer trips count for more.
 struct Merged {
   SoftPart soft;
   ArgPart arg;
   float thr;
 };
-template <int MODE>
+template <int MODE, int AT>
 __device__ __forceinline__ Merged merge_slot(const KParams& p, const RecordRange& q, int i, int g, int sub) {
   constexpr bool kSample = (MODE == kEnsembleSample || MODE == kLogitSample);
-  constexpr int kAtOnce = kSample ? 4 : 8;  // (argmaxes are compared one after the other, so that fewer trips count for more)
+  constexpr int kAtOnce = AT;
   const int slots = record_slots<MODE>(p);
   Merged m;
   m.soft.ref = -INFINITY;
@@ -1069,7 +1072,7 @@ __device__ __forceinline__ void decide_and_publish(const KParams& p, Finish& fin
   if (kSample && i < slots && lane % g == 0) d = draft_logit<DT, MODE>(p, base, i, pis, at);  // (asked for before the records are)
   const float thr = masked ? mask_bound(p, __ldcg(&p.mask_key[uidx])) : -INFINITY;
   if (i >= slots) q.count = 0;
-  const Merged m = merge_slot<MODE>(p, q, i, g, lane % g);
+  const Merged m = merge_slot<MODE, 8>(p, q, i, g, lane % g);
   if (i < slots && lane % g == 0) {
     if (kSample) {
       fin.fsoft[i] = m.soft;
