@@ -418,12 +418,13 @@ __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst&
   constexpr int NR = ENS ? NCH : 2;         // vectors of a step kept in registers
   constexpr int US = (NR == 2) ? 2 : 1;     // steps fetched at a time
   // Slow vectors are finished where they are, which is the shorter chain, or behind the (up to 32) steps that have them, fetched again, where
-  // the call in the loop costs registers.  Where they are and behind, device time in us: two models, 64 rows of 9 x 151936 80.7 and 81.6, one
-  // row 16.1 and 16.8; three, 16 rows of 6 x 50001 unaligned 32.2 and 33.0; four, 32 rows of 7 x 128256 65.2 and 62.5; logit level, 200 rows of
-  // 5 x 2 x 128256 138.5 and 136.8, 48 of 3 x 128256 with a mask 94.7 and 88.0.  Eight channels entry by entry over the warp (`kShared`), with nothing live across
-  // the call: by the lane that left a vector out the kernel spilled 400 bytes a thread around it, and five models took, by the lane and over
-  // the warp, 7 rows of 5 x 32000 47.1 and 37.5, 40 of 50001 120.4 and 106.5, the same in fp32 165.9 and 145.5, 60 of 64000 99.8 and 102.1.
-  constexpr bool kShared = ENS && NCH == 8, kLater = kShared || !ENS || (NCH == 4 && AL);
+  // the call in the loop costs registers: by the lane that left them out (`kLater`) or entry by entry over the warp (`kShared`), with nothing live
+  // across the call.  Device time in us, where they are / behind, by the lane / over the warp: two models, 16-bit, 60 rows of 5 x 64000 36.9 / 36.7 /
+  // 37.4, at temperature 0.7 35.9 / 36.4 / 36.6, 7 rows of 32000 14.9 / 15.1 / 15.2; fp32 46.9 / 44.3 / 44.9; three, 60 rows aligned 57.7 / 52.8 / 54.1,
+  // fp32 70.7 / 67.5 / 70.4; four, 66.7 / 61.6 / 63.1; 40 rows of 50001 unaligned of three 54.1 / 52.9 / 51.7 (fp32 72.2 / 71.1 / 70.8), of four 66.3 / 63.8 /
+  // 62.6 (fp32 89.4 / 88.6 / 89.7); logit level, 60 rows of two 37.0 / 35.4 / 38.0, of three with a mask 71.9 / 66.0 / 66.4.  Eight channels (five
+  // models) by the lane and over the warp: 7 rows of 32000 47.1 / 37.5, 40 of 50001 120.4 / 106.5, fp32 165.9 / 145.5; 60 of 64000 99.8 / 102.1.
+  constexpr bool kShared = ENS && (NCH == 8 || (NCH == 4 && !AL)), kLater = kShared || !ENS || NCH == 4 || DT == COS_DTYPE_F32;
   const int lane = threadIdx.x & 31;
   const f32x2 c2 = pack2(p.cT, p.cT);
   const VecRange whole = whole_vectors<DT, AL>(p.V);
