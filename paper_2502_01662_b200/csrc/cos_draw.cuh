@@ -406,8 +406,8 @@ __device__ __noinline__ void slow_entries(const DrawConst& p, const DrawUnit<NCH
 // The steps [s_lo, s_hi) of a position by one warp, in chunks of cs steps: per channel the sum over the tokens with a positive mass,
 // for every chunk NCH sums to the records from the rec-th on, and to part the normaliser's share, of all chunks together (both in the cluster's first block).
 // The fast loop adds vectors up in fp32, up to 32 of a lane, and leaves those with a big entry, and the ragged ends, to slow_vector.
-// What bounds it: instruction issue (counted at logit level, 128 rows of 256000 tokens: 211 instructions a step, 0.53 of the issue
-// slots of the average multiprocessor, 0.67 of the busiest).  Loads in flight do not: fetching a step as soon as a place is free,
+// What bounds it: instruction issue (counted at logit level, 128 rows of 256000 tokens: 220 instructions a step, 0.55 of the issue
+// slots of the average multiprocessor, 0.70 of the busiest).  Loads in flight do not: fetching a step as soon as a place is free,
 // so that two are always on their way, gained nothing with two channels and lost 2 to 7 % with four.
 template <int DT, bool ENS, int NCH, bool AL, int FORM>
 __device__ __forceinline__ void draw_sweep_as(const KParams& p, const DrawConst& kc, const DrawUnit<NCH>& u, int cs, int s_lo, int s_hi, double* acc,
